@@ -90,6 +90,50 @@ def _requests(case):
     return [int(x) for x in lens], [int(x) for x in ks]
 
 
+# --------------------------------------------------------------------------- inputs, from a generator alone
+def _weights(s, gen):
+    """Per layer a dict of matrices, the embedding table and the output matrix."""
+    def matrix(n, k):
+        return torch.empty((n, k), dtype=torch.bfloat16, device="cuda").normal_(0.0, STD, generator=gen)
+
+    sizes = dict(wq=(s.q_dim, s.d_model), wk=(s.kv_dim, s.d_model), wv=(s.kv_dim, s.d_model), wo=(s.d_model, s.q_dim),
+                 wg=(s.d_ffn, s.d_model), wu=(s.d_ffn, s.d_model), wd=(s.d_model, s.d_ffn))
+    return [{n: matrix(*d) for n, d in sizes.items()} for _ in range(s.n_layers)], matrix(s.vocab, s.d_model), matrix(s.vocab, s.d_model)
+
+
+def _prefix_block(s, gen, lens):
+    """Cached prefixes: random K and V rows (std 0.02 sqrt(d), what a prefill of these weights leaves behind).  One block
+    of rows serves all: a request and layer take it from a row of their own, _prefix_row."""
+    rows = max(lens) + s.n_layers + 8 * len(lens)
+    return torch.empty((2, rows, s.kv_dim), dtype=torch.bfloat16, device="cuda").normal_(0.0, STD * math.sqrt(s.d_model), generator=gen)
+
+
+def _prefix_row(layer, i):
+    return layer + 8 * i
+
+
+def _round(case, s, ks, gen):
+    """Tokens (pending and drafts) and uniforms of all rows; the edge model's distributions, as peaked as the target's,
+    and the drafts drawn from them."""
+    rows = sum(ks) + len(ks)
+    tokens = torch.randint(s.vocab, (rows,), dtype=torch.int32, device="cuda", generator=gen).cpu()
+    u = (torch.randint(1 << 24, (rows,), device="cuda", generator=gen).float() * 2.0 ** -24).cpu()
+    q = None
+    if case["mode"] != "greedy":
+        q = torch.empty((sum(ks), s.vocab), device="cuda").normal_(0.0, FINAL_GAIN * STD * math.sqrt(s.d_model), generator=gen)
+        q = torch.softmax(q, 1)
+        drafts = torch.multinomial(q, 1, generator=gen)[:, 0].to(torch.int32).cpu()
+        row = qrow = 0
+        for k in ks:
+            tokens[row + 1:row + 1 + k] = drafts[qrow:qrow + k]
+            row, qrow = row + k + 1, qrow + k
+    return tokens, u, q
+
+
+def _prompt(case, s, gen):
+    return torch.randint(s.vocab, (case["n"],), dtype=torch.int32, device="cuda", generator=gen).cpu()
+
+
 # --------------------------------------------------------------------------- the server's side: model and caches
 class Model:
     """A target model behind a context of the library, with random weights made on the GPU."""
@@ -105,23 +149,14 @@ class Model:
         self.weights = torch.empty(size.weights_bytes, dtype=torch.uint8, device=dev)
         self.kv = torch.zeros(size.kv_bytes // 2, dtype=torch.bfloat16, device=dev)
         self.workspace = torch.zeros(size.workspace_bytes, dtype=torch.uint8, device=dev)
-        keep = []
-
-        def matrix(n, k):
-            keep.append(torch.empty((n, k), dtype=torch.bfloat16, device=dev).normal_(0.0, STD, generator=gen))
-            return keep[-1].data_ptr()
-
-        def gain(v):
-            keep.append(torch.full((s.d_model,), v, device=dev))
-            return keep[-1].data_ptr()
-
+        mats, emb, head = _weights(s, gen)
+        one, final = (torch.full((s.d_model,), v, device=dev) for v in (1.0, FINAL_GAIN))
         layers = (binding.LayerWeights * s.n_layers)()
-        for l in layers:
-            l.wq, l.wk, l.wv = matrix(s.q_dim, s.d_model), matrix(s.kv_dim, s.d_model), matrix(s.kv_dim, s.d_model)
-            l.wo = matrix(s.d_model, s.q_dim)
-            l.wg, l.wu, l.wd = matrix(s.d_ffn, s.d_model), matrix(s.d_ffn, s.d_model), matrix(s.d_model, s.d_ffn)
-            l.attn_norm, l.ffn_norm = gain(1.0), gain(1.0)
-        w = binding.Weights(matrix(s.vocab, s.d_model), matrix(s.vocab, s.d_model), gain(FINAL_GAIN), layers)
+        for l, m in zip(layers, mats):
+            for name, t in m.items():
+                setattr(l, name, t.data_ptr())
+            l.attn_norm = l.ffn_norm = one.data_ptr()
+        w = binding.Weights(emb.data_ptr(), head.data_ptr(), final.data_ptr(), layers)
         mem = binding.Mem(self.weights.data_ptr(), size.weights_bytes, self.kv.data_ptr(), size.kv_bytes,
                           self.workspace.data_ptr(), size.workspace_bytes)
         stream = ctypes.c_void_p(torch.cuda.current_stream(dev).cuda_stream)
@@ -144,14 +179,11 @@ class Model:
 
 
 def _write_prefix(model, shape, gen, reqs, lens):
-    """Cached prefixes: random K and V rows (std 0.02 sqrt(d), what a prefill of these weights leaves behind).  One block
-    of rows serves all: a request and layer take it from a row of their own."""
-    rows = max(lens) + shape.n_layers + 8 * len(reqs)
-    block = torch.empty((2, rows, shape.kv_dim), dtype=torch.bfloat16, pin_memory=True)
-    block.copy_(torch.empty(block.shape, dtype=torch.bfloat16, device="cuda").normal_(0.0, STD * math.sqrt(shape.d_model), generator=gen))
+    block = _prefix_block(shape, gen, lens)
+    block = torch.empty(block.shape, dtype=torch.bfloat16, pin_memory=True).copy_(block)
     for i, (req, P) in enumerate(zip(reqs, lens)):
         for layer in range(shape.n_layers):
-            at = layer + 8 * i
+            at = _prefix_row(layer, i)
             model.check(model.lib.pipesd_debug_write_kv(model.handle, req, layer, 0, P, block[0, at].data_ptr(), block[1, at].data_ptr()))
 
 
@@ -159,25 +191,15 @@ class Round:
     """The items of one pipesd_verify call and the arrays they point into."""
 
     def __init__(self, case, shape, reqs, ks, gen):
-        greedy, n, V = case["mode"] == "greedy", len(reqs), shape.vocab
+        greedy, n = case["mode"] == "greedy", len(reqs)
         self.items, self.results = (binding.VerifyItem * n)(), (binding.VerifyResult * n)()
         self.flags = 0
-        rows = sum(ks) + n
-        self.tokens = torch.randint(V, (rows,), dtype=torch.int32, device="cuda", generator=gen).cpu()
-        self.u = (torch.randint(1 << 24, (rows,), device="cuda", generator=gen).float() * 2.0 ** -24).cpu()
-        self.q = None
-        if not greedy:
-            # the edge model's distributions, as peaked as the target's; the drafts are drawn from them
-            self.q = torch.empty((sum(ks), V), device="cuda").normal_(0.0, FINAL_GAIN * STD * math.sqrt(shape.d_model), generator=gen)
-            self.q = torch.softmax(self.q, 1)
-            drafts = torch.multinomial(self.q, 1, generator=gen)[:, 0].to(torch.int32).cpu()
-            if case["q"] == "host":
-                self.flags |= binding.Q_HOST
-                self.q = torch.empty(self.q.shape, pin_memory=True).copy_(self.q)
+        self.tokens, self.u, self.q = _round(case, shape, ks, gen)
+        if not greedy and case["q"] == "host":
+            self.flags |= binding.Q_HOST
+            self.q = torch.empty(self.q.shape, pin_memory=True).copy_(self.q)
         row = qrow = 0
         for i, (req, k) in enumerate(zip(reqs, ks)):
-            if not greedy:
-                self.tokens[row + 1:row + 1 + k] = drafts[qrow:qrow + k]
             self.items[i] = binding.VerifyItem(req, k, binding.MODE_GREEDY if greedy else binding.MODE_STOCHASTIC, 0,
                                                self.tokens[row:].data_ptr(), None if greedy else self.q[qrow:].data_ptr(),
                                                self.u[row:].data_ptr())
@@ -200,7 +222,7 @@ def prepare(case, seed):
         n = case["n"]
         st.model = Model(shape, gen, (n + PAGE - 1) // PAGE, 1, case["max_rows"], n)
         st.req, st.n = st.model.open(), n
-        st.prompt = torch.randint(shape.vocab, (n,), dtype=torch.int32, device="cuda", generator=gen).cpu()
+        st.prompt = _prompt(case, shape, gen)
         st.logits = torch.zeros(shape.vocab, pin_memory=True)
         return st
     lens, ks = _requests(case)
@@ -262,6 +284,86 @@ def work(case):
         bytes_ += 2 * (s.n_layers * per_layer + head) + 2 * rows * s.d_model + kv_row * (cached + rows) + 4 * rows * s.vocab + q
         flops += 2 * rows * (s.n_layers * per_layer + head) + 4 * s.n_layers * s.q_dim * pairs
     return {"bytes": bytes_, "flops": flops}
+
+
+class _Plain:
+    """The model in 64-bit torch.  K and V are rounded to bf16 where they are cached: that is what the cache holds."""
+
+    def __init__(self, shape, gen):
+        self.s = shape
+        self.layers, self.emb, self.head = _weights(shape, gen)
+        self.cache = []                    # per request, per layer: [K, V], each [positions, kv heads, head_dim]
+
+    def norm(self, x):
+        return x * torch.rsqrt((x * x).mean(1, keepdim=True) + self.s.rms_eps)
+
+    def forward(self, chunks):
+        """The requests' next tokens (None: none); returns the rows after the last layer, final norm included."""
+        s, hd, half, group = self.s, self.s.head_dim, self.s.head_dim // 2, self.s.n_q_heads // self.s.n_kv_heads
+        sizes = [len(c) for c in chunks]
+        starts = [self.cache[i][0][0].shape[0] for i in range(len(chunks))]
+        pos = torch.cat([torch.arange(p, p + n, device="cuda", dtype=torch.float64) for p, n in zip(starts, sizes)])
+        angle = pos[:, None, None] * float(s.rope_base) ** (-torch.arange(half, device="cuda", dtype=torch.float64) * 2 / hd)
+        c, z = angle.cos(), angle.sin()
+
+        def turn(v):
+            a, b = v[..., :half], v[..., half:]
+            return torch.cat([a * c - b * z, b * c + a * z], -1)
+
+        x = self.emb[torch.cat(chunks).long().cuda()].double()
+        for l, m in enumerate(self.layers):
+            h = self.norm(x)
+            q, k, v = ((h @ m[n].double().T).view(len(x), -1, hd) for n in ("wq", "wk", "wv"))
+            q, k, v = turn(q), turn(k).bfloat16().double(), v.bfloat16().double()
+            out, at = [], 0
+            for i, (p, n) in enumerate(zip(starts, sizes)):
+                kv = self.cache[i][l] = [torch.cat([old, new[at:at + n]]) for old, new in zip(self.cache[i][l], (k, v))]
+                kk, vv = (t.repeat_interleave(group, 1).transpose(0, 1) for t in kv)
+                score = q[at:at + n].transpose(0, 1) @ kk.transpose(1, 2) / math.sqrt(hd)
+                later = torch.arange(p + n, device="cuda")[None, :] > torch.arange(p, p + n, device="cuda")[:, None]
+                out.append((score.masked_fill_(later, -math.inf).softmax(2) @ vv).transpose(0, 1).reshape(n, -1))
+                del kk, vv, score
+                at += n
+            x = x + torch.cat(out) @ m["wo"].double().T
+            h = self.norm(x)
+            x = x + (torch.nn.functional.silu(h @ m["wg"].double().T) * (h @ m["wu"].double().T)) @ m["wd"].double().T
+        return self.norm(x) * FINAL_GAIN
+
+    def logits(self, rows):
+        return torch.cat([rows @ w.double().T for w in self.head.split(16384)], 1)
+
+    def pool(self, n_pages):
+        """The first request's cache as the library lays it out (include/pipesd.h, pages handed out in order)."""
+        s, out = self.s, torch.zeros((self.s.n_layers, n_pages, 2, self.s.n_kv_heads, PAGE // 8, self.s.head_dim // 8, 8, 8), dtype=torch.float64)
+        for l, kv in enumerate(self.cache[0]):
+            for j, t in enumerate(kv):
+                t = torch.nn.functional.pad(t, (0, 0, 0, 0, 0, n_pages * PAGE - t.shape[0]))
+                out[l, :, j] = t.view(n_pages, PAGE // 8, 8, s.n_kv_heads, s.head_dim // 8, 8).permute(0, 3, 1, 4, 2, 5).cpu()
+        return out.view(-1)
+
+
+def exact(case, seed):
+    """`run` in 64 bits: logits, and the cache of a single request.  Decisions (whole numbers) are left out."""
+    s = synth.SHAPES[case["shape"]]
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    m = _Plain(s, gen)
+    empty = torch.zeros((0, s.n_kv_heads, s.head_dim), dtype=torch.float64, device="cuda")
+    if case["op"] == "prefill":
+        m.cache = [[[empty, empty] for _ in range(s.n_layers)]]
+        rows = m.forward([_prompt(case, s, gen)])
+        return {"logits": m.logits(rows[-1:])[0].cpu(), "kv": m.pool((case["n"] + PAGE - 1) // PAGE)}
+    lens, ks = _requests(case)
+    block = _prefix_block(s, gen, lens)
+    for i, P in enumerate(lens):
+        m.cache.append([[block[j, _prefix_row(l, i):_prefix_row(l, i) + P].double().view(P, s.n_kv_heads, s.head_dim) for j in (0, 1)]
+                        for l in range(s.n_layers)])
+    turns = 2 if case["commit"] == "device" else 1
+    for tokens in [_round(case, s, ks, gen)[0] for _ in range(turns)]:
+        rows = m.forward(list(tokens.split([k + 1 for k in ks])))
+    out = {"results": [None] * turns, "logits": m.logits(rows).cpu()}
+    if len(ks) == 1:
+        out["kv"] = m.pool((lens[0] + 2 * (max(ks) + 1)) // PAGE + 1)
+    return out
 
 
 def tolerance(case):
