@@ -165,7 +165,7 @@ int32_t pipesd_req_len(pipesd_ctx *ctx, int32_t req, int32_t *len);
 
 /* Append n prompt tokens (host ids) to the request's cache -- the accepted prefix that every NAV pass runs against
  * (Sec. 2.2: the drafts are checked against the prefix accepted so far): the same layer stack as verify, run in chunks of
- * at most min(max_rows, 32) rows, no acceptance step.  If last_logits (host, vocab floats) is non-null it
+ * up to max(max_rows, min(max_seq, 1024)) rows, no acceptance step.  If last_logits (host, vocab floats) is non-null it
  * receives the logits of the final position; the call then synchronises. */
 int32_t pipesd_prefill(pipesd_ctx *ctx, int32_t req, const int32_t *tokens, int32_t n, float *last_logits);
 

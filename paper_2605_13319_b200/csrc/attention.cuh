@@ -110,7 +110,7 @@ static inline int attn_rows_n(int rows_per_kv_head) {    // N of a CTA that hold
 // number of 128-key tiles.  The plan fixes the order a row's keys are summed in: a function of the pass's composition
 // and the device, the same every time that composition is verified.
 struct AttnSplit { int splits, keys_per_split, short_tail; };
-static inline AttnSplit attn_split_plan(int total_keys, int page_size, int units, const int* slots) {
+static inline AttnSplit attn_split_plan(int total_keys, int page_size, int units, const int* slots, int max_splits = kAttnMaxSplits) {
     auto chunk_of = [&](int s) {
         const int ch = (total_keys + s - 1) / s;
         return (ch + page_size - 1) / page_size * page_size;
@@ -120,7 +120,7 @@ static inline AttnSplit attn_split_plan(int total_keys, int page_size, int units
     AttnSplit p = {1, chunk_of(1), 0};
     for (int cls = 1; cls >= 0; --cls) {
         int s = slots[cls] / (units > 0 ? units : 1);
-        s = s > kAttnMaxSplits ? kAttnMaxSplits : s;
+        s = s > max_splits ? max_splits : s;
         s = s > by_keys ? by_keys : s;
         s = s < 1 ? 1 : s;
         const int t = tiles_of(s);
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
     const int sp = blockIdx.x;                                     // key split of this CTA
     if (sp >= nsplit) return;
     const int Hkv = a.Hkv, Hq = a.Hq;
-    const int kvh = blockIdx.y % Hkv, rg = blockIdx.y / Hkv;
+    const int kvh = blockIdx.y % Hkv, rg = a.row_groups - 1 - blockIdx.y / Hkv;   // the latest rows see the most keys: first
     const int G = Hq / Hkv;
     const int R = G * rows;
     const int rho0 = rg * a.rows_cap;
@@ -217,9 +217,12 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
     if (N > a.n_max) return;
     const int NG = N / 8, NB = N / 16;
     const int total = base + rows;
+    // query rows are numbered (chunk row, query head): a group's last row bounds the keys that any of its rows sees, so the
+    // early groups of a prompt chunk stop short of the chunk's own later keys
+    const int seen = min(total, base + (rho0 + n_rows - 1) / G + 1);
     AttnCtx c;
-    c.k0 = min(sp * chunk, total);
-    c.k1 = min(c.k0 + chunk, total);
+    c.k0 = min(sp * chunk, seen);
+    c.k1 = min(c.k0 + chunk, seen);
     c.kbase = a.kv_pool + kv_index(a.layer, a.n_pages, 0, 0, Hkv, kvh, a.page_size, 0, HD, 0);
     c.page_stride = (size_t)2 * Hkv * a.page_size * HD;
     c.v_off = (size_t)Hkv * a.page_size * HD;
@@ -285,7 +288,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             if (tid < SM::kOnes / 4) reinterpret_cast<uint32_t*>(ones)[tid] = 0x3F803F80u;
             for (int n = tid; n < N; n += kAttnWorkers) {
                 const int rho = rho0 + n;
-                hz[n] = n < n_rows ? base + rho % rows : -1;
+                hz[n] = n < n_rows ? base + rho / G : -1;
                 m_ref[n] = -INFINITY;
             }
             pdl_wait();
@@ -300,7 +303,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
                     const int idx = idx0 + u * kAttnWorkers, n = idx / HG, g = idx % HG;
                     x[u][0] = x[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
                     if (idx < N * HG && n < n_rows) {
-                        const int rho = rho0 + n, gq = rho / rows, r = rho % rows;
+                        const int rho = rho0 + n, gq = rho % G, r = rho / G;
                         const float4* qp = reinterpret_cast<const float4*>(a.q + ((size_t)(row0 + r) * Hq + kvh * G + gq) * HD + g * 8);
                         x[u][0] = qp[0];
                         x[u][1] = qp[1];
@@ -523,7 +526,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             // there (its token, its head's first k16 step) is worked out once per row, into the maxima's array
             uint32_t* otab = reinterpret_cast<uint32_t*>(wm);
             if (nsplit == 1 && tid < n_rows) {
-                const int rho = rho0 + tid, gq = rho / rows, r_in = rho % rows;
+                const int rho = rho0 + tid, gq = rho % G, r_in = rho / G;
                 otab[tid] = act_index_row(row0 + r_in, ((kvh * G + gq) * HD) >> 4, KSo, NTo, a.xd_tbs);
             }
             const uint32_t ocol = act_index_col(kt, NTo, a.xd_tbs), olo = act_index_lo(a.xd_tbs);
@@ -613,7 +616,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             }
         }
         if (lane < HD / 4) {
-            const int rho = rho0 + rl, gq = rho / rows, r_in = rho % rows;
+            const int rho = rho0 + rl, gq = rho % G, r_in = rho / G;
             const int col = (kvh * G + gq) * HD + lane * 4;
             const float inv = 1.f / den;
             if (a.xd_tbs > 0) {

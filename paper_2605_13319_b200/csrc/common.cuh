@@ -33,6 +33,22 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint4& a, ui
         : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b0), "r"(b1));
 }
 
+// A fragment of m16n8k16 from a 16x16 bf16 tile stored as four contiguous 8x8 core matrices in the order (rows 0-7, k 0-7),
+// (rows 0-7, k 8-15), (rows 8-15, k 0-7), (rows 8-15, k 8-15); `addr` = the tile's shared address + ldmatrix_a16_lane().
+// The lanes name the matrices in the MMA's register order (second and third exchanged): in storage order the four
+// registers would have to be shuffled before every MMA.
+// (volatile: stays behind the barrier wait that precedes it, and in order with the MMAs -- issue it ahead of them.)
+__device__ __forceinline__ uint32_t ldmatrix_a16_lane(int lane) {
+    return (uint32_t)((lane & 7) * 16 + ((lane >> 3) & 1) * 256 + (lane >> 4) * 128);
+}
+__device__ __forceinline__ uint4 ldmatrix_a16(uint32_t addr) {
+    uint4 a;
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w)
+                 : "r"(addr));
+    return a;
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -91,6 +107,33 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
             else if (now - t0 > 2000000000ull) return false;
         }
     }
+}
+// The same for a barrier that threads of other CTAs of the cluster arrive on, and one such arrival (`bar` = dsmem_addr).
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity) {
+    uint64_t t0 = 0;
+    for (uint32_t it = 0;; ++it) {
+        uint32_t ok;
+        asm volatile(
+            "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+            : "=r"(ok)
+            : "r"(bar), "r"(parity)
+            : "memory");
+        if (ok) return true;
+        if ((it & 1023u) == 1023u) {
+            const uint64_t now = global_ns();
+            if (t0 == 0) t0 = now;
+            else if (now - t0 > 2000000000ull) return false;
+        }
+    }
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// A remote arrival that orders nothing of this thread's own: it passes on a phase that the copy engine completed in this
+// CTA's shared memory (the data are there before that phase turns).  The releasing form above drains the thread's memory
+// operations first, 600 cycles and more, which a thread that reports every ring stage cannot afford.
+__device__ __forceinline__ void mbar_forward_cluster(uint32_t bar) {
+    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 // Contiguous global -> shared copy by the copy engine; completion is counted in bytes on `bar`.
 // Both addresses 16-byte aligned, size a multiple of 16.

@@ -3,11 +3,12 @@
 //
 // The weight matrix is the wide operand: a 16-row x 16-column tile of W is the A fragment of a
 // warp-level m16n8k16 MMA and the (few) token rows are the narrow N dimension.  W is repacked once
-// at context creation into fragment order, 4 KB per (128-row block, k16 step), so that a chunk of
-// consecutive k-steps of a row block is one contiguous run in HBM.
+// at context creation, 4 KB per (128-row block, k16 step), so that a chunk of consecutive k-steps of a
+// row block is one contiguous run in HBM; the order inside is the tcgen05 operand's, which ldmatrix reads
+// just as well, so that this kernel and the dense one share one copy of the weights.
 // One producer lane streams those runs into a shared-memory ring with bulk asynchronous copies
 // (cp.async.bulk + mbarrier transaction counts); four consumer warps, two row tiles each, read their
-// fragments back with conflict-free 16-byte loads and issue the MMAs.  The ring is the kernel's
+// fragments back with ldmatrix (conflict free: 512 contiguous bytes) and issue the MMAs.  The ring is the kernel's
 // memory-level parallelism, and because weights do not depend on the previous kernel it is filled
 // BEFORE the programmatic-dependent-launch wait: the weight stream of kernel n+1 starts while kernel n
 // is still draining.
@@ -119,36 +120,30 @@ struct PackSrc {
     int hd;                 // head width (kQkvRope)
 };
 
-// Repack into MMA A-fragment order: packed[((rb*KS + ks)*8 + tile)*32 + lane] =
-//   { W[r][c], W[r][c+1] | W[r+8][c], W[r+8][c+1] | W[r][c+8], W[r][c+9] | W[r+8][c+8], W[r+8][c+9] }
-// with r = (rb*8 + tile)*16 + lane/4 in packed-row numbering, c = ks*16 + 2*(lane%4); packed rows map to
-// logical rows per `mode`; rows beyond the sources (padding of the last row block) are zero.
+// Repack into the order both projection kernels read.  Per (128-row block rb, k16 step) 4 KB: the K-major, unswizzled
+// operand layout of tcgen05.mma -- 8x8 "core matrices" (8 rows x 16 bytes, contiguous), the two k halves of a row
+// group 128 bytes apart, row groups 256 bytes apart.  A 16-row tile is then 512 contiguous bytes of four core matrices,
+// which one ldmatrix.x4 turns into the A fragment of an m16n8k16 MMA.  Packed rows map to logical rows per `mode` (a
+// rotary pair / a gate-up pair sits in rows i and i + 8 of a 16-row tile); rows beyond the sources are zero.
 __global__ void gemm_pack_kernel(PackSrc src, uint4* __restrict__ packed, int n_rows, int K) {
     const int KS = K / 16;
-    const int n_rt = (n_rows + 127) / 128 * 8;
-    const size_t total = (size_t)n_rt * KS * 32;
-    auto fetch = [&](int pr, int c, uint32_t& lo, uint32_t& hi) {
-        lo = hi = 0u;
-        if (pr >= n_rows) return;
-        int lr, which = 0;
-        if (src.mode == kSwiglu) { which = (pr & 15) < 8 ? 0 : 1; lr = gu_feature(pr); }
-        else {
-            lr = src.mode == kQkvRope ? qkv_logical_row(pr, src.hd) : pr;
-            while (which < 2 && lr >= src.rows[which]) { lr -= src.rows[which]; ++which; }
-        }
-        const uint16_t* w = src.w[which] + (size_t)lr * K + c;
-        lo = pack2(w[0], w[1]);
-        hi = pack2(w[8], w[9]);
-    };
+    const int n_rb = (n_rows + 127) / 128;
+    const size_t total = (size_t)n_rb * 128 * KS * 2;        // 16-byte pieces
     for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int lane = (int)(i & 31);
-        const size_t tile = i >> 5;
-        const int ks = (int)(tile % KS), rt = (int)(tile / KS);
-        const int r = rt * 16 + (lane >> 2), c = ks * 16 + 2 * (lane & 3);
-        uint4 v;
-        fetch(r, c, v.x, v.z);
-        fetch(r + 8, c, v.y, v.w);
-        packed[(((size_t)(rt >> 3) * KS + ks) * 8 + (rt & 7)) * 32 + lane] = v;
+        const int kgq = (int)(i % (2 * KS));                 // k8 group along the row
+        const int pr = (int)(i / (2 * KS));                  // packed row
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (pr < n_rows) {
+            int lr, which = 0;
+            if (src.mode == kSwiglu) { which = (pr & 15) < 8 ? 0 : 1; lr = gu_feature(pr); }
+            else {
+                lr = src.mode == kQkvRope ? qkv_logical_row(pr, src.hd) : pr;
+                while (which < 2 && lr >= src.rows[which]) { lr -= src.rows[which]; ++which; }
+            }
+            v = *reinterpret_cast<const uint4*>(src.w[which] + (size_t)lr * K + 8 * kgq);
+        }
+        const int rb = pr >> 7, r = pr & 127, ks = kgq >> 1, kg = kgq & 1;
+        packed[((size_t)rb * KS + ks) * 256 + ((r >> 3) * 2 + kg) * 8 + (r & 7)] = v;
     }
 }
 
@@ -350,27 +345,32 @@ __global__ void __launch_bounds__(kGemmThreads, kGemmCtasPerSm) gemm_wstream_ker
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[j][nt][e] = 0.f;
 
+        const uint32_t a_off = (uint32_t)(warp * 1024) + ldmatrix_a16_lane(lane);
         int st = 0;
         uint32_t ph = 0;
         for (int c = 0; c < nchunks; ++c) {
             ok = mbar_wait(full0 + 8 * st, ph);
             if (!ok) break;
-            const unsigned char* wst = smem + st * kStageBytes;
-            const unsigned char* bst = wst + kGemmWStage;
+            const uint32_t wst = smem_base + st * kStageBytes;
+            const unsigned char* bst = smem + st * kStageBytes + kGemmWStage;
             int kc = nks - c * kGemmKC;
             kc = kc < kGemmKC ? kc : kGemmKC;
 #pragma unroll
             for (int k = 0; k < kGemmKC; ++k) {
                 if (k < kc) {
-                    const uint4 a0 = *reinterpret_cast<const uint4*>(wst + ((k * 8 + warp * 2) * 32 + lane) * 16);
-                    const uint4 a1 = *reinterpret_cast<const uint4*>(wst + ((k * 8 + warp * 2 + 1) * 32 + lane) * 16);
+                    const uint4 a0 = ldmatrix_a16(wst + k * 4096 + a_off), a1 = ldmatrix_a16(wst + k * 4096 + 512 + a_off);
+                    uint4 b[NT];
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt) b[nt] = *reinterpret_cast<const uint4*>(bst + ((k * NT + nt) * 32 + lane) * 16);
 #pragma unroll
                     for (int nt = 0; nt < NT; ++nt) {
-                        const uint4 b = *reinterpret_cast<const uint4*>(bst + ((k * NT + nt) * 32 + lane) * 16);
-                        mma_bf16_16816(acc[0][nt], a0, b.x, b.y);
-                        mma_bf16_16816(acc[1][nt], a1, b.x, b.y);
-                        mma_bf16_16816(acc[0][nt], a0, b.z, b.w);
-                        mma_bf16_16816(acc[1][nt], a1, b.z, b.w);
+                        mma_bf16_16816(acc[0][nt], a0, b[nt].x, b[nt].y);
+                        mma_bf16_16816(acc[1][nt], a1, b[nt].x, b[nt].y);
+                    }
+#pragma unroll
+                    for (int nt = 0; nt < NT; ++nt) {
+                        mma_bf16_16816(acc[0][nt], a0, b[nt].z, b[nt].w);
+                        mma_bf16_16816(acc[1][nt], a1, b[nt].z, b[nt].w);
                     }
                 }
             }

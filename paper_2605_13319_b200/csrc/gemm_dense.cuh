@@ -1,183 +1,193 @@
-// Dense weight-streaming GEMM for passes of more than 32 rows (a batch of requests, a prefill chunk):
+// Dense weight-streaming GEMM for passes of more than 32 rows (a batch of requests, a prompt chunk):
 // y[M,N] = x[M,K] . W[N,K]^T on the tcgen05 tensor cores, with the same fused epilogues as the small-M kernel.
 //
-// One CTA = one 128-row block of W x one token block of up to 160 tokens x the whole of K: no split-K, so a
-// result element is summed in one fixed order (k ascending; within a k16 step the bf16 hi term, then the lo term)
-// whatever the batch, and every weight byte is read once per token block.  The weight tile is the M = 128 side of
-// the MMA (A operand, K-major, packed at context creation in the operand's own core-matrix order); the tokens are
-// the N side (B operand): activations arrive as split-bf16 hi and lo tiles in operand order ("xd" arrays, written
-// by the producing kernel's epilogue), two MMAs per k16 step into one fp32 accumulator in tensor memory
-// (128 lanes = weight rows, one column per token).
-// Two CTAs share an SM (half of its shared memory and tensor memory each), so that one's epilogue runs under the
-// other's main loop.
-// Warp 0: one lane streams (weights, activations) chunks into a shared-memory ring with bulk copies (weights before
-// the dependent-launch wait).  Warp 1: one lane issues the MMAs; tcgen05.commit frees a ring stage / hands the
-// accumulator over.  Warps 2-5: the input's RMSNorm factors while the ring streams, then the epilogue: tcgen05.ld
-// (thread = weight row, registers = 16 tokens at a time) and the mode's arithmetic.
+// A pair of CTAs (cta_group::2) = 256 rows of W x a block of up to 256 tokens x one K slice.  The weights are the M side of
+// the MMA (128 rows from each CTA's shared memory), the tokens the N side (each CTA holds half of the block): activations
+// arrive as split-bf16 hi and lo tiles in operand order ("xd" arrays, written by the producing kernel's epilogue), two
+// MMAs per k16 step into one fp32 accumulator.
+// What bounds it: the tensor pipe takes N/2 cycles per MMA, but every MMA fetches its operands from shared memory at 128 B
+// per cycle (32 cycles for a CTA's 128 weight rows, N/4 for N tokens), and the copies into the ring need the same
+// bandwidth.  One CTA alone with 128 x 256 tiles would want 344 cycles of shared memory per k16 step against 256 of math,
+// and 20 KB of L2 per step; a pair halves the token side: 224 against 256 cycles, 12 KB.
+// Sums: the tensor pipe truncates each accumulation, so a long K in one accumulator drifts (7b shape, layer 31's K after a
+// 160-token prompt: relative L1 error 3.6e-3 with one accumulator over all of K, 2.6e-3 with the small-M kernel's slices).
+// Every kDenseChunk k16 steps the epilogue warps take the accumulator into registers and add there, rounding to nearest,
+// while the MMAs go on in the other of two accumulators.
+// K slices: where row pairs x token blocks leave SMs idle, S <= 4 pairs form a cluster and share K; the partial tiles cross
+// the cluster through distributed shared memory (into the drained ring), each pair sums and finishes every S-th 16-token
+// column block, slices in order.
+// Warp 0: one lane streams (weights, activations) into the ring (weights before the dependent-launch wait).  Warp 1: one
+// lane of the even CTA issues the MMAs, one of the odd CTA passes "this stage has landed here" on to it; tcgen05.commit
+// frees a stage / hands an accumulator over in both CTAs.  Warp 2: tensor memory.  Warps 4-11: accumulators and epilogue
+// (thread = weight row x half of the tokens).
 #pragma once
+#include <algorithm>
+
 #include "common.cuh"
 #include "gemm.cuh"
 #include "tcgen05.cuh"
 
 namespace pipesd {
 
-constexpr int kDenseThreads = 192;
-constexpr int kDenseEpi = 128;            // threads of warps 2-5
-constexpr int kDenseMaxTok = 160;         // tokens per CTA: columns of the accumulator (a multiple of 16)
-constexpr int kDenseMaxStages = 7;
-constexpr int kDenseTail = 128 + 4 * kDenseMaxTok + 4 * 4 * 16;   // barriers, tensor-memory base | rstd[160] | sums of squares [4 warps][16]
-constexpr int kDenseSmemHalf = (228 * 1024) / 2 - 1024;          // dynamic shared memory of a CTA when two share an SM
-constexpr int kDenseSmemWhole = 227 * 1024;                      // ... when it has the SM to itself
-static_assert(8 * (2 * kDenseMaxStages + 1) + 4 <= 128, "barriers and the tensor-memory slot fill the first 128 bytes of the tail");
-
-// ---- weights in tensor-core operand order --------------------------------------------------------------------
-// Per (128-row block rb, k16 step ks) 4 KB: the K-major, unswizzled operand layout of tcgen05.mma -- 8x8
-// "core matrices" (8 rows x 16 bytes, contiguous), the two k halves of a row group 128 bytes apart, row groups
-// 256 bytes apart.  Packed rows map to logical rows per `mode` exactly as in gemm_pack_kernel (a rotary pair /
-// a gate-up pair sits in rows i and i + 8 of a 16-row tile); rows beyond the sources are zero.
-__global__ void gemm_pack_umma_kernel(PackSrc src, uint4* __restrict__ packed, int n_rows, int K) {
-    const int KS = K / 16;
-    const int n_rb = (n_rows + 127) / 128;
-    const size_t total = (size_t)n_rb * 128 * KS * 2;        // 16-byte pieces
-    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
-        const int kgq = (int)(i % (2 * KS));                 // k8 group along the row
-        const int pr = (int)(i / (2 * KS));                  // packed row
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (pr < n_rows) {
-            int lr, which = 0;
-            if (src.mode == kSwiglu) { which = (pr & 15) < 8 ? 0 : 1; lr = gu_feature(pr); }
-            else {
-                lr = src.mode == kQkvRope ? qkv_logical_row(pr, src.hd) : pr;
-                while (which < 2 && lr >= src.rows[which]) { lr -= src.rows[which]; ++which; }
-            }
-            v = *reinterpret_cast<const uint4*>(src.w[which] + (size_t)lr * K + 8 * kgq);
-        }
-        const int rb = pr >> 7, r = pr & 127, ks = kgq >> 1, kg = kgq & 1;
-        packed[((size_t)rb * KS + ks) * 256 + ((r >> 3) * 2 + kg) * 8 + (r & 7)] = v;
-    }
-}
+constexpr int kDenseThreads = 384;
+constexpr int kDenseMaxHalf = 128;        // tokens per CTA of a pair (half of a token block): a multiple of 16
+constexpr int kDenseMaxSlices = 4;        // K slices: pairs per cluster (8 CTAs, the portable limit)
+constexpr int kDenseMaxStages = 9;
+constexpr int kDenseChunk = 32;           // k16 steps per accumulator
+constexpr int kDenseTail = 256 + 4 * 2 * kDenseMaxHalf + 4 * 2 * 4 * 16;   // barriers, tensor-memory base | rstd | sums of squares [2][4 warps][16]
+constexpr int kDenseSmem = 227 * 1024;    // the CTA has its SM to itself
+static_assert(8 * (2 * kDenseMaxStages + 4) + 4 <= 256, "barriers and the tensor-memory slot fill the first 256 bytes of the tail");
 
 // ---- "xd" activation arrays: the K-major B operand of tcgen05.mma, in global memory ---------------------------
-// Token blocks of TBS tokens (a multiple of 16).  Per (token block, k16 step): the bf16 hi tile then the lo tile,
-// TBS * 32 bytes each, cut into 8x8 core matrices: element (token t, k) of a tile at
-// ((t / 8) * 2 + (k / 8) % 2) * 128 + (t % 8) * 16 + (k % 8) * 2.  A chunk of consecutive k16 steps of a token block
-// is one contiguous run.  (xd_store_one and act_store_one, next to the fragment-order stores, write these.)
-struct XdPlan { int tbs, n_tb; };          // tokens per block, blocks
-// Host: the token blocks of a GEMM with N output rows over M tokens on a device of n_sm SMs.  The tensor cores bound
-// the kernel: an SM's time is about (CTAs it runs) x (a per-step cost that grows with the tokens of a block: fetch of
-// the weight tile + fetch of and product with the token tile), so the plan is the block count that minimises
-// ceil(CTAs / n_sm) x (32 + 3/4 tokens per block) -- few, large blocks unless they leave SMs idle or a last wave nearly
-// empty; the fewest blocks among equals.  A function of (M, N, n_sm) alone: producer and consumer derive the same plan.
-static inline XdPlan dense_plan(int M, int N, int n_sm) {
-    const int RB = (N + 127) / 128;
-    const int lo = (M + kDenseMaxTok - 1) / kDenseMaxTok, hi = (M + 15) / 16;
-    XdPlan best = {kDenseMaxTok, lo < 1 ? 1 : lo};
+// Blocks of `tbs` tokens (a multiple of 16), one per CTA of a pair.  Per (block, k16 step): the bf16 hi tile then the lo
+// tile, tbs * 32 bytes each, cut into 8x8 core matrices: element (token t, k) of a tile at
+// ((t / 8) * 2 + (k / 8) % 2) * 128 + (t % 8) * 16 + (k % 8) * 2.  A chunk of consecutive k16 steps of a block is one
+// contiguous run.  (xd_store_one and act_store_one, next to the fragment-order stores, write these.)
+struct DensePlan {
+    int tbs;      // tokens per CTA; a token block is 2 * tbs
+    int n_tb;     // token blocks
+    int S;        // K slices
+};
+// Host: token blocks and K slices of a GEMM of N output rows and depth K over M tokens.  pairs[S] = pairs of CTAs the device
+// keeps resident at once in clusters of S pairs.  The model, in cycles of 1.9 GHz, is fitted to kernels timed alone (K =
+// 4096 and 11008, cold weights): a k16 step costs 110 + 0.05 per token of the block (issue, hand-over of stages), or the
+// tensor pipe's 1 per token, 1.3 with all SMs at it (the clock drops under the power cap), or the weights' stream from
+// HBM (173 for 4 KB per SM at the copy peak, shared by the token blocks that read the same rows); a wave adds 7600 + 40
+// per token (launch, first stages, epilogue), slices another 1500.  Measured against the model, us: 12288 x 4096, 306
+// tokens in two blocks of 160: 67 (66), three of 128: 61 (58); 4096 x 11008, 48 tokens in three slices: 22.8 (21).
+// A function of its arguments alone: producer and consumer derive the same plan.
+static inline DensePlan dense_plan(int M, int N, int K, const int* pairs) {
+    const int RBP = ((N + 127) / 128 + 1) / 2, KS = K / 16;
+    const int lo = (M + 2 * kDenseMaxHalf - 1) / (2 * kDenseMaxHalf);
+    DensePlan best = {kDenseMaxHalf, lo < 1 ? 1 : lo, 1};
     double best_cost = 1e300;
-    for (int n = lo < 1 ? 1 : lo; n <= hi && n <= lo + 16; ++n) {
-        const int tbs = ((M + n - 1) / n + 15) / 16 * 16;
-        const int n_tb = (M + tbs - 1) / tbs;
-        const double cost = (double)((RB * n_tb + n_sm - 1) / n_sm) * (32.0 + 0.75 * tbs);
-        if (cost < best_cost - 1e-9) { best_cost = cost; best.tbs = tbs; best.n_tb = n_tb; }
+    for (int n = lo < 1 ? 1 : lo; n <= lo + 8; ++n) {
+        const int tbs = ((M + 2 * n - 1) / (2 * n) + 15) / 16 * 16, tok = 2 * tbs;
+        const int n_tb = (M + tok - 1) / tok;
+        if (n_tb != n) continue;
+        for (int S = 1; S <= kDenseMaxSlices && (S == 1 || KS / S >= 16); ++S) {
+            const long units = (long)RBP * n_tb * S;
+            const long waves = (units + pairs[S] - 1) / pairs[S];
+            const double occ = (double)units / (waves * pairs[S]);
+            const double step = std::max({110.0 + 0.05 * tok, tok * (1.0 + 0.3 * occ), 173.0 * occ / n_tb});
+            const double cost = waves * ((KS + S - 1) / S * step + 7600.0 + 40.0 * tok + (S > 1 ? 1500.0 : 0.0));
+            if (cost < best_cost * (1.0 - 1e-9)) { best_cost = cost; best = DensePlan{tbs, n_tb, S}; }
+        }
     }
     return best;
 }
-// Host: the ring of a launch of `ctas` CTAs.  More CTAs than SMs: two per SM, each with half of the shared memory
-// and stages of two k16 steps; otherwise a CTA has its SM to itself and keeps twice the bytes in flight.
+// Host: the ring.  As much of the shared memory as it gets.  A stage costs the issuer some 340 cycles of waiting and
+// committing beside its MMAs, so small steps are taken eight at a time (4096 x 11008, 32 tokens per CTA, us: 94 with two
+// steps a stage, 51.5 with four, 46.7 with eight; 80 tokens: 98, 70.3, 70.7; 64 tokens: 103, 63.1, 65.1).
 struct DenseRing { int kc, stages; size_t smem; };
-static inline DenseRing dense_ring(int tbs, int ctas, int n_sm) {
+static inline DenseRing dense_ring(int tbs) {
     DenseRing r;
-    const bool whole = ctas <= n_sm;
-    r.kc = whole ? 4 : 2;
+    r.kc = tbs <= 48 ? 8 : 4;
     const int stage = r.kc * (4096 + tbs * 64);
-    const int s = ((whole ? kDenseSmemWhole : kDenseSmemHalf) - kDenseTail) / stage;
+    const int s = (kDenseSmem - kDenseTail) / stage;
     r.stages = s > kDenseMaxStages ? kDenseMaxStages : s;
     r.smem = (size_t)r.stages * stage + kDenseTail;
     return r;
 }
-__host__ __device__ constexpr int dense_tmem_cols(int tbs) {
+__host__ __device__ constexpr int dense_tmem_cols(int tbs) {      // two accumulators of 2 * tbs columns
     int c = 32;
-    while (c < tbs) c *= 2;
+    while (c < 4 * tbs) c *= 2;
     return c;
 }
 
 struct DenseArgs {
-    GemmArgs g;         // W = weights in operand order; xf = input xd array; the mode's outputs as for the small-M kernel
+    GemmArgs g;         // W = packed weights; xf = input xd array; S = K slices; the mode's outputs as for the small-M kernel
     int kc;             // k16 steps per ring stage (g.stages stages)
-    int tbs_in;         // token block size of the input array and of this launch
-    int tbs_out;        // token block size of the xd array this launch produces (kResid, kSwiglu)
+    int tbs_in;         // block size of the input array and of this launch
+    int tbs_out;        // block size of the xd array this launch produces (kResid, kSwiglu)
+    int tb0, n_tb;      // first token block of the launch, token blocks
+    int out_row0;       // kPlain: the token whose result is row 0 of the output (earlier tokens are not stored)
 };
 
-// grid (128-row blocks, token blocks), block 192.  The bound of 256 threads x 2 CTAs caps a thread at 128 registers:
-// a CTA's six warps put two on one register partition of the SM (a quarter of the register file), and two CTAs must
-// fit there side by side.
+// grid (2 * S * row pairs * n_tb), clusters of 2 * S: cluster rank = 2 * slice + CTA of the pair.  The token blocks of a
+// row pair are neighbours in the launch order, so that they read its weights from HBM once.
 template <int MODE>
-__global__ void __launch_bounds__(256, 2) gemm_dense_kernel(const DenseArgs da) {
+__global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const DenseArgs da) {
     const GemmArgs& a = da.g;
     extern __shared__ __align__(128) unsigned char smem[];
-    const int TBS = da.tbs_in;
-    const int KC = da.kc;
-    const int w_stage = KC * 4096, b_stage = KC * TBS * 64;
-    const int stage_bytes = w_stage + b_stage;
+    const int TBS = da.tbs_in, NT = 2 * TBS;                           // tokens per CTA / per block
+    const int KC = da.kc, S = a.S;
+    const int w_stage = KC * 4096, stage_bytes = w_stage + KC * TBS * 64;
     const int stages = a.stages;
     unsigned char* tail = smem + stages * stage_bytes;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);                // full[7], empty[7], acc_full
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 8 * (2 * kDenseMaxStages + 1));
-    float* rstd_s = reinterpret_cast<float*>(tail + 128);              // [TBS]
-    float* ssq_s = rstd_s + kDenseMaxTok;                              // [4 warps][16 tokens]
+    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);                // full[9], empty[9], acc_full[2], acc_empty[2]
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 8 * (2 * kDenseMaxStages + 4));
+    float* rstd_s = reinterpret_cast<float*>(tail + 256);              // [NT]
+    float* ssq_s = rstd_s + 2 * kDenseMaxHalf;                         // [2 halves][4 warps][16 tokens]
     const uint32_t smem_base = smem_u32(smem);
-    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kDenseMaxStages, acc_full = full0 + 16 * kDenseMaxStages;
+    const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kDenseMaxStages;
+    const uint32_t acc_full = full0 + 16 * kDenseMaxStages, acc_empty = acc_full + 16;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int rb = blockIdx.x, tb = blockIdx.y;
-    const int KS = a.KS, nchunks = (KS + KC - 1) / KC;
-    const int tok0 = tb * TBS;
+    const uint32_t rank = cluster_ctarank();
+    const int r = (int)(rank & 1), s = (int)(rank >> 1);
+    const int cid = blockIdx.x / (2 * S);
+    const int tb = da.tb0 + cid % da.n_tb, rbp = cid / da.n_tb;
+    const int RB = (a.N + 127) / 128, rb = 2 * rbp + r;                // an odd RB: the last odd CTA computes a copy, stored by nobody
+    const int KS = a.KS;
+    const int ks0 = (int)(((long)KS * s) / S), ks1 = (int)(((long)KS * (s + 1)) / S);
+    const int nks = ks1 - ks0;
+    const int n_chunk = (nks + kDenseChunk - 1) / kDenseChunk;
+    const int tok0 = tb * NT;
     const uint32_t tmem_cols = (uint32_t)dense_tmem_cols(TBS);
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < stages; ++i) {
-            mbar_init(full0 + 8 * i, 1);
+            mbar_init(full0 + 8 * i, r == 0 ? 2 : 1);                  // the copies; in the even CTA also the odd one's report
             mbar_init(empty0 + 8 * i, 1);
         }
-        mbar_init(acc_full, 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(acc_full + 8 * i, 1);
+            mbar_init(acc_empty + 8 * i, 16);                          // one arrival per epilogue warp of the pair
+        }
         fence_mbar_init();
     }
-    if (warp == 1) {
-        tmem_alloc(smem_u32(tmem_slot), tmem_cols);
+    if (warp == 2) {
+        tmem2_alloc(smem_u32(tmem_slot), tmem_cols);
         tc_fence_before();
     }
-    __syncthreads();
+    cluster_sync_all();                                                // barriers of all CTAs are in place
     pdl_launch_dependents();
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
 
+    // ring stages of KC steps, in the order all roles walk them (kDenseChunk is a multiple of KC, so that only the slice's
+    // last stage is shorter)
+    const int n_stage = (nks + KC - 1) / KC;
     bool ok = true;
     if (warp == 0) {
-        // ---------------- producer: lane 0 streams (weights, activations) chunks into the ring
+        // ---------------- producer: lane 0 streams (weights, activations) into the ring
         if (lane == 0) {
-            const unsigned char* wsrc = reinterpret_cast<const unsigned char*>(a.W) + (size_t)rb * KS * 4096;
-            const unsigned char* bsrc = reinterpret_cast<const unsigned char*>(a.xf) + (size_t)tb * KS * (TBS * 64);
-            auto chunk_ks = [&](int c) { int r = KS - c * KC; return r < KC ? r : KC; };
-            const int pre = nchunks < stages ? nchunks : stages;
+            const unsigned char* wsrc = reinterpret_cast<const unsigned char*>(a.W) + ((size_t)min(rb, RB - 1) * KS + ks0) * 4096;
+            const unsigned char* bsrc = reinterpret_cast<const unsigned char*>(a.xf) + ((size_t)(2 * tb + r) * KS + ks0) * (TBS * 64);
+            auto steps = [&](int c) { return min(KC, nks - c * KC); };
             const uint64_t pol = l2_evict_first_policy();
+            auto weights = [&](int c, int st) {
+                const int kc = steps(c);
+                mbar_expect_tx(full0 + 8 * st, (uint32_t)kc * (4096 + TBS * 64));
+                // weights that other token blocks read as well stay in L2 like any line; read once, they leave first
+                if (da.n_tb == 1) bulk_g2s_hint(smem_base + st * stage_bytes, wsrc + (size_t)c * w_stage, (uint32_t)kc * 4096, full0 + 8 * st, pol);
+                else bulk_g2s(smem_base + st * stage_bytes, wsrc + (size_t)c * w_stage, (uint32_t)kc * 4096, full0 + 8 * st);
+            };
+            auto tokens = [&](int c, int st) {
+                bulk_g2s(smem_base + st * stage_bytes + w_stage, bsrc + (size_t)c * (KC * TBS * 64), (uint32_t)steps(c) * (TBS * 64), full0 + 8 * st);
+            };
             // weights do not depend on the previous kernel: start them before the dependency wait
-            for (int c = 0; c < pre; ++c) {
-                const int kc = chunk_ks(c);
-                mbar_expect_tx(full0 + 8 * c, (uint32_t)kc * (4096 + TBS * 64));
-                bulk_g2s_hint(smem_base + c * stage_bytes, wsrc + (size_t)c * w_stage, (uint32_t)kc * 4096, full0 + 8 * c, pol);
-            }
+            const int pre = n_stage < stages ? n_stage : stages;
+            for (int c = 0; c < pre; ++c) weights(c, c);
             pdl_wait();
-            for (int c = 0; c < pre; ++c) {
-                const int kc = chunk_ks(c);
-                bulk_g2s(smem_base + c * stage_bytes + w_stage, bsrc + (size_t)c * b_stage, (uint32_t)kc * TBS * 64, full0 + 8 * c);
-            }
+            for (int c = 0; c < pre; ++c) tokens(c, c);
             int issued = pre, st = 0;
             uint32_t ph = 0;
-            for (int c = pre; c < nchunks; ++c) {
-                const int kc = chunk_ks(c);
+            for (int c = pre; c < n_stage; ++c) {
                 ok = mbar_wait(empty0 + 8 * st, ph);
                 if (!ok) break;
-                mbar_expect_tx(full0 + 8 * st, (uint32_t)kc * (4096 + TBS * 64));
-                bulk_g2s_hint(smem_base + st * stage_bytes, wsrc + (size_t)c * w_stage, (uint32_t)kc * 4096, full0 + 8 * st, pol);
-                bulk_g2s(smem_base + st * stage_bytes + w_stage, bsrc + (size_t)c * b_stage, (uint32_t)kc * TBS * 64, full0 + 8 * st);
+                weights(c, st);
+                tokens(c, st);
                 issued = c + 1;
                 if (++st == stages) { st = 0; ph ^= 1u; }
             }
@@ -188,125 +198,187 @@ __global__ void __launch_bounds__(256, 2) gemm_dense_kernel(const DenseArgs da) 
                     mbar_wait(full0 + 8 * (c % stages), (c / stages) & 1);
             }
         }
-    } else if (warp == 1) {
-        // ---------------- MMA issuer
-        if (lane == 0) {
-            const uint32_t idesc = umma_idesc_bf16(128, TBS, 0, 0);
+        __syncwarp();
+    } else if (warp == 1 && r == 0) {
+        // ---------------- MMA issuer of the pair
+        if (elect_one()) {
+            const uint32_t idesc = umma_idesc_bf16(256, NT, 0, 0);
+            const uint16_t mask = (uint16_t)(3u << rank);              // this CTA and its peer
+            const uint32_t lo_step = (uint32_t)(TBS * 32) >> 4;        // hi tile -> lo tile, in descriptor units
             int st = 0;
             uint32_t ph = 0;
-            for (int c = 0; c < nchunks; ++c) {
-                ok = mbar_wait(full0 + 8 * st, ph);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t wst = smem_base + st * stage_bytes, bst = wst + w_stage;
-                int kc = KS - c * KC;
-                kc = kc < KC ? kc : KC;
-                for (int k = 0; k < kc; ++k) {
-                    const uint64_t ad = umma_desc(wst + k * 4096, 128, 256);
-                    umma_bf16(tmem, ad, umma_desc(bst + (k * 2) * TBS * 32, 128, 256), idesc, (c > 0 || k > 0) ? 1u : 0u);
-                    umma_bf16(tmem, ad, umma_desc(bst + (k * 2 + 1) * TBS * 32, 128, 256), idesc, 1u);
+            for (int ch = 0; ch < n_chunk && ok; ++ch) {
+                if (ch >= 2) ok = mbar_wait_cluster(acc_empty + 8 * (ch & 1), (uint32_t)((ch >> 1) - 1) & 1u);
+                const uint32_t d = tmem + (uint32_t)((ch & 1) * NT);
+                const int k_end = min(nks, (ch + 1) * kDenseChunk);
+                for (int k = ch * kDenseChunk; k < k_end && ok; k += KC) {
+                    ok = mbar_wait(full0 + 8 * st, ph);                // landed in both CTAs
+                    if (!ok) break;
+                    tc_fence_after();
+                    uint64_t ad = umma_desc(smem_base + st * stage_bytes, 128, 256);
+                    uint64_t bd = umma_desc(smem_base + st * stage_bytes + w_stage, 128, 256);
+                    const int kc = min(KC, k_end - k);
+                    uint32_t acc = k > ch * kDenseChunk ? 1u : 0u;
+                    for (int i = 0; i < kc; ++i) {
+                        umma2_bf16(d, ad, bd, idesc, acc);
+                        umma2_bf16(d, ad, bd + lo_step, idesc, 1u);
+                        ad += 4096 >> 4;
+                        bd += 2 * lo_step;
+                        acc = 1u;
+                    }
+                    umma2_commit(empty0 + 8 * st, mask);               // the stage is free in both CTAs when these MMAs have read it
+                    if (++st == stages) { st = 0; ph ^= 1u; }
                 }
-                umma_commit(empty0 + 8 * st);      // the stage is free when these MMAs have read it
+                if (ok) umma2_commit(acc_full + 8 * (ch & 1), mask);
+            }
+            if (!ok && a.err) atomicExch(a.err, 7);
+        }
+        __syncwarp();
+    } else if (warp == 1) {
+        // ---------------- odd CTA: report landed stages to the issuer
+        if (lane == 0) {
+            int st = 0;
+            uint32_t ph = 0;
+            for (int c = 0; c < n_stage && ok; ++c) {
+                ok = mbar_wait(full0 + 8 * st, ph);
+                if (ok) mbar_forward_cluster(dsmem_addr(full0 + 8 * st, rank ^ 1u));
                 if (++st == stages) { st = 0; ph ^= 1u; }
             }
-            if (ok) umma_commit(acc_full);
-            else if (a.err) atomicExch(a.err, 7);
+            if (!ok && a.err) atomicExch(a.err, 8);
         }
+        __syncwarp();
+    }
+    if (warp < 4) {
+        if (S > 1) { cluster_sync_all(); cluster_sync_all(); }
     } else {
-        // ---------------- epilogue warps: thread = weight row (tensor-memory lane 32 * (warp % 4) + lane)
-        const int et = threadIdx.x - 64;                               // 0..127
-        const int quarter = warp & 3;
+        // ---------------- epilogue warps: thread = weight row (tensor-memory lane 32 * (warp % 4) + lane) x one CTA's tokens
+        const int et = threadIdx.x - 128;                              // 0..255
+        const int quarter = warp & 3, half = et >> 7;
         const int row = quarter * 32 + lane;                           // row within the block
         const int pr = rb * 128 + row;                                 // packed row
         const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
         pdl_wait();
         if (a.ssq_in != nullptr) {
-            for (int tl = et; tl < TBS; tl += kDenseEpi) {
+            for (int tl = et; tl < NT; tl += 256) {
                 const int tok = tok0 + tl;
                 float ss = 0.f;
-                if (tok < a.M)
+                if (tok < a.M) {
+#pragma unroll 8
                     for (int b = 0; b < a.n_ssq; ++b) ss += a.ssq_in[(size_t)b * a.M + tok];
+                }
                 rstd_s[tl] = rsqrtf(ss / (float)a.d_in + a.eps);
             }
         }
-        asm volatile("bar.sync 1, %0;" ::"n"(kDenseEpi) : "memory");
+        asm volatile("bar.sync 1, 256;" ::: "memory");
+        // ---- accumulators: chunk by chunk from tensor memory into registers
+        const int ncb = TBS / 16;
+        float acc[kDenseMaxHalf / 16][16];
+#pragma unroll
+        for (int cb = 0; cb < kDenseMaxHalf / 16; ++cb)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) acc[cb][i] = 0.f;
+        const uint32_t lead_empty = dsmem_addr(acc_empty, rank & ~1u);
+        for (int ch = 0; ch < n_chunk; ++ch) {
+            if (ok) ok = mbar_wait(acc_full + 8 * (ch & 1), (uint32_t)(ch >> 1) & 1u);
+            ok = __all_sync(0xffffffffu, ok);
+            tc_fence_after();
+            const uint32_t t = tmem + lane_sel + (uint32_t)((ch & 1) * NT + half * TBS);
+#pragma unroll
+            for (int cb = 0; cb < kDenseMaxHalf / 16; ++cb) {
+                if (cb < ncb) {
+                    float v[16];
+                    tmem_ld16(t + cb * 16, v);
+                    tmem_ld_wait16(v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) acc[cb][i] += v[i];
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(lead_empty + 8 * (ch & 1));
+        }
+        if (!ok && a.err && lane == 0) atomicExch(a.err, 9);
+        __syncwarp();
+
         // per-row constants of the mode
-        float gain = 0.f;
-        if (MODE == kResid && pr < a.N) gain = a.gain_next[pr];
-        const int half_hd = a.hd / 2;
-        int lr = 0, head = 0, dim = 0;
-        if (MODE == kQkvRope) { lr = qkv_logical_row(pr, a.hd); head = lr / a.hd; dim = lr % a.hd; }
-        ok = mbar_wait(acc_full, 0);
-        ok = __all_sync(0xffffffffu, ok);
-        tc_fence_after();
         const bool row_live = pr < a.N;
         const int prc = row_live ? pr : a.N - 1;
+        float gain = 0.f;
+        if (MODE == kResid) gain = a.gain_next[prc];
+        const int half_hd = a.hd / 2;
+        int lr = 0, head = 0, dim = 0;
+        if (MODE == kQkvRope) { lr = qkv_logical_row(prc, a.hd); head = lr / a.hd; dim = lr % a.hd; }
         // the activation output: this thread's column of the consumer's xd array; a 16-token column block of the
         // accumulator lies inside one of its token blocks (block sizes and block starts are multiples of 16)
         const int k_out = MODE == kSwiglu ? gu_feature(prc) : prc;
         const int KS_out = (MODE == kSwiglu ? a.N / 2 : a.N) / 16;
         uint16_t* act_out = MODE == kSwiglu ? a.xf_act : a.xf_out;
         const uint32_t ocol = act_index_col(k_out, 0, da.tbs_out), olo = act_index_lo(da.tbs_out);
-        for (int cb = 0; cb < TBS / 16; ++cb) {
-            float v[16];
-            tmem_ld16(tmem + lane_sel + cb * 16, v);
-            // what the mode reads per element, fetched for the 16 tokens at once (independent loads, clamped addresses)
-            // while the accumulator columns arrive
-            float e0[16], e1[16];
-            long long rk[16];
-            if (MODE == kResid) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) e0[i] = a.x[(size_t)min(tok0 + cb * 16 + i, a.M - 1) * a.N + prc];
-            } else if (MODE == kQkvRope) {
-                const bool rot = head < a.Hq + a.Hkv, cached = head >= a.Hq;
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    const int tokc = min(tok0 + cb * 16 + i, a.M - 1);
-                    e0[i] = rot ? a.cs[(size_t)tokc * half_hd + (dim % half_hd)] : 1.f;
-                    e1[i] = rot ? a.sn[(size_t)tokc * half_hd + (dim % half_hd)] : 0.f;
-                    rk[i] = cached ? a.row_kvoff[tokc] : 0;
-                }
-            }
-            const uint32_t orow = (MODE == kResid || MODE == kSwiglu) ? act_index_row(tok0 + cb * 16, 0, KS_out, 0, da.tbs_out) + ocol : 0u;
-            tmem_ld_wait();
+
+        auto half_sync = [&]() {
+            if (half == 0) asm volatile("bar.sync 2, 128;" ::: "memory");
+            else asm volatile("bar.sync 3, 128;" ::: "memory");
+        };
+        // the mode's arithmetic for 16 tokens (column block b of the token block), run by the 128 threads of a half
+        auto finish = [&](int b, const float (&v)[16]) {
+            const int tokb = tok0 + b * 16;
+            const uint32_t orow = (MODE == kResid || MODE == kSwiglu) ? act_index_row(tokb, 0, KS_out, 0, da.tbs_out) + ocol : 0u;
             float sq[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int tl = cb * 16 + i, tok = tok0 + tl;
-                float x = ok ? v[i] : 0.f;
-                if (a.ssq_in != nullptr) x *= rstd_s[tl];
-                const bool live = tok < a.M && row_live;
-                sq[i] = 0.f;
-                if (MODE == kPlain) {
-                    if (live) a.out[(size_t)tok * a.N + pr] = x;
-                } else if (MODE == kResid) {
-                    float xn = 0.f;
-                    if (live) {
-                        xn = e0[i] + x;
-                        a.x[(size_t)tok * a.N + pr] = xn;
-                        act_store_at(act_out, orow + (uint32_t)((i >> 3) * 128 + (i & 7) * 8), olo, xn * gain);
+            for (int g = 0; g < 2; ++g) {
+                // what the mode reads per element, fetched for eight tokens at once (independent loads, clamped addresses)
+                float e0[8], e1[8];
+                long long rk[8];
+                if (MODE == kResid) {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) e0[i] = a.x[(size_t)min(tokb + g * 8 + i, a.M - 1) * a.N + prc];
+                } else if (MODE == kQkvRope) {
+                    const bool rot = head < a.Hq + a.Hkv, cached = head >= a.Hq;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int tokc = min(tokb + g * 8 + i, a.M - 1);
+                        e0[i] = rot ? a.cs[(size_t)tokc * half_hd + (dim % half_hd)] : 1.f;
+                        e1[i] = rot ? a.sn[(size_t)tokc * half_hd + (dim % half_hd)] : 0.f;
+                        rk[i] = cached ? a.row_kvoff[tokc] : 0;
                     }
-                    sq[i] = xn * xn;
-                } else {
-                    // both remaining modes pair row i (< 8) with row i + 8 of a 16-row tile
-                    const float partner = __shfl_xor_sync(0xffffffffu, x, 8);
-                    if (MODE == kSwiglu) {
-                        if ((row & 15) < 8 && live) {
-                            const float act = x / (1.f + expf(-x)) * partner;      // own = gate, partner = up
-                            act_store_at(act_out, orow + (uint32_t)((i >> 3) * 128 + (i & 7) * 8), olo, act);
+                }
+#pragma unroll
+                for (int i8 = 0; i8 < 8; ++i8) {
+                    const int i = g * 8 + i8, tok = tokb + i;
+                    float x = ok ? v[i] : 0.f;
+                    if (a.ssq_in != nullptr) x *= rstd_s[b * 16 + i];
+                    const bool live = tok < a.M && row_live;
+                    if (MODE == kPlain) {
+                        if (live && tok >= da.out_row0) a.out[(size_t)(tok - da.out_row0) * a.N + pr] = x;
+                    } else if (MODE == kResid) {
+                        float xn = 0.f;
+                        if (live) {
+                            xn = e0[i8] + x;
+                            a.x[(size_t)tok * a.N + pr] = xn;
+                            act_store_at(act_out, orow + (uint32_t)(g * 128 + i8 * 8), olo, xn * gain);
                         }
-                    } else if (live) {                                           // kQkvRope
-                        // q and k heads are rotated (cos = 1, sin = 0 for v heads)
-                        const float val = (row & 15) < 8 ? x * e0[i] - partner * e1[i] : x * e0[i] + partner * e1[i];
-                        if (head < a.Hq) {
-                            a.q_out[((size_t)tok * a.Hq + head) * a.hd + dim] = val;
-                        } else {
-                            const int kv = head < a.Hq + a.Hkv ? 0 : 1;
-                            const int kvh = kv ? head - a.Hq - a.Hkv : head - a.Hq;
-                            const size_t per_head = (size_t)a.page_size * a.hd;
-                            const size_t off = (size_t)a.layer * a.n_pages * 2 * a.Hkv * per_head + (size_t)rk[i] +
-                                               ((size_t)kv * a.Hkv + kvh) * per_head + kv_col_offset(dim);
-                            a.kv_pool[off] = f32_to_bf16_bits(val);
+                        sq[i] = xn * xn;
+                    } else {
+                        // both remaining modes pair row i (< 8) with row i + 8 of a 16-row tile
+                        const float partner = __shfl_xor_sync(0xffffffffu, x, 8);
+                        if (MODE == kSwiglu) {
+                            if ((row & 15) < 8 && live) {
+                                const float act = x / (1.f + expf(-x)) * partner;      // own = gate, partner = up
+                                act_store_at(act_out, orow + (uint32_t)(g * 128 + i8 * 8), olo, act);
+                            }
+                        } else if (live) {                                           // kQkvRope
+                            // q and k heads are rotated (cos = 1, sin = 0 for v heads)
+                            const float val = (row & 15) < 8 ? x * e0[i8] - partner * e1[i8] : x * e0[i8] + partner * e1[i8];
+                            if (head < a.Hq) {
+                                a.q_out[((size_t)tok * a.Hq + head) * a.hd + dim] = val;
+                            } else {
+                                const int kv = head < a.Hq + a.Hkv ? 0 : 1;
+                                const int kvh = kv ? head - a.Hq - a.Hkv : head - a.Hq;
+                                const size_t per_head = (size_t)a.page_size * a.hd;
+                                const size_t off = (size_t)a.layer * a.n_pages * 2 * a.Hkv * per_head + (size_t)rk[i8] +
+                                                   ((size_t)kv * a.Hkv + kvh) * per_head + kv_col_offset(dim);
+                                a.kv_pool[off] = f32_to_bf16_bits(val);
+                            }
                         }
                     }
                 }
@@ -325,22 +397,54 @@ __global__ void __launch_bounds__(256, 2) gemm_dense_kernel(const DenseArgs da) 
                     }
                 }
                 sq[0] += __shfl_xor_sync(0xffffffffu, sq[0], 16);
-                if (lane < 16) ssq_s[quarter * 16 + lane] = sq[0];       // lane l: token l of the column block
-                asm volatile("bar.sync 1, %0;" ::"n"(kDenseEpi) : "memory");
-                if (et < 16) {
-                    const int tl = cb * 16 + et, tok = tok0 + tl;
-                    if (tok < a.M)
-                        a.ssq_out[(size_t)rb * a.M + tok] = ssq_s[et] + ssq_s[16 + et] + ssq_s[32 + et] + ssq_s[48 + et];
-                }
-                asm volatile("bar.sync 1, %0;" ::"n"(kDenseEpi) : "memory");
+                float* hs = ssq_s + half * 64;
+                if (lane < 16) hs[quarter * 16 + lane] = sq[0];          // lane l: token l of the column block
+                half_sync();
+                const int ht = et & 127;
+                if (ht < 16 && tokb + ht < a.M && rb < RB)
+                    a.ssq_out[(size_t)rb * a.M + tokb + ht] = hs[ht] + hs[16 + ht] + hs[32 + ht] + hs[48 + ht];
+                half_sync();
             }
+        };
+
+        // ---- the sums leave the registers for the ring's place (the pair's MMAs are done, its copies consumed), where the
+        // epilogue reads 16 tokens at a time: column block b of the token block belongs to slice b % S of the same CTA of
+        // a pair, which receives it as [b / S][slice][16 tokens][128 rows].  With one slice a thread reads back its own.
+        if (S > 1) cluster_sync_all();                                 // ... in every CTA of the cluster
+        float* own = reinterpret_cast<float*>(smem);
+#pragma unroll
+        for (int cb = 0; cb < kDenseMaxHalf / 16; ++cb) {
+            if (cb < ncb) {
+                const int b = half * ncb + cb;
+                const uint32_t dst = dsmem_addr(smem_base + (uint32_t)(((b / S) * S + s) * 8192 + row * 4), (uint32_t)((b % S) * 2 + r));
+#pragma unroll
+                for (int i = 0; i < 16; ++i) {
+                    if (S > 1) dsmem_st_f32(dst + i * 512, acc[cb][i]);
+                    else own[(b * 16 + i) * 128 + row] = acc[cb][i];
+                }
+            }
+        }
+        if (S > 1) cluster_sync_all();
+        const int j0 = S > 1 ? half : half * ncb, j1 = S > 1 ? (2 * ncb - s + S - 1) / S : (half + 1) * ncb, dj = S > 1 ? 2 : 1;
+#pragma unroll 1
+        for (int j = j0; j < j1; j += dj) {
+            float v[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) v[i] = own[(size_t)(j * S) * 2048 + i * 128 + row];
+#pragma unroll 1
+            for (int q = 1; q < S; ++q) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[i] += own[(size_t)(j * S + q) * 2048 + i * 128 + row];
+            }
+            finish(j * S + s, v);
         }
         tc_fence_before();
     }
-    __syncthreads();
-    if (warp == 1) {
+    __syncwarp();
+    cluster_sync_all();                // nobody arrives on or reads from a CTA that has left
+    if (warp == 2) {
         tc_fence_after();
-        tmem_dealloc(tmem, tmem_cols);
+        tmem2_dealloc(tmem, tmem_cols);
     }
 }
 

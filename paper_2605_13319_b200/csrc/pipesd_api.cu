@@ -39,8 +39,7 @@ struct Request {
 };
 
 struct GemmW {
-    uint4* packed = nullptr;     // MMA-fragment order (small-M kernel)
-    uint4* packed_u = nullptr;   // tensor-core operand order (dense kernel; only when max_rows > 32)
+    uint4* packed = nullptr;     // operand order of both projection kernels (gemm_pack_kernel)
     int N = 0, K = 0;
 };
 
@@ -48,6 +47,11 @@ struct LayerW {
     GemmW qkv, o, gu, dn;
     float *n1 = nullptr, *n2 = nullptr;
 };
+
+// Rows of a prompt chunk.  A chunk streams every weight once per token block, so it pays to be long: at 32 rows a chunk
+// is bound by that stream (7b shape, 2048 tokens: 64 chunks of 4.5 ms, 286 ms), at a thousand by the tensor cores.  What
+// it costs is workspace, about 110 KB per row at the 7b shape.
+constexpr int kPrefillRows = 1024;
 
 // Fixed offsets of the per-call metadata block (same layout in pinned host staging and on device).
 struct MetaLayout {
@@ -77,6 +81,7 @@ MetaLayout meta_layout(int max_rows, int max_items) {
 
 struct Derived {
     int Nqkv, qd, kvd, max_pages, max_items;
+    int row_cap;         // rows of the largest pass: a verify call's, or a prompt chunk's
     size_t part_floats;  // floats in each of the two KV staging arrays
 };
 
@@ -89,11 +94,16 @@ Derived derive(const pipesd_model_cfg& c) {
     // multiple of four entries with one spare group
     d.max_pages = ((c.max_seq + c.page_size - 1) / c.page_size + 3) / 4 * 4 + 4;
     d.max_items = std::min(c.max_requests, c.max_rows);
+    d.row_cap = std::max(c.max_rows, std::min(c.max_seq, kPrefillRows));
     // two staging arrays for pipesd_debug_read_kv / write_kv: 256 positions of K and of V per round
     size_t best = (size_t)256 * d.kvd / 2 + 64;
     d.part_floats = best;
     return d;
 }
+
+// Partial attention results the workspace holds: every row, head and split of a verify pass.  A prompt chunk of more rows
+// takes fewer splits (with one split there are no partials).
+size_t attn_part_slots(const pipesd_model_cfg& c) { return (size_t)c.max_rows * c.n_q_heads * kAttnMaxSplits; }
 
 struct WsLayout {
     size_t x, xf_h, qbuf, xf_attn, xf_act, logits, partA, partB, ssqA, ssqB, o_part, m_part, l_part, tickets, cs, sn, kvoff, stats, results, meta,
@@ -104,21 +114,21 @@ WsLayout ws_layout(const pipesd_model_cfg& c, const Derived& d) {
     WsLayout w;
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes); return r; };
-    const size_t M = c.max_rows;
+    const size_t M = d.row_cap, Mv = c.max_rows;
     w.x = take(4 * M * c.d_model);
-    // split-bf16 activation arrays: 4 bytes per element, token count padded to whole token blocks (of up to 160 tokens
-    // plus rounding in the dense kernel's layout)
-    w.xf_h = take(4 * (M + 176) * c.d_model);
+    // split-bf16 activation arrays: 4 bytes per element, token count padded to whole token blocks of the dense kernel
+    constexpr size_t kPad = 2 * kDenseMaxHalf + 16;
+    w.xf_h = take(4 * (M + kPad) * c.d_model);
     w.qbuf = take(4 * M * d.qd);
-    w.xf_attn = take(4 * (M + 176) * d.qd);
-    w.xf_act = take(4 * (M + 176) * c.d_ffn);
-    w.logits = take(4 * M * c.vocab);
+    w.xf_attn = take(4 * (M + kPad) * d.qd);
+    w.xf_act = take(4 * (M + kPad) * c.d_ffn);
+    w.logits = take(4 * Mv * c.vocab);
     w.partA = take(4 * d.part_floats);
     w.partB = take(4 * d.part_floats);
     const size_t nssq = (c.d_model + 127) / 128;
     w.ssqA = take(4 * nssq * M);
     w.ssqB = take(4 * nssq * M);
-    const size_t slots = M * c.n_q_heads * kAttnMaxSplits;               // one per (row, head, key split)
+    const size_t slots = attn_part_slots(c);                             // one per (row, head, key split)
     w.o_part = take(4 * slots * c.head_dim);
     w.m_part = take(4 * slots);
     w.l_part = take(4 * slots);
@@ -126,11 +136,11 @@ WsLayout ws_layout(const pipesd_model_cfg& c, const Derived& d) {
     w.cs = take(4 * M * (c.head_dim / 2));
     w.sn = take(4 * M * (c.head_dim / 2));
     w.kvoff = take(8 * M);
-    w.stats = take(sizeof(RowStat) * M * kStatSplits);
+    w.stats = take(sizeof(RowStat) * Mv * kStatSplits);
     w.results = take(sizeof(RejectOut) * d.max_items + 16);   // + the device error word, read back with the results
-    w.meta = take(meta_layout(c.max_rows, d.max_items).total);
+    w.meta = take(meta_layout(d.row_cap, d.max_items).total);
     w.block_tab = take(4 * (size_t)c.max_requests * d.max_pages);
-    w.qstage = take(4 * M * c.vocab);
+    w.qstage = take(4 * Mv * c.vocab);
     w.req_state = take(sizeof(ReqState) * (size_t)c.max_requests);
     w.never_flag = take(16);
     w.total = o;
@@ -140,12 +150,11 @@ WsLayout ws_layout(const pipesd_model_cfg& c, const Derived& d) {
 size_t packed_bytes(int N, int K) { return align_up(gemm_packed_bytes(N, K)); }
 
 size_t weights_bytes(const pipesd_model_cfg& c, const Derived& d) {
-    const size_t copies = c.max_rows > 32 ? 2 : 1;      // passes of more than 32 rows read the weights in another order
-    size_t per_layer = copies * (packed_bytes(d.Nqkv, c.d_model) + packed_bytes(c.d_model, d.qd) +
-                                 packed_bytes(2 * c.d_ffn, c.d_model) + packed_bytes(c.d_model, c.d_ffn)) +
+    size_t per_layer = packed_bytes(d.Nqkv, c.d_model) + packed_bytes(c.d_model, d.qd) +
+                       packed_bytes(2 * c.d_ffn, c.d_model) + packed_bytes(c.d_model, c.d_ffn) +
                        2 * align_up(4 * (size_t)c.d_model);
     return (size_t)c.n_layers * per_layer + align_up((size_t)c.vocab * c.d_model * 2) +
-           copies * packed_bytes(c.vocab, c.d_model) + align_up(4 * (size_t)c.d_model);
+           packed_bytes(c.vocab, c.d_model) + align_up(4 * (size_t)c.d_model);
 }
 
 size_t kv_bytes(const pipesd_model_cfg& c) {
@@ -164,7 +173,7 @@ cudaError_t init_attrs_current_device() {
     const void* dense_fns[4] = {(const void*)gemm_dense_kernel<kPlain>, (const void*)gemm_dense_kernel<kQkvRope>,
                                 (const void*)gemm_dense_kernel<kResid>, (const void*)gemm_dense_kernel<kSwiglu>};
     for (const void* fn : dense_fns) {
-        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kDenseSmemWhole)) != cudaSuccess) return e;
+        if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kDenseSmem)) != cudaSuccess) return e;
         if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess) return e;
     }
     e = cudaFuncSetAttribute(attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -227,7 +236,7 @@ struct pipesd_ctx {
     pipesd_model_cfg cfg;
     Derived dv;
     WsLayout ws;
-    MetaLayout ml;
+    MetaLayout ml, ml_long;      // of a pass of up to max_rows rows / of a longer prompt chunk (a small pass uploads a small block)
     cudaStream_t st = nullptr;
     // device
     uint16_t* emb = nullptr;
@@ -257,7 +266,7 @@ struct pipesd_ctx {
     int last_rows = 0;
     int attn_slots[kAttnMaxRows / 16 + 1][2] = {};   // [query rows / 16][cut-down third ring slot]: CTAs of the attention
                                                      // kernel the device keeps resident at once
-    int n_sm = 148;             // SMs of the context's device
+    int dense_pairs[kDenseMaxSlices + 1] = {};   // [K slices]: CTA pairs of the dense kernel the device keeps resident at once
     bool force_dense = false;   // harness switch: the dense kernels also for passes of at most 32 rows
     bool pass_dense = false;    // the pass being enqueued runs on the dense kernels
     // bytes of the O and gate/up weights the attention kernel pulls into L2 once its K/V has landed (measured: all of O
@@ -275,7 +284,7 @@ struct pipesd_ctx {
     template <typename T>
     T* W(size_t off) const { return reinterpret_cast<T*>(wsp + off); }
     int* err_word() const { return reinterpret_cast<int*>(wsp + ws.results + sizeof(RejectOut) * dv.max_items); }
-    PassMeta pass_meta() const {
+    PassMeta pass_meta(const MetaLayout& ml) const {
         PassMeta m;
         const char* b = wsp + ws.meta;
         m.row_item = (const int32_t*)(b + ml.row_item);
@@ -315,12 +324,13 @@ int cuda_fail(pipesd_ctx* c, cudaError_t e, const char* where) {
 
 template <int MODE>
 cudaError_t dense_launch_mode(const DenseArgs& da, dim3 grid, size_t smem, cudaStream_t st) {
-    return launch_pdl(gemm_dense_kernel<MODE>, grid, dim3(kDenseThreads), smem, st, da);
+    return launch_pdl_cluster(gemm_dense_kernel<MODE>, grid, dim3(kDenseThreads), smem, st, 2 * da.g.S, da);
 }
 
-// Launch one weight-streaming GEMM with accounting (and event timing when profiling is on).  next_N: output rows of
-// the GEMM that consumes this one's activation output (0: none): its token-block plan fixes the layout written.
-int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, int next_N) {
+// Launch one weight-streaming GEMM with accounting (and event timing when profiling is on).  next_N, next_K: output rows and
+// depth of the GEMM that consumes this one's activation output (0: none): its token-block plan fixes the layout written.
+// first_row (dense, kPlain): results are wanted from this row on and stored from the start of the output.
+int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, int next_N, int next_K, int first_row = 0) {
     a.err = ctx->err_word();
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ctx->time_gemms) {
@@ -337,18 +347,23 @@ int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, in
         CU(cudaEventRecord(e0, ctx->st));
     }
     if (ctx->pass_dense) {
-        const XdPlan pin = dense_plan(a.M, a.N, ctx->n_sm);
+        const DensePlan pin = dense_plan(a.M, a.N, K, ctx->dense_pairs);
+        const int tb0 = first_row / (2 * pin.tbs);
         DenseArgs da = {};
         da.g = a;
-        da.g.W = w.packed_u;
+        da.g.W = w.packed;
         da.g.KS = K / 16;
-        const dim3 grid((a.N + 127) / 128, pin.n_tb);
-        const DenseRing ring = dense_ring(pin.tbs, (int)(grid.x * grid.y), ctx->n_sm);
+        da.g.S = pin.S;
+        const dim3 grid(2 * pin.S * (((a.N + 127) / 128 + 1) / 2) * (pin.n_tb - tb0));
+        const DenseRing ring = dense_ring(pin.tbs);
         da.g.stages = ring.stages;
         da.kc = ring.kc;
         da.g.pf = L2Prefetch{};
         da.tbs_in = pin.tbs;
-        da.tbs_out = next_N > 0 ? dense_plan(a.M, next_N, ctx->n_sm).tbs : 0;
+        da.tb0 = tb0;
+        da.n_tb = pin.n_tb - tb0;
+        da.out_row0 = first_row;
+        da.tbs_out = next_N > 0 ? dense_plan(a.M, next_N, next_K, ctx->dense_pairs).tbs : 0;
         const size_t smem = ring.smem;
         cudaError_t e;
         switch (mode) {
@@ -421,8 +436,10 @@ void shrink_pages(pipesd_ctx* c, Request& r, int keep_len) {
     }
 }
 
-// Upload the metadata of one pass and run the layer stack over M rows.
-int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, bool want_logits, bool want_reject) {
+// Upload the metadata of one pass and run the layer stack over M rows.  Logits are wanted of the last n_logits rows (of
+// all rows unless the pass is a prompt chunk of more than 32).
+int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, bool want_reject) {
+    const bool want_logits = n_logits > 0;
     const pipesd_model_cfg& c = ctx->cfg;
     const Derived& dv = ctx->dv;
     const int n_items = (int)items.size();
@@ -434,7 +451,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, bool want_logi
     ctx->stage = (ctx->stage + 1) % pipesd_ctx::kStages;
     CU(cudaEventSynchronize(ctx->ev_meta[sidx]));
     char* hm = ctx->h_meta[sidx];
-    const MetaLayout& ml = ctx->ml;
+    const MetaLayout& ml = M <= c.max_rows ? ctx->ml : ctx->ml_long;
     auto I = [&](size_t off) { return reinterpret_cast<int32_t*>(hm + off); };
     float* hu = reinterpret_cast<float*>(hm + ml.u);
     RejectItem* hr = reinterpret_cast<RejectItem*>(hm + ml.rej);
@@ -481,8 +498,11 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, bool want_logi
         const int R_i = it.rows * (c.n_q_heads / c.n_kv_heads);                  // query rows per KV head
         const int rg_i = (R_i + rows_cap - 1) / rows_cap;
         const int units_i = (int)std::min(1.0e9, std::ceil(pass_work / (double)total));
+        // splits whose partial results the workspace can hold beside those of the items before (all 16, in a verify pass)
+        const size_t room = attn_part_slots(c) - std::min<size_t>(part0, attn_part_slots(c));
+        const int max_splits = (int)std::min<size_t>(kAttnMaxSplits, room / ((size_t)it.rows * c.n_q_heads));
         const AttnSplit sp = attn_split_plan(total, c.page_size, std::max(units_i, c.n_kv_heads * rg_i),
-                                             ctx->attn_slots[attn_rows_n(std::min(R_i, rows_cap)) / 16]);
+                                             ctx->attn_slots[attn_rows_n(std::min(R_i, rows_cap)) / 16], max_splits);
         const int nsplit = sp.splits, chunk = sp.keys_per_split;
         if (chunk > kAttnTile + kAttnShortTail) all_short = false;
         I(ml.it_slot)[i] = it.slot;
@@ -516,7 +536,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, bool want_logi
     CU(cudaEventRecord(ctx->ev_meta[sidx], ctx->st));
 
     // ---- layer stack
-    const PassMeta meta = ctx->pass_meta();
+    const PassMeta meta = ctx->pass_meta(ml);
     cudaStream_t st = ctx->st;
     float* x = ctx->W<float>(ctx->ws.x);
     uint32_t* xf_h = ctx->W<uint32_t>(ctx->ws.xf_h);
@@ -533,11 +553,12 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, bool want_logi
     const int hd = c.head_dim, Hq = c.n_q_heads, Hkv = c.n_kv_heads, d = c.d_model, F = c.d_ffn;
     const int n_ssq = (d + 127) / 128;
 
-    // Passes of more than 32 rows run their GEMMs on the dense kernels (every weight byte read once per block of up to 160
+    // Passes of more than 32 rows run their GEMMs on the dense kernels (every weight byte read once per block of up to 256
     // tokens); their activation arrays are in that kernel's operand order, with the token block size of the consumer.
-    ctx->pass_dense = ctx->layers[0].qkv.packed_u != nullptr && (M > 32 || ctx->force_dense);
+    ctx->pass_dense = M > 32 || ctx->force_dense;
     const bool dense = ctx->pass_dense;
-    const int tbs_qkv = dense ? dense_plan(M, dv.Nqkv, ctx->n_sm).tbs : 0, tbs_o = dense ? dense_plan(M, d, ctx->n_sm).tbs : 0;
+    const int tbs_qkv = dense ? dense_plan(M, dv.Nqkv, d, ctx->dense_pairs).tbs : 0,
+              tbs_o = dense ? dense_plan(M, d, dv.qd, ctx->dense_pairs).tbs : 0;
     // Every kernel of the chain is launched with programmatic stream serialisation: it may start while its
     // predecessor drains and blocks in griddepcontrol.wait before touching the predecessor's output.
     {
@@ -589,7 +610,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, bool want_logi
             a.q_out = qbuf; a.kv_pool = ctx->kv_pool; a.cs = cs; a.sn = sn;
             a.row_kvoff = ctx->W<long long>(ctx->ws.kvoff);
             a.Hq = Hq; a.Hkv = Hkv; a.hd = hd; a.layer = l; a.n_pages = c.n_pages; a.page_size = c.page_size;
-            int rc_ = launch_gemm(ctx, kQkvRope, lw.qkv, a, d, 0);
+            int rc_ = launch_gemm(ctx, kQkvRope, lw.qkv, a, d, 0, 0);
             if (rc_) return rc_;
         }
         { int rc_ = launch_attn(l); if (rc_) return rc_; }
@@ -598,7 +619,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, bool want_logi
             a.xf = (const uint4*)xf_attn; a.N = d; a.ssq_in = nullptr;
             a.x = x; a.xf_out = (uint16_t*)xf_h; a.gain_next = lw.n2; a.ssq_out = ssqB;
             a.pf = gemm_prefetch_of(lw.gu.packed, M, 2 * F, d, pf_depth);
-            int rc_ = launch_gemm(ctx, kResid, lw.o, a, dv.qd, 2 * F);
+            int rc_ = launch_gemm(ctx, kResid, lw.o, a, dv.qd, 2 * F, d);
             if (rc_) return rc_;
         }
         {   // act = silu(W_g . norm(x)) * (W_u . norm(x))
@@ -606,7 +627,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, bool want_logi
             a.xf = (const uint4*)xf_h; a.N = 2 * F; a.ssq_in = ssqB;
             a.xf_act = (uint16_t*)xf_act;
             a.pf = gemm_prefetch_of(lw.dn.packed, M, d, F, pf_depth);
-            int rc_ = launch_gemm(ctx, kSwiglu, lw.gu, a, d, d);
+            int rc_ = launch_gemm(ctx, kSwiglu, lw.gu, a, d, d, F);
             if (rc_) return rc_;
         }
         {   // x += W_d . act; xf_h = x * (next layer's attention gain | final gain); ssqA
@@ -617,24 +638,24 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, bool want_logi
             a.ssq_out = ssqA;
             if (l + 1 < c.n_layers) a.pf = gemm_prefetch_of(ctx->layers[l + 1].qkv.packed, M, dv.Nqkv, d, pf_depth);
             else if (want_logits) a.pf = gemm_prefetch_of(ctx->lm.packed, M, c.vocab, d, pf_depth);
-            int rc_ = launch_gemm(ctx, kResid, lw.dn, a, F, l + 1 < c.n_layers ? dv.Nqkv : c.vocab);
+            int rc_ = launch_gemm(ctx, kResid, lw.dn, a, F, l + 1 < c.n_layers ? dv.Nqkv : c.vocab, d);
             if (rc_) return rc_;
         }
     }
     if (want_logits) {
-        ctx->n_launch += 1 + (want_reject ? 1 : 0);   // row_stats, accept_sample
         float* logits = ctx->W<float>(ctx->ws.logits);
         RowStat* stats = ctx->W<RowStat>(ctx->ws.stats);
         {
             GemmArgs a = base;
             a.xf = (const uint4*)xf_h; a.N = c.vocab; a.ssq_in = ssqA; a.out = logits;
-            int rc_ = launch_gemm(ctx, kPlain, ctx->lm, a, d, 0);
+            int rc_ = launch_gemm(ctx, kPlain, ctx->lm, a, d, 0, 0, M - n_logits);
             if (rc_) return rc_;
         }
-        // plain launches from here on: they start after the GEMM has fully completed
-        row_stats_kernel<<<dim3(M, kStatSplits), 256, 0, st>>>(c.vocab, logits, stats);
-        ctx->last_rows = M;
+        ctx->last_rows = n_logits;
         if (want_reject) {
+            ctx->n_launch += 2;
+            // a plain launch: it starts after the GEMM has fully completed
+            row_stats_kernel<<<dim3(M, kStatSplits), 256, 0, st>>>(c.vocab, logits, stats);
             CU(launch_pdl_cluster(accept_sample_kernel, dim3(kSampleCluster, n_items), dim3(kSampleThreads), 0, st,
                                   kSampleCluster, (const float*)logits, c.vocab, (const RowStat*)stats,
                                   reinterpret_cast<const RejectItem*>(ctx->wsp + ctx->ws.meta + ml.rej), meta.row_tok,
@@ -690,6 +711,7 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
     ctx->dv = derive(*cfg);
     ctx->ws = ws_layout(*cfg, ctx->dv);
     ctx->ml = meta_layout(cfg->max_rows, ctx->dv.max_items);
+    ctx->ml_long = meta_layout(ctx->dv.row_cap, ctx->dv.max_items);
     ctx->st = (cudaStream_t)cuda_stream;
     const pipesd_model_cfg& c = ctx->cfg;
     const Derived& dv = ctx->dv;
@@ -712,7 +734,21 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
             cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, c.device) != cudaSuccess ||
             cudaDeviceGetAttribute(&thr_sm, cudaDevAttrMaxThreadsPerMultiProcessor, c.device) != cudaSuccess)
             return bail(PIPESD_E_CUDA);
-        ctx->n_sm = n_sm;
+        for (int S = 1; S <= kDenseMaxSlices; ++S) {
+            cudaLaunchConfig_t lc = {};
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = 2 * S;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            lc.gridDim = dim3(2 * S * n_sm);
+            lc.blockDim = dim3(kDenseThreads);
+            lc.dynamicSmemBytes = kDenseSmem;
+            lc.attrs = at;
+            lc.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, gemm_dense_kernel<kQkvRope>, &lc) != cudaSuccess) return bail(PIPESD_E_CUDA);
+            ctx->dense_pairs[S] = std::max(1, n * S);
+        }
         cudaFuncAttributes fa;
         if (cudaFuncGetAttributes(&fa, c.head_dim == 128 ? (const void*)attn_kernel<128> : (const void*)attn_kernel<64>) != cudaSuccess)
             return bail(PIPESD_E_CUDA);
@@ -733,7 +769,7 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
     ctx->kv_pool = (uint16_t*)mem->kv;
     ctx->wsp = (char*)mem->workspace;
     for (int i = 0; i < pipesd_ctx::kStages; ++i) {
-        if (cudaHostAlloc((void**)&ctx->h_meta[i], ctx->ml.total, cudaHostAllocDefault) != cudaSuccess)
+        if (cudaHostAlloc((void**)&ctx->h_meta[i], ctx->ml_long.total, cudaHostAllocDefault) != cudaSuccess)
             return bail(PIPESD_E_CUDA);
         if (cudaEventCreateWithFlags(&ctx->ev_meta[i], cudaEventDisableTiming) != cudaSuccess)
             return bail(PIPESD_E_CUDA);
@@ -764,10 +800,6 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
         int blocks = (int)std::min<size_t>((total + 255) / 256, 148 * 16);
         g.packed = (uint4*)take(gemm_packed_bytes(N, K));
         gemm_pack_kernel<<<blocks, 256, 0, st>>>(ps, g.packed, N, K);
-        if (c.max_rows > 32) {
-            g.packed_u = (uint4*)take(gemm_packed_bytes(N, K));
-            gemm_pack_umma_kernel<<<blocks, 256, 0, st>>>(ps, g.packed_u, N, K);
-        }
     };
     ctx->emb = (uint16_t*)take((size_t)c.vocab * c.d_model * 2);
     if (cudaMemcpyAsync(ctx->emb, w->tok_emb, (size_t)c.vocab * c.d_model * 2, cudaMemcpyDeviceToDevice, st) !=
@@ -905,13 +937,18 @@ int32_t pipesd_prefill(pipesd_ctx* ctx, int32_t req, const int32_t* tokens, int3
         return fail(ctx, PIPESD_E_OOM_PAGES, "pipesd_prefill");
     int rc = grow_pages(ctx, req, r.len + n);
     if (rc != PIPESD_OK) return rc;
-    const int chunk = std::min(ctx->cfg.max_rows, kMaxItemRows);
+    // Up to 32 tokens are a pass of the small-M kernels; more of them go through the dense kernels in equal chunks of up to
+    // row_cap rows, the last of which leaves logits of its last rows only.
+    const int small = std::min(ctx->cfg.max_rows, kMaxItemRows);
+    const int n_chunks = (n + ctx->dv.row_cap - 1) / ctx->dv.row_cap;
+    const int chunk = n <= kMaxItemRows ? small : (n + n_chunks - 1) / n_chunks;
+    const int n_logits = (n - 1) % small + 1;
     for (int done = 0; done < n; done += chunk) {
         int rows = std::min(chunk, n - done);
         bool last = done + rows == n;
         std::vector<ItemDesc> items(1);
         items[0] = ItemDesc{req, rows, 2, 0, tokens + done, nullptr, nullptr, r.len, kCommitNone, 0};
-        rc = run_pass(ctx, items, last && last_logits, false);
+        rc = run_pass(ctx, items, last && last_logits ? n_logits : 0, false);
         if (rc != PIPESD_OK) return rc;
         r.len += rows;
         r.pending = -1;
@@ -920,7 +957,7 @@ int32_t pipesd_prefill(pipesd_ctx* ctx, int32_t req, const int32_t* tokens, int3
             if (rc != PIPESD_OK) return rc;
         }
         if (last && last_logits) {
-            CU(cudaMemcpyAsync(last_logits, ctx->W<float>(ctx->ws.logits) + (size_t)(rows - 1) * ctx->cfg.vocab,
+            CU(cudaMemcpyAsync(last_logits, ctx->W<float>(ctx->ws.logits) + (size_t)(n_logits - 1) * ctx->cfg.vocab,
                                4 * (size_t)ctx->cfg.vocab, cudaMemcpyDeviceToHost, ctx->st));
             rc = pipesd_ctx_sync(ctx);
             if (rc != PIPESD_OK) return rc;
@@ -992,7 +1029,7 @@ int32_t pipesd_verify(pipesd_ctx* ctx, int32_t n_req, const pipesd_verify_item* 
         items[i] = ItemDesc{it.req, it.k + 1, it.mode, it.k, it.tokens, q, it.u, base, commit, r.pending};
         fl[i] = pipesd_ctx::InflightItem{it.req, it.k, commit};
     }
-    int rc = run_pass(ctx, items, true, true);
+    int rc = run_pass(ctx, items, M, true);
     if (rc != PIPESD_OK) return rc;
     rc = push_inflight(ctx, results, std::move(fl));
     if (rc != PIPESD_OK) return rc;
@@ -1258,7 +1295,7 @@ int32_t pipesd_gemm_run(const void* packed, const float* x, float* y, void* scra
 int32_t pipesd_debug_force_dense(pipesd_ctx* ctx, int32_t on) {
     if (!ctx) return PIPESD_E_INVALID;
     if (on && ctx->cfg.max_rows <= 32)
-        return fail(ctx, PIPESD_E_INVALID, "pipesd_debug_force_dense: the context keeps no weights in the dense kernel's order (max_rows <= 32)");
+        return fail(ctx, PIPESD_E_INVALID, "pipesd_debug_force_dense: the context was made for passes of at most 32 rows");
     ctx->force_dense = on != 0;
     return PIPESD_OK;
 }
