@@ -290,6 +290,18 @@ __device__ __forceinline__ void act_store_at(uint16_t* dst, uint32_t idx, uint32
     dst[idx] = h;
     dst[idx + lo] = l;
 }
+__device__ __forceinline__ uint4 bf16x8(const float* v) {
+    return make_uint4(pack2(f32_to_bf16_bits(v[0]), f32_to_bf16_bits(v[1])), pack2(f32_to_bf16_bits(v[2]), f32_to_bf16_bits(v[3])),
+                      pack2(f32_to_bf16_bits(v[4]), f32_to_bf16_bits(v[5])), pack2(f32_to_bf16_bits(v[6]), f32_to_bf16_bits(v[7])));
+}
+// Eight consecutive k of one token in an xd array: 16 bytes of hi terms and, `lo` elements on, 16 bytes of lo terms.
+__device__ __forceinline__ void act_store_8(uint16_t* dst, uint32_t lo, const float* v) {
+    uint16_t h[8], l[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) split_bf16(v[i], h[i], l[i]);
+    *reinterpret_cast<uint4*>(dst) = make_uint4(pack2(h[0], h[1]), pack2(h[2], h[3]), pack2(h[4], h[5]), pack2(h[6], h[7]));
+    *reinterpret_cast<uint4*>(dst + lo) = make_uint4(pack2(l[0], l[1]), pack2(l[2], l[3]), pack2(l[4], l[5]), pack2(l[6], l[7]));
+}
 // Store one activation in whichever layout its consumer reads: tbs > 0: an xd array with that block size; tbs == 0:
 // the small-M kernel's fragment order with NT token tiles per block.
 __device__ __forceinline__ void act_store_one(uint16_t* dst, int tok, int k, float v, int KS, int NT, int tbs) {

@@ -19,7 +19,7 @@
 // Warp 0: one lane streams (weights, activations) into the ring (weights before the dependent-launch wait).  Warp 1: one
 // lane of the even CTA issues the MMAs, one of the odd CTA passes "this stage has landed here" on to it; tcgen05.commit
 // frees a stage / hands an accumulator over in both CTAs.  Warp 2: tensor memory.  Warps 4-11: accumulators and epilogue
-// (thread = weight row x half of the tokens).
+// (thread = weight row x half of the tokens, then token x weight rows).
 #pragma once
 #include <algorithm>
 
@@ -34,7 +34,8 @@ constexpr int kDenseMaxHalf = 128;        // tokens per CTA of a pair (half of a
 constexpr int kDenseMaxSlices = 4;        // K slices: pairs per cluster (8 CTAs, the portable limit)
 constexpr int kDenseMaxStages = 9;
 constexpr int kDenseChunk = 32;           // k16 steps per accumulator
-constexpr int kDenseTail = 256 + 4 * 2 * kDenseMaxHalf + 4 * 2 * 4 * 16;   // barriers, tensor-memory base | rstd | sums of squares [2][4 warps][16]
+constexpr int kDenseRow = 132;            // floats of a token's 128 results in shared memory: eight tokens on eight bank groups
+constexpr int kDenseTail = 256 + 4 * 2 * kDenseMaxHalf;   // barriers, tensor-memory base | rstd
 constexpr int kDenseSmem = 227 * 1024;    // the CTA has its SM to itself
 static_assert(8 * (2 * kDenseMaxStages + 4) + 4 <= 256, "barriers and the tensor-memory slot fill the first 256 bytes of the tail");
 
@@ -118,7 +119,6 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const Dens
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);                // full[9], empty[9], acc_full[2], acc_empty[2]
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 8 * (2 * kDenseMaxStages + 4));
     float* rstd_s = reinterpret_cast<float*>(tail + 256);              // [NT]
-    float* ssq_s = rstd_s + 2 * kDenseMaxHalf;                         // [2 halves][4 warps][16 tokens]
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kDenseMaxStages;
     const uint32_t acc_full = full0 + 16 * kDenseMaxStages, acc_empty = acc_full + 16;
@@ -255,7 +255,6 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const Dens
         const int et = threadIdx.x - 128;                              // 0..255
         const int quarter = warp & 3, half = et >> 7;
         const int row = quarter * 32 + lane;                           // row within the block
-        const int pr = rb * 128 + row;                                 // packed row
         const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
         pdl_wait();
         if (a.ssq_in != nullptr) {
@@ -300,143 +299,155 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const Dens
         if (!ok && a.err && lane == 0) atomicExch(a.err, 9);
         __syncwarp();
 
-        // per-row constants of the mode
-        const bool row_live = pr < a.N;
-        const int prc = row_live ? pr : a.N - 1;
-        float gain = 0.f;
-        if (MODE == kResid) gain = a.gain_next[prc];
+        // ---- the sums leave the registers for the ring's place (the pair's MMAs are done, its copies consumed), token by
+        // token: column block b (16 tokens) of the token block belongs to slice b % S of the same CTA of a pair, which
+        // receives it as [b / S][slice][16 tokens][128 rows], a token padded to kDenseRow floats
+        float* stage_s = reinterpret_cast<float*>(smem);
+        if (S > 1) {
+            cluster_sync_all();                                        // ... in every CTA of the cluster
+#pragma unroll
+            for (int cb = 0; cb < kDenseMaxHalf / 16; ++cb) {
+                if (cb < ncb) {
+                    const int b = half * ncb + cb;
+                    const uint32_t dst = dsmem_addr(smem_base + (uint32_t)(((((b / S) * S + s) * 16) * kDenseRow + row) * 4), (uint32_t)((b % S) * 2 + r));
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) dsmem_st_f32(dst + i * (kDenseRow * 4), acc[cb][i]);
+                }
+            }
+            cluster_sync_all();
+        } else {
+#pragma unroll
+            for (int cb = 0; cb < kDenseMaxHalf / 16; ++cb) {
+                if (cb < ncb) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) stage_s[((half * ncb + cb) * 16 + i) * kDenseRow + row] = acc[cb][i];
+                }
+            }
+            asm volatile("bar.sync 1, 256;" ::: "memory");
+        }
+
+        // ---- the mode's arithmetic.  A warp takes eight tokens: lane = token (lane % 8) x two 16-row tiles (lane / 8 and
+        // that + 4), so that a thread holds a tile's rotary pairs, gate/up pairs or a whole k16 step of the next GEMM's
+        // input, and everything it loads and stores is in pieces of 16 bytes, eight lanes to a 128-byte line of an xd array.
+        // (Thread = row and two-byte stores instead: 1024 tokens at the 7b shape, us, QKV 260, gate/up 356, O and down 113.)
+        const int tk = lane & 7, tq = lane >> 3;
         const int half_hd = a.hd / 2;
-        int lr = 0, head = 0, dim = 0;
-        if (MODE == kQkvRope) { lr = qkv_logical_row(prc, a.hd); head = lr / a.hd; dim = lr % a.hd; }
-        // the activation output: this thread's column of the consumer's xd array; a 16-token column block of the
-        // accumulator lies inside one of its token blocks (block sizes and block starts are multiples of 16)
-        const int k_out = MODE == kSwiglu ? gu_feature(prc) : prc;
         const int KS_out = (MODE == kSwiglu ? a.N / 2 : a.N) / 16;
         uint16_t* act_out = MODE == kSwiglu ? a.xf_act : a.xf_out;
-        const uint32_t ocol = act_index_col(k_out, 0, da.tbs_out), olo = act_index_lo(da.tbs_out);
-
-        auto half_sync = [&]() {
-            if (half == 0) asm volatile("bar.sync 2, 128;" ::: "memory");
-            else asm volatile("bar.sync 3, 128;" ::: "memory");
-        };
-        // the mode's arithmetic for 16 tokens (column block b of the token block), run by the 128 threads of a half
-        auto finish = [&](int b, const float (&v)[16]) {
-            const int tokb = tok0 + b * 16;
-            const uint32_t orow = (MODE == kResid || MODE == kSwiglu) ? act_index_row(tokb, 0, KS_out, 0, da.tbs_out) + ocol : 0u;
-            float sq[16];
+        const uint32_t olo = act_index_lo(da.tbs_out);
+        const int n_blk = (2 * ncb - s + S - 1) / S;                   // this slice's column blocks
+#pragma unroll 1
+        for (int it = warp - 4; it < 2 * n_blk; it += 8) {
+            const int blk = it >> 1, tl16 = (it & 1) * 8 + tk;
+            const int tl = (blk * S + s) * 16 + tl16, tok = tok0 + tl, tokc = min(tok, a.M - 1);
+            const bool live = tok < a.M;
+            // what the mode reads of global memory, for both tiles, in flight together
+            float4 g0[2][4], g1[2][4];
+            long long rk = 0;
 #pragma unroll
-            for (int g = 0; g < 2; ++g) {
-                // what the mode reads per element, fetched for eight tokens at once (independent loads, clamped addresses)
-                float e0[8], e1[8];
-                long long rk[8];
+            for (int h = 0; h < 2; ++h) {
+                const int pr0 = min(rb * 128 + (tq + 4 * h) * 16, a.N - 16);
                 if (MODE == kResid) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) e0[i] = a.x[(size_t)min(tokb + g * 8 + i, a.M - 1) * a.N + prc];
+                    for (int j = 0; j < 4; ++j) {
+                        g0[h][j] = *reinterpret_cast<const float4*>(a.x + (size_t)tokc * a.N + pr0 + 4 * j);
+                        g1[h][j] = *reinterpret_cast<const float4*>(a.gain_next + pr0 + 4 * j);
+                    }
                 } else if (MODE == kQkvRope) {
-                    const bool rot = head < a.Hq + a.Hkv, cached = head >= a.Hq;
+                    const size_t o = (size_t)tokc * half_hd + (pr0 % a.hd) / 2;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const int tokc = min(tokb + g * 8 + i, a.M - 1);
-                        e0[i] = rot ? a.cs[(size_t)tokc * half_hd + (dim % half_hd)] : 1.f;
-                        e1[i] = rot ? a.sn[(size_t)tokc * half_hd + (dim % half_hd)] : 0.f;
-                        rk[i] = cached ? a.row_kvoff[tokc] : 0;
+                    for (int j = 0; j < 2; ++j) {
+                        g0[h][j] = *reinterpret_cast<const float4*>(a.cs + o + 4 * j);
+                        g1[h][j] = *reinterpret_cast<const float4*>(a.sn + o + 4 * j);
+                    }
+                }
+            }
+            if (MODE == kQkvRope) rk = a.row_kvoff[tokc];
+            const float scale = a.ssq_in != nullptr ? rstd_s[tl] : 1.f;
+            float ss = 0.f;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int tile = tq + 4 * h, pr0 = rb * 128 + tile * 16;
+                const bool on = live && pr0 < a.N;                     // N is a multiple of 16
+                float v[16];
+                const float* sp = stage_s + (size_t)(blk * S * 16 + tl16) * kDenseRow + tile * 16;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) *reinterpret_cast<float4*>(v + 4 * j) = *reinterpret_cast<const float4*>(sp + 4 * j);
+#pragma unroll 1
+                for (int q = 1; q < S; ++q) {                          // slices in order
+                    sp += 16 * kDenseRow;
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float4 p = *reinterpret_cast<const float4*>(sp + 4 * j);
+                        v[4 * j] += p.x; v[4 * j + 1] += p.y; v[4 * j + 2] += p.z; v[4 * j + 3] += p.w;
                     }
                 }
 #pragma unroll
-                for (int i8 = 0; i8 < 8; ++i8) {
-                    const int i = g * 8 + i8, tok = tokb + i;
-                    float x = ok ? v[i] : 0.f;
-                    if (a.ssq_in != nullptr) x *= rstd_s[b * 16 + i];
-                    const bool live = tok < a.M && row_live;
-                    if (MODE == kPlain) {
-                        if (live && tok >= da.out_row0) a.out[(size_t)(tok - da.out_row0) * a.N + pr] = x;
-                    } else if (MODE == kResid) {
-                        float xn = 0.f;
-                        if (live) {
-                            xn = e0[i8] + x;
-                            a.x[(size_t)tok * a.N + pr] = xn;
-                            act_store_at(act_out, orow + (uint32_t)(g * 128 + i8 * 8), olo, xn * gain);
+                for (int i = 0; i < 16; ++i) v[i] = ok ? v[i] * scale : 0.f;
+                if (MODE == kPlain) {
+                    if (on && tok >= da.out_row0) {
+                        float4* op = reinterpret_cast<float4*>(a.out + (size_t)(tok - da.out_row0) * a.N + pr0);
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) op[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+                    }
+                } else if (MODE == kResid) {
+                    if (on) {
+                        float4* xp = reinterpret_cast<float4*>(a.x + (size_t)tok * a.N + pr0);
+                        float y[16];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const float4 n = make_float4(g0[h][j].x + v[4 * j], g0[h][j].y + v[4 * j + 1], g0[h][j].z + v[4 * j + 2], g0[h][j].w + v[4 * j + 3]);
+                            xp[j] = n;
+                            ss += n.x * n.x + n.y * n.y + n.z * n.z + n.w * n.w;
+                            y[4 * j] = n.x * g1[h][j].x; y[4 * j + 1] = n.y * g1[h][j].y; y[4 * j + 2] = n.z * g1[h][j].z; y[4 * j + 3] = n.w * g1[h][j].w;
                         }
-                        sq[i] = xn * xn;
+                        uint16_t* op = act_out + act_index_row(tok, pr0 >> 4, KS_out, 0, da.tbs_out);
+                        act_store_8(op, olo, y);
+                        act_store_8(op + 64, olo, y + 8);
+                    }
+                } else if (MODE == kSwiglu) {
+                    if (on) {
+                        const int f0 = gu_feature(pr0);
+                        float y[8];
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) y[i] = v[i] / (1.f + expf(-v[i])) * v[i + 8];      // rows 0-7 gate, 8-15 up
+                        act_store_8(act_out + act_index_row(tok, f0 >> 4, KS_out, 0, da.tbs_out) + (f0 & 8) * 8, olo, y);
+                    }
+                } else if (on) {                                       // kQkvRope: rows 0-7 are dims 8 tau .., rows 8-15 their partners
+                    const int head = pr0 / a.hd, d0 = (pr0 % a.hd) / 2;
+                    float lo8[8], hi8[8];
+                    const float* c8 = reinterpret_cast<const float*>(g0[h]);
+                    const float* s8 = reinterpret_cast<const float*>(g1[h]);
+                    const bool rot = head < a.Hq + a.Hkv;              // v heads are not rotated
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        lo8[i] = rot ? v[i] * c8[i] - v[i + 8] * s8[i] : v[i];
+                        hi8[i] = rot ? v[i + 8] * c8[i] + v[i] * s8[i] : v[i + 8];
+                    }
+                    if (head < a.Hq) {
+                        float4* qp = reinterpret_cast<float4*>(a.q_out + ((size_t)tok * a.Hq + head) * a.hd + d0);
+                        float4* qh = reinterpret_cast<float4*>(a.q_out + ((size_t)tok * a.Hq + head) * a.hd + half_hd + d0);
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            qp[j] = make_float4(lo8[4 * j], lo8[4 * j + 1], lo8[4 * j + 2], lo8[4 * j + 3]);
+                            qh[j] = make_float4(hi8[4 * j], hi8[4 * j + 1], hi8[4 * j + 2], hi8[4 * j + 3]);
+                        }
                     } else {
-                        // both remaining modes pair row i (< 8) with row i + 8 of a 16-row tile
-                        const float partner = __shfl_xor_sync(0xffffffffu, x, 8);
-                        if (MODE == kSwiglu) {
-                            if ((row & 15) < 8 && live) {
-                                const float act = x / (1.f + expf(-x)) * partner;      // own = gate, partner = up
-                                act_store_at(act_out, orow + (uint32_t)(g * 128 + i8 * 8), olo, act);
-                            }
-                        } else if (live) {                                           // kQkvRope
-                            // q and k heads are rotated (cos = 1, sin = 0 for v heads)
-                            const float val = (row & 15) < 8 ? x * e0[i8] - partner * e1[i8] : x * e0[i8] + partner * e1[i8];
-                            if (head < a.Hq) {
-                                a.q_out[((size_t)tok * a.Hq + head) * a.hd + dim] = val;
-                            } else {
-                                const int kv = head < a.Hq + a.Hkv ? 0 : 1;
-                                const int kvh = kv ? head - a.Hq - a.Hkv : head - a.Hq;
-                                const size_t per_head = (size_t)a.page_size * a.hd;
-                                const size_t off = (size_t)a.layer * a.n_pages * 2 * a.Hkv * per_head + (size_t)rk[i8] +
-                                                   ((size_t)kv * a.Hkv + kvh) * per_head + kv_col_offset(dim);
-                                a.kv_pool[off] = f32_to_bf16_bits(val);
-                            }
-                        }
+                        const int kv = head < a.Hq + a.Hkv ? 0 : 1;
+                        const int kvh = kv ? head - a.Hq - a.Hkv : head - a.Hq;
+                        const size_t per_head = (size_t)a.page_size * a.hd;
+                        uint16_t* kp = a.kv_pool + (size_t)a.layer * a.n_pages * 2 * a.Hkv * per_head + (size_t)rk + ((size_t)kv * a.Hkv + kvh) * per_head;
+                        *reinterpret_cast<uint4*>(kp + kv_col_offset(d0)) = bf16x8(lo8);
+                        *reinterpret_cast<uint4*>(kp + kv_col_offset(half_hd + d0)) = bf16x8(hi8);
                     }
                 }
             }
             if (MODE == kResid) {
-                // sums of squares of the new rows over the block's 128 rows, per token: over the warp's 32 rows by
-                // recursive halving (lane i ends up with token i's sum, lanes 16-31 mirror 0-15), then over the four
-                // warps in order
-#pragma unroll
-                for (int w = 8; w >= 1; w >>= 1) {
-                    const bool upper = (lane & w) != 0;
-#pragma unroll
-                    for (int i = 0; i < w; ++i) {
-                        const float keep = upper ? sq[i + w] : sq[i], give = upper ? sq[i] : sq[i + w];
-                        sq[i] = keep + __shfl_xor_sync(0xffffffffu, give, w);
-                    }
-                }
-                sq[0] += __shfl_xor_sync(0xffffffffu, sq[0], 16);
-                float* hs = ssq_s + half * 64;
-                if (lane < 16) hs[quarter * 16 + lane] = sq[0];          // lane l: token l of the column block
-                half_sync();
-                const int ht = et & 127;
-                if (ht < 16 && tokb + ht < a.M && rb < RB)
-                    a.ssq_out[(size_t)rb * a.M + tokb + ht] = hs[ht] + hs[16 + ht] + hs[32 + ht] + hs[48 + ht];
-                half_sync();
+                // sum of squares of the token's 128 new values: the lanes that share the token
+                ss += __shfl_xor_sync(0xffffffffu, ss, 8);
+                ss += __shfl_xor_sync(0xffffffffu, ss, 16);
+                if (tq == 0 && live && rb < RB) a.ssq_out[(size_t)rb * a.M + tok] = ss;
             }
-        };
-
-        // ---- the sums leave the registers for the ring's place (the pair's MMAs are done, its copies consumed), where the
-        // epilogue reads 16 tokens at a time: column block b of the token block belongs to slice b % S of the same CTA of
-        // a pair, which receives it as [b / S][slice][16 tokens][128 rows].  With one slice a thread reads back its own.
-        if (S > 1) cluster_sync_all();                                 // ... in every CTA of the cluster
-        float* own = reinterpret_cast<float*>(smem);
-#pragma unroll
-        for (int cb = 0; cb < kDenseMaxHalf / 16; ++cb) {
-            if (cb < ncb) {
-                const int b = half * ncb + cb;
-                const uint32_t dst = dsmem_addr(smem_base + (uint32_t)(((b / S) * S + s) * 8192 + row * 4), (uint32_t)((b % S) * 2 + r));
-#pragma unroll
-                for (int i = 0; i < 16; ++i) {
-                    if (S > 1) dsmem_st_f32(dst + i * 512, acc[cb][i]);
-                    else own[(b * 16 + i) * 128 + row] = acc[cb][i];
-                }
-            }
-        }
-        if (S > 1) cluster_sync_all();
-        const int j0 = S > 1 ? half : half * ncb, j1 = S > 1 ? (2 * ncb - s + S - 1) / S : (half + 1) * ncb, dj = S > 1 ? 2 : 1;
-#pragma unroll 1
-        for (int j = j0; j < j1; j += dj) {
-            float v[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = own[(size_t)(j * S) * 2048 + i * 128 + row];
-#pragma unroll 1
-            for (int q = 1; q < S; ++q) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] += own[(size_t)(j * S + q) * 2048 + i * 128 + row];
-            }
-            finish(j * S + s, v);
         }
         tc_fence_before();
     }
