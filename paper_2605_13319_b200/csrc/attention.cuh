@@ -18,9 +18,9 @@
 // and is read by the tensor cores as it is.  Q and P are fp32 values split into bf16 hi + lo terms (two MMAs into
 // the same accumulator); K and V are the cache's bf16.
 // Warps 0-7: one thread per key of a tile (= tensor-memory lane; warps w and w+4 share a lane quarter and take
-// alternate 16-row column blocks): masking, the running maximum (a row's reference maximum only moves when the
-// tile's maximum exceeds it by more than 2^8, so that O^T is rarely rescaled), exponentials, P written back as the
-// next MMA's B operand.  Warp 8: bulk copies of the K/V pages (a ring of three slots, K0 V0 K1 V1 ...; tiles of keys
+// alternate 8-row column blocks): masking, exponentials relative to the score of the split's first key (any reference will
+// do that keeps p in range; a row's maximum is only looked for when a score exceeds its reference by 2^40 and O^T has to
+// be rescaled), P written back as the next MMA's B operand.  Warp 8: bulk copies of the K/V pages (a ring of three slots, K0 V0 K1 V1 ...; tiles of keys
 // that were cached before this pass do not depend on the preceding QKV projection and are requested before the
 // dependent-launch wait) and the MMA issue (one thread).  Every wait is bounded and raises the device error word.
 #pragma once
@@ -36,7 +36,8 @@ constexpr int kAttnTile = 128;              // keys per tile = M of the MMAs
 constexpr int kAttnMaxRows = 112;           // query rows per CTA (N of the MMAs; what fits beside the ring); more rows: more row groups
 constexpr int kAttnMaxSplits = 16;          // key splits of one request
 constexpr int kAttnShortTail = 112;         // keys of the second tile up to which the third ring slot is cut down
-constexpr float kAttnLazyRescale = 8.f;     // log2 units by which a tile's maximum may exceed the reference maximum
+constexpr float kAttnMaxExcess = 40.f;      // log2 units by which a score may exceed its row's reference: P, O^T and the
+                                            // denominators stay below 2^60 and, next to a p of at least 1, lose nothing below
 
 // Wait for a barrier phase.  Bounded by a try count (each try suspends for a hardware-chosen time; 2^22 of them take
 // seconds), so that a protocol error cannot hang the GPU: the caller raises the error word and carries on.
@@ -62,6 +63,17 @@ __device__ __forceinline__ float fast_exp2(float x) {   // 2^x, relative error 2
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+// One barrier of the worker warps that also tells whether any of their threads said yes.
+__device__ __forceinline__ bool attn_workers_any(bool mine) {
+    uint32_t any;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.aligned.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+        : "=r"(any)
+        : "r"((uint32_t)mine), "n"(kAttnWorkers)
+        : "memory");
+    return any != 0;
 }
 
 // Shared-memory plan of one CTA with N query rows (a multiple of 16).  K and V tiles travel through a ring of three
@@ -147,17 +159,19 @@ struct AttnCtx {
 // belong to one KV head are contiguous in the pool, already in operand order, so every page the tile touches is one
 // bulk copy (lane l takes the l-th page), counted in bytes on the barrier.  Whole 8-row groups are copied: the rows
 // of the last group at or beyond k1 are masked (K) or cleared (V) by the consumers.
+// A function of its own (not inlined at its four places): a launch runs this kernel's code once or twice per SM, so what it
+// executes comes from the L2 rather than the instruction caches, and its size is time (see attn_kernel).
 template <int HD>
-__device__ __forceinline__ void attn_issue_tile(const AttnCtx& c, int kv, uint32_t dst, uint32_t bar, int j0) {
+__device__ __noinline__ void attn_issue_tile(const uint16_t* src0, const int32_t* bt, size_t page_stride, int page_size, int k1, uint32_t dst,
+                                             uint32_t bar, int j0) {
     const int lane = threadIdx.x & 31;
-    const int j1 = (min(j0 + kAttnTile, c.k1) + 7) & ~7;
+    const int j1 = (min(j0 + kAttnTile, k1) + 7) & ~7;
     if (lane == 0) mbar_expect_tx(bar, (uint32_t)(j1 - j0) * (HD * 2));
     __syncwarp();
-    const int pidx = j0 / c.page_size + lane;                              // page of the request
-    const int js = max(j0, pidx * c.page_size), je = min(j1, (pidx + 1) * c.page_size);
+    const int pidx = j0 / page_size + lane;                                // page of the request
+    const int js = max(j0, pidx * page_size), je = min(j1, (pidx + 1) * page_size);
     if (js < je) {
-        const uint16_t* src = c.kbase + (size_t)c.bt[pidx] * c.page_stride + (kv ? c.v_off : 0) +
-                              (size_t)(js - pidx * c.page_size) * HD;
+        const uint16_t* src = src0 + (size_t)bt[pidx] * page_stride + (size_t)(js - pidx * page_size) * HD;
         bulk_g2s(dst + (uint32_t)(js - j0) * (HD * 2), src, (uint32_t)(je - js) * (HD * 2), bar);
     }
 }
@@ -241,17 +255,21 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
     unsigned char* p_lo = p_hi + SM::p_bytes(N);
     float* wm = reinterpret_cast<float*>(p_lo + SM::p_bytes(N));   // [4][N] maxima of a tile per lane quarter
     int* hz = reinterpret_cast<int*>(wm + 4 * N);                  // [N] last visible key of a row (-1: padding row)
-    float* m_ref = reinterpret_cast<float*>(hz + N);               // [N] reference maximum of a row
+    float* m_ref = reinterpret_cast<float*>(hz + N);               // [N] reference score of a row
     float* alpha = m_ref + N;                                      // [N] rescale factor of a row for this tile
     float* Fl = alpha + N;                                         // [N] the CTA's partial denominators
     unsigned long long* bars = reinterpret_cast<unsigned long long*>(Fl + N);   // full[3], s_full[2], p_full, pv_done
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 7);
-    int* s_flag = reinterpret_cast<int*>(tmem_slot + 1);           // a row's reference maximum moved: rescale
-    int* s_last = s_flag + 1;
+    int* s_last = reinterpret_cast<int*>(tmem_slot + 1);
     const uint32_t bar_full = smem_u32(bars), bar_s = bar_full + 24, bar_p = bar_full + 40, bar_pv = bar_full + 48;
     const uint32_t tmem_cols = (uint32_t)attn_tmem_cols(N);
     const uint32_t ring_a = smem_u32(ring);
     auto slot_addr = [&](int i) { return ring_a + (uint32_t)(i % 3) * SM::kTileBytes; };   // ring slot of item i (K_t: 2t, V_t: 2t+1)
+
+    auto issue_item = [&](int i) {
+        attn_issue_tile<HD>(c.kbase + (i & 1 ? c.v_off : 0), c.bt, c.page_stride, c.page_size, c.k1, slot_addr(i), bar_full + 8 * (i % 3),
+                            c.k0 + (i >> 1) * kAttnTile);
+    };
 
     bool ok = true;
     uint32_t tmem_held = 0;        // tensor memory to give back before leaving, if any (address 0 is a valid one)
@@ -276,16 +294,19 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             // kernel: they are requested now, the others after the dependency has resolved.
             const int early_tiles = base >= c.k1 ? ntiles : (base - c.k0) / kAttnTile;      // whole tiles below `base`
             const int first = ntiles > 1 ? 3 : 2;                                            // items requested up front
+#pragma unroll 1
             for (int i = 0; i < first; ++i)
-                if ((i >> 1) < early_tiles) attn_issue_tile<HD>(c, i & 1, slot_addr(i), bar_full + 8 * (i % 3), c.k0 + (i >> 1) * kAttnTile);
+                if ((i >> 1) < early_tiles) issue_item(i);
             tmem_alloc(smem_u32(tmem_slot), tmem_cols);
             tc_fence_before();
             pdl_wait();
+#pragma unroll 1
             for (int i = 0; i < first; ++i)
-                if ((i >> 1) >= early_tiles) attn_issue_tile<HD>(c, i & 1, slot_addr(i), bar_full + 8 * (i % 3), c.k0 + (i >> 1) * kAttnTile);
+                if ((i >> 1) >= early_tiles) issue_item(i);
         } else {
             // operands that do not depend on the predecessor: the ones, the rows' horizons and initial state
             if (tid < SM::kOnes / 4) reinterpret_cast<uint32_t*>(ones)[tid] = 0x3F803F80u;
+#pragma unroll 1
             for (int n = tid; n < N; n += kAttnWorkers) {
                 const int rho = rho0 + n;
                 hz[n] = n < n_rows ? base + rho / G : -1;
@@ -296,6 +317,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             // piece (row n, k group g) at ((n/8) * HG + g) * 128 + (n%8) * 16.  Two pieces per thread and step, all
             // loads of a step in flight together.
             const float scale = rsqrtf((float)HD) * 1.4426950408889634f;   // scores in the log2 domain: p = 2^(s - m)
+#pragma unroll 1
             for (int idx0 = tid; idx0 < N * HG; idx0 += 2 * kAttnWorkers) {
                 float4 x[2][2];
 #pragma unroll
@@ -315,12 +337,12 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
                     if (idx >= N * HG) break;
                     const float v[8] = {x[u][0].x * scale, x[u][0].y * scale, x[u][0].z * scale, x[u][0].w * scale,
                                         x[u][1].x * scale, x[u][1].y * scale, x[u][1].z * scale, x[u][1].w * scale};
-                    uint16_t h[8], l[8];
+                    uint32_t h[4], l[4];
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) split_bf16(v[i], h[i], l[i]);
+                    for (int i = 0; i < 4; ++i) split_bf16x2(v[2 * i], v[2 * i + 1], h[i], l[i]);
                     const uint32_t off = (uint32_t)(((n >> 3) * HG + g) * 128 + (n & 7) * 16);
-                    *reinterpret_cast<uint4*>(q_hi + off) = make_uint4(pack2(h[0], h[1]), pack2(h[2], h[3]), pack2(h[4], h[5]), pack2(h[6], h[7]));
-                    *reinterpret_cast<uint4*>(q_lo + off) = make_uint4(pack2(l[0], l[1]), pack2(l[2], l[3]), pack2(l[4], l[5]), pack2(l[6], l[7]));
+                    *reinterpret_cast<uint4*>(q_hi + off) = make_uint4(h[0], h[1], h[2], h[3]);
+                    *reinterpret_cast<uint4*>(q_lo + off) = make_uint4(l[0], l[1], l[2], l[3]);
                 }
             }
             fence_proxy_async_smem();      // the tensor cores read these through the asynchronous proxy
@@ -341,26 +363,27 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             const uint64_t ones_desc = umma_desc(smem_u32(ones), 128, 256);
             auto issue_qk = [&](int t) {       // S^T[t & 1] = K_t . Q^T
                 const uint32_t ka = slot_addr(2 * t), d = t_S + (uint32_t)((t & 1) * N);
-#pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk)
-                    umma_bf16(d, umma_desc(ka + kk * 256, 128, HG * 128), umma_desc(qh + kk * 256, 128, HG * 128), idesc_qk, kk > 0);
-#pragma unroll
-                for (int kk = 0; kk < HD / 16; ++kk)
-                    umma_bf16(d, umma_desc(ka + kk * 256, 128, HG * 128), umma_desc(ql + kk * 256, 128, HG * 128), idesc_qk, 1);
+                uint64_t kd = umma_desc(ka, 128, HG * 128), hd_ = umma_desc(qh, 128, HG * 128), ld_ = umma_desc(ql, 128, HG * 128);
+#pragma unroll 2
+                for (int kk = 0; kk < HD / 16; ++kk) {
+                    umma_bf16(d, kd, hd_, idesc_qk, kk > 0);
+                    umma_bf16(d, kd, ld_, idesc_qk, 1);
+                    kd += 256 >> 4; hd_ += 256 >> 4; ld_ += 256 >> 4;
+                }
                 umma_commit(bar_s + 8 * (t & 1));
             };
             auto full_wait = [&](int i) { return attn_wait_warp(bar_full + 8 * (i % 3), (uint32_t)(i / 3) & 1u); };
             auto request = [&](int i) {        // ring item i, if the split has it
-                if ((i >> 1) < ntiles) attn_issue_tile<HD>(c, i & 1, slot_addr(i), bar_full + 8 * (i % 3), c.k0 + (i >> 1) * kAttnTile);
+                if ((i >> 1) < ntiles) issue_item(i);
             };
-            ok = full_wait(0);
-            if (ok && lane == 0) { tc_fence_after(); issue_qk(0); }
-            for (int t = 0; t < ntiles && ok; ++t) {
+#pragma unroll 1
+            for (int t = -1; t < ntiles && ok; ++t) {
                 if (t + 1 < ntiles) {
                     ok = full_wait(2 * t + 2);                                           // K of tile t+1 has landed
                     // S^T[(t+1) & 1] was last read for tile t-1: free once P of tile t-1 was announced (seen below)
                     if (ok && lane == 0) { tc_fence_after(); issue_qk(t + 1); }
                 }
+                if (t < 0) continue;
                 if (ok) ok = attn_wait_warp(bar_s + 8 * (t & 1), (uint32_t)(t >> 1) & 1u);   // K_t has been read
                 if (ok && t + 1 < ntiles) request(2 * t + 3);                            // V of tile t+1 into K_t's slot
                 if (ok) ok = attn_wait_warp(bar_p, (uint32_t)t & 1u);                    // P of tile t is written (and O^T rescaled)
@@ -370,16 +393,19 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
                     const uint32_t va = slot_addr(2 * t + 1);
                     const int n_valid = min(kAttnTile, c.k1 - (c.k0 + t * kAttnTile));
                     const int n16 = (n_valid + 15) / 16;
+                    uint64_t vd = umma_desc(va, HG * 128, 128), bh = umma_desc(ph, NG * 128, 128), bl = umma_desc(pl, NG * 128, 128);
+                    uint32_t acc = t > 0 ? 1u : 0u;
+#pragma unroll 1
                     for (int ks = 0; ks < n16; ++ks) {
-                        const uint64_t vd = umma_desc(va + ks * 2 * HG * 128, HG * 128, 128);
-                        const uint64_t bh = umma_desc(ph + ks * 2 * NG * 128, NG * 128, 128);
-                        const uint64_t bl = umma_desc(pl + ks * 2 * NG * 128, NG * 128, 128);
-                        const uint32_t acc = (t > 0 || ks > 0) ? 1u : 0u;
                         umma_bf16(t_O, vd, bh, idesc_pv, acc);
                         umma_bf16(t_O, vd, bl, idesc_pv, 1);
                         umma_bf16(t_L, ones_desc, bh, idesc_pv, acc);
                         umma_bf16(t_L, ones_desc, bl, idesc_pv, 1);
+                        vd += (2 * HG * 128) >> 4; bh += (uint64_t)((2 * NG * 128) >> 4); bl += (uint64_t)((2 * NG * 128) >> 4);
+                        acc = 1u;
                     }
+                }
+                if (ok && lane == 0) {
                     umma_commit(bar_pv);
                 }
                 if (ok && t == ntiles - 1) {
@@ -405,99 +431,118 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             const int quarter = warp & 3, half = warp >> 2;
             const int kt = quarter * 32 + lane;                         // key within the tile
             const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
+#pragma unroll 1
             for (int t = 0; t < ntiles; ++t) {
                 const int j = c.k0 + t * kAttnTile + kt;                // this thread's key
                 const int n_valid = min(kAttnTile, c.k1 - (c.k0 + t * kAttnTile));
                 const uint32_t t_St = t_S + (uint32_t)((t & 1) * N);
-                if (tid == 0) *s_flag = 0;
                 if (ok) ok = attn_wait_warp(bar_s + 8 * (t & 1), (uint32_t)(t >> 1) & 1u);
                 tc_fence_after();
                 const bool need_mask = c.k0 + (t + 1) * kAttnTile - 1 > base || n_valid < kAttnTile;   // CTA-uniform
-                // ---- pass 1: the tile's maximum per row (over the 32 keys of the warp, then over the lane quarters)
-                for (int cu = half; cu < NG; cu += 2) {
-                    float s[8];
-                    tmem_ld8(t_St + lane_sel + cu * 8, s);
-                    tmem_ld_wait();
-                    float mine = -INFINITY;
+                // A row's reference: the score of the split's first key, if the row sees it (else it sees none of the split).
+                // Softmax does not mind which: the largest p of the row is then at least 1, and no p may exceed
+                // 2^kAttnMaxExcess, so that everything stays far inside the range of fp32 and of the bf16 terms.
+                if (t == 0) {
+                    if (quarter == 0) {
+#pragma unroll 1
+    #pragma unroll 1
+                    for (int cu = half; cu < NG; cu += 2) {
+                            float s[8];
+                            tmem_ld8(t_St + cu * 8, s);
+                            tmem_ld_wait8(s);
+                            if (lane == 0) {
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        float v = s[i];
-                        if (need_mask && !(j < c.k1 && j <= hz[cu * 8 + i])) v = -INFINITY;
-                        if (!ok) v = -INFINITY;
-                        const float wmax = warp_max_redux(v);
-                        if (lane == i) mine = wmax;
+                                for (int i = 0; i < 8; ++i) m_ref[cu * 8 + i] = ok && j <= hz[cu * 8 + i] ? s[i] : -INFINITY;
+                            }
+                        }
                     }
-                    if (lane < 8) wm[quarter * N + cu * 8 + lane] = mine;
+                    asm volatile("bar.sync 1, %0;" ::"n"(kAttnWorkers) : "memory");
                 }
-                asm volatile("bar.sync 1, %0;" ::"n"(kAttnWorkers) : "memory");
-                if (tid < N) {
-                    const float tmax = fmaxf(fmaxf(wm[tid], wm[N + tid]), fmaxf(wm[2 * N + tid], wm[3 * N + tid]));
-                    const float m_old = m_ref[tid];
-                    float al = 1.f;
-                    if (tmax > -INFINITY) {
-                        if (m_old == -INFINITY) m_ref[tid] = tmax;             // nothing accumulated for this row so far
-                        else if (tmax > m_old + kAttnLazyRescale) { m_ref[tid] = tmax; al = fast_exp2(m_old - tmax); *s_flag = 1; }
-                    }
-                    alpha[tid] = al;
-                }
-                asm volatile("bar.sync 1, %0;" ::"n"(kAttnWorkers) : "memory");
                 // the previous tile's second product has read P (and updated O^T, L): P may be overwritten
                 if (t > 0 && ok) ok = attn_wait_warp(bar_pv, (uint32_t)(t - 1) & 1u);
                 tc_fence_after();
-                if (*s_flag && t > 0 && ok) {
-                    // ---- a reference maximum moved: rescale the rows' columns of O^T and L (2N columns from t_O)
-                    for (int cb = half; cb < 2 * NB; cb += 2) {
-                        float o[16];
-                        tmem_ld16(t_O + lane_sel + cb * 16, o);
-                        tmem_ld_wait();
+                // ---- p = 2^(s - reference), written as the MN-major B operand (hi and lo terms):
+                // piece (key group kg, row group g, key) at ((kg * NG + g) * 8 + key % 8) * 16 holds 8 rows.
+                // Done again, once, where some score exceeds its reference by too much.
+#pragma unroll 1
+                for (int again = 0;; ++again) {
+                    bool over = false;
+#pragma unroll 1
+                    for (int cu = half; cu < NG; cu += 2) {
+                        float s[8], mr[8];
+                        tmem_ld8(t_St + lane_sel + cu * 8, s);
+                        *reinterpret_cast<float4*>(mr) = *reinterpret_cast<const float4*>(m_ref + cu * 8);
+                        *reinterpret_cast<float4*>(mr + 4) = *reinterpret_cast<const float4*>(m_ref + cu * 8 + 4);
+                        tmem_ld_wait8(s);
+                        uint32_t hw[4], lw[4];
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) o[i] *= alpha[(cb * 16 + i) % N];
-                        tmem_st16(t_O + lane_sel + cb * 16, o);
-                    }
-                    tmem_st_wait();
-                }
-                // ---- pass 2: p = 2^(s - reference maximum), written as the MN-major B operand (hi and lo terms):
-                // piece (key group kg, row group g, key) at ((kg * NG + g) * 8 + key % 8) * 16 holds 8 rows
-                for (int cu = half; cu < NG; cu += 2) {
-                    float s[8];
-                    tmem_ld8(t_St + lane_sel + cu * 8, s);
-                    tmem_ld_wait();
-                    uint32_t hw[4], lw[4];
+                        for (int i = 0; i < 8; i += 2) {
+                            float p2[2];
 #pragma unroll
-                    for (int i = 0; i < 8; i += 2) {
-                        float p2[2];
-#pragma unroll
-                        for (int e = 0; e < 2; ++e) {
-                            const int n = cu * 8 + i + e;
-                            const float mr = m_ref[n];
-                            float v = s[i + e];
-                            if (need_mask && !(j < c.k1 && j <= hz[n])) v = -INFINITY;
-                            p2[e] = (ok && mr > -INFINITY) ? fast_exp2(v - mr) : 0.f;      // masked: 2^-inf = 0
+                            for (int e = 0; e < 2; ++e) {
+                                float v = s[i + e];
+                                if (need_mask && !(j < c.k1 && j <= hz[cu * 8 + i + e])) v = -INFINITY;
+                                over |= v > mr[i + e] + kAttnMaxExcess;
+                                p2[e] = (ok && mr[i + e] > -INFINITY) ? fast_exp2(v - mr[i + e]) : 0.f;      // masked: 2^-inf = 0
+                            }
+                            split_bf16x2(p2[0], p2[1], hw[i >> 1], lw[i >> 1]);
                         }
-                        uint16_t h0, l0, h1, l1;
-                        split_bf16(p2[0], h0, l0);
-                        split_bf16(p2[1], h1, l1);
-                        hw[i >> 1] = pack2(h0, h1);
-                        lw[i >> 1] = pack2(l0, l1);
+                        const uint32_t off = (uint32_t)((((kt >> 3) * NG + cu) * 8 + (kt & 7)) * 16);
+                        *reinterpret_cast<uint4*>(p_hi + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+                        *reinterpret_cast<uint4*>(p_lo + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
                     }
-                    const uint32_t off = (uint32_t)((((kt >> 3) * NG + cu) * 8 + (kt & 7)) * 16);
-                    *reinterpret_cast<uint4*>(p_hi + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                    *reinterpret_cast<uint4*>(p_lo + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-                }
-                // V rows at and beyond the split's end must be finite (P is 0 there, but 0 * NaN is not): cleared, once
-                // the tile's V rows have landed (the copy may bring garbage rows of the last 8-row group)
-                if (n_valid < kAttnTile) {
-                    if (ok) ok = attn_wait_warp(bar_full + 8 * ((2 * t + 1) % 3), (uint32_t)((2 * t + 1) / 3) & 1u);
-                    if (half == 0 && kt >= n_valid && kt < ((n_valid + 15) & ~15)) {
-                        unsigned char* v_tile = ring + ((2 * t + 1) % 3) * SM::kTileBytes;
+                    // V rows at and beyond the split's end must be finite (P is 0 there, but 0 * NaN is not): cleared, once
+                    // the tile's V rows have landed (the copy may bring garbage rows of the last 8-row group)
+                    if (n_valid < kAttnTile) {
+                        if (ok) ok = attn_wait_warp(bar_full + 8 * ((2 * t + 1) % 3), (uint32_t)((2 * t + 1) / 3) & 1u);
+                        if (half == 0 && kt >= n_valid && kt < ((n_valid + 15) & ~15)) {
+                            unsigned char* v_tile = ring + ((2 * t + 1) % 3) * SM::kTileBytes;
 #pragma unroll
-                        for (int g = 0; g < HG; ++g)
-                            *reinterpret_cast<uint4*>(v_tile + ((kt >> 3) * HG + g) * 128 + (kt & 7) * 16) = make_uint4(0, 0, 0, 0);
+                            for (int g = 0; g < HG; ++g)
+                                *reinterpret_cast<uint4*>(v_tile + ((kt >> 3) * HG + g) * 128 + (kt & 7) * 16) = make_uint4(0, 0, 0, 0);
+                        }
+                    }
+                    fence_proxy_async_smem();
+                    tc_fence_before();
+                    if (!attn_workers_any(over && ok && again == 0)) break;
+                    // ---- rare: the rows' references move up to the tile's maxima (over the 32 keys of the warp, then over
+                    // the lane quarters), what has been summed is rescaled, and P is written again
+#pragma unroll 1
+                    for (int cu = half; cu < NG; cu += 2) {
+                        float s[8];
+                        tmem_ld8(t_St + lane_sel + cu * 8, s);
+                        tmem_ld_wait8(s);
+                        float mine = -INFINITY;
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            float v = s[i];
+                            if (need_mask && !(j < c.k1 && j <= hz[cu * 8 + i])) v = -INFINITY;
+                            const float wmax = warp_max_redux(v);
+                            if (lane == i) mine = wmax;
+                        }
+                        if (lane < 8) wm[quarter * N + cu * 8 + lane] = mine;
+                    }
+                    asm volatile("bar.sync 1, %0;" ::"n"(kAttnWorkers) : "memory");
+                    if (tid < N) {
+                        const float tmax = fmaxf(fmaxf(wm[tid], wm[N + tid]), fmaxf(wm[2 * N + tid], wm[3 * N + tid]));
+                        const float m_old = m_ref[tid], m_new = fmaxf(m_old, tmax);
+                        m_ref[tid] = m_new;
+                        alpha[tid] = m_new > m_old ? fast_exp2(m_old - m_new) : 1.f;       // from -inf: nothing summed so far, 0
+                    }
+                    asm volatile("bar.sync 1, %0;" ::"n"(kAttnWorkers) : "memory");
+                    if (t > 0) {
+#pragma unroll 1
+                        for (int cb = half; cb < 2 * NB; cb += 2) {                  // O^T and L: 2N columns from t_O
+                            float o[16];
+                            tmem_ld16(t_O + lane_sel + cb * 16, o);
+                            tmem_ld_wait16(o);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) o[i] *= alpha[(cb < NB ? cb : cb - NB) * 16 + i];
+                            tmem_st16(t_O + lane_sel + cb * 16, o);
+                        }
+                        tmem_st_wait();
                     }
                 }
-                fence_proxy_async_smem();
-                tc_fence_before();
-                asm volatile("bar.sync 1, %0;" ::"n"(kAttnWorkers) : "memory");
                 if (tid == 0) mbar_arrive(bar_p);
             }
             // ---- the CTA's partial result: O^T (thread = head dimension) and L (lanes 0-7 hold all rows' sums)
@@ -506,6 +551,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             if (quarter == 0) {
                 // the column blocks go to the two warps of the quarter the other way round than O^T's below, so that with
                 // one block the denominators are stored by a warp that has no O^T columns to store
+#pragma unroll 1
                 for (int cb = half ^ 1; cb < NB; cb += 2) {
                     float l[16];
                     tmem_ld16(t_L + cb * 16, l);
@@ -531,6 +577,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             }
             const uint32_t ocol = act_index_col(kt, NTo, a.xd_tbs), olo = act_index_lo(a.xd_tbs);
             if (nsplit == 1) asm volatile("bar.sync 1, %0;" ::"n"(kAttnWorkers) : "memory");     // the sums and the table
+#pragma unroll 1
             for (int cb = half; cb < NB; cb += 2) {
                 float o[16];
                 tmem_ld16(t_O + lane_sel + cb * 16, o);
@@ -559,7 +606,9 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
     } else {
         // empty split: contributes nothing (finite zeros, so the merge can read it unconditionally)
         pdl_wait();
+#pragma unroll 1
         for (int i = tid; i < n_rows * HD; i += kAttnThreads) a.o_part[(slot0 + (size_t)(i / HD) * nsplit + sp) * HD + i % HD] = 0.f;
+#pragma unroll 1
         for (int i = tid; i < n_rows; i += kAttnThreads) {
             a.m_part[slot0 + (size_t)i * nsplit + sp] = -INFINITY;
             a.l_part[slot0 + (size_t)i * nsplit + sp] = 0.f;
@@ -586,6 +635,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
     // use (one trip to the L2 for up to kMergeBatch splits): lane j fetches split j's maximum and denominator, every
     // lane its four columns of each split's numerator; the sums run in split order.
     constexpr int kMergeBatch = 10;
+#pragma unroll 1
     for (int rl = warp; rl < n_rows; rl += kAttnThreads / 32) {
         const size_t sl0 = slot0 + (size_t)rl * nsplit;
         const float m_mine = lane < nsplit ? __ldcg(a.m_part + sl0 + lane) : -INFINITY;
@@ -617,16 +667,19 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
         }
         if (lane < HD / 4) {
             const int rho = rho0 + rl, gq = rho % G, r_in = rho / G;
-            const int col = (kvh * G + gq) * HD + lane * 4;
+            const int dk = lane * 4;                                 // column within the head
             const float inv = 1.f / den;
-            if (a.xd_tbs > 0) {
-                xd_store_one(a.xf_out, row0 + r_in, col, num.x * inv, KSo, a.xd_tbs);
-                xd_store_one(a.xf_out, row0 + r_in, col + 1, num.y * inv, KSo, a.xd_tbs);
-                xd_store_one(a.xf_out, row0 + r_in, col + 2, num.z * inv, KSo, a.xd_tbs);
-                xd_store_one(a.xf_out, row0 + r_in, col + 3, num.w * inv, KSo, a.xd_tbs);
-            } else {
-                xf_store_pair(reinterpret_cast<uint32_t*>(a.xf_out), row0 + r_in, col, num.x * inv, num.y * inv, KSo, NTo);
-                xf_store_pair(reinterpret_cast<uint32_t*>(a.xf_out), row0 + r_in, col + 2, num.z * inv, num.w * inv, KSo, NTo);
+            const uint32_t idx = act_index_row(row0 + r_in, ((kvh * G + gq) * HD) >> 4, KSo, NTo, a.xd_tbs) + act_index_col(dk, NTo, a.xd_tbs);
+            uint32_t h[2], l[2];
+            split_bf16x2(num.x * inv, num.y * inv, h[0], l[0]);
+            split_bf16x2(num.z * inv, num.w * inv, h[1], l[1]);
+            // columns dk, dk + 1 are neighbours in either layout; dk + 2 follows them in an xd array, one lane (16 bytes) on in
+            // fragment order
+            const uint32_t lo = act_index_lo(a.xd_tbs), next = a.xd_tbs > 0 ? 2 : 8;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                *reinterpret_cast<uint32_t*>(a.xf_out + idx + e * next) = h[e];
+                *reinterpret_cast<uint32_t*>(a.xf_out + idx + e * next + lo) = l[e];
             }
         }
     }

@@ -108,6 +108,12 @@ __device__ __forceinline__ void tmem_ld_wait16(float (&r)[16]) {
                  :
                  : "memory");
 }
+__device__ __forceinline__ void tmem_ld_wait8(float (&r)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(r[0]), "+f"(r[1]), "+f"(r[2]), "+f"(r[3]), "+f"(r[4]), "+f"(r[5]), "+f"(r[6]), "+f"(r[7])
+                 :
+                 : "memory");
+}
 // True in one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
     uint32_t p;

@@ -273,3 +273,31 @@ def test_host_side_errors_and_page_accounting():
     ctx.prefill(r1, synth.make_prefix(shape, 40, 0))                  # pages came back
     assert ctx.req_len(r1) == 40
     ctx.close()
+
+
+@pytest.mark.parametrize("n_kv_heads,k", [(4, 4), (2, 16)])
+@pytest.mark.parametrize("loud", ["first", "second"])
+def test_attention_scores_of_wide_range(n_kv_heads, k, loud):
+    """Cached keys whose scores lie hundreds of powers of two apart, the loud ones in the first or in the second 128-key tile
+    of every split (16 splits of 256 keys): the reference a row's exponentials are taken from has to move, before anything
+    has been summed and after."""
+    from paper_2605_13319_b200 import binding
+    shape, P = synth.TINY.scaled(name=f"tiny-kv{n_kv_heads}", n_kv_heads=n_kv_heads), 4090
+    w = synth.make_weights(shape, 5)
+    orc = oracle.Oracle(shape, w, P + 32)
+    ctx = binding.Context(shape, w, n_pages=(P + 32) // 16 + 1, max_seq=P + 32, max_draft=16, poison=True)
+    req = ctx.req_open()
+    tile = np.arange(P) // 128 % 2
+    scale = np.where(tile == (1 if loud == "second" else 0), 400.0, 1.0).astype(np.float32)
+    for l in range(shape.n_layers):
+        kb, vb = synth.make_synthetic_kv(shape, P, 5, l)
+        kb = synth.f32_to_bf16(synth.bf16_to_f32(kb) * scale[:, None])
+        ctx.debug_write_kv(req, l, 0, kb, vb)
+        orc.set_synthetic_kv(l, kb, vb)
+    orc.set_len(P)
+    toks, q, u, _ = draft_inputs(orc, shape, k, 1.0, 5)
+    ref = orc.verify(toks, q, u)
+    ctx.verify([dict(req=req, tokens=toks, q=q, u=u)], flags=binding.Q_HOST)
+    # a score of 500 carries an error of 2^-17 of itself, 4e-3, and the probabilities e^s as much in relative terms
+    assert logit_rel_err(ctx.debug_get_logits(k + 1), ref["logits"]).max() < LOGIT_TOL
+    ctx.close()
