@@ -12,7 +12,7 @@
 //   S^T[128 keys x N rows] = K_tile[128 x hd] . Q^T[hd x N]          A = K rows from the cache, B = Q
 //   O^T[hd x N rows]      += V_tile^T[hd x 128 keys] . P^T[128 x N]   A = V rows from the cache, B = P
 //   L  [  * x N rows]      += 1[* x 128 keys] . P^T[128 x N]          the softmax denominators, by the same P
-// with S^T (twice: two tiles in flight), O^T and L in tensor memory (4N columns).  The cache stores, per page and
+// with S^T (twice: two tiles in flight), O^T and L in tensor memory.  The cache stores, per page and
 // head, the rows in 8-row groups of 8-element pieces ([slot/8][hd/8][slot%8][8]), which IS the operand order of
 // both products (K-major for the first, MN-major for the second): a page lands in shared memory by one bulk copy
 // and is read by the tensor cores as it is.  Q and P are fp32 values split into bf16 hi + lo terms (two MMAs into
@@ -35,6 +35,8 @@ constexpr int kAttnThreads = kAttnWorkers + 32;
 constexpr int kAttnTile = 128;              // keys per tile = M of the MMAs
 constexpr int kAttnMaxRows = 112;           // query rows per CTA (N of the MMAs; what fits beside the ring); more rows: more row groups
 constexpr int kAttnMaxSplits = 16;          // key splits of one request
+constexpr int kAttnMaxSlots = 4;            // tile slots of the K/V ring
+constexpr int kAttnBigCols = kAttnMaxRows / 16;   // 8-row column blocks per worker warp of the large variant (the small one: 1, 16 rows)
 constexpr int kAttnShortTail = 112;         // keys of the second tile up to which the third ring slot is cut down
 constexpr float kAttnMaxExcess = 40.f;      // log2 units by which a score may exceed its row's reference: P, O^T and the
                                             // denominators stay below 2^60 and, next to a p of at least 1, lose nothing below
@@ -77,7 +79,7 @@ __device__ __forceinline__ bool attn_workers_any(bool mine) {
 }
 
 // Shared-memory plan of one CTA with N query rows (a multiple of 16).  K and V tiles travel through a ring of three
-// slots in the order K0 V0 K1 V1 ...: two of a whole tile each and a third of `slot_c` bytes (a whole tile, or less
+// slots in the order K0 V0 K1 V1 ...: two of a whole tile each and a third (a whole tile, or less
 // when no CTA of the launch has more than two tiles, the second of at most kAttnShortTail keys: the K/V of such a
 // CTA are then requested in full before the first product starts).
 template <int HD>
@@ -88,25 +90,46 @@ struct AttnSmem {
     __host__ __device__ static constexpr int p_bytes(int N) { return kAttnTile * N * 2; }   // hi or lo
     __host__ __device__ static constexpr int small_bytes(int N) { return 8 * N * 4 + 128; } // warp maxima [4][N], horizon, reference
                                                                                             // maximum, factor, sums [N] each; barriers
-    __host__ __device__ static constexpr size_t bytes(int N, int slot_c) {
-        return (size_t)kOnes + 2 * kTileBytes + slot_c + 2 * q_bytes(N) + 2 * p_bytes(N) + small_bytes(N);
+    __host__ __device__ static constexpr size_t bytes(int N, int ring) {
+        return (size_t)kOnes + ring + 2 * q_bytes(N) + 2 * p_bytes(N) + small_bytes(N);
     }
 };
 
-// Tensor-memory columns of a CTA with N query rows: S^T twice, O^T and L, N columns each, as a power of two >= 32.
+// An MMA of up to about 48 rows costs the same as one of 16 (fetch of the 128-row A operand, issue), so the hi and lo terms of
+// Q, and of P, stand side by side as one operand of 2N rows -- half the MMAs, and the two halves of the result are added
+// where it is read -- as long as the wider accumulators fit tensor memory: 8N columns up to 64 rows; up to 80 rows for P
+// only, 6N; else the terms take turns, 4N.  (Batch of 16 at the 7b shape: 24 MMAs of 42 cycles per tile instead of 48.)
+__host__ __device__ constexpr bool attn_wide_q(int N) { return N <= 64; }
+__host__ __device__ constexpr bool attn_wide_p(int N) { return N <= 80; }
+// Tensor-memory columns of a CTA with N query rows: S^T twice, O^T and L, as a power of two >= 32.
 __host__ __device__ constexpr int attn_tmem_cols(int N) {
     int c = 32;
-    while (c < 4 * N) c *= 2;
+    while (c < 2 * N * (attn_wide_q(N) ? 2 : 1) + 2 * N * (attn_wide_p(N) ? 2 : 1)) c *= 2;
     return c;
 }
-static inline int attn_slot_c_bytes(int hd, bool short_tail) { return (short_tail ? kAttnShortTail : kAttnTile) * hd * 2; }
+// The ring: three slots of a tile (the third cut down where no split of the launch has more than two tiles, the second a
+// short one), or four where that costs no resident CTA.  With three, the next K tile is only requested when the present
+// V tile has been read, and its 3 us are waited for once per tile (8b shape, 17 rows: 3.9 us per tile).
+static inline int attn_ring_bytes(int hd, int slots, bool short_tail) {
+    const int tile = kAttnTile * hd * 2;
+    return slots == 4 ? 4 * tile : 2 * tile + (short_tail ? kAttnShortTail * hd * 2 : tile);
+}
+static inline size_t attn_smem_bytes_raw(int hd, int N, int ring) {
+    return hd == 128 ? AttnSmem<128>::bytes(N, ring) : AttnSmem<64>::bytes(N, ring);
+}
+constexpr int kAttnSmemMax = 227 * 1024;
+static inline int attn_ring_slots(int hd, int N) {
+    const size_t three = attn_smem_bytes_raw(hd, N, attn_ring_bytes(hd, 3, false)), four = attn_smem_bytes_raw(hd, N, attn_ring_bytes(hd, 4, false));
+    const int cap = N > 16 ? 1 : 2;                              // CTAs per SM by registers
+    auto per_sm = [&](size_t b) { const int n = (int)((size_t)(228 * 1024) / (b + 1024)); return n > cap ? cap : n; };
+    return four <= (size_t)kAttnSmemMax && per_sm(four) >= per_sm(three) ? 4 : 3;
+}
 // Dynamic shared memory to ask for: the plan above, padded so that the CTAs an SM can hold never want more than the
 // SM's 512 tensor-memory columns together (the allocation instruction blocks until its columns are free).
 static inline size_t attn_smem_bytes(int hd, int N, bool short_tail) {
-    const int sc = attn_slot_c_bytes(hd, short_tail);
-    const size_t need = hd == 128 ? AttnSmem<128>::bytes(N, sc) : AttnSmem<64>::bytes(N, sc);
+    const size_t need = attn_smem_bytes_raw(hd, N, attn_ring_bytes(hd, attn_ring_slots(hd, N), short_tail));
     const int max_ctas = 512 / attn_tmem_cols(N);
-    const size_t floor_ = (size_t)(227 * 1024) / (max_ctas + 1) + 1;
+    const size_t floor_ = (size_t)kAttnSmemMax / (max_ctas + 1) + 1;
     return need > floor_ ? need : floor_;
 }
 static inline int attn_rows_n(int rows_per_kv_head) {    // N of a CTA that holds this many query rows
@@ -183,7 +206,8 @@ struct AttnArgs {
     int layer, n_pages, page_size, M, Hq, Hkv;
     int rows_cap;              // query rows per row group (kAttnMaxRows, or 16 for a batch whose requests have up to 32)
     int n_max;                 // N the launch's shared memory was sized for
-    int slot_c;                // bytes of the ring's third slot
+    int ring, slots;           // bytes and slots of the K/V ring
+    int share_merge;           // every CTA of the launch is resident: the CTAs of a group merge its rows together
     int row_groups;
     float* o_part;             // partial results: [slot][hd], slot = it_part0 + ((kv head * R + row) * splits + split)
     float* m_part;             // [slot]
@@ -199,11 +223,12 @@ struct AttnArgs {
     int* err;
 };
 
-// grid (max splits of the launch, n_kv_heads * row_groups, n_items), block 288.  The register bound is what lets two CTAs
-// share an SM: a CTA's nine warps put three on one of the SM's four register partitions (16K registers each), and two
-// such triples must fit it.
-template <int HD>
-__global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a) {
+// grid (max splits of the launch, n_kv_heads * row_groups, n_items), block 288.  CU = 1: launches of up to 16 query rows per
+// CTA; the register bound is what lets two CTAs share an SM (a CTA's nine warps put three on one of the SM's four register
+// partitions, 16K registers each, and two such triples must fit it).  CU = kAttnBigCols: more rows, one CTA per SM, and
+// a worker's share of a tile's P, up to 56 values, stays in registers until the previous product is through.
+template <int HD, int CU>
+__global__ void __launch_bounds__(kAttnThreads, CU == 1 ? 3 : 1) attn_kernel(const AttnArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     using SM = AttnSmem<HD>;
     constexpr int HG = HD / 8;                                      // 8-element pieces of a row
@@ -248,26 +273,29 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
 
     // ---- shared memory: the ones come first (the tensor cores read a few KB past them, see below)
     unsigned char* ones = smem;
-    unsigned char* ring = ones + SM::kOnes;                        // slots 0, 1: a whole tile; slot 2: a.slot_c bytes
-    unsigned char* q_hi = ring + 2 * SM::kTileBytes + a.slot_c;
+    unsigned char* ring = ones + SM::kOnes;                        // a.slots slots of a tile (of three, the last may be shorter)
+    unsigned char* q_hi = ring + a.ring;
     unsigned char* q_lo = q_hi + SM::q_bytes(N);
     unsigned char* p_hi = q_lo + SM::q_bytes(N);
-    unsigned char* p_lo = p_hi + SM::p_bytes(N);
-    float* wm = reinterpret_cast<float*>(p_lo + SM::p_bytes(N));   // [4][N] maxima of a tile per lane quarter
+    float* wm = reinterpret_cast<float*>(p_hi + 2 * SM::p_bytes(N));   // [4][N] maxima of a tile per lane quarter
     int* hz = reinterpret_cast<int*>(wm + 4 * N);                  // [N] last visible key of a row (-1: padding row)
     float* m_ref = reinterpret_cast<float*>(hz + N);               // [N] reference score of a row
     float* alpha = m_ref + N;                                      // [N] rescale factor of a row for this tile
     float* Fl = alpha + N;                                         // [N] the CTA's partial denominators
-    unsigned long long* bars = reinterpret_cast<unsigned long long*>(Fl + N);   // full[3], s_full[2], p_full, pv_done
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 7);
+    unsigned long long* bars = reinterpret_cast<unsigned long long*>(Fl + N);   // full[4], s_full[2], p_full, pv_done
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 8);
     int* s_last = reinterpret_cast<int*>(tmem_slot + 1);
-    const uint32_t bar_full = smem_u32(bars), bar_s = bar_full + 24, bar_p = bar_full + 40, bar_pv = bar_full + 48;
+    const uint32_t bar_full = smem_u32(bars), bar_s = bar_full + 32, bar_p = bar_full + 48, bar_pv = bar_full + 56;
     const uint32_t tmem_cols = (uint32_t)attn_tmem_cols(N);
     const uint32_t ring_a = smem_u32(ring);
-    auto slot_addr = [&](int i) { return ring_a + (uint32_t)(i % 3) * SM::kTileBytes; };   // ring slot of item i (K_t: 2t, V_t: 2t+1)
+    const int slots = a.slots;
+    // ring item i (K_t: 2t, V_t: 2t+1) lives in slot i % slots
+    auto slot_of = [&](int i) { return slots == 4 ? i & 3 : i % 3; };
+    auto turn_of = [&](int i) { return (uint32_t)(slots == 4 ? i >> 2 : i / 3) & 1u; };
+    auto slot_addr = [&](int i) { return ring_a + (uint32_t)slot_of(i) * SM::kTileBytes; };
 
     auto issue_item = [&](int i) {
-        attn_issue_tile<HD>(c.kbase + (i & 1 ? c.v_off : 0), c.bt, c.page_stride, c.page_size, c.k1, slot_addr(i), bar_full + 8 * (i % 3),
+        attn_issue_tile<HD>(c.kbase + (i & 1 ? c.v_off : 0), c.bt, c.page_stride, c.page_size, c.k1, slot_addr(i), bar_full + 8 * slot_of(i),
                             c.k0 + (i >> 1) * kAttnTile);
     };
 
@@ -286,14 +314,14 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
         if (warp == 8) {
             // ---------------- barriers, the first three items of the ring, tensor memory
             if (lane == 0) {
-                for (int i = 0; i < 7; ++i) mbar_init(bar_full + 8 * i, 1);
+                for (int i = 0; i < 8; ++i) mbar_init(bar_full + 8 * i, 1);
                 fence_mbar_init();
             }
             __syncwarp();
             // Items made only of keys cached before this pass do not depend on the QKV projection that precedes this
             // kernel: they are requested now, the others after the dependency has resolved.
             const int early_tiles = base >= c.k1 ? ntiles : (base - c.k0) / kAttnTile;      // whole tiles below `base`
-            const int first = ntiles > 1 ? 3 : 2;                                            // items requested up front
+            const int first = min(2 * ntiles, slots);                                           // items requested up front
 #pragma unroll 1
             for (int i = 0; i < first; ++i)
                 if ((i >> 1) < early_tiles) issue_item(i);
@@ -350,29 +378,30 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
         __syncthreads();                   // barriers, Q, ones and the tensor-memory base are in place
         tc_fence_after();
         tmem = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
-        const uint32_t t_S = tmem, t_O = tmem + 2u * (uint32_t)N, t_L = tmem + 3u * (uint32_t)N;   // S^T twice, O^T, L
+        const bool wide_q = attn_wide_q(N), wide_p = attn_wide_p(N);
+        const int NS = wide_q ? 2 * N : N, NO = wide_p ? 2 * N : N;                                // columns of S^T / of O^T and L
+        const uint32_t t_S = tmem, t_O = tmem + 2u * (uint32_t)NS, t_L = t_O + (uint32_t)NO;       // S^T twice, O^T, L
 
         if (warp == 8) {
-            // ---------------- copies and MMA issue.  Ring item i (K_t: 2t, V_t: 2t+1) lives in slot i % 3 and may be
-            // requested once item i - 3 has been read: a K tile by the first product of its tile (s_full), a V tile by
-            // the second (pv_done).  The first product of tile t+1 is issued ahead of the second of tile t.
-            const uint32_t idesc_qk = umma_idesc_bf16(128, N, 0, 0), idesc_pv = umma_idesc_bf16(128, N, 1, 1);
-            const uint32_t qh = smem_u32(q_hi), ql = smem_u32(q_lo), ph = smem_u32(p_hi), pl = smem_u32(p_lo);
+            // ---------------- copies and MMA issue.  Ring item i may be requested once item i - slots has been read: a K tile
+            // by the first product of its tile (s_full), a V tile by the second (pv_done).  The first product of tile t+1 is issued ahead of the second of tile t.
+            const uint32_t idesc_qk = umma_idesc_bf16(128, NS, 0, 0), idesc_pv = umma_idesc_bf16(128, NO, 1, 1);
+            const uint32_t qh = smem_u32(q_hi), ql = smem_u32(q_lo), ph = smem_u32(p_hi);
             // the denominators' A operand: 16 keys x 8 rows of ones; the other 120 rows of the MMA read whatever follows
             // in shared memory (the ring) and land in tensor-memory lanes that nobody reads
             const uint64_t ones_desc = umma_desc(smem_u32(ones), 128, 256);
             auto issue_qk = [&](int t) {       // S^T[t & 1] = K_t . Q^T
-                const uint32_t ka = slot_addr(2 * t), d = t_S + (uint32_t)((t & 1) * N);
-                uint64_t kd = umma_desc(ka, 128, HG * 128), hd_ = umma_desc(qh, 128, HG * 128), ld_ = umma_desc(ql, 128, HG * 128);
-#pragma unroll 2
+                const uint32_t d = t_S + (uint32_t)((t & 1) * NS);
+                uint64_t kd = umma_desc(slot_addr(2 * t), 128, HG * 128), hd_ = umma_desc(qh, 128, HG * 128), ld_ = umma_desc(ql, 128, HG * 128);
+#pragma unroll 4
                 for (int kk = 0; kk < HD / 16; ++kk) {
                     umma_bf16(d, kd, hd_, idesc_qk, kk > 0);
-                    umma_bf16(d, kd, ld_, idesc_qk, 1);
+                    if (!wide_q) umma_bf16(d, kd, ld_, idesc_qk, 1);
                     kd += 256 >> 4; hd_ += 256 >> 4; ld_ += 256 >> 4;
                 }
                 umma_commit(bar_s + 8 * (t & 1));
             };
-            auto full_wait = [&](int i) { return attn_wait_warp(bar_full + 8 * (i % 3), (uint32_t)(i / 3) & 1u); };
+            auto full_wait = [&](int i) { return attn_wait_warp(bar_full + 8 * slot_of(i), turn_of(i)); };
             auto request = [&](int i) {        // ring item i, if the split has it
                 if ((i >> 1) < ntiles) issue_item(i);
             };
@@ -381,31 +410,33 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
                 if (t + 1 < ntiles) {
                     ok = full_wait(2 * t + 2);                                           // K of tile t+1 has landed
                     // S^T[(t+1) & 1] was last read for tile t-1: free once P of tile t-1 was announced (seen below)
-                    if (ok && lane == 0) { tc_fence_after(); issue_qk(t + 1); }
+                    if (ok && elect_one()) { tc_fence_after(); issue_qk(t + 1); }
                 }
                 if (t < 0) continue;
                 if (ok) ok = attn_wait_warp(bar_s + 8 * (t & 1), (uint32_t)(t >> 1) & 1u);   // K_t has been read
-                if (ok && t + 1 < ntiles) request(2 * t + 3);                            // V of tile t+1 into K_t's slot
+                if (ok) request(2 * t + slots);                                          // into K_t's slot
                 if (ok) ok = attn_wait_warp(bar_p, (uint32_t)t & 1u);                    // P of tile t is written (and O^T rescaled)
                 if (ok) ok = full_wait(2 * t + 1);                                       // V of tile t has landed
-                if (ok && lane == 0) {
+                if (ok && elect_one()) {
                     tc_fence_after();
                     const uint32_t va = slot_addr(2 * t + 1);
                     const int n_valid = min(kAttnTile, c.k1 - (c.k0 + t * kAttnTile));
                     const int n16 = (n_valid + 15) / 16;
-                    uint64_t vd = umma_desc(va, HG * 128, 128), bh = umma_desc(ph, NG * 128, 128), bl = umma_desc(pl, NG * 128, 128);
+                    // P: hi and lo row groups side by side, 2 * NG of them per key group
+                    uint64_t vd = umma_desc(va, HG * 128, 128), pd = umma_desc(ph, 2 * NG * 128, 128);
                     uint32_t acc = t > 0 ? 1u : 0u;
-#pragma unroll 1
+#pragma unroll 2
                     for (int ks = 0; ks < n16; ++ks) {
-                        umma_bf16(t_O, vd, bh, idesc_pv, acc);
-                        umma_bf16(t_O, vd, bl, idesc_pv, 1);
-                        umma_bf16(t_L, ones_desc, bh, idesc_pv, acc);
-                        umma_bf16(t_L, ones_desc, bl, idesc_pv, 1);
-                        vd += (2 * HG * 128) >> 4; bh += (uint64_t)((2 * NG * 128) >> 4); bl += (uint64_t)((2 * NG * 128) >> 4);
+                        umma_bf16(t_O, vd, pd, idesc_pv, acc);
+                        umma_bf16(t_L, ones_desc, pd, idesc_pv, acc);
+                        if (!wide_p) {
+                            umma_bf16(t_O, vd, pd + (uint64_t)((NG * 128) >> 4), idesc_pv, 1);
+                            umma_bf16(t_L, ones_desc, pd + (uint64_t)((NG * 128) >> 4), idesc_pv, 1);
+                        }
+                        vd += (2 * HG * 128) >> 4;
+                        pd += (uint64_t)((4 * NG * 128) >> 4);
                         acc = 1u;
                     }
-                }
-                if (ok && lane == 0) {
                     umma_commit(bar_pv);
                 }
                 if (ok && t == ntiles - 1) {
@@ -421,7 +452,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
                 }
                 if (ok && t + 2 < ntiles) {
                     ok = attn_wait_warp(bar_pv, (uint32_t)t & 1u);                       // V_t has been read
-                    if (ok) request(2 * t + 4);                                          // K of tile t+2 into V_t's slot
+                    if (ok) request(2 * t + 1 + slots);                                  // into V_t's slot
                 }
             }
             if (!ok && a.err && lane == 0) atomicExch(a.err, 3);
@@ -435,21 +466,32 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             for (int t = 0; t < ntiles; ++t) {
                 const int j = c.k0 + t * kAttnTile + kt;                // this thread's key
                 const int n_valid = min(kAttnTile, c.k1 - (c.k0 + t * kAttnTile));
-                const uint32_t t_St = t_S + (uint32_t)((t & 1) * N);
+                const uint32_t t_St = t_S + (uint32_t)((t & 1) * NS);
                 if (ok) ok = attn_wait_warp(bar_s + 8 * (t & 1), (uint32_t)(t >> 1) & 1u);
                 tc_fence_after();
                 const bool need_mask = c.k0 + (t + 1) * kAttnTile - 1 > base || n_valid < kAttnTile;   // CTA-uniform
                 // A row's reference: the score of the split's first key, if the row sees it (else it sees none of the split).
                 // Softmax does not mind which: the largest p of the row is then at least 1, and no p may exceed
                 // 2^kAttnMaxExcess, so that everything stays far inside the range of fp32 and of the bf16 terms.
+                // eight columns of S^T: rows of Q's hi terms, and of its lo terms where they have columns of their own
+                auto read_s = [&](uint32_t at, float (&s)[8]) {
+                    float l[8];
+                    tmem_ld8(at, s);
+                    if (wide_q) tmem_ld8(at + (uint32_t)N, l);
+                    tmem_ld_wait8(s);
+                    if (wide_q) {
+                        tmem_ld_wait8(l);
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) s[i] += l[i];
+                    }
+                };
                 if (t == 0) {
                     if (quarter == 0) {
 #pragma unroll 1
     #pragma unroll 1
                     for (int cu = half; cu < NG; cu += 2) {
                             float s[8];
-                            tmem_ld8(t_St + cu * 8, s);
-                            tmem_ld_wait8(s);
+                            read_s(t_St + cu * 8, s);
                             if (lane == 0) {
 #pragma unroll
                                 for (int i = 0; i < 8; ++i) m_ref[cu * 8 + i] = ok && j <= hz[cu * 8 + i] ? s[i] : -INFINITY;
@@ -458,45 +500,57 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
                     }
                     asm volatile("bar.sync 1, %0;" ::"n"(kAttnWorkers) : "memory");
                 }
-                // the previous tile's second product has read P (and updated O^T, L): P may be overwritten
-                if (t > 0 && ok) ok = attn_wait_warp(bar_pv, (uint32_t)(t - 1) & 1u);
-                tc_fence_after();
-                // ---- p = 2^(s - reference), written as the MN-major B operand (hi and lo terms):
-                // piece (key group kg, row group g, key) at ((kg * NG + g) * 8 + key % 8) * 16 holds 8 rows.
-                // Done again, once, where some score exceeds its reference by too much.
+                // ---- p = 2^(s - reference) as bf16 hi and lo terms, in registers: this part runs under the previous tile's
+                // second product.  Done again, once, where some score exceeds its reference by too much.
 #pragma unroll 1
                 for (int again = 0;; ++again) {
                     bool over = false;
-#pragma unroll 1
-                    for (int cu = half; cu < NG; cu += 2) {
-                        float s[8], mr[8];
-                        tmem_ld8(t_St + lane_sel + cu * 8, s);
-                        *reinterpret_cast<float4*>(mr) = *reinterpret_cast<const float4*>(m_ref + cu * 8);
-                        *reinterpret_cast<float4*>(mr + 4) = *reinterpret_cast<const float4*>(m_ref + cu * 8 + 4);
-                        tmem_ld_wait8(s);
-                        uint32_t hw[4], lw[4];
+                    uint32_t hw[CU][4], lw[CU][4];
 #pragma unroll
-                        for (int i = 0; i < 8; i += 2) {
-                            float p2[2];
+                    for (int q = 0; q < CU; ++q) {
+                        const int cu = half + 2 * q;
+                        if (cu < NG) {
+                            float sc[8], mr[8];
+                            read_s(t_St + lane_sel + cu * 8, sc);
+                            *reinterpret_cast<float4*>(mr) = *reinterpret_cast<const float4*>(m_ref + cu * 8);
+                            *reinterpret_cast<float4*>(mr + 4) = *reinterpret_cast<const float4*>(m_ref + cu * 8 + 4);
+                            if (need_mask) {
 #pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                float v = s[i + e];
-                                if (need_mask && !(j < c.k1 && j <= hz[cu * 8 + i + e])) v = -INFINITY;
-                                over |= v > mr[i + e] + kAttnMaxExcess;
-                                p2[e] = (ok && mr[i + e] > -INFINITY) ? fast_exp2(v - mr[i + e]) : 0.f;      // masked: 2^-inf = 0
+                                for (int i = 0; i < 8; ++i)
+                                    if (!(j < c.k1 && j <= hz[cu * 8 + i])) sc[i] = -INFINITY;
                             }
-                            split_bf16x2(p2[0], p2[1], hw[i >> 1], lw[i >> 1]);
+#pragma unroll
+                            for (int i = 0; i < 8; i += 2) {
+                                float p2[2];
+#pragma unroll
+                                for (int e = 0; e < 2; ++e) {
+                                    over |= sc[i + e] > mr[i + e] + kAttnMaxExcess;
+                                    p2[e] = (ok && mr[i + e] > -INFINITY) ? fast_exp2(sc[i + e] - mr[i + e]) : 0.f;    // masked: 2^-inf = 0
+                                }
+                                split_bf16x2(p2[0], p2[1], hw[q][i >> 1], lw[q][i >> 1]);
+                            }
                         }
-                        const uint32_t off = (uint32_t)((((kt >> 3) * NG + cu) * 8 + (kt & 7)) * 16);
-                        *reinterpret_cast<uint4*>(p_hi + off) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-                        *reinterpret_cast<uint4*>(p_lo + off) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+                    }
+                    // the previous tile's second product has read P (and updated O^T, L): P may be overwritten
+                    if (t > 0 && again == 0 && ok) ok = attn_wait_warp(bar_pv, (uint32_t)(t - 1) & 1u);
+                    tc_fence_after();
+                    // the MN-major B operand: piece (key group kg, row group g, key) at ((kg * 2 NG + g) * 8 + key % 8) * 16 holds
+                    // 8 rows, their lo terms in row group NG + g
+#pragma unroll
+                    for (int q = 0; q < CU; ++q) {
+                        const int cu = half + 2 * q;
+                        if (cu < NG) {
+                            const uint32_t off = (uint32_t)((((kt >> 3) * 2 * NG + cu) * 8 + (kt & 7)) * 16);
+                            *reinterpret_cast<uint4*>(p_hi + off) = make_uint4(hw[q][0], hw[q][1], hw[q][2], hw[q][3]);
+                            *reinterpret_cast<uint4*>(p_hi + off + NG * 128) = make_uint4(lw[q][0], lw[q][1], lw[q][2], lw[q][3]);
+                        }
                     }
                     // V rows at and beyond the split's end must be finite (P is 0 there, but 0 * NaN is not): cleared, once
                     // the tile's V rows have landed (the copy may bring garbage rows of the last 8-row group)
                     if (n_valid < kAttnTile) {
-                        if (ok) ok = attn_wait_warp(bar_full + 8 * ((2 * t + 1) % 3), (uint32_t)((2 * t + 1) / 3) & 1u);
+                        if (ok) ok = attn_wait_warp(bar_full + 8 * slot_of(2 * t + 1), turn_of(2 * t + 1));
                         if (half == 0 && kt >= n_valid && kt < ((n_valid + 15) & ~15)) {
-                            unsigned char* v_tile = ring + ((2 * t + 1) % 3) * SM::kTileBytes;
+                            unsigned char* v_tile = ring + slot_of(2 * t + 1) * SM::kTileBytes;
 #pragma unroll
                             for (int g = 0; g < HG; ++g)
                                 *reinterpret_cast<uint4*>(v_tile + ((kt >> 3) * HG + g) * 128 + (kt & 7) * 16) = make_uint4(0, 0, 0, 0);
@@ -510,8 +564,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
 #pragma unroll 1
                     for (int cu = half; cu < NG; cu += 2) {
                         float s[8];
-                        tmem_ld8(t_St + lane_sel + cu * 8, s);
-                        tmem_ld_wait8(s);
+                        read_s(t_St + lane_sel + cu * 8, s);
                         float mine = -INFINITY;
 #pragma unroll
                         for (int i = 0; i < 8; ++i) {
@@ -532,12 +585,12 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
                     asm volatile("bar.sync 1, %0;" ::"n"(kAttnWorkers) : "memory");
                     if (t > 0) {
 #pragma unroll 1
-                        for (int cb = half; cb < 2 * NB; cb += 2) {                  // O^T and L: 2N columns from t_O
+                        for (int cb = half; cb < 2 * NO / 16; cb += 2) {             // O^T and L: all columns from t_O
                             float o[16];
                             tmem_ld16(t_O + lane_sel + cb * 16, o);
                             tmem_ld_wait16(o);
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) o[i] *= alpha[(cb < NB ? cb : cb - NB) * 16 + i];
+                            for (int i = 0; i < 16; ++i) o[i] *= alpha[(cb % NB) * 16 + i];
                             tmem_st16(t_O + lane_sel + cb * 16, o);
                         }
                         tmem_st_wait();
@@ -548,14 +601,25 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
             // ---- the CTA's partial result: O^T (thread = head dimension) and L (lanes 0-7 hold all rows' sums)
             if (ok) ok = attn_wait_warp(bar_pv, (uint32_t)(ntiles - 1) & 1u);
             tc_fence_after();
+            // sixteen columns of O^T or L: the products with P's hi terms, and those with its lo terms where they are apart
+            auto read_16 = [&](uint32_t at, float (&v)[16]) {
+                tmem_ld16(at, v);
+                tmem_ld_wait16(v);
+                if (wide_p) {
+                    float l[16];
+                    tmem_ld16(at + (uint32_t)N, l);
+                    tmem_ld_wait16(l);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) v[i] += l[i];
+                }
+            };
             if (quarter == 0) {
                 // the column blocks go to the two warps of the quarter the other way round than O^T's below, so that with
                 // one block the denominators are stored by a warp that has no O^T columns to store
 #pragma unroll 1
                 for (int cb = half ^ 1; cb < NB; cb += 2) {
                     float l[16];
-                    tmem_ld16(t_L + cb * 16, l);
-                    tmem_ld_wait();
+                    read_16(t_L + cb * 16, l);
                     if (lane == 0) {
 #pragma unroll
                         for (int i = 0; i < 16; ++i) Fl[cb * 16 + i] = ok ? l[i] : 0.f;
@@ -580,8 +644,7 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
 #pragma unroll 1
             for (int cb = half; cb < NB; cb += 2) {
                 float o[16];
-                tmem_ld16(t_O + lane_sel + cb * 16, o);
-                tmem_ld_wait();
+                read_16(t_O + lane_sel + cb * 16, o);
                 if (kt < HD) {
 #pragma unroll
                     for (int i = 0; i < 16; ++i) {
@@ -617,16 +680,31 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
     }
     if (nsplit == 1) { release_tmem(); return; }
 
-    // ---- the last CTA of this (request, KV head, row group) to arrive merges the splits, in split order
-    // (the barrier above orders the whole CTA's stores before thread 0's ticket, a release; the ticket is also an acquire,
-    // and the barrier below orders it before everybody's loads of the other CTAs' partials)
+    // ---- merge of the splits, in split order.  Either the last CTA of this (request, KV head, row group) to arrive does it,
+    // and nobody waits for anybody; or, where every CTA of the launch is resident and a group has more rows than one round
+    // of warps (nine) takes, all CTAs of the group wait for each other's partials and take every nsplit-th row each (68
+    // rows x 13 splits, 450 KB, take one SM 14 us).
+    // (the barrier above orders the whole CTA's stores before thread 0's ticket, a release; the ticket or the poll is also an
+    // acquire, and the barrier below orders it before everybody's loads of the other CTAs' partials)
+    const bool share = a.share_merge && n_rows > kAttnThreads / 32;
     if (tid == 0) {
+        // arrivals in the low half, in shared merges also departures in the high half; zero again when the last is through
         int* ticket = a.tickets + ((size_t)item * Hkv + kvh) * a.row_groups + rg;
         int t;
         asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
-        const int last = (t == nsplit - 1);
-        if (last) *ticket = 0;                                   // self-cleaning: ready for the next launch
-        *s_last = last;
+        int go = (t == nsplit - 1);
+        if (share) {
+            for (uint32_t it = 0; it < (1u << 20) && !go; ++it) {
+                asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(t) : "l"(ticket) : "memory");
+                go = (t & 0xffff) == nsplit;
+            }
+            if (!go && a.err) atomicExch(a.err, 10);
+            asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 65536;" : "=r"(t) : "l"(ticket) : "memory");
+            if ((t >> 16) == nsplit - 1) *ticket = 0;
+        } else if (go) {
+            *ticket = 0;                                         // self-cleaning: ready for the next launch
+        }
+        *s_last = go;
     }
     __syncthreads();
     release_tmem();
@@ -635,8 +713,9 @@ __global__ void __launch_bounds__(kAttnThreads, 3) attn_kernel(const AttnArgs a)
     // use (one trip to the L2 for up to kMergeBatch splits): lane j fetches split j's maximum and denominator, every
     // lane its four columns of each split's numerator; the sums run in split order.
     constexpr int kMergeBatch = 10;
+    const int rl_step = share ? nsplit : 1;
 #pragma unroll 1
-    for (int rl = warp; rl < n_rows; rl += kAttnThreads / 32) {
+    for (int rl = share ? sp + warp * nsplit : warp; rl < n_rows; rl += rl_step * (kAttnThreads / 32)) {
         const size_t sl0 = slot0 + (size_t)rl * nsplit;
         const float m_mine = lane < nsplit ? __ldcg(a.m_part + sl0 + lane) : -INFINITY;
         const float l_mine = lane < nsplit ? __ldcg(a.l_part + sl0 + lane) : 0.f;

@@ -167,6 +167,11 @@ constexpr int kMaxDevices = 64;
 std::mutex g_dev_mu;
 bool g_dev_ready[kMaxDevices] = {false};
 
+const void* attn_fn(int hd, bool big) {
+    if (big) return hd == 128 ? (const void*)attn_kernel<128, kAttnBigCols> : (const void*)attn_kernel<64, kAttnBigCols>;
+    return hd == 128 ? (const void*)attn_kernel<128, 1> : (const void*)attn_kernel<64, 1>;
+}
+
 cudaError_t init_attrs_current_device() {
     cudaError_t e;
     if ((e = gemm_init_attrs()) != cudaSuccess) return e;
@@ -176,14 +181,12 @@ cudaError_t init_attrs_current_device() {
         if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kDenseSmem)) != cudaSuccess) return e;
         if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess) return e;
     }
-    e = cudaFuncSetAttribute(attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_smem_bytes(128, kAttnMaxRows, false));
-    if (e != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(attn_kernel<128>, cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)attn_smem_bytes(64, kAttnMaxRows, false));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(attn_kernel<64>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    for (int hd : {64, 128})
+        for (bool big : {false, true}) {
+            if ((e = cudaFuncSetAttribute(attn_fn(hd, big), cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmemMax)) != cudaSuccess) return e;
+            if ((e = cudaFuncSetAttribute(attn_fn(hd, big), cudaFuncAttributePreferredSharedMemoryCarveout, 100)) != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
 int ensure_device_ready() {
@@ -455,7 +458,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
     auto I = [&](size_t off) { return reinterpret_cast<int32_t*>(hm + off); };
     float* hu = reinterpret_cast<float*>(hm + ml.u);
     RejectItem* hr = reinterpret_cast<RejectItem*>(hm + ml.rej);
-    int row = 0, part0 = 0, max_nsplit = 1, u0 = 0;
+    int row = 0, part0 = 0, max_nsplit = 1, u0 = 0, attn_ctas = 0;
     bool all_short = true;       // no split of the pass has more than two key tiles, the second a short one
     // attention work of the pass in (keys x CTA groups): a request gets the share of the device's resident CTAs that its
     // keys are of the pass's, so that the CTAs of the whole pass fill one wave
@@ -513,6 +516,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
         I(ml.it_chunk)[i] = chunk;
         I(ml.it_part0)[i] = part0;
         max_nsplit = std::max(max_nsplit, nsplit);
+        attn_ctas += nsplit * c.n_kv_heads * rg_i;
         part0 += it.rows * c.n_q_heads * nsplit;
         hr[i].row0 = row;
         hr[i].k = it.k;
@@ -587,7 +591,9 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
         AttnArgs aa = {};
         aa.q = qbuf; aa.meta = meta; aa.kv_pool = ctx->kv_pool;
         aa.layer = l; aa.n_pages = c.n_pages; aa.page_size = c.page_size; aa.M = M; aa.Hq = Hq; aa.Hkv = Hkv;
-        aa.rows_cap = rows_cap; aa.n_max = n_max; aa.slot_c = attn_slot_c_bytes(hd, all_short); aa.row_groups = row_groups;
+        aa.rows_cap = rows_cap; aa.n_max = n_max; aa.row_groups = row_groups;
+        aa.slots = attn_ring_slots(hd, n_max); aa.ring = attn_ring_bytes(hd, aa.slots, all_short);
+        aa.share_merge = attn_ctas <= ctx->attn_slots[n_max / 16][all_short ? 1 : 0];
         aa.o_part = o_part; aa.m_part = m_part; aa.l_part = l_part; aa.tickets = ctx->W<int>(ctx->ws.tickets);
         aa.xf_out = (uint16_t*)xf_attn; aa.xd_tbs = tbs_o; aa.err = ctx->err_word();
         if (!dense) {
@@ -597,8 +603,14 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
             aa.pf_ptr[1] = reinterpret_cast<const unsigned char*>(lw.gu.packed);
             aa.pf_len[1] = std::min(gemm_packed_bytes(2 * F, d), ctx->pf_attn[1]);
         }
-        if (hd == 128) CU(launch_pdl(attn_kernel<128>, ag, dim3(kAttnThreads), asmem, st, aa));
-        else CU(launch_pdl(attn_kernel<64>, ag, dim3(kAttnThreads), asmem, st, aa));
+        const dim3 ab(kAttnThreads);
+        if (n_max <= 16) {
+            if (hd == 128) CU(launch_pdl(attn_kernel<128, 1>, ag, ab, asmem, st, aa));
+            else CU(launch_pdl(attn_kernel<64, 1>, ag, ab, asmem, st, aa));
+        } else {
+            if (hd == 128) CU(launch_pdl(attn_kernel<128, kAttnBigCols>, ag, ab, asmem, st, aa));
+            else CU(launch_pdl(attn_kernel<64, kAttnBigCols>, ag, ab, asmem, st, aa));
+        }
         ctx->n_launch += 1;
         return PIPESD_OK;
     };
@@ -749,14 +761,13 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
             if (cudaOccupancyMaxActiveClusters(&n, gemm_dense_kernel<kQkvRope>, &lc) != cudaSuccess) return bail(PIPESD_E_CUDA);
             ctx->dense_pairs[S] = std::max(1, n * S);
         }
-        cudaFuncAttributes fa;
-        if (cudaFuncGetAttributes(&fa, c.head_dim == 128 ? (const void*)attn_kernel<128> : (const void*)attn_kernel<64>) != cudaSuccess)
-            return bail(PIPESD_E_CUDA);
-        // registers: allocated per warp (in units of 512), and a CTA's warps are dealt to the SM's four register
-        // partitions in turn, so the fullest partition binds
-        const int regs_warp = (fa.numRegs * 32 + 511) / 512 * 512;
-        const int warps_part = (kAttnThreads / 32 + 3) / 4;
-        for (int qt = 1; qt <= kAttnMaxRows / 16; ++qt)
+        for (int qt = 1; qt <= kAttnMaxRows / 16; ++qt) {
+            cudaFuncAttributes fa;
+            if (cudaFuncGetAttributes(&fa, attn_fn(c.head_dim, qt > 1)) != cudaSuccess) return bail(PIPESD_E_CUDA);
+            // registers: allocated per warp (in units of 512), and a CTA's warps are dealt to the SM's four register
+            // partitions in turn, so the fullest partition binds
+            const int regs_warp = (fa.numRegs * 32 + 511) / 512 * 512;
+            const int warps_part = (kAttnThreads / 32 + 3) / 4;
             for (int short_tail = 0; short_tail < 2; ++short_tail) {
                 const size_t smem_cta = attn_smem_bytes(c.head_dim, 16 * qt, short_tail != 0) + fa.sharedSizeBytes + smem_rsv;
                 int per_sm = (int)(smem_sm / smem_cta);
@@ -765,6 +776,7 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
                 per_sm = std::min(per_sm, 512 / attn_tmem_cols(16 * qt));
                 ctx->attn_slots[qt][short_tail] = std::max(1, per_sm) * n_sm;
             }
+        }
     }
     ctx->kv_pool = (uint16_t*)mem->kv;
     ctx->wsp = (char*)mem->workspace;
