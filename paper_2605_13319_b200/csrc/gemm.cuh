@@ -82,6 +82,9 @@ static inline GemmPlan gemm_plan(int M, int N, int K) {
         if (s > 1 && p.KS / s < 2 * kGemmKC) break;
         if ((long)p.RB * s <= kGemmWave) best = s;
     }
+    // Between half and a whole wave of row blocks (two slices would not fit it): slices of a fifth instead, two to three waves
+    // of short CTAs, whose starts and ends overlap (8b shape, gate/up of 17 rows, 224 row blocks: pass 5145 -> 5025 us).
+    if (best == 1 && 2 * p.RB > kGemmWave && p.RB < kGemmWave && p.KS >= 5 * 2 * kGemmKC) best = 5;
     p.S = best;
     // ring depth: as deep as the shared memory of an SM allows for the number of CTAs it will hold.  A clustered
     // GEMM always leaves room for three CTAs per SM, even when it brings fewer: at two 113 KB CTAs per SM a B200
@@ -92,7 +95,9 @@ static inline GemmPlan gemm_plan(int M, int N, int K) {
     // (7b, 17 rows: 3.81 ms with five stages, 4.00 ms with three), so those keep the depth by CTA count.
     long ctas = (long)p.RB * p.S * p.TB;
     int per_sm = (int)((ctas + 147) / 148);
-    if (p.S > 1 && p.NT <= 2) per_sm = kGemmCtasPerSm;
+    // A launch of at most one CTA per SM keeps room for one other only: its ring is all the SM has in flight (1b shape, k = 8,
+    // O and down of 128 CTAs: pass 1070 -> 1009 us with five stages instead of three).
+    if (p.S > 1 && p.NT <= 2) per_sm = ctas <= 148 ? 2 : kGemmCtasPerSm;
     per_sm = per_sm < 1 ? 1 : (per_sm > kGemmCtasPerSm ? kGemmCtasPerSm : per_sm);
     int budget = (227 * 1024) / per_sm - 1024 - kGemmSmemTail - gemm_recv_bytes(p.NT, p.S);
     p.stages = budget / gemm_stage_bytes(p.NT);
@@ -140,7 +145,9 @@ __global__ void gemm_pack_kernel(PackSrc src, uint4* __restrict__ packed, int n_
                 lr = src.mode == kQkvRope ? qkv_logical_row(pr, src.hd) : pr;
                 while (which < 2 && lr >= src.rows[which]) { lr -= src.rows[which]; ++which; }
             }
-            v = *reinterpret_cast<const uint4*>(src.w[which] + (size_t)lr * K + 8 * kgq);
+            const uint16_t* w = src.w[which] + (size_t)lr * K + 8 * kgq;
+            if (((uintptr_t)w & 15) == 0) v = *reinterpret_cast<const uint4*>(w);
+            else v = make_uint4(pack2(w[0], w[1]), pack2(w[2], w[3]), pack2(w[4], w[5]), pack2(w[6], w[7]));   // a view at an odd offset
         }
         const int rb = pr >> 7, r = pr & 127, ks = kgq >> 1, kg = kgq & 1;
         packed[((size_t)rb * KS + ks) * 256 + ((r >> 3) * 2 + kg) * 8 + (r & 7)] = v;

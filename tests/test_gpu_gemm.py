@@ -41,6 +41,27 @@ def test_gemm_matches_oracle(M, N, K):
     assert np.abs(y.cpu().numpy() - want2).max() < 3e-5 * scale * 12
 
 
+@pytest.mark.parametrize("M,N,K,offset", [
+    (17, 28672, 640, 0), (9, 28432, 656, 0),      # more than half a wave of row blocks: slices of a fifth, two to three waves
+    (9, 2048, 2048, 0),                           # at most one CTA per SM: the deeper ring
+    (5, 272, 256, 1), (5, 272, 256, 4),           # weights at an address that is no multiple of 16 bytes
+])
+def test_gemm_plans_and_alignment(M, N, K, offset):
+    import torch
+    from paper_2605_13319_b200 import binding
+    dev = torch.device("cuda", 0)
+    W = synth.normal_bf16((N, K), 13, 40 + M, 0.02)
+    x = synth.normal_f32((M, K), 13, 80 + M, 1.0)
+    want = oracle.linear(W, x.astype(np.float64))
+    flat = torch.zeros(N * K + 8, dtype=torch.int16, device=dev)
+    flat[offset:offset + N * K] = torch.from_numpy(W.view(np.int16)).to(dev).reshape(-1)
+    packed = binding.gemm_pack(flat[offset:offset + N * K].view(N, K))
+    y = torch.full((M, N), float("nan"), device=dev)
+    binding.gemm_run(packed, torch.from_numpy(x).to(dev), y, binding.gemm_scratch(M, N, K, dev), N, K)
+    torch.cuda.synchronize()
+    assert np.abs(y.cpu().numpy() - want).max() < 3e-5 * 0.02 * np.sqrt(K) * 4      # as above
+
+
 def test_gemm_rejects_bad_shapes():
     from paper_2605_13319_b200 import binding
     L = binding.lib()
