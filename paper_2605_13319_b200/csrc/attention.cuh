@@ -15,8 +15,8 @@
 // with S^T (twice: two tiles in flight), O^T and L in tensor memory.  The cache stores, per page and
 // head, the rows in 8-row groups of 8-element pieces ([slot/8][hd/8][slot%8][8]), which IS the operand order of
 // both products (K-major for the first, MN-major for the second): a page lands in shared memory by one bulk copy
-// and is read by the tensor cores as it is.  Q and P are fp32 values split into bf16 hi + lo terms (two MMAs into
-// the same accumulator); K and V are the cache's bf16.
+// and is read by the tensor cores as it is.  Q and P are fp32 values split into bf16 hi + lo terms (see
+// attn_wide_q); K and V are the cache's bf16.
 // Warps 0-7: one thread per key of a tile (= tensor-memory lane; warps w and w+4 share a lane quarter and take
 // alternate 8-row column blocks): masking, exponentials relative to the score of the split's first key (any reference will
 // do that keeps p in range; a row's maximum is only looked for when a score exceeds its reference by 2^40 and O^T has to
@@ -683,7 +683,9 @@ __global__ void __launch_bounds__(kAttnThreads, CU == 1 ? 3 : 1) attn_kernel(con
     // ---- merge of the splits, in split order.  Either the last CTA of this (request, KV head, row group) to arrive does it,
     // and nobody waits for anybody; or, where every CTA of the launch is resident and a group has more rows than one round
     // of warps (nine) takes, all CTAs of the group wait for each other's partials and take every nsplit-th row each (68
-    // rows x 13 splits, 450 KB, take one SM 14 us).
+    // rows x 13 splits, 450 KB, take one SM 14 us).  The wait ends although other launches may hold SMs: a group's CTAs are
+    // neighbours in the grid, so of each launch at most one group, 16 CTAs, is only partly on the device, and every other
+    // one runs to its end; and it is bounded.
     // (the barrier above orders the whole CTA's stores before thread 0's ticket, a release; the ticket or the poll is also an
     // acquire, and the barrier below orders it before everybody's loads of the other CTAs' partials)
     const bool share = a.share_merge && n_rows > kAttnThreads / 32;

@@ -266,15 +266,6 @@ __device__ __forceinline__ void xf_store_one(uint16_t* xf, int tok, int k, float
 // Token blocks of `tbs` tokens (a multiple of 16).  Per (token block, k16 step): the bf16 hi tile then the lo tile,
 // tbs * 32 bytes each, cut into 8x8 core matrices: element (token t, k) of a tile at
 // ((t / 8) * 2 + (k / 8) % 2) * 128 + (t % 8) * 16 + (k % 8) * 2.
-__device__ __forceinline__ void xd_store_one(uint16_t* xd, int tok, int k, float v, int KS, int tbs) {
-    const int tb = tok / tbs, tl = tok % tbs;
-    uint16_t h, l;
-    split_bf16(v, h, l);
-    unsigned char* b = reinterpret_cast<unsigned char*>(xd) + ((size_t)tb * KS + (k >> 4)) * (size_t)(tbs * 64) +
-                       (((tl >> 3) * 2 + ((k >> 3) & 1)) * 128 + (tl & 7) * 16 + (k & 7) * 2);
-    *reinterpret_cast<uint16_t*>(b) = h;
-    *reinterpret_cast<uint16_t*>(b + tbs * 32) = l;
-}
 // In either layout an element's index (in 16-bit units) is the sum of a part fixed by its token and the first k16 step
 // ks0 of a block of columns, and a part fixed by the column's offset dk inside that block; the lo half follows the hi
 // half at a fixed distance.  Epilogues that walk tokens x columns compute each part once instead of dividing per element.
@@ -310,13 +301,6 @@ __device__ __forceinline__ void act_store_8(uint16_t* dst, uint32_t lo, const fl
     *reinterpret_cast<uint4*>(dst) = make_uint4(pack2(h[0], h[1]), pack2(h[2], h[3]), pack2(h[4], h[5]), pack2(h[6], h[7]));
     *reinterpret_cast<uint4*>(dst + lo) = make_uint4(pack2(l[0], l[1]), pack2(l[2], l[3]), pack2(l[4], l[5]), pack2(l[6], l[7]));
 }
-// Store one activation in whichever layout its consumer reads: tbs > 0: an xd array with that block size; tbs == 0:
-// the small-M kernel's fragment order with NT token tiles per block.
-__device__ __forceinline__ void act_store_one(uint16_t* dst, int tok, int k, float v, int KS, int NT, int tbs) {
-    if (tbs > 0) xd_store_one(dst, tok, k, v, KS, tbs);
-    else xf_store_one(dst, tok, k, v, KS, NT);
-}
-
 // ---- thread-block clusters: barrier and distributed shared memory --------------------------------
 __device__ __forceinline__ uint32_t cluster_ctarank() {
     uint32_t r;

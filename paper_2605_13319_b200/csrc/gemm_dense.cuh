@@ -43,7 +43,7 @@ static_assert(8 * (2 * kDenseMaxStages + 4) + 4 <= 256, "barriers and the tensor
 // Blocks of `tbs` tokens (a multiple of 16), one per CTA of a pair.  Per (block, k16 step): the bf16 hi tile then the lo
 // tile, tbs * 32 bytes each, cut into 8x8 core matrices: element (token t, k) of a tile at
 // ((t / 8) * 2 + (k / 8) % 2) * 128 + (t % 8) * 16 + (k % 8) * 2.  A chunk of consecutive k16 steps of a block is one
-// contiguous run.  (xd_store_one and act_store_one, next to the fragment-order stores, write these.)
+// contiguous run.  (act_index_row / act_index_col and act_store_8, next to the fragment-order stores, write these.)
 struct DensePlan {
     int tbs;      // tokens per CTA; a token block is 2 * tbs
     int n_tb;     // token blocks
@@ -76,6 +76,12 @@ static inline DensePlan dense_plan(int M, int N, int K, const int* pairs) {
         }
     }
     return best;
+}
+// The same where only the results of rows first_row .. M-1 are wanted (a prompt's last rows): blocks for that many rows.
+static inline DensePlan dense_plan_from(int M, int first_row, int N, int K, const int* pairs) {
+    DensePlan p = dense_plan(M - first_row, N, K, pairs);
+    p.n_tb = (M + 2 * p.tbs - 1) / (2 * p.tbs);
+    return p;
 }
 // Host: the ring.  As much of the shared memory as it gets.  A stage costs the issuer some 340 cycles of waiting and
 // committing beside its MMAs, so small steps are taken eight at a time (4096 x 11008, 32 tokens per CTA, us: 94 with two

@@ -35,11 +35,12 @@ __global__ void __launch_bounds__(kEmbedThreads) embed_kernel(float* __restrict_
             ss += a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w;
             const float4 g = *reinterpret_cast<const float4*>(gain + e);
             if (tbs > 0) {
-                uint16_t* xd = reinterpret_cast<uint16_t*>(xf_out);
-                xd_store_one(xd, row, e, a.x * g.x, KS, tbs);
-                xd_store_one(xd, row, e + 1, a.y * g.y, KS, tbs);
-                xd_store_one(xd, row, e + 2, a.z * g.z, KS, tbs);
-                xd_store_one(xd, row, e + 3, a.w * g.w, KS, tbs);
+                uint16_t* xd = reinterpret_cast<uint16_t*>(xf_out) + act_index_row(row, e >> 4, KS, 0, tbs) + act_index_col(e & 15, 0, tbs);
+                uint2 h, l;                                          // four neighbours of one 16-byte piece
+                split_bf16x2(a.x * g.x, a.y * g.y, h.x, l.x);
+                split_bf16x2(a.z * g.z, a.w * g.w, h.y, l.y);
+                *reinterpret_cast<uint2*>(xd) = h;
+                *reinterpret_cast<uint2*>(xd + act_index_lo(tbs)) = l;
             } else {
                 xf_store_pair(xf_out, row, e, a.x * g.x, a.y * g.y, KS, NT);
                 xf_store_pair(xf_out, row, e + 2, a.z * g.z, a.w * g.w, KS, NT);

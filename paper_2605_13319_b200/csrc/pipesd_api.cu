@@ -332,8 +332,9 @@ cudaError_t dense_launch_mode(const DenseArgs& da, dim3 grid, size_t smem, cudaS
 
 // Launch one weight-streaming GEMM with accounting (and event timing when profiling is on).  next_N, next_K: output rows and
 // depth of the GEMM that consumes this one's activation output (0: none): its token-block plan fixes the layout written.
-// first_row (dense, kPlain): results are wanted from this row on and stored from the start of the output.
-int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, int next_N, int next_K, int first_row = 0) {
+// first_row (dense, kPlain): results are wanted from this row on and stored from the start of the output; next_first: the
+// same of the consumer.
+int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, int next_N, int next_K, int first_row = 0, int next_first = 0) {
     a.err = ctx->err_word();
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     if (ctx->time_gemms) {
@@ -350,7 +351,7 @@ int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, in
         CU(cudaEventRecord(e0, ctx->st));
     }
     if (ctx->pass_dense) {
-        const DensePlan pin = dense_plan(a.M, a.N, K, ctx->dense_pairs);
+        const DensePlan pin = dense_plan_from(a.M, first_row, a.N, K, ctx->dense_pairs);
         const int tb0 = first_row / (2 * pin.tbs);
         DenseArgs da = {};
         da.g = a;
@@ -366,7 +367,7 @@ int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, in
         da.tb0 = tb0;
         da.n_tb = pin.n_tb - tb0;
         da.out_row0 = first_row;
-        da.tbs_out = next_N > 0 ? dense_plan(a.M, next_N, next_K, ctx->dense_pairs).tbs : 0;
+        da.tbs_out = next_N > 0 ? dense_plan_from(a.M, next_first, next_N, next_K, ctx->dense_pairs).tbs : 0;
         const size_t smem = ring.smem;
         cudaError_t e;
         switch (mode) {
@@ -650,7 +651,8 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
             a.ssq_out = ssqA;
             if (l + 1 < c.n_layers) a.pf = gemm_prefetch_of(ctx->layers[l + 1].qkv.packed, M, dv.Nqkv, d, pf_depth);
             else if (want_logits) a.pf = gemm_prefetch_of(ctx->lm.packed, M, c.vocab, d, pf_depth);
-            int rc_ = launch_gemm(ctx, kResid, lw.dn, a, F, l + 1 < c.n_layers ? dv.Nqkv : c.vocab, d);
+            int rc_ = launch_gemm(ctx, kResid, lw.dn, a, F, l + 1 < c.n_layers ? dv.Nqkv : c.vocab, d, 0,
+                                  l + 1 < c.n_layers || !want_logits ? 0 : M - n_logits);
             if (rc_) return rc_;
         }
     }

@@ -28,6 +28,7 @@ __global__ void __launch_bounds__(256) row_stats_kernel(int V, const float* __re
     const float* lr = logits + (size_t)row * V;
     float m = -INFINITY;
     int arg = 0x7fffffff;
+#pragma unroll 8
     for (int j = j0 + threadIdx.x; j < j1; j += 256) {
         const float v = lr[j];
         if (v > m) { m = v; arg = j; }
@@ -48,6 +49,7 @@ __global__ void __launch_bounds__(256) row_stats_kernel(int V, const float* __re
     for (int w = 1; w < 8; ++w)
         if (sm_m[w] > m || (sm_m[w] == m && sm_a[w] < arg)) { m = sm_m[w]; arg = sm_a[w]; }
     double z = 0.0;
+#pragma unroll 8
     for (int j = j0 + threadIdx.x; j < j1; j += 256) z += (double)expf(lr[j] - m);
     z = warp_sum_d(z);
     if ((threadIdx.x & 31) == 0) sm_z[threadIdx.x >> 5] = z;
@@ -193,15 +195,34 @@ __global__ void __launch_bounds__(kSampleThreads) accept_sample_kernel(const flo
     const int j0 = min(V, (rank * kWarps + warp) * R), j1 = min(V, j0 + R);
     bool use_q = n_acc < it.k;
     const float* qr = use_q ? it.q + (size_t)n_acc * V : nullptr;
-    auto term = [&](int j) -> double {
-        if (j >= j1) return 0.0;
-        double r = exp((double)lr[j] - m) * inv_z;
-        if (use_q) r = fmax(0.0, r - (double)qr[j]);
-        return r;
+    // The terms of kDrawBatch steps of 32 ids, this lane's: all loads in flight together, then the exponentials (one step at a
+    // time each costs a trip to the L2; 34 us at 128256 ids, where a walk has 16 steps).
+    constexpr int kDrawBatch = 8;
+    auto terms = [&](int j, double (&t)[kDrawBatch]) {
+        float l[kDrawBatch], q[kDrawBatch];
+#pragma unroll
+        for (int i = 0; i < kDrawBatch; ++i) {
+            const bool in = j + 32 * i < j1;
+            l[i] = in ? lr[j + 32 * i] : 0.f;
+            q[i] = in && use_q ? qr[j + 32 * i] : 0.f;
+        }
+#pragma unroll
+        for (int i = 0; i < kDrawBatch; ++i) {
+            t[i] = 0.0;
+            if (j + 32 * i < j1) {
+                t[i] = exp((double)l[i] - m) * inv_z;
+                if (use_q) t[i] = fmax(0.0, t[i] - (double)q[i]);
+            }
+        }
     };
     for (int attempt = 0; attempt < 2; ++attempt) {
         double loc = 0.0;
-        for (int j = j0 + lane; j < j1; j += 32) loc += term(j);
+        for (int j = j0 + lane; j < j1; j += 32 * kDrawBatch) {
+            double t[kDrawBatch];
+            terms(j, t);
+#pragma unroll
+            for (int i = 0; i < kDrawBatch; ++i) loc += t[i];
+        }
         const double wsum = warp_sum_d(loc);
         if (lane == 0) s_warp[warp] = wsum;
         __syncthreads();
@@ -244,18 +265,26 @@ __global__ void __launch_bounds__(kSampleThreads) accept_sample_kernel(const flo
         if (mine) {
             double run = before;
             int tok = -1, last_mass = -1;
-            for (int c = j0; c < j1 && tok < 0; c += 32) {
-                double inc = term(c + lane);
-                const unsigned mass = __ballot_sync(0xffffffffu, inc > 0.0);
-                if (mass) last_mass = c + 31 - __clz(mass);
+            for (int c0 = j0; c0 < j1 && tok < 0; c0 += 32 * kDrawBatch) {
+                double ts[kDrawBatch];
+                terms(c0 + lane, ts);
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    double t = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += t;
+                for (int i = 0; i < kDrawBatch; ++i) {
+                    const int c = c0 + 32 * i;
+                    if (c < j1 && tok < 0) {
+                        double inc = ts[i];
+                        const unsigned mass = __ballot_sync(0xffffffffu, inc > 0.0);
+                        if (mass) last_mass = c + 31 - __clz(mass);
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            double t = __shfl_up_sync(0xffffffffu, inc, o);
+                            if (lane >= o) inc += t;
+                        }
+                        const unsigned hit = __ballot_sync(0xffffffffu, run + inc > target && c + lane < j1);
+                        if (hit) tok = c + __ffs(hit) - 1;
+                        run += __shfl_sync(0xffffffffu, inc, 31);
+                    }
                 }
-                const unsigned hit = __ballot_sync(0xffffffffu, run + inc > target && c + lane < j1);
-                if (hit) tok = c + __ffs(hit) - 1;
-                run += __shfl_sync(0xffffffffu, inc, 31);
             }
             if (tok < 0) tok = last_mass;    // the walk's rounding fell short of the range's total: its last id with mass
             if (lane == 0) emit(n_acc, tok);
