@@ -25,3 +25,14 @@ def pytest_collection_modifyitems(config, items):
         for it in items:
             if "gpu" in it.keywords:
                 it.add_marker(skip)
+
+
+@pytest.fixture(autouse=True)
+def _collect_after_gpu_test(request):
+    """A test that catches an error keeps its frame, and with it a context's device buffers, alive in a reference cycle.
+    They go with the test, not whenever the collector next runs -- which may be between two readings of the allocator in
+    a later one."""
+    yield
+    if "gpu" in request.node.keywords:
+        import gc
+        gc.collect()
