@@ -247,6 +247,13 @@ int32_t pipesd_gemm_run(const void *packed, const float *x, float *y, void *scra
  * projections a large batch runs; the attention's key splits still follow the pass's composition, so the two agree
  * to rounding and in their decisions, not in every bit); needs max_rows > 32 (PIPESD_E_INVALID otherwise). */
 int32_t pipesd_debug_force_dense(pipesd_ctx *ctx, int32_t on);
+/* The dense kernel on its own, in a given plan: y[M,N] = x[M,K] . W[N,K]^T as pipesd_gemm_run computes it, with blocks of
+ * 2 * tokens_per_cta tokens (tokens_per_cta: a multiple of 16 up to 128) and K cut into `slices` (1..4) slices.  scratch:
+ * device, of pipesd_debug_gemm_dense_scratch_bytes(M, K, tokens_per_cta) bytes, 16-byte aligned.  PIPESD_E_INVALID (0
+ * bytes) for arguments outside these limits. */
+uint64_t pipesd_debug_gemm_dense_scratch_bytes(int32_t M, int32_t K, int32_t tokens_per_cta);
+int32_t pipesd_debug_gemm_dense(const void *packed, const float *x, float *y, void *scratch, int32_t M, int32_t N, int32_t K,
+                                int32_t tokens_per_cta, int32_t slices, void *cuda_stream);
 /* CTAs of the attention kernel that the context's device keeps resident at once for a request with this many query
  * rows per KV head: out2 (host) = {with the whole third ring slot, with the cut-down one} -- the two numbers
  * pipesd_debug_attn_split takes. */

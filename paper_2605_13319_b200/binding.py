@@ -97,6 +97,8 @@ _SIGNATURES = {
     "pipesd_sched_trigger_step": (i32, [ctypes.POINTER(ctypes.c_double), ctypes.c_double, ctypes.c_double,
                                         ctypes.c_double, ctypes.POINTER(i32)]),
     "pipesd_debug_force_dense": (i32, [vp, i32]),
+    "pipesd_debug_gemm_dense_scratch_bytes": (u64, [i32, i32, i32]),
+    "pipesd_debug_gemm_dense": (i32, [vp, vp, vp, vp, i32, i32, i32, i32, i32, vp]),
     "pipesd_debug_attn_slots": (i32, [vp, i32, ctypes.POINTER(ctypes.c_int32)]),
     "pipesd_debug_attn_split": (i32, [i32, i32, ctypes.POINTER(ctypes.c_int32), i32, ctypes.POINTER(ctypes.c_int32)]),
     "pipesd_debug_req_state": (i32, [vp, i32, ctypes.POINTER(ctypes.c_int32)]),
@@ -376,6 +378,21 @@ def gemm_run_static(packed, x, y, N, K, stream=None):
     rc = lib().pipesd_gemm_run_static(packed.data_ptr(), x.data_ptr(), y.data_ptr(), M, N, K, vp(st.cuda_stream))
     if rc != OK:
         raise PipesdError(rc, "pipesd_gemm_run_static")
+
+
+def debug_gemm_dense(packed, x, y, scratch, N, K, tokens_per_cta, slices):
+    """The dense projection kernel alone, in a given plan.  scratch: uint8 tensor of at least
+    pipesd_debug_gemm_dense_scratch_bytes(M, K, tokens_per_cta) bytes."""
+    import torch
+    M = x.shape[0]
+    assert x.dtype == torch.float32 and y.dtype == torch.float32 and x.is_contiguous() and y.is_contiguous()
+    assert x.shape[1] == K and tuple(y.shape) == (M, N)
+    assert scratch.numel() * scratch.element_size() >= lib().pipesd_debug_gemm_dense_scratch_bytes(M, K, tokens_per_cta)
+    st = torch.cuda.current_stream(x.device)
+    rc = lib().pipesd_debug_gemm_dense(packed.data_ptr(), x.data_ptr(), y.data_ptr(), scratch.data_ptr(), M, N, K,
+                                       tokens_per_cta, slices, vp(st.cuda_stream))
+    if rc != OK:
+        raise PipesdError(rc, "pipesd_debug_gemm_dense")
 
 
 def debug_attn_split(total_keys: int, page_size: int, resident_ctas, units: int):

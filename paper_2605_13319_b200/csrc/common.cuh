@@ -137,12 +137,6 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity)
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// A remote arrival that orders nothing of this thread's own: it passes on a phase that the copy engine completed in this
-// CTA's shared memory (the data are there before that phase turns).  The releasing form above drains the thread's memory
-// operations first, 600 cycles and more, which a thread that reports every ring stage cannot afford.
-__device__ __forceinline__ void mbar_forward_cluster(uint32_t bar) {
-    asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
-}
 // Contiguous global -> shared copy by the copy engine; completion is counted in bytes on `bar`.
 // Both addresses 16-byte aligned, size a multiple of 16.
 __device__ __forceinline__ void bulk_g2s(uint32_t dst_smem, const void* src, uint32_t bytes, uint32_t bar) {

@@ -7,7 +7,7 @@
 // MMAs per k16 step into one fp32 accumulator.
 // What bounds it: the tensor pipe takes N/2 cycles per MMA, but every MMA fetches its operands from shared memory at 128 B
 // per cycle (32 cycles for a CTA's 128 weight rows, N/4 for N tokens), and the copies into the ring need the same
-// bandwidth.  One CTA alone with 128 x 256 tiles would want 344 cycles of shared memory per k16 step against 256 of math,
+// bandwidth.  One CTA alone with 128 x 256 tiles would want 352 cycles of shared memory per k16 step against 256 of math,
 // and 20 KB of L2 per step; a pair halves the token side: 224 against 256 cycles, 12 KB.
 // Sums: the tensor pipe truncates each accumulation, so a long K in one accumulator drifts (7b shape, layer 31's K after a
 // 160-token prompt: relative L1 error 3.6e-3 with one accumulator over all of K, 2.6e-3 with the small-M kernel's slices).
@@ -16,11 +16,16 @@
 // K slices: where row pairs x token blocks leave SMs idle, S <= 4 pairs form a cluster and share K; the partial tiles cross
 // the cluster through distributed shared memory (into the drained ring), each pair sums and finishes every S-th 16-token
 // column block, slices in order.
-// Warp 0: one lane streams (weights, activations) into the ring (weights before the dependent-launch wait).  Warp 1: one
-// lane of the even CTA issues the MMAs, one of the odd CTA passes "this stage has landed here" on to it; tcgen05.commit
-// frees a stage / hands an accumulator over in both CTAs.  Warp 2: tensor memory.  Warps 4-11: accumulators and epilogue
-// (thread = weight row x half of the tokens, then token x weight rows).
+// Warp 0: one lane of each CTA streams (weights, activations) into its ring (weights before the dependent-launch wait), by
+// tensor copies of the pair (cta_group::2) whose bytes count on the EVEN CTA's barrier: that barrier alone tells the issuer
+// that a stage has landed in both.  (A thread of the odd CTA that waits for its own copies and then arrives remotely is
+// either unordered, if the arrival is relaxed, or slow: the release takes 600 cycles; 1024 rows x 12288 x 4096, us: relaxed
+// 167, released by three threads in turn 181, this 167.)  Warp 1 of the even CTA: one lane issues the MMAs;
+// tcgen05.commit frees a stage / hands an accumulator over in both CTAs.  Warp 2: tensor memory.  Warps 4-11: accumulators
+// and epilogue (thread = weight row x half of the tokens, then token x weight rows).
 #pragma once
+#include <cuda.h>
+
 #include <algorithm>
 
 #include "common.cuh"
@@ -102,8 +107,12 @@ __host__ __device__ constexpr int dense_tmem_cols(int tbs) {      // two accumul
     return c;
 }
 
+// Packed weights and xd arrays as the copy engine sees them: rows of 1 KB, of which a run of k16 steps is a box.  Maps for
+// boxes of 8 and 4 steps (the stages' sizes) and for single steps (the remainder of a slice).
+struct RunMaps { CUtensorMap by8, by4, by1; };
 struct DenseArgs {
-    GemmArgs g;         // W = packed weights; xf = input xd array; S = K slices; the mode's outputs as for the small-M kernel
+    RunMaps w, t;       // weights, tokens (the input xd array)
+    GemmArgs g;         // S = K slices; the mode's outputs as for the small-M kernel; W and xf are not read
     int kc;             // k16 steps per ring stage (g.stages stages)
     int tbs_in;         // block size of the input array and of this launch
     int tbs_out;        // block size of the xd array this launch produces (kResid, kSwiglu)
@@ -111,10 +120,24 @@ struct DenseArgs {
     int out_row0;       // kPlain: the token whose result is row 0 of the output (earlier tokens are not stored)
 };
 
+// fp32 x[M][K] -> an xd array of blocks of tbs tokens (the component entry point; in a pass the producing kernels write it).
+// One thread per (token, eight k).
+__global__ void xd_format_kernel(const float* __restrict__ x, uint16_t* __restrict__ xd, int M, int K, int tbs) {
+    const int KS = K / 16, per_tok = K / 8;
+    const size_t n = (size_t)M * per_tok;
+    for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+        const int tok = (int)(i / per_tok), k = 8 * (int)(i % per_tok);
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = x[(size_t)tok * K + k + e];
+        act_store_8(xd + act_index_row(tok, k >> 4, KS, 0, tbs) + act_index_col(k & 15, 0, tbs), act_index_lo(tbs), v);
+    }
+}
+
 // grid (2 * S * row pairs * n_tb), clusters of 2 * S: cluster rank = 2 * slice + CTA of the pair.  The token blocks of a
 // row pair are neighbours in the launch order, so that they read its weights from HBM once.
 template <int MODE>
-__global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const DenseArgs da) {
+__global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const __grid_constant__ DenseArgs da) {
     const GemmArgs& a = da.g;
     extern __shared__ __align__(128) unsigned char smem[];
     const int TBS = da.tbs_in, NT = 2 * TBS;                           // tokens per CTA / per block
@@ -143,7 +166,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const Dens
 
     if (threadIdx.x == 0) {
         for (int i = 0; i < stages; ++i) {
-            mbar_init(full0 + 8 * i, r == 0 ? 2 : 1);                  // the copies; in the even CTA also the odd one's report
+            mbar_init(full0 + 8 * i, 1);                               // the even CTA's: bytes of both CTAs' copies (the odd one's is not used)
             mbar_init(empty0 + 8 * i, 1);
         }
         for (int i = 0; i < 2; ++i) {
@@ -155,6 +178,10 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const Dens
     if (warp == 2) {
         tmem2_alloc(smem_u32(tmem_slot), tmem_cols);
         tc_fence_before();
+    }
+    if (threadIdx.x == 96) {
+        tensor_map_prefetch(KC == 8 ? &da.w.by8 : &da.w.by4);
+        tensor_map_prefetch(KC == 8 ? &da.t.by8 : &da.t.by4);
     }
     cluster_sync_all();                                                // barriers of all CTAs are in place
     pdl_launch_dependents();
@@ -168,19 +195,34 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const Dens
     if (warp == 0) {
         // ---------------- producer: lane 0 streams (weights, activations) into the ring
         if (lane == 0) {
-            const unsigned char* wsrc = reinterpret_cast<const unsigned char*>(a.W) + ((size_t)min(rb, RB - 1) * KS + ks0) * 4096;
-            const unsigned char* bsrc = reinterpret_cast<const unsigned char*>(a.xf) + ((size_t)(2 * tb + r) * KS + ks0) * (TBS * 64);
+            const int wrow = (min(rb, RB - 1) * KS + ks0) * 4, trow = ((2 * tb + r) * KS + ks0) * (TBS / 16);     // in rows of 1 KB
+            const uint32_t lead_full = dsmem_addr(full0, rank & ~1u);
             auto steps = [&](int c) { return min(KC, nks - c * KC); };
+            auto box = [](int left) { return left >= 8 ? 8 : left >= 4 ? 4 : 1; };                   // steps of the next copy
             const uint64_t pol = l2_evict_first_policy();
             auto weights = [&](int c, int st) {
                 const int kc = steps(c);
-                mbar_expect_tx(full0 + 8 * st, (uint32_t)kc * (4096 + TBS * 64));
+                const uint32_t dst = smem_base + st * stage_bytes, bar = lead_full + 8 * st;
+                // the other CTA's bytes may count before this: the phase cannot complete without this arrival
+                if (r == 0) mbar_expect_tx(full0 + 8 * st, 2u * (uint32_t)kc * (4096 + TBS * 64));
                 // weights that other token blocks read as well stay in L2 like any line; read once, they leave first
-                if (da.n_tb == 1) bulk_g2s_hint(smem_base + st * stage_bytes, wsrc + (size_t)c * w_stage, (uint32_t)kc * 4096, full0 + 8 * st, pol);
-                else bulk_g2s(smem_base + st * stage_bytes, wsrc + (size_t)c * w_stage, (uint32_t)kc * 4096, full0 + 8 * st);
+                for (int i = 0; i < kc;) {
+                    const int n = box(kc - i);
+                    const CUtensorMap* m = n == 8 ? &da.w.by8 : n == 4 ? &da.w.by4 : &da.w.by1;
+                    if (da.n_tb == 1) tensor2_g2s_hint(dst + i * 4096, m, wrow + (c * KC + i) * 4, bar, pol);
+                    else tensor2_g2s(dst + i * 4096, m, wrow + (c * KC + i) * 4, bar);
+                    i += n;
+                }
             };
             auto tokens = [&](int c, int st) {
-                bulk_g2s(smem_base + st * stage_bytes + w_stage, bsrc + (size_t)c * (KC * TBS * 64), (uint32_t)steps(c) * (TBS * 64), full0 + 8 * st);
+                const int kc = steps(c);
+                const uint32_t dst = smem_base + st * stage_bytes + w_stage, bar = lead_full + 8 * st;
+                for (int i = 0; i < kc;) {
+                    const int n = box(kc - i);
+                    const CUtensorMap* m = n == 8 ? &da.t.by8 : n == 4 ? &da.t.by4 : &da.t.by1;
+                    tensor2_g2s(dst + i * (TBS * 64), m, trow + (c * KC + i) * (TBS / 16), bar);
+                    i += n;
+                }
             };
             // weights do not depend on the previous kernel: start them before the dependency wait
             const int pre = n_stage < stages ? n_stage : stages;
@@ -199,9 +241,11 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const Dens
             }
             if (!ok) {
                 if (a.err) atomicExch(a.err, 6);
-                // give up: let every copy already issued land before this CTA's shared memory is released
-                for (int c = issued > stages ? issued - stages : 0; c < issued; ++c)
-                    mbar_wait(full0 + 8 * (c % stages), (c / stages) & 1);
+                // give up: let every copy already issued land before shared memory is released (the odd CTA's count here too,
+                // and it stays for the even one at the cluster barrier below)
+                if (r == 0)
+                    for (int c = issued > stages ? issued - stages : 0; c < issued; ++c)
+                        mbar_wait(full0 + 8 * (c % stages), (c / stages) & 1);
             }
         }
         __syncwarp();
@@ -238,19 +282,6 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const Dens
                 if (ok) umma2_commit(acc_full + 8 * (ch & 1), mask);
             }
             if (!ok && a.err) atomicExch(a.err, 7);
-        }
-        __syncwarp();
-    } else if (warp == 1) {
-        // ---------------- odd CTA: report landed stages to the issuer
-        if (lane == 0) {
-            int st = 0;
-            uint32_t ph = 0;
-            for (int c = 0; c < n_stage && ok; ++c) {
-                ok = mbar_wait(full0 + 8 * st, ph);
-                if (ok) mbar_forward_cluster(dsmem_addr(full0 + 8 * st, rank ^ 1u));
-                if (++st == stages) { st = 0; ph ^= 1u; }
-            }
-            if (!ok && a.err) atomicExch(a.err, 8);
         }
         __syncwarp();
     }

@@ -41,6 +41,7 @@ struct Request {
 struct GemmW {
     uint4* packed = nullptr;     // operand order of both projection kernels (gemm_pack_kernel)
     int N = 0, K = 0;
+    RunMaps maps;                // the same for the dense kernel's copies
 };
 
 struct LayerW {
@@ -110,6 +111,8 @@ struct WsLayout {
         block_tab, qstage, req_state, never_flag, total;
 };
 
+constexpr size_t kXdPad = 2 * kDenseMaxHalf + 16;
+
 WsLayout ws_layout(const pipesd_model_cfg& c, const Derived& d) {
     WsLayout w;
     size_t o = 0;
@@ -117,11 +120,10 @@ WsLayout ws_layout(const pipesd_model_cfg& c, const Derived& d) {
     const size_t M = d.row_cap, Mv = c.max_rows;
     w.x = take(4 * M * c.d_model);
     // split-bf16 activation arrays: 4 bytes per element, token count padded to whole token blocks of the dense kernel
-    constexpr size_t kPad = 2 * kDenseMaxHalf + 16;
-    w.xf_h = take(4 * (M + kPad) * c.d_model);
+    w.xf_h = take(4 * (M + kXdPad) * c.d_model);
     w.qbuf = take(4 * M * d.qd);
-    w.xf_attn = take(4 * (M + kPad) * d.qd);
-    w.xf_act = take(4 * (M + kPad) * c.d_ffn);
+    w.xf_attn = take(4 * (M + kXdPad) * d.qd);
+    w.xf_act = take(4 * (M + kXdPad) * c.d_ffn);
     w.logits = take(4 * Mv * c.vocab);
     w.partA = take(4 * d.part_floats);
     w.partB = take(4 * d.part_floats);
@@ -200,6 +202,29 @@ int ensure_device_ready() {
     return PIPESD_OK;
 }
 
+// A contiguous device array cut into k16 steps of `step_bytes` (a multiple of 1 KB), as maps for the dense kernel's copies.
+bool make_run_maps(RunMaps* m, const void* base, size_t bytes, size_t step_bytes) {
+    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const Encode encode = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? (Encode)fn : (Encode) nullptr;
+    }();
+    if (!encode) return false;
+    CUtensorMap* maps[3] = {&m->by8, &m->by4, &m->by1};
+    const int steps[3] = {8, 4, 1};
+    for (int i = 0; i < 3; ++i) {
+        const cuuint64_t dims[2] = {256, bytes / 1024}, strides[1] = {1024};
+        const cuuint32_t box[2] = {256, (cuuint32_t)(step_bytes / 1024 * steps[i])}, ones[2] = {1, 1};
+        if (encode(maps[i], CU_TENSOR_MAP_DATA_TYPE_UINT32, 2, (void*)base, dims, strides, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return false;
+    }
+    return true;
+}
+
 int check_cfg(const pipesd_model_cfg* c) {
     if (!c) return PIPESD_E_INVALID;
     if (c->n_layers < 1 || c->d_model < 16 || c->n_q_heads < 1 || c->n_kv_heads < 1 || c->d_ffn < 16 ||
@@ -269,6 +294,7 @@ struct pipesd_ctx {
     int last_rows = 0;
     int attn_slots[kAttnMaxRows / 16 + 1][2] = {};   // [query rows / 16][cut-down third ring slot]: CTAs of the attention
                                                      // kernel the device keeps resident at once
+    RunMaps xd_maps[3][kDenseMaxHalf / 16];      // [xf_h, xf_attn, xf_act][tokens per block / 16 - 1]
     int dense_pairs[kDenseMaxSlices + 1] = {};   // [K slices]: CTA pairs of the dense kernel the device keeps resident at once
     bool force_dense = false;   // harness switch: the dense kernels also for passes of at most 32 rows
     bool pass_dense = false;    // the pass being enqueued runs on the dense kernels
@@ -355,7 +381,9 @@ int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, in
         const int tb0 = first_row / (2 * pin.tbs);
         DenseArgs da = {};
         da.g = a;
-        da.g.W = w.packed;
+        const int src = a.xf == ctx->W<uint4>(ctx->ws.xf_h) ? 0 : a.xf == ctx->W<uint4>(ctx->ws.xf_attn) ? 1 : 2;
+        da.w = w.maps;
+        da.t = ctx->xd_maps[src][pin.tbs / 16 - 1];
         da.g.KS = K / 16;
         da.g.S = pin.S;
         const dim3 grid(2 * pin.S * (((a.N + 127) / 128 + 1) / 2) * (pin.n_tb - tb0));
@@ -802,6 +830,12 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
     char* wp = (char*)mem->weights;
     size_t off = 0;
     auto take = [&](size_t bytes) { char* p = wp + off; off += align_up(bytes); return p; };
+    bool maps_ok = true;
+    for (int tbs = 16; tbs <= kDenseMaxHalf; tbs += 16) {
+        const size_t at[3] = {ctx->ws.xf_h, ctx->ws.xf_attn, ctx->ws.xf_act}, k[3] = {(size_t)c.d_model, (size_t)dv.qd, (size_t)c.d_ffn};
+        for (int i = 0; i < 3; ++i)
+            maps_ok = maps_ok && make_run_maps(&ctx->xd_maps[i][tbs / 16 - 1], ctx->wsp + at[i], 4 * (dv.row_cap + kXdPad) * k[i], 64 * (size_t)tbs);
+    }
     auto pack = [&](GemmW& g, int N, int K, int mode, std::initializer_list<std::pair<const void*, int>> srcs) {
         g.N = N;
         g.K = K;
@@ -814,6 +848,7 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
         int blocks = (int)std::min<size_t>((total + 255) / 256, 148 * 16);
         g.packed = (uint4*)take(gemm_packed_bytes(N, K));
         gemm_pack_kernel<<<blocks, 256, 0, st>>>(ps, g.packed, N, K);
+        maps_ok = maps_ok && make_run_maps(&g.maps, g.packed, gemm_packed_bytes(N, K), 4096);
     };
     ctx->emb = (uint16_t*)take((size_t)c.vocab * c.d_model * 2);
     if (cudaMemcpyAsync(ctx->emb, w->tok_emb, (size_t)c.vocab * c.d_model * 2, cudaMemcpyDeviceToDevice, st) !=
@@ -837,7 +872,7 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
     pack(ctx->lm, c.vocab, c.d_model, kPlain, {{w->lm_head, c.vocab}});
     ctx->final_norm = (float*)take(4 * (size_t)c.d_model);
     cudaMemcpyAsync(ctx->final_norm, w->final_norm, 4 * (size_t)c.d_model, cudaMemcpyDeviceToDevice, st);
-    if (cudaGetLastError() != cudaSuccess) return bail(PIPESD_E_CUDA);
+    if (!maps_ok || cudaGetLastError() != cudaSuccess) return bail(PIPESD_E_CUDA);
 
     ctx->reqs.resize(c.max_requests);
     ctx->free_pages.resize(c.n_pages);
@@ -1304,6 +1339,43 @@ int32_t pipesd_gemm_run(const void* packed, const float* x, float* y, void* scra
     if (!packed || !x || !y || !scratch || M < 1 || N < 16 || K < 16 || N % 16 || K % 16) return PIPESD_E_INVALID;
     if (ensure_device_ready() != PIPESD_OK) return PIPESD_E_CUDA;
     return gemm_run_with_scratch(packed, x, y, scratch, M, N, K, (cudaStream_t)cuda_stream);
+}
+
+static bool dense_forced_ok(int M, int N, int K, int tbs, int slices) {
+    return M >= 1 && N >= 16 && K >= 16 && N % 16 == 0 && K % 16 == 0 && tbs >= 16 && tbs <= kDenseMaxHalf && tbs % 16 == 0 &&
+           slices >= 1 && slices <= kDenseMaxSlices && slices <= K / 16;
+}
+static int dense_forced_blocks(int M, int tbs) { return (M + 2 * tbs - 1) / (2 * tbs); }
+
+uint64_t pipesd_debug_gemm_dense_scratch_bytes(int32_t M, int32_t K, int32_t tokens_per_cta) {
+    if (!dense_forced_ok(M, 16, K, tokens_per_cta, 1)) return 0;
+    return align_up((size_t)dense_forced_blocks(M, tokens_per_cta) * 2 * tokens_per_cta * K * 4);
+}
+
+int32_t pipesd_debug_gemm_dense(const void* packed, const float* x, float* y, void* scratch, int32_t M, int32_t N, int32_t K,
+                                int32_t tokens_per_cta, int32_t slices, void* cuda_stream) {
+    if (!packed || !x || !y || !scratch || !dense_forced_ok(M, N, K, tokens_per_cta, slices)) return PIPESD_E_INVALID;
+    if (ensure_device_ready() != PIPESD_OK) return PIPESD_E_CUDA;
+    cudaStream_t st = (cudaStream_t)cuda_stream;
+    const size_t pieces = (size_t)M * (K / 8);
+    xd_format_kernel<<<(int)std::min<size_t>((pieces + 255) / 256, 148 * 8), 256, 0, st>>>(x, (uint16_t*)scratch, M, K, tokens_per_cta);
+    DenseArgs da = {};
+    if (!make_run_maps(&da.w, packed, gemm_packed_bytes(N, K), 4096) ||
+        !make_run_maps(&da.t, scratch, pipesd_debug_gemm_dense_scratch_bytes(M, K, tokens_per_cta), 64 * (size_t)tokens_per_cta))
+        return PIPESD_E_CUDA;
+    da.g.M = M;
+    da.g.N = N;
+    da.g.KS = K / 16;
+    da.g.S = slices;
+    da.g.out = y;
+    const DenseRing ring = dense_ring(tokens_per_cta);
+    da.g.stages = ring.stages;
+    da.kc = ring.kc;
+    da.tbs_in = tokens_per_cta;
+    da.n_tb = dense_forced_blocks(M, tokens_per_cta);
+    const dim3 grid(2 * slices * (((N + 127) / 128 + 1) / 2) * da.n_tb);
+    if (dense_launch_mode<kPlain>(da, grid, ring.smem, st) != cudaSuccess) return PIPESD_E_CUDA;
+    return cudaGetLastError() == cudaSuccess ? PIPESD_OK : PIPESD_E_CUDA;
 }
 
 int32_t pipesd_debug_force_dense(pipesd_ctx* ctx, int32_t on) {

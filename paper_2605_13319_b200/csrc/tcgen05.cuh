@@ -1,5 +1,7 @@
 // Thin wrappers around the 5th-generation tensor-core instructions (tcgen05) and tensor memory, as inline PTX.
 #pragma once
+#include <cuda.h>
+
 #include "common.cuh"
 
 namespace pipesd {
@@ -52,6 +54,19 @@ __device__ __forceinline__ void umma2_commit(uint32_t bar, uint16_t mask) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"(mask)
                  : "memory");
 }
+// Tile copy (box of the map at row `row`, column 0) into this CTA's shared memory; the bytes count on `bar`, a barrier of
+// either CTA of the pair (dsmem_addr).
+__device__ __forceinline__ void tensor2_g2s(uint32_t dst_smem, const CUtensorMap* map, int row, uint32_t bar) {
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];" ::"r"(dst_smem),
+                 "l"(map), "r"(bar), "r"(0), "r"(row)
+                 : "memory");
+}
+__device__ __forceinline__ void tensor2_g2s_hint(uint32_t dst_smem, const CUtensorMap* map, int row, uint32_t bar, uint64_t pol) {
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4}], [%2], %5;" ::"r"(dst_smem),
+                 "l"(map), "r"(bar), "r"(0), "r"(row), "l"(pol)
+                 : "memory");
+}
+__device__ __forceinline__ void tensor_map_prefetch(const CUtensorMap* map) { asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
