@@ -11,8 +11,8 @@
 // and 20 KB of L2 per step; a pair halves the token side: 224 against 256 cycles, 12 KB.
 // Sums: the tensor pipe truncates each accumulation, so a long K in one accumulator drifts (7b shape, layer 31's K after a
 // 160-token prompt: relative L1 error 3.6e-3 with one accumulator over all of K, 2.6e-3 with the small-M kernel's slices).
-// Every kDenseChunk k16 steps the epilogue warps take the accumulator into registers and add there, rounding to nearest,
-// while the MMAs go on in the other of two accumulators.
+// Every dense_chunk k16 steps the epilogue warps take the accumulator into registers and add there, rounding to nearest,
+// while the MMAs go on in another accumulator: of two, or of four where tensor memory holds them (up to 64 tokens per CTA).
 // K slices: where row pairs x token blocks leave SMs idle, S <= 4 pairs form a cluster and share K; the partial tiles cross
 // the cluster through distributed shared memory (into the drained ring), each pair sums and finishes every S-th 16-token
 // column block, slices in order.
@@ -38,11 +38,11 @@ constexpr int kDenseThreads = 384;
 constexpr int kDenseMaxHalf = 128;        // tokens per CTA of a pair (half of a token block): a multiple of 16
 constexpr int kDenseMaxSlices = 4;        // K slices: pairs per cluster (8 CTAs, the portable limit)
 constexpr int kDenseMaxStages = 9;
-constexpr int kDenseChunk = 32;           // k16 steps per accumulator
 constexpr int kDenseRow = 132;            // floats of a token's 128 results in shared memory: eight tokens on eight bank groups
 constexpr int kDenseTail = 256 + 4 * 2 * kDenseMaxHalf;   // barriers, tensor-memory base | rstd
 constexpr int kDenseSmem = 227 * 1024;    // the CTA has its SM to itself
-static_assert(8 * (2 * kDenseMaxStages + 4) + 4 <= 256, "barriers and the tensor-memory slot fill the first 256 bytes of the tail");
+constexpr int kDenseMaxAccs = 4;
+static_assert(8 * (2 * kDenseMaxStages + 2 * kDenseMaxAccs) + 4 <= 256, "barriers and the tensor-memory slot fill the first 256 bytes of the tail");
 
 // ---- "xd" activation arrays: the K-major B operand of tcgen05.mma, in global memory ---------------------------
 // Blocks of `tbs` tokens (a multiple of 16), one per CTA of a pair.  Per (block, k16 step): the bf16 hi tile then the lo
@@ -88,6 +88,12 @@ static inline DensePlan dense_plan_from(int M, int first_row, int N, int K, cons
     p.n_tb = (M + 2 * p.tbs - 1) / (2 * p.tbs);
     return p;
 }
+// Host: k16 steps per accumulator: an eighth of K, as deep as the small-M kernel sums at the most slices it takes, so that a
+// prompt's rows are as exact here as there; 8 at least and 32 at most.  (Logits of a 203-token prompt against 64 bits, mean
+// over seeds: 1b shape, K = 2048, 3.6e-4 with 32 steps, 3.0e-4 with 16, 3.1e-4 with the small-M kernel; tiny shape, K = 256
+// and 688, 4.0e-5 with 16 or 32, 3.0e-5 with 8, 3.1e-5 with the small-M kernel.  8 steps everywhere would cost a tenth to a
+// third, as the accumulator changes hands more often.)
+static inline int dense_chunk(int KS) { return KS >= 256 ? 32 : KS >= 128 ? 16 : 8; }
 // Host: the ring.  As much of the shared memory as it gets.  A stage costs the issuer some 340 cycles of waiting and
 // committing beside its MMAs, so small steps are taken eight at a time (4096 x 11008, 32 tokens per CTA, us: 94 with two
 // steps a stage, 51.5 with four, 46.7 with eight; 80 tokens: 98, 70.3, 70.7; 64 tokens: 103, 63.1, 65.1).
@@ -101,9 +107,12 @@ static inline DenseRing dense_ring(int tbs) {
     r.smem = (size_t)r.stages * stage + kDenseTail;
     return r;
 }
-__host__ __device__ constexpr int dense_tmem_cols(int tbs) {      // two accumulators of 2 * tbs columns
+// Accumulators of 2 * tbs columns, taken in turn.  With two, the MMAs of a third chunk wait for the epilogue warps to have read
+// the first: commit, loads and a releasing remote arrival, about the time of 16 steps at few tokens.
+__host__ __device__ constexpr int dense_accs(int tbs) { return 2 * tbs * kDenseMaxAccs <= 512 ? kDenseMaxAccs : 2; }
+__host__ __device__ constexpr int dense_tmem_cols(int tbs) {
     int c = 32;
-    while (c < 4 * tbs) c *= 2;
+    while (c < dense_accs(tbs) * 2 * tbs) c *= 2;
     return c;
 }
 
@@ -114,6 +123,7 @@ struct DenseArgs {
     RunMaps w, t;       // weights, tokens (the input xd array)
     GemmArgs g;         // S = K slices; the mode's outputs as for the small-M kernel; W and xf are not read
     int kc;             // k16 steps per ring stage (g.stages stages)
+    int chunk;          // k16 steps per accumulator, a multiple of kc
     int tbs_in;         // block size of the input array and of this launch
     int tbs_out;        // block size of the xd array this launch produces (kResid, kSwiglu)
     int tb0, n_tb;      // first token block of the launch, token blocks
@@ -141,16 +151,17 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const __gr
     const GemmArgs& a = da.g;
     extern __shared__ __align__(128) unsigned char smem[];
     const int TBS = da.tbs_in, NT = 2 * TBS;                           // tokens per CTA / per block
-    const int KC = da.kc, S = a.S;
+    const int KC = da.kc, CH = da.chunk, S = a.S;
     const int w_stage = KC * 4096, stage_bytes = w_stage + KC * TBS * 64;
     const int stages = a.stages;
     unsigned char* tail = smem + stages * stage_bytes;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);                // full[9], empty[9], acc_full[2], acc_empty[2]
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 8 * (2 * kDenseMaxStages + 4));
+    uint64_t* bars = reinterpret_cast<uint64_t*>(tail);                // full[9], empty[9], acc_full[4], acc_empty[4]
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tail + 8 * (2 * kDenseMaxStages + 2 * kDenseMaxAccs));
     float* rstd_s = reinterpret_cast<float*>(tail + 256);              // [NT]
     const uint32_t smem_base = smem_u32(smem);
     const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * kDenseMaxStages;
-    const uint32_t acc_full = full0 + 16 * kDenseMaxStages, acc_empty = acc_full + 16;
+    const uint32_t acc_full = full0 + 16 * kDenseMaxStages, acc_empty = acc_full + 8 * kDenseMaxAccs;
+    const int n_acc = dense_accs(TBS), acc_sh = n_acc == 4 ? 2 : 1;    // chunk ch: accumulator ch % n_acc, turn ch >> acc_sh
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const int r = (int)(rank & 1), s = (int)(rank >> 1);
@@ -160,7 +171,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const __gr
     const int KS = a.KS;
     const int ks0 = (int)(((long)KS * s) / S), ks1 = (int)(((long)KS * (s + 1)) / S);
     const int nks = ks1 - ks0;
-    const int n_chunk = (nks + kDenseChunk - 1) / kDenseChunk;
+    const int n_chunk = (nks + CH - 1) / CH;
     const int tok0 = tb * NT;
     const uint32_t tmem_cols = (uint32_t)dense_tmem_cols(TBS);
 
@@ -169,7 +180,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const __gr
             mbar_init(full0 + 8 * i, 1);                               // the even CTA's: bytes of both CTAs' copies (the odd one's is not used)
             mbar_init(empty0 + 8 * i, 1);
         }
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < n_acc; ++i) {
             mbar_init(acc_full + 8 * i, 1);
             mbar_init(acc_empty + 8 * i, 16);                          // one arrival per epilogue warp of the pair
         }
@@ -188,7 +199,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const __gr
     tc_fence_after();
     const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
 
-    // ring stages of KC steps, in the order all roles walk them (kDenseChunk is a multiple of KC, so that only the slice's
+    // ring stages of KC steps, in the order all roles walk them (CH is a multiple of KC, so that only the slice's
     // last stage is shorter)
     const int n_stage = (nks + KC - 1) / KC;
     bool ok = true;
@@ -258,17 +269,18 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const __gr
             int st = 0;
             uint32_t ph = 0;
             for (int ch = 0; ch < n_chunk && ok; ++ch) {
-                if (ch >= 2) ok = mbar_wait_cluster(acc_empty + 8 * (ch & 1), (uint32_t)((ch >> 1) - 1) & 1u);
-                const uint32_t d = tmem + (uint32_t)((ch & 1) * NT);
-                const int k_end = min(nks, (ch + 1) * kDenseChunk);
-                for (int k = ch * kDenseChunk; k < k_end && ok; k += KC) {
+                const int ac = ch & (n_acc - 1);
+                if (ch >= n_acc) ok = mbar_wait_cluster(acc_empty + 8 * ac, (uint32_t)((ch >> acc_sh) - 1) & 1u);
+                const uint32_t d = tmem + (uint32_t)(ac * NT);
+                const int k_end = min(nks, (ch + 1) * CH);
+                for (int k = ch * CH; k < k_end && ok; k += KC) {
                     ok = mbar_wait(full0 + 8 * st, ph);                // landed in both CTAs
                     if (!ok) break;
                     tc_fence_after();
                     uint64_t ad = umma_desc(smem_base + st * stage_bytes, 128, 256);
                     uint64_t bd = umma_desc(smem_base + st * stage_bytes + w_stage, 128, 256);
                     const int kc = min(KC, k_end - k);
-                    uint32_t acc = k > ch * kDenseChunk ? 1u : 0u;
+                    uint32_t acc = k > ch * CH ? 1u : 0u;
                     for (int i = 0; i < kc; ++i) {
                         umma2_bf16(d, ad, bd, idesc, acc);
                         umma2_bf16(d, ad, bd + lo_step, idesc, 1u);
@@ -279,7 +291,7 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const __gr
                     umma2_commit(empty0 + 8 * st, mask);               // the stage is free in both CTAs when these MMAs have read it
                     if (++st == stages) { st = 0; ph ^= 1u; }
                 }
-                if (ok) umma2_commit(acc_full + 8 * (ch & 1), mask);
+                if (ok) umma2_commit(acc_full + 8 * ac, mask);
             }
             if (!ok && a.err) atomicExch(a.err, 7);
         }
@@ -315,10 +327,11 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const __gr
             for (int i = 0; i < 16; ++i) acc[cb][i] = 0.f;
         const uint32_t lead_empty = dsmem_addr(acc_empty, rank & ~1u);
         for (int ch = 0; ch < n_chunk; ++ch) {
-            if (ok) ok = mbar_wait(acc_full + 8 * (ch & 1), (uint32_t)(ch >> 1) & 1u);
+            const int ac = ch & (n_acc - 1);
+            if (ok) ok = mbar_wait(acc_full + 8 * ac, (uint32_t)(ch >> acc_sh) & 1u);
             ok = __all_sync(0xffffffffu, ok);
             tc_fence_after();
-            const uint32_t t = tmem + lane_sel + (uint32_t)((ch & 1) * NT + half * TBS);
+            const uint32_t t = tmem + lane_sel + (uint32_t)(ac * NT + half * TBS);
 #pragma unroll
             for (int cb = 0; cb < kDenseMaxHalf / 16; ++cb) {
                 if (cb < ncb) {
@@ -331,7 +344,8 @@ __global__ void __launch_bounds__(kDenseThreads, 1) gemm_dense_kernel(const __gr
             }
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(lead_empty + 8 * (ch & 1));
+            // only where a later chunk waits for it: the releasing arrival costs 600 cycles
+            if (lane == 0 && ch + n_acc < n_chunk) mbar_arrive_cluster(lead_empty + 8 * ac);
         }
         if (!ok && a.err && lane == 0) atomicExch(a.err, 9);
         __syncwarp();

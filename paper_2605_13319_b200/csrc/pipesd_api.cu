@@ -390,6 +390,7 @@ int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, in
         const DenseRing ring = dense_ring(pin.tbs);
         da.g.stages = ring.stages;
         da.kc = ring.kc;
+        da.chunk = dense_chunk(K / 16);
         da.g.pf = L2Prefetch{};
         da.tbs_in = pin.tbs;
         da.tb0 = tb0;
@@ -1371,6 +1372,7 @@ int32_t pipesd_debug_gemm_dense(const void* packed, const float* x, float* y, vo
     const DenseRing ring = dense_ring(tokens_per_cta);
     da.g.stages = ring.stages;
     da.kc = ring.kc;
+    da.chunk = dense_chunk(K / 16);
     da.tbs_in = tokens_per_cta;
     da.n_tb = dense_forced_blocks(M, tokens_per_cta);
     const dim3 grid(2 * slices * (((N + 127) / 128 + 1) / 2) * da.n_tb);

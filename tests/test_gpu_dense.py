@@ -37,6 +37,32 @@ def test_dense_plans(tokens_per_cta, slices):
             assert np.abs(y.cpu().numpy() - want).max() < 3e-5 * 0.02 * np.sqrt(K) * 4, (N, K, M)
 
 
+@pytest.mark.parametrize("N,K", [(256, 256), (272, 688), (512, 1024), (2048, 2048), (4096, 4096)])
+def test_dense_sums_as_exact_as_small_m(N, K):
+    """The tensor pipe truncates where it adds, so depth costs precision: the rms error of rows through this kernel may not
+    exceed the small-M kernel's, whose K slices are an eighth of K here (5 % for another order of sums)."""
+    import torch
+    from paper_2605_13319_b200 import binding
+    dev, M = torch.device("cuda", 0), 32
+    W = synth.normal_bf16((N, K), 19, 5, 0.02)
+    packed = binding.gemm_pack(torch.from_numpy(W.view(np.int16)).to(dev))
+    x = synth.normal_f32((M, K), 19, 6, 1.0)
+    want = oracle.linear(W, x.astype(np.float64))
+    xd, y = torch.from_numpy(x).to(dev), torch.empty((M, N), device=dev)
+
+    def rms():
+        torch.cuda.synchronize()
+        return np.sqrt(np.mean((y.cpu().numpy() - want) ** 2))
+
+    binding.gemm_run(packed, xd, y, binding.gemm_scratch(M, N, K, dev), N, K)
+    small = rms()
+    scratch = torch.zeros(binding.lib().pipesd_debug_gemm_dense_scratch_bytes(M, K, 16), dtype=torch.uint8, device=dev)
+    binding.debug_gemm_dense(packed, xd, y, scratch, N, K, 16, 1)
+    dense = rms()
+    print(f"rms error {N} x {K}: small-M {small:.3e}, dense {dense:.3e}")
+    assert dense < 1.05 * small
+
+
 def test_dense_rejects_bad_plans():
     from paper_2605_13319_b200 import binding
     L = binding.lib()
