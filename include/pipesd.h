@@ -254,6 +254,10 @@ int32_t pipesd_debug_force_dense(pipesd_ctx *ctx, int32_t on);
 uint64_t pipesd_debug_gemm_dense_scratch_bytes(int32_t M, int32_t K, int32_t tokens_per_cta);
 int32_t pipesd_debug_gemm_dense(const void *packed, const float *x, float *y, void *scratch, int32_t M, int32_t N, int32_t K,
                                 int32_t tokens_per_cta, int32_t slices, void *cuda_stream);
+/* Harness switch: how often (0..65536) a CTA of the attention kernel looks whether the other key splits of its rows are
+ * done before it leaves its share of their merge to the last one.  Results do not depend on it, bit for bit: at 0 the last
+ * one merges all rows, as it does where other work keeps the splits from running at the same time. */
+int32_t pipesd_debug_merge_polls(pipesd_ctx *ctx, int32_t polls);
 /* CTAs of the attention kernel that the context's device keeps resident at once for a request with this many query
  * rows per KV head: out2 (host) = {with the whole third ring slot, with the cut-down one} -- the two numbers
  * pipesd_debug_attn_split takes. */

@@ -97,6 +97,7 @@ _SIGNATURES = {
     "pipesd_sched_trigger_step": (i32, [ctypes.POINTER(ctypes.c_double), ctypes.c_double, ctypes.c_double,
                                         ctypes.c_double, ctypes.POINTER(i32)]),
     "pipesd_debug_force_dense": (i32, [vp, i32]),
+    "pipesd_debug_merge_polls": (i32, [vp, i32]),
     "pipesd_debug_gemm_dense_scratch_bytes": (u64, [i32, i32, i32]),
     "pipesd_debug_gemm_dense": (i32, [vp, vp, vp, vp, i32, i32, i32, i32, i32, vp]),
     "pipesd_debug_attn_slots": (i32, [vp, i32, ctypes.POINTER(ctypes.c_int32)]),
@@ -284,6 +285,9 @@ class Context:
 
     def debug_force_dense(self, on: bool):
         self._check(lib().pipesd_debug_force_dense(self._h, int(on)), "pipesd_debug_force_dense")
+
+    def debug_merge_polls(self, polls: int):
+        self._check(lib().pipesd_debug_merge_polls(self._h, polls), "pipesd_debug_merge_polls")
 
     def debug_attn_slots(self, rows_per_kv_head: int):
         out = (ctypes.c_int32 * 2)()

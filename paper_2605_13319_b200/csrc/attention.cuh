@@ -3,8 +3,10 @@
 // to each other.  The keys of a request are cut into up to 16 splits ("split-K"), one CTA each; a CTA leaves an
 // un-normalised partial output with its reference maximum and sum in global memory (a few MB that stay in L2),
 // takes a ticket, and the last CTA of a (request, KV head, row group) to arrive merges the splits in split order
-// and writes the result straight into the output projection's input format -- nobody waits for anybody, and a CTA
-// that is not the last one leaves its SM to the next kernel at once.
+// and writes the result straight into the output projection's input format, so that a CTA that is not the last one
+// leaves its SM to the next kernel at once.  Where all CTAs of a launch fit the device together and a group has many rows,
+// the others stay for a moment and take a share of the rows; what they do not take the last one merges, so that no CTA's
+// result depends on another one being on the device.
 //
 // One CTA = one KV head of one request x one key split x up to 112 query rows, where the rows are all (query head
 // of the group, chunk row) pairs that share the KV head (GQA).  The keys are on the M side of the MMAs, the (few)
@@ -38,6 +40,8 @@ constexpr int kAttnMaxSplits = 16;          // key splits of one request
 constexpr int kAttnMaxSlots = 4;            // tile slots of the K/V ring
 constexpr int kAttnBigCols = kAttnMaxRows / 16;   // 8-row column blocks per worker warp of the large variant (the small one: 1, 16 rows)
 constexpr int kAttnShortTail = 112;         // keys of the second tile up to which the third ring slot is cut down
+constexpr int kAttnMergePolls = 128;        // looks a CTA takes at the ticket before it leaves its share of a merge to the last one
+                                            // (0.3-0.5 us each; splits of one length end within a few us of each other)
 constexpr float kAttnMaxExcess = 40.f;      // log2 units by which a score may exceed its row's reference: P, O^T and the
                                             // denominators stay below 2^60 and, next to a p of at least 1, lose nothing below
 
@@ -207,7 +211,8 @@ struct AttnArgs {
     int rows_cap;              // query rows per row group (kAttnMaxRows, or 16 for a batch whose requests have up to 32)
     int n_max;                 // N the launch's shared memory was sized for
     int ring, slots;           // bytes and slots of the K/V ring
-    int share_merge;           // every CTA of the launch is resident: the CTAs of a group merge its rows together
+    int share_merge;           // all CTAs of the launch fit the device together: the CTAs of a group merge its rows together
+    int merge_polls;           // kAttnMergePolls, or the harness's limit
     int row_groups;
     float* o_part;             // partial results: [slot][hd], slot = it_part0 + ((kv head * R + row) * splits + split)
     float* m_part;             // [slot]
@@ -284,7 +289,7 @@ __global__ void __launch_bounds__(kAttnThreads, CU == 1 ? 3 : 1) attn_kernel(con
     float* Fl = alpha + N;                                         // [N] the CTA's partial denominators
     unsigned long long* bars = reinterpret_cast<unsigned long long*>(Fl + N);   // full[4], s_full[2], p_full, pv_done
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 8);
-    int* s_last = reinterpret_cast<int*>(tmem_slot + 1);
+    unsigned* s_mine = reinterpret_cast<unsigned*>(tmem_slot + 1);
     const uint32_t bar_full = smem_u32(bars), bar_s = bar_full + 32, bar_p = bar_full + 48, bar_pv = bar_full + 56;
     const uint32_t tmem_cols = (uint32_t)attn_tmem_cols(N);
     const uint32_t ring_a = smem_u32(ring);
@@ -680,44 +685,56 @@ __global__ void __launch_bounds__(kAttnThreads, CU == 1 ? 3 : 1) attn_kernel(con
     }
     if (nsplit == 1) { release_tmem(); return; }
 
-    // ---- merge of the splits, in split order.  Either the last CTA of this (request, KV head, row group) to arrive does it,
-    // and nobody waits for anybody; or, where every CTA of the launch is resident and a group has more rows than one round
-    // of warps (nine) takes, all CTAs of the group wait for each other's partials and take every nsplit-th row each (68
-    // rows x 13 splits, 450 KB, take one SM 14 us).  The wait ends although other launches may hold SMs: a group's CTAs are
-    // neighbours in the grid, so of each launch at most one group, 16 CTAs, is only partly on the device, and every other
-    // one runs to its end; and it is bounded.
+    // ---- merge of the splits, in split order, by the last CTA of this (request, KV head, row group) to arrive; or, where all
+    // CTAs of the launch fit the device together and a group has more rows than one round of warps (nine) takes, by all CTAs
+    // of the group, every nsplit-th row each (68 rows x 13 splits, 450 KB, take one SM 14 us).  Nobody depends on that: a CTA
+    // that does not see all the others arrive within merge_polls looks, because other work holds the SMs they need, marks
+    // its rows as not taken and leaves; the last one finds the marks in its ticket and merges those rows too.
     // (the barrier above orders the whole CTA's stores before thread 0's ticket, a release; the ticket or the poll is also an
     // acquire, and the barrier below orders it before everybody's loads of the other CTAs' partials)
     const bool share = a.share_merge && n_rows > kAttnThreads / 32;
     if (tid == 0) {
-        // arrivals in the low half, in shared merges also departures in the high half; zero again when the last is through
-        int* ticket = a.tickets + ((size_t)item * Hkv + kvh) * a.row_groups + rg;
-        int t;
-        asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;" : "=r"(t) : "l"(ticket) : "memory");
-        int go = (t == nsplit - 1);
-        if (share) {
-            for (uint32_t it = 0; it < (1u << 20) && !go; ++it) {
-                asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(t) : "l"(ticket) : "memory");
-                go = (t & 0xffff) == nsplit;
+        // one byte of arrivals, one of departures (shared merges), 16 marks; zero again when the last is through
+        unsigned* ticket = reinterpret_cast<unsigned*>(a.tickets) + ((size_t)item * Hkv + kvh) * a.row_groups + rg;
+        auto ticket_add = [&](unsigned v) {
+            unsigned t;
+            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(t) : "l"(ticket), "r"(v) : "memory");
+            return t;
+        };
+        unsigned t = ticket_add(1u);
+        const bool last = (t & 0xffu) == (unsigned)nsplit - 1u;
+        unsigned mine = 0u;                                      // bit s: the rows of split s's share are this CTA's to merge
+        if (!share) {
+            mine = last ? 1u : 0u;
+            if (last) *ticket = 0u;                              // self-cleaning: ready for the next launch
+        } else {
+            bool all = last;
+            for (int it = 0; it < a.merge_polls && !all; ++it) {
+                unsigned seen_t;
+                asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen_t) : "l"(ticket) : "memory");
+                all = (seen_t & 0xffu) == (unsigned)nsplit;
             }
-            if (!go && a.err) atomicExch(a.err, 10);
-            asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 65536;" : "=r"(t) : "l"(ticket) : "memory");
-            if ((t >> 16) == nsplit - 1) *ticket = 0;
-        } else if (go) {
-            *ticket = 0;                                         // self-cleaning: ready for the next launch
+            if (last) mine = t >> 16;
+            t = ticket_add(all ? 0x100u : 0x100u + (0x10000u << sp));
+            // (a mark that comes after the last arrival is seen by nobody, and all partials are there)
+            if ((t & 0xffu) == (unsigned)nsplit) mine |= 1u << sp;
+            if (((t >> 8) & 0xffu) == (unsigned)nsplit - 1u) *ticket = 0u;
         }
-        *s_last = go;
+        *s_mine = mine;
     }
     __syncthreads();
     release_tmem();
-    if (!*s_last) return;
+    const unsigned mine = *s_mine;
+    if (mine == 0u) return;
     // warp = row, lane = four columns: one round covers nine rows.  All of a row's loads are issued before the first
     // use (one trip to the L2 for up to kMergeBatch splits): lane j fetches split j's maximum and denominator, every
     // lane its four columns of each split's numerator; the sums run in split order.
     constexpr int kMergeBatch = 10;
     const int rl_step = share ? nsplit : 1;
 #pragma unroll 1
-    for (int rl = share ? sp + warp * nsplit : warp; rl < n_rows; rl += rl_step * (kAttnThreads / 32)) {
+    for (unsigned left = mine; left != 0u; left &= left - 1u)
+#pragma unroll 1
+    for (int rl = (share ? __ffs(left) - 1 : 0) + warp * rl_step; rl < n_rows; rl += rl_step * (kAttnThreads / 32)) {
         const size_t sl0 = slot0 + (size_t)rl * nsplit;
         const float m_mine = lane < nsplit ? __ldcg(a.m_part + sl0 + lane) : -INFINITY;
         const float l_mine = lane < nsplit ? __ldcg(a.l_part + sl0 + lane) : 0.f;

@@ -296,6 +296,7 @@ struct pipesd_ctx {
                                                      // kernel the device keeps resident at once
     RunMaps xd_maps[3][kDenseMaxHalf / 16];      // [xf_h, xf_attn, xf_act][tokens per block / 16 - 1]
     int dense_pairs[kDenseMaxSlices + 1] = {};   // [K slices]: CTA pairs of the dense kernel the device keeps resident at once
+    int merge_polls = kAttnMergePolls;
     bool force_dense = false;   // harness switch: the dense kernels also for passes of at most 32 rows
     bool pass_dense = false;    // the pass being enqueued runs on the dense kernels
     // bytes of the O and gate/up weights the attention kernel pulls into L2 once its K/V has landed (measured: all of O
@@ -623,6 +624,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
         aa.layer = l; aa.n_pages = c.n_pages; aa.page_size = c.page_size; aa.M = M; aa.Hq = Hq; aa.Hkv = Hkv;
         aa.rows_cap = rows_cap; aa.n_max = n_max; aa.row_groups = row_groups;
         aa.slots = attn_ring_slots(hd, n_max); aa.ring = attn_ring_bytes(hd, aa.slots, all_short);
+        aa.merge_polls = ctx->merge_polls;
         aa.share_merge = attn_ctas <= ctx->attn_slots[n_max / 16][all_short ? 1 : 0];
         aa.o_part = o_part; aa.m_part = m_part; aa.l_part = l_part; aa.tickets = ctx->W<int>(ctx->ws.tickets);
         aa.xf_out = (uint16_t*)xf_attn; aa.xd_tbs = tbs_o; aa.err = ctx->err_word();
@@ -1385,6 +1387,12 @@ int32_t pipesd_debug_force_dense(pipesd_ctx* ctx, int32_t on) {
     if (on && ctx->cfg.max_rows <= 32)
         return fail(ctx, PIPESD_E_INVALID, "pipesd_debug_force_dense: the context was made for passes of at most 32 rows");
     ctx->force_dense = on != 0;
+    return PIPESD_OK;
+}
+
+int32_t pipesd_debug_merge_polls(pipesd_ctx* ctx, int32_t polls) {
+    if (!ctx || polls < 0 || polls > 65536) return fail(ctx, PIPESD_E_INVALID, "pipesd_debug_merge_polls");
+    ctx->merge_polls = polls;
     return PIPESD_OK;
 }
 

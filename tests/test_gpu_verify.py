@@ -301,3 +301,29 @@ def test_attention_scores_of_wide_range(n_kv_heads, k, loud):
     # a score of 500 carries an error of 2^-17 of itself, 4e-3, and the probabilities e^s as much in relative terms
     assert logit_rel_err(ctx.debug_get_logits(k + 1), ref["logits"]).max() < LOGIT_TOL
     ctx.close()
+
+
+@pytest.mark.parametrize("n_kv_heads,k,P", [(4, 16, 4090), (2, 16, 4090), (1, 8, 1000), (2, 4, 300)])
+def test_merge_without_waiting(n_kv_heads, k, P):
+    """Key splits whose CTAs do not see each other finish (other work holds the SMs) leave their rows to the last one: the
+    same bits as when all of them merge together, whatever share is left, and no error.  Up to 16 splits, 10 to 68 rows."""
+    from paper_2605_13319_b200 import binding
+    shape = synth.TINY.scaled(name=f"tiny-kv{n_kv_heads}", n_kv_heads=n_kv_heads)
+    w = synth.make_weights(shape, 6)
+    ctx = binding.Context(shape, w, n_pages=(P + 32) // 16 + 1, max_seq=P + 32, max_draft=16, poison=True)
+    req = ctx.req_open()
+    for l in range(shape.n_layers):
+        ctx.debug_write_kv(req, l, 0, *synth.make_synthetic_kv(shape, P, 6, l))
+    toks = synth.make_prefix(shape, k + 1, 6)
+    q = np.full((k, shape.vocab), 1.0 / shape.vocab, np.float32)
+    item = dict(req=req, tokens=toks, q=q, u=synth.make_accept_uniforms(k, 6))
+    want = None
+    for polls in (128, 0, 0, 1, 2, 3, 5, 8, 0, 128):
+        ctx.debug_merge_polls(polls)
+        ctx.verify([item], flags=binding.Q_HOST)
+        got = ctx.debug_get_logits(k + 1)
+        want = got if want is None else want
+        assert np.isfinite(got).all() and np.array_equal(got, want), polls
+        ctx.kv_rollback([req], [0])
+        ctx.debug_set_len(req, P)
+    ctx.close()
