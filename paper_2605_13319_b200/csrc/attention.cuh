@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(kAttnThreads, CU == 1 ? 3 : 1) attn_kernel(con
     unsigned char* q_lo = q_hi + SM::q_bytes(N);
     unsigned char* p_hi = q_lo + SM::q_bytes(N);
     float* wm = reinterpret_cast<float*>(p_hi + 2 * SM::p_bytes(N));   // [4][N] maxima of a tile per lane quarter
-    int* hz = reinterpret_cast<int*>(wm + 4 * N);                  // [N] last visible key of a row (-1: padding row)
+    int* hz = reinterpret_cast<int*>(wm + 4 * N);                  // [N] last visible key of a row
     float* m_ref = reinterpret_cast<float*>(hz + N);               // [N] reference score of a row
     float* alpha = m_ref + N;                                      // [N] rescale factor of a row for this tile
     float* Fl = alpha + N;                                         // [N] the CTA's partial denominators
@@ -342,7 +342,8 @@ __global__ void __launch_bounds__(kAttnThreads, CU == 1 ? 3 : 1) attn_kernel(con
 #pragma unroll 1
             for (int n = tid; n < N; n += kAttnWorkers) {
                 const int rho = rho0 + n;
-                hz[n] = n < n_rows ? base + rho / G : -1;
+                // (a padding row has scores of 0; it sees every key, so that its reference is 0 too and nothing exceeds that)
+                hz[n] = n < n_rows ? base + rho / G : 0x7fffffff;
                 m_ref[n] = -INFINITY;
             }
             pdl_wait();
@@ -493,8 +494,7 @@ __global__ void __launch_bounds__(kAttnThreads, CU == 1 ? 3 : 1) attn_kernel(con
                 if (t == 0) {
                     if (quarter == 0) {
 #pragma unroll 1
-    #pragma unroll 1
-                    for (int cu = half; cu < NG; cu += 2) {
+                        for (int cu = half; cu < NG; cu += 2) {
                             float s[8];
                             read_s(t_St + cu * 8, s);
                             if (lane == 0) {
