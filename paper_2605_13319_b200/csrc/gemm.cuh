@@ -82,9 +82,9 @@ static inline GemmPlan gemm_plan(int M, int N, int K) {
         if (s > 1 && p.KS / s < 2 * kGemmKC) break;
         if ((long)p.RB * s <= kGemmWave) best = s;
     }
-    // Between half and a whole wave of row blocks (two slices would not fit it): slices of a fifth instead, two to three waves
-    // of short CTAs, whose starts and ends overlap (8b shape, gate/up of 17 rows, 224 row blocks: pass 5145 -> 5025 us).
-    if (best == 1 && 2 * p.RB > kGemmWave && p.RB < kGemmWave && p.KS >= 5 * 2 * kGemmKC) best = 5;
+    // Between half and a whole wave of row blocks no two slices fit it, and more CTAs than a wave do not pay (8b shape, gate/up of
+    // 224 row blocks, us a pass of 3, 9 and 17 rows: one slice 3434, 3612, 5030; two 3756, 4008, 5248; three 3493, 3700, 4943;
+    // five 3560, 3730, 4927; 32000 x 4096 alone, 9 rows: one 47, five 56).
     p.S = best;
     // ring depth: as deep as the shared memory of an SM allows for the number of CTAs it will hold.  A clustered
     // GEMM always leaves room for three CTAs per SM, even when it brings fewer: at two 113 KB CTAs per SM a B200

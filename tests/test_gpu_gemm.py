@@ -42,7 +42,7 @@ def test_gemm_matches_oracle(M, N, K):
 
 
 @pytest.mark.parametrize("M,N,K,offset", [
-    (17, 28672, 640, 0), (9, 28432, 656, 0),      # more than half a wave of row blocks: slices of a fifth, two to three waves
+    (17, 28672, 640, 0), (9, 28432, 656, 0),      # between half and a whole wave of row blocks: one slice
     (9, 2048, 2048, 0),                           # at most one CTA per SM: the deeper ring
     (5, 272, 256, 1), (5, 272, 256, 4),           # weights at an address that is no multiple of 16 bytes
 ])
