@@ -847,10 +847,8 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
         ps.hd = c.head_dim;
         int i = 0;
         for (auto& s : srcs) { ps.w[i] = (const uint16_t*)s.first; ps.rows[i] = s.second; ++i; }
-        size_t total = (size_t)((N + 127) / 128 * 8) * (K / 16) * 32;
-        int blocks = (int)std::min<size_t>((total + 255) / 256, 148 * 16);
         g.packed = (uint4*)take(gemm_packed_bytes(N, K));
-        gemm_pack_kernel<<<blocks, 256, 0, st>>>(ps, g.packed, N, K);
+        gemm_pack_kernel<<<gemm_pack_grid(N, K), kPackThreads, 0, st>>>(ps, g.packed, N, K);
         maps_ok = maps_ok && make_run_maps(&g.maps, g.packed, gemm_packed_bytes(N, K), 4096);
     };
     ctx->emb = (uint16_t*)take((size_t)c.vocab * c.d_model * 2);
@@ -1311,9 +1309,7 @@ int32_t pipesd_gemm_pack(const void* W, void* packed, int32_t N, int32_t K, void
     ps.mode = kPlain;
     ps.w[0] = (const uint16_t*)W;
     ps.rows[0] = N;
-    size_t total = (size_t)((N + 127) / 128 * 8) * (K / 16) * 32;
-    int blocks = (int)std::min<size_t>((total + 255) / 256, 148 * 16);
-    gemm_pack_kernel<<<blocks, 256, 0, (cudaStream_t)cuda_stream>>>(ps, (uint4*)packed, N, K);
+    gemm_pack_kernel<<<gemm_pack_grid(N, K), kPackThreads, 0, (cudaStream_t)cuda_stream>>>(ps, (uint4*)packed, N, K);
     return cudaGetLastError() == cudaSuccess ? PIPESD_OK : PIPESD_E_CUDA;
 }
 
