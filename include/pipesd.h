@@ -165,7 +165,10 @@ int32_t pipesd_req_len(pipesd_ctx *ctx, int32_t req, int32_t *len);
 
 /* Append n prompt tokens (host ids) to the request's cache -- the accepted prefix that every NAV pass runs against
  * (Sec. 2.2: the drafts are checked against the prefix accepted so far): the same layer stack as verify, run in chunks of
- * up to max(max_rows, min(max_seq, 1024)) rows, no acceptance step.  If last_logits (host, vocab floats) is non-null it
+ * up to max(max_rows, min(max_seq, 1024)) rows, no acceptance step.  Prompts that begin alike leave K and V that agree to
+ * rounding, not bit for bit, unless they also have the same length: the chunks, and with them the order of sums, follow
+ * the length.  The workspace holds a chunk: per row 8 bytes for each of d_model and the query width and 4 for d_ffn,
+ * 112 MB for 1024 rows at 4096, 4096 and 11008.  If last_logits (host, vocab floats) is non-null it
  * receives the logits of the final position; the call then synchronises. */
 int32_t pipesd_prefill(pipesd_ctx *ctx, int32_t req, const int32_t *tokens, int32_t n, float *last_logits);
 
@@ -242,10 +245,13 @@ int32_t pipesd_gemm_run(const void *packed, const float *x, float *y, void *scra
                         int32_t K, void *cuda_stream);
 
 /* Harness switch.  Passes of more than 32 rows run their projections on the dense tensor-core kernel, smaller passes
- * on the small-M weight-streaming kernel; the two sum in different orders, so their results agree to rounding, not
- * bit for bit.  on != 0 makes every pass of the context use the dense kernel (so that a request verified alone runs the
- * projections a large batch runs; the attention's key splits still follow the pass's composition, so the two agree
- * to rounding and in their decisions, not in every bit); needs max_rows > 32 (PIPESD_E_INVALID otherwise). */
+ * on the small-M weight-streaming kernel.  The small-M kernel sums a row in an order that follows the weights' shape alone;
+ * the dense kernel cuts K into slices by the pass's row count as well, so that a row's projections agree to rounding, not
+ * bit for bit, between passes of different row counts (and between the kernels).  on != 0 makes every pass of the context
+ * use the dense kernel; on > 1 also gives passes of fewer rows the slices of a pass of `on` rows, so that a request
+ * verified alone runs the very projections of a batch of that many rows (the attention's key splits still follow the pass's
+ * composition, so the two agree to rounding and in their decisions, not in every bit).  Needs max_rows > 32
+ * (PIPESD_E_INVALID otherwise). */
 int32_t pipesd_debug_force_dense(pipesd_ctx *ctx, int32_t on);
 /* The dense kernel on its own, in a given plan: y[M,N] = x[M,K] . W[N,K]^T as pipesd_gemm_run computes it, with blocks of
  * 2 * tokens_per_cta tokens (tokens_per_cta: a multiple of 16 up to 128) and K cut into `slices` (1..4) slices.  scratch:

@@ -283,7 +283,8 @@ class Context:
         self._check(lib().pipesd_debug_req_state(self._h, req, out), "pipesd_debug_req_state")
         return tuple(out)
 
-    def debug_force_dense(self, on: bool):
+    def debug_force_dense(self, on: int):
+        """0: off; 1: every pass on the dense kernel; n > 1: planned like a pass of n rows."""
         self._check(lib().pipesd_debug_force_dense(self._h, int(on)), "pipesd_debug_force_dense")
 
     def debug_merge_polls(self, polls: int):

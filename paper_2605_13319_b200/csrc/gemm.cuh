@@ -76,7 +76,7 @@ static inline GemmPlan gemm_plan(int M, int N, int K) {
     // One resident wave if possible: every CTA streams from the first microsecond and the next kernel's
     // CTAs find room to prefetch.  Largest K split that still fits the wave of a single token block.  The
     // split depends on (N, K) only, never on M: the order in which a result element is summed is then the
-    // same whether a request is verified alone or inside a batch (bit-identical decisions).
+    // same in every pass that runs on this kernel.
     int best = 1;
     for (int s = 1; s <= kGemmMaxSplit && s <= p.KS; ++s) {
         if (s > 1 && p.KS / s < 2 * kGemmKC) break;

@@ -82,9 +82,10 @@ static inline DensePlan dense_plan(int M, int N, int K, const int* pairs) {
     }
     return best;
 }
-// The same where only the results of rows first_row .. M-1 are wanted (a prompt's last rows): blocks for that many rows.
-static inline DensePlan dense_plan_from(int M, int first_row, int N, int K, const int* pairs) {
-    DensePlan p = dense_plan(M - first_row, N, K, pairs);
+// The same where only the results of rows first_row .. M-1 are wanted (a prompt's last rows): blocks for that many rows, or,
+// if that is more, slices and block size of a pass of plan_rows rows (0: of this pass).
+static inline DensePlan dense_plan_from(int M, int first_row, int plan_rows, int N, int K, const int* pairs) {
+    DensePlan p = dense_plan(M - first_row > plan_rows ? M - first_row : plan_rows, N, K, pairs);
     p.n_tb = (M + 2 * p.tbs - 1) / (2 * p.tbs);
     return p;
 }

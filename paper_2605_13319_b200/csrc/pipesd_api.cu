@@ -297,7 +297,8 @@ struct pipesd_ctx {
     RunMaps xd_maps[3][kDenseMaxHalf / 16];      // [xf_h, xf_attn, xf_act][tokens per block / 16 - 1]
     int dense_pairs[kDenseMaxSlices + 1] = {};   // [K slices]: CTA pairs of the dense kernel the device keeps resident at once
     int merge_polls = kAttnMergePolls;
-    bool force_dense = false;   // harness switch: the dense kernels also for passes of at most 32 rows
+    bool force_dense = false;   // harness switch: the dense kernels also for passes of at most 32 rows ...
+    int plan_rows = 0;          // ... with the plans of a pass of this many rows
     bool pass_dense = false;    // the pass being enqueued runs on the dense kernels
     // bytes of the O and gate/up weights the attention kernel pulls into L2 once its K/V has landed (measured: all of O
     // and 16 MB of gate/up; more gains nothing, an SM takes data in only about 1.4 times faster than HBM delivers it)
@@ -378,7 +379,7 @@ int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, in
         CU(cudaEventRecord(e0, ctx->st));
     }
     if (ctx->pass_dense) {
-        const DensePlan pin = dense_plan_from(a.M, first_row, a.N, K, ctx->dense_pairs);
+        const DensePlan pin = dense_plan_from(a.M, first_row, ctx->plan_rows, a.N, K, ctx->dense_pairs);
         const int tb0 = first_row / (2 * pin.tbs);
         DenseArgs da = {};
         da.g = a;
@@ -397,7 +398,7 @@ int launch_gemm(pipesd_ctx* ctx, int mode, const GemmW& w, GemmArgs a, int K, in
         da.tb0 = tb0;
         da.n_tb = pin.n_tb - tb0;
         da.out_row0 = first_row;
-        da.tbs_out = next_N > 0 ? dense_plan_from(a.M, next_first, next_N, next_K, ctx->dense_pairs).tbs : 0;
+        da.tbs_out = next_N > 0 ? dense_plan_from(a.M, next_first, ctx->plan_rows, next_N, next_K, ctx->dense_pairs).tbs : 0;
         const size_t smem = ring.smem;
         cudaError_t e;
         switch (mode) {
@@ -592,8 +593,8 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
     // tokens); their activation arrays are in that kernel's operand order, with the token block size of the consumer.
     ctx->pass_dense = M > 32 || ctx->force_dense;
     const bool dense = ctx->pass_dense;
-    const int tbs_qkv = dense ? dense_plan(M, dv.Nqkv, d, ctx->dense_pairs).tbs : 0,
-              tbs_o = dense ? dense_plan(M, d, dv.qd, ctx->dense_pairs).tbs : 0;
+    const int tbs_qkv = dense ? dense_plan_from(M, 0, ctx->plan_rows, dv.Nqkv, d, ctx->dense_pairs).tbs : 0,
+              tbs_o = dense ? dense_plan_from(M, 0, ctx->plan_rows, d, dv.qd, ctx->dense_pairs).tbs : 0;
     // Every kernel of the chain is launched with programmatic stream serialisation: it may start while its
     // predecessor drains and blocks in griddepcontrol.wait before touching the predecessor's output.
     {
@@ -1383,6 +1384,7 @@ int32_t pipesd_debug_force_dense(pipesd_ctx* ctx, int32_t on) {
     if (on && ctx->cfg.max_rows <= 32)
         return fail(ctx, PIPESD_E_INVALID, "pipesd_debug_force_dense: the context was made for passes of at most 32 rows");
     ctx->force_dense = on != 0;
+    ctx->plan_rows = on > 1 ? std::min(on, ctx->dv.row_cap) : 0;
     return PIPESD_OK;
 }
 

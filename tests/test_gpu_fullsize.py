@@ -250,7 +250,7 @@ def test_7b_ragged_batch_of_32_requests(seven_b):
     # follow the pass's composition, so the two runs agree to rounding; a decision may differ only where its margin (or
     # its distance to a CDF edge) under the batch's own logits is inside the tie band, and such flips are counted
     inv = Tally()
-    ctx.debug_force_dense(True)       # the kernels the batch of more than 32 rows ran on
+    ctx.debug_force_dense(rows)       # the kernels the batch of more than 32 rows ran on, with its plans
     row = 0
     for i in range(n):
         k = int(ks[i])
@@ -265,7 +265,7 @@ def test_7b_ragged_batch_of_32_requests(seven_b):
         row += k + 1
     assert inv.len_flip + inv.tok_flip <= 4, inv.report()
     print("\nbatch vs alone: " + inv.report())
-    ctx.debug_force_dense(False)
+    ctx.debug_force_dense(0)
     print("\n" + tally.report())
     for it in items:
         ctx.req_close(it["req"])

@@ -139,13 +139,14 @@ def test_batched_ragged_verify_and_batch_invariance(n_kv_heads):
         k = int(ks[i])
         assert logit_rel_err(logits[row:row + k + 1], ref["logits"]).max() < LOGIT_TOL
         tally.check(got[i], ref, ref["logits"], q, u, where=f"request {i}")
-        # alone, on the kernels the batch ran on (more than 32 rows: the dense ones), then on the small-pass kernels
-        ctx.debug_force_dense(True)
+        # alone, on the kernels the batch ran on (more than 32 rows: the dense ones, with the batch's plans), then on the
+        # small-pass kernels
+        ctx.debug_force_dense(len(logits))
         (alone,) = ctx.verify([solo[i]], flags=binding.Q_HOST)
         inv.check(alone, decisions_from_logits(logits[row:row + k + 1], items[i]), logits[row:row + k + 1], q, u,
                   where=f"request {i}: alone vs in the batch")
         assert logit_rel_err(ctx.debug_get_logits(k + 1), ref["logits"]).max() < LOGIT_TOL
-        ctx.debug_force_dense(False)
+        ctx.debug_force_dense(0)
         ctx.kv_rollback([solo[i]["req"]], [0])
         ctx.debug_set_len(solo[i]["req"], int(lens[i]))
         (small,) = ctx.verify([solo[i]], flags=binding.Q_HOST)
@@ -326,4 +327,37 @@ def test_merge_without_waiting(n_kv_heads, k, P):
         assert np.isfinite(got).all() and np.array_equal(got, want), polls
         ctx.kv_rollback([req], [0])
         ctx.debug_set_len(req, P)
+    ctx.close()
+
+
+@pytest.mark.parametrize("n_req", [6, 12])
+def test_alone_with_the_batch_plans_is_bit_identical(n_req):
+    """Requests of one key split (so that the attention sums alike too): alone, with the projections planned for the batch's
+    rows, each leaves the very logits it had in the batch.  At these widths the K slices of three projections differ between
+    the plans of 2 to 17 rows and those of the batch."""
+    from paper_2605_13319_b200 import binding
+    shape = synth.TINY.scaled(name="tiny-wide", d_model=1024, d_ffn=2048, vocab=2048)
+    lens, ks, _ = synth.ragged_requests(7, n_req, 20, 100, 1, 16)
+    rows = int(ks.sum()) + n_req
+    assert rows > 32
+    w = synth.make_weights(shape, 7)
+    ctx = binding.Context(shape, w, n_pages=n_req * 9, max_requests=n_req, max_rows=rows, max_seq=128, poison=True)
+    items = []
+    for i in range(n_req):
+        P, k = int(lens[i]), int(ks[i])
+        req = ctx.req_open()
+        ctx.prefill(req, synth.make_prefix(shape, P, 7, request=i))
+        items.append(dict(req=req, tokens=synth.tokens_i32(k + 1, 7, 900 + i, shape.vocab), u=synth.make_accept_uniforms(k, 7, i),
+                          q=np.full((k, shape.vocab), 1.0 / shape.vocab, np.float32)))
+    ctx.verify(items, flags=binding.Q_HOST)
+    want = ctx.debug_get_logits(rows)
+    ctx.kv_rollback([it["req"] for it in items], [0] * n_req)
+    ctx.debug_force_dense(rows)
+    row = 0
+    for i, it in enumerate(items):
+        ctx.debug_set_len(it["req"], int(lens[i]))
+        ctx.verify([it], flags=binding.Q_HOST)
+        assert np.array_equal(ctx.debug_get_logits(int(ks[i]) + 1), want[row:row + int(ks[i]) + 1]), i
+        ctx.kv_rollback([it["req"]], [0])
+        row += int(ks[i]) + 1
     ctx.close()
