@@ -7,7 +7,6 @@
 namespace pipesd {
 
 constexpr int kMaxItemRows = 32;   // rows (k+1, or a prefill chunk) one request contributes to a pass
-constexpr int kMaxSplits = 32;     // split-K partitions of one request's KV range
 
 __device__ __forceinline__ float bf16_bits_to_f32(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
 
@@ -60,11 +59,6 @@ __device__ __forceinline__ uint4 ldmatrix_a16(uint32_t addr) {
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
 __device__ __forceinline__ double warp_sum_d(double v) {
@@ -156,11 +150,6 @@ __device__ __forceinline__ void bulk_g2s_hint(uint32_t dst_smem, const void* src
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;" ::"r"(dst_smem),
                  "l"(src), "r"(bytes), "r"(bar), "l"(pol)
                  : "memory");
-}
-// Hint: pull a contiguous global range into L2 (no destination, no completion to wait for).  Address 16-byte
-// aligned, size a multiple of 16.
-__device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes) {
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 // What a kernel pulls into L2 on behalf of its successor while its own demand on HBM ebbs (its tail: split-K
 // reduction, epilogue, grid hand-over leave HBM idle for several microseconds).  The successor's weights are cut
@@ -301,11 +290,6 @@ __device__ __forceinline__ uint32_t cluster_ctarank() {
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
     return r;
 }
-__device__ __forceinline__ uint32_t cluster_nctaid_x() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(r));
-    return r;
-}
 // Every thread of every CTA of the cluster must execute this (hardware barrier, release/acquire).
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
@@ -315,11 +299,6 @@ __device__ __forceinline__ uint32_t dsmem_addr(uint32_t local_smem_addr, uint32_
     uint32_t r;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_smem_addr), "r"(rank));
     return r;
-}
-__device__ __forceinline__ float dsmem_ld_f32(uint32_t addr) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr));
-    return v;
 }
 __device__ __forceinline__ void dsmem_st_f32(uint32_t addr, float v) {
     asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");

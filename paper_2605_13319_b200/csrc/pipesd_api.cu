@@ -111,6 +111,7 @@ struct WsLayout {
         block_tab, qstage, req_state, never_flag, total;
 };
 
+size_t ticket_bytes(const pipesd_model_cfg& c, const Derived& d) { return 4 * (size_t)d.row_cap * c.n_q_heads; }
 constexpr size_t kXdPad = 2 * kDenseMaxHalf + 16;
 
 WsLayout ws_layout(const pipesd_model_cfg& c, const Derived& d) {
@@ -134,7 +135,7 @@ WsLayout ws_layout(const pipesd_model_cfg& c, const Derived& d) {
     w.o_part = take(4 * slots * c.head_dim);
     w.m_part = take(4 * slots);
     w.l_part = take(4 * slots);
-    w.tickets = take(4 * M * c.n_q_heads);   // one per (item, KV head, row group); zero between launches
+    w.tickets = take(ticket_bytes(c, d));    // one per (item, KV head, row group); zero between launches
     w.cs = take(4 * M * (c.head_dim / 2));
     w.sn = take(4 * M * (c.head_dim / 2));
     w.kvoff = take(8 * M);
@@ -340,6 +341,12 @@ namespace {
 int fail(pipesd_ctx* c, int code, const char* what) {
     if (c) c->err = std::string(pipesd_strerror(code)) + ": " + what;
     return code;
+}
+
+// The device error word and the attention tickets start at zero, and again after an error (the tickets reset themselves in use).
+cudaError_t clear_device_flags(pipesd_ctx* c) {
+    const cudaError_t e = cudaMemsetAsync(c->err_word(), 0, 4, c->st);
+    return e != cudaSuccess ? e : cudaMemsetAsync(c->wsp + c->ws.tickets, 0, ticket_bytes(c->cfg, c->dv), c->st);
 }
 
 int cuda_fail(pipesd_ctx* c, cudaError_t e, const char* where) {
@@ -825,10 +832,7 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
             return bail(PIPESD_E_CUDA);
 
     cudaStream_t st = ctx->st;
-    // the device error word and the attention tickets start at zero (the tickets reset themselves after use)
-    if (cudaMemsetAsync(ctx->err_word(), 0, 4, st) != cudaSuccess) return bail(PIPESD_E_CUDA);
-    if (cudaMemsetAsync(ctx->wsp + ctx->ws.tickets, 0, 4 * (size_t)c.max_rows * c.n_q_heads, st) != cudaSuccess)
-        return bail(PIPESD_E_CUDA);
+    if (clear_device_flags(ctx) != cudaSuccess) return bail(PIPESD_E_CUDA);
 
     // ---- repack the weights into the library's own layout
     char* wp = (char*)mem->weights;
@@ -912,8 +916,7 @@ int32_t pipesd_ctx_sync(pipesd_ctx* ctx) {
             }
         }
         ctx->inflight.clear();
-        cudaMemsetAsync(ctx->err_word(), 0, 4, ctx->st);
-        cudaMemsetAsync(ctx->wsp + ctx->ws.tickets, 0, 4 * (size_t)ctx->cfg.max_rows * ctx->cfg.n_q_heads, ctx->st);
+        clear_device_flags(ctx);
         char msg[96];
         snprintf(msg, sizeof msg, "a device-side wait timed out (kernel error word %d)", dev_err);
         return fail(ctx, PIPESD_E_CUDA, msg);

@@ -37,6 +37,30 @@ def test_prefill_lengths(n, n_kv_heads, max_rows):
     ctx.close()
 
 
+def test_prefill_wide():
+    """Widths of the 7b shape, where the projections of a long chunk run with blocks of up to 256 tokens: a chunk of 1024 rows
+    and one of 750 on top of it, rows of every layer's K and V and the last logits against the CPU checker."""
+    from paper_2605_13319_b200 import binding
+    shape = synth.TINY.scaled(name="wide", d_model=4096, n_q_heads=32, n_kv_heads=32, head_dim=128, d_ffn=5504, vocab=512)
+    w = synth.make_weights(shape, 8)
+    n = 1024 + 750
+    prefix = synth.make_prefix(shape, n, 8)
+    orc = oracle.Oracle(shape, w, n)
+    ctx = binding.Context(shape, w, n_pages=n // 16 + 1, max_seq=n, poison=True)
+    req = ctx.req_open()
+    for part in (prefix[:1024], prefix[1024:]):
+        want = orc.prefill(part, want_last_logits=True)
+        got = ctx.prefill(req, part, want_last_logits=True)
+        assert logit_rel_err(got[None], np.reshape(want, (1, -1))).max() < 1e-3
+    for layer in range(shape.n_layers):
+        kg, vg = ctx.debug_read_kv(req, layer, 0, n)
+        for i, bits in enumerate((kg, vg)):
+            got, want = synth.bf16_to_f32(bits), np.stack([orc.get_kv(layer, p)[i] for p in range(n)])
+            # one bf16 step where a rounding boundary was crossed (2^-7 of the value at most), 2e-4 accumulated below it
+            assert np.all(np.abs(got - want) <= 2.0 ** -7 * np.maximum(np.abs(got), np.abs(want)) + 2e-4 * np.abs(want).max())
+    ctx.close()
+
+
 def test_prefill_chunks_agree():
     """Two chunks of the longest kind (1024 rows at most, cut in equal parts) against the same prompt fed in two calls."""
     from paper_2605_13319_b200 import binding
