@@ -56,8 +56,14 @@ def test_prefill_wide():
         kg, vg = ctx.debug_read_kv(req, layer, 0, n)
         for i, bits in enumerate((kg, vg)):
             got, want = synth.bf16_to_f32(bits), np.stack([orc.get_kv(layer, p)[i] for p in range(n)])
-            # one bf16 step where a rounding boundary was crossed (2^-7 of the value at most), 2e-4 accumulated below it
-            assert np.all(np.abs(got - want) <= 2.0 ** -7 * np.maximum(np.abs(got), np.abs(want)) + 2e-4 * np.abs(want).max())
+            # The bounds of the full-size test.  Layer 0 sees identical inputs: an element differs by one bf16 step where a
+            # rounding boundary was crossed (2^-7 of the value at most; here 4 elements in 10,000).  Such a step in a large
+            # element of K moves a score by 2^-7 |q| |k|, a few percent, and where that key has most of a row's weight, the
+            # row's whole attention output by as much: in layer 1 single rows are off by two steps, so an element is held
+            # to 2e-2 of the largest and the mean to twice what prompts of 32-row passes show (1.6e-4; here 1.1e-4).
+            diff, slack, l1 = np.abs(got - want), *((2e-5, 1e-4) if layer == 0 else (2e-2, 3.2e-4))
+            assert np.all(diff <= 2.0 ** -7 * np.maximum(np.abs(got), np.abs(want)) + slack * np.abs(want).max()), (layer, i)
+            assert diff.sum() < l1 * np.abs(want).sum(), (layer, i)
     ctx.close()
 
 
