@@ -264,6 +264,9 @@ int32_t pipesd_debug_gemm_dense(const void *packed, const float *x, float *y, vo
  * done before it leaves its share of their merge to the last one.  Results do not depend on it, bit for bit: at 0 the last
  * one merges all rows, as it does where other work keeps the splits from running at the same time. */
 int32_t pipesd_debug_merge_polls(pipesd_ctx *ctx, int32_t polls);
+/* Host only: how pipesd_prefill cuts a prompt of n tokens (1..max_seq): *rows of the chunk behind its first `done`, and the
+ * last *logits rows of the last chunk whose logits it keeps. */
+int32_t pipesd_debug_prefill_chunk(const pipesd_model_cfg *cfg, int32_t n, int32_t done, int32_t *rows, int32_t *logits);
 /* CTAs of the attention kernel that the context's device keeps resident at once for a request with this many query
  * rows per KV head: out2 (host) = {with the whole third ring slot, with the cut-down one} -- the two numbers
  * pipesd_debug_attn_split takes. */

@@ -98,6 +98,7 @@ _SIGNATURES = {
                                         ctypes.c_double, ctypes.POINTER(i32)]),
     "pipesd_debug_force_dense": (i32, [vp, i32]),
     "pipesd_debug_merge_polls": (i32, [vp, i32]),
+    "pipesd_debug_prefill_chunk": (i32, [ctypes.POINTER(ModelCfg), i32, i32, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]),
     "pipesd_debug_gemm_dense_scratch_bytes": (u64, [i32, i32, i32]),
     "pipesd_debug_gemm_dense": (i32, [vp, vp, vp, vp, i32, i32, i32, i32, i32, vp]),
     "pipesd_debug_attn_slots": (i32, [vp, i32, ctypes.POINTER(ctypes.c_int32)]),

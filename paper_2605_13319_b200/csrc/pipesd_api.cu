@@ -450,6 +450,16 @@ int push_inflight(pipesd_ctx* ctx, pipesd_verify_result* dst, std::vector<pipesd
     return PIPESD_OK;
 }
 
+// Rows of the chunk of a prompt of n tokens that follows the first `done`.  Up to 32 tokens are passes of the small-M kernels;
+// more of them go through the dense kernels in chunks of up to row_cap rows, no two of which differ by more than one, so that
+// none is as short as a small-M pass: the last one leaves logits of its last rows only, which the dense kernels alone can do.
+int prompt_chunk(const pipesd_model_cfg& c, const Derived& d, int n, int done) {
+    if (n <= kMaxItemRows) return std::min(std::min(c.max_rows, kMaxItemRows), n - done);
+    const int chunks = (n - 1) / d.row_cap + 1;
+    return n / chunks + (done < (n % chunks) * (n / chunks + 1) ? 1 : 0);
+}
+int prompt_logits(const pipesd_model_cfg& c, int n) { return (n - 1) % std::min(c.max_rows, kMaxItemRows) + 1; }
+
 // Make sure the request owns pages for `need_len` positions. All-or-nothing is checked by the caller.
 int pages_needed(const pipesd_ctx* c, const Request& r, int need_len) {
     int need = (need_len + c->cfg.page_size - 1) / c->cfg.page_size;
@@ -991,14 +1001,9 @@ int32_t pipesd_prefill(pipesd_ctx* ctx, int32_t req, const int32_t* tokens, int3
         return fail(ctx, PIPESD_E_OOM_PAGES, "pipesd_prefill");
     int rc = grow_pages(ctx, req, r.len + n);
     if (rc != PIPESD_OK) return rc;
-    // Up to 32 tokens are a pass of the small-M kernels; more of them go through the dense kernels in equal chunks of up to
-    // row_cap rows, the last of which leaves logits of its last rows only.
-    const int small = std::min(ctx->cfg.max_rows, kMaxItemRows);
-    const int n_chunks = (n + ctx->dv.row_cap - 1) / ctx->dv.row_cap;
-    const int chunk = n <= kMaxItemRows ? small : (n + n_chunks - 1) / n_chunks;
-    const int n_logits = (n - 1) % small + 1;
-    for (int done = 0; done < n; done += chunk) {
-        int rows = std::min(chunk, n - done);
+    const int n_logits = prompt_logits(ctx->cfg, n);
+    for (int done = 0, rows; done < n; done += rows) {
+        rows = prompt_chunk(ctx->cfg, ctx->dv, n, done);
         bool last = done + rows == n;
         std::vector<ItemDesc> items(1);
         items[0] = ItemDesc{req, rows, 2, 0, tokens + done, nullptr, nullptr, r.len, kCommitNone, 0};
@@ -1394,6 +1399,13 @@ int32_t pipesd_debug_force_dense(pipesd_ctx* ctx, int32_t on) {
 int32_t pipesd_debug_merge_polls(pipesd_ctx* ctx, int32_t polls) {
     if (!ctx || polls < 0 || polls > 65536) return fail(ctx, PIPESD_E_INVALID, "pipesd_debug_merge_polls");
     ctx->merge_polls = polls;
+    return PIPESD_OK;
+}
+
+int32_t pipesd_debug_prefill_chunk(const pipesd_model_cfg* cfg, int32_t n, int32_t done, int32_t* rows, int32_t* logits) {
+    if (check_cfg(cfg) != PIPESD_OK || n < 1 || n > cfg->max_seq || done < 0 || done >= n || !rows || !logits) return PIPESD_E_INVALID;
+    *rows = prompt_chunk(*cfg, derive(*cfg), n, done);
+    *logits = prompt_logits(*cfg, n);
     return PIPESD_OK;
 }
 

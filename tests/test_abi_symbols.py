@@ -75,3 +75,28 @@ def test_attention_key_split_plan():
     import pytest
     with pytest.raises(binding.PipesdError):
         binding.debug_attn_split(100, 12, b200, 8)
+
+
+def test_prefill_chunks():
+    """A prompt is covered whole; beyond 32 tokens no chunk is as short as a small-M pass (33 rows at least), none longer than
+    the workspace holds, and the last one has the rows whose logits are kept -- also of prompts of a million tokens and odd
+    max_rows."""
+    rows, logits = ctypes.c_int32(), ctypes.c_int32()
+    for max_rows in (2, 13, 17, 31, 32, 96, 1500, 4096):
+        small = min(max_rows, 32)
+        for n in (1, 2, 13, 14, 31, 32, 33, 64, 1024, 1025, 1500, 2048, 2049, 4097, 5000, 1047557, 1048577, 2994197, 3000000):
+            for max_seq in (n, n + 777):
+                cfg = binding.ModelCfg(2, 256, 4, 4, 64, 688, 1024, 1e-5, 10000.0, 16, 1, 1, 1, max_rows, max_seq, 0, 0)
+                cap, done, sizes = max(max_rows, min(max_seq, 1024)), 0, []
+                while done < n:
+                    assert binding.lib().pipesd_debug_prefill_chunk(ctypes.byref(cfg), n, done, ctypes.byref(rows), ctypes.byref(logits)) == 0
+                    sizes.append(rows.value)
+                    assert rows.value > 0
+                    done += rows.value
+                assert done == n and max(sizes) <= cap
+                assert logits.value == (n - 1) % small + 1 <= sizes[-1]
+                if n > 32:
+                    assert min(sizes) > 32 and max(sizes) - min(sizes) <= 1 and len(sizes) == -(-n // cap)
+                else:
+                    assert max(sizes) <= small
+    assert binding.lib().pipesd_debug_prefill_chunk(ctypes.byref(cfg), n, n, ctypes.byref(rows), ctypes.byref(logits)) == binding.E_INVALID
