@@ -22,9 +22,10 @@
 // Warps 0-7: one thread per key of a tile (= tensor-memory lane; warps w and w+4 share a lane quarter and take
 // alternate 8-row column blocks): masking, exponentials relative to the score of the split's first key (any reference will
 // do that keeps p in range; a row's maximum is only looked for when a score exceeds its reference by 2^40 and O^T has to
-// be rescaled), P written back as the next MMA's B operand.  Warp 8: bulk copies of the K/V pages (a ring of three slots, K0 V0 K1 V1 ...; tiles of keys
-// that were cached before this pass do not depend on the preceding QKV projection and are requested before the
-// dependent-launch wait) and the MMA issue (one thread).  Every wait is bounded and raises the device error word.
+// be rescaled), P written back as the next MMA's B operand.  Warp 8: bulk copies of the K/V pages (a ring of three or four
+// slots, K0 V0 K1 V1 ...; tiles of keys that were cached before this pass do not depend on the preceding QKV projection and
+// are requested before the dependent-launch wait) and the MMA issue (one thread).  Every wait is bounded and raises the
+// device error word, but for the shared merge's, which needs nobody to give up.
 #pragma once
 #include "common.cuh"
 #include "layers.cuh"
@@ -82,10 +83,9 @@ __device__ __forceinline__ bool attn_workers_any(bool mine) {
     return any != 0;
 }
 
-// Shared-memory plan of one CTA with N query rows (a multiple of 16).  K and V tiles travel through a ring of three
-// slots in the order K0 V0 K1 V1 ...: two of a whole tile each and a third (a whole tile, or less
-// when no CTA of the launch has more than two tiles, the second of at most kAttnShortTail keys: the K/V of such a
-// CTA are then requested in full before the first product starts).
+// Shared-memory plan of one CTA with N query rows (a multiple of 16).  K and V tiles travel through a ring of three or four
+// slots (attn_ring_bytes) in the order K0 V0 K1 V1 ...; a cut-down third one, where no CTA of the launch has more than two
+// tiles and the second at most kAttnShortTail keys, still takes such a CTA's K/V in full before the first product starts.
 template <int HD>
 struct AttnSmem {
     static constexpr int kTileBytes = kAttnTile * HD * 2;            // one K or V tile
@@ -464,7 +464,7 @@ __global__ void __launch_bounds__(kAttnThreads, CU == 1 ? 3 : 1) attn_kernel(con
             if (!ok && a.err && lane == 0) atomicExch(a.err, 3);
         } else {
             // ---------------- thread = key of the tile (tensor-memory lane 32 * quarter + lane); the two warps of a
-            // lane quarter take alternate 16-row column blocks
+            // lane quarter take alternate 8-row column blocks
             const int quarter = warp & 3, half = warp >> 2;
             const int kt = quarter * 32 + lane;                         // key within the tile
             const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
@@ -732,7 +732,7 @@ __global__ void __launch_bounds__(kAttnThreads, CU == 1 ? 3 : 1) attn_kernel(con
     constexpr int kMergeBatch = 10;
     const int rl_step = share ? nsplit : 1;
 #pragma unroll 1
-    for (unsigned left = mine; left != 0u; left &= left - 1u)
+    for (unsigned left = mine; left != 0u; left &= left - 1u)    // shares to merge, one after the other
 #pragma unroll 1
     for (int rl = (share ? __ffs(left) - 1 : 0) + warp * rl_step; rl < n_rows; rl += rl_step * (kAttnThreads / 32)) {
         const size_t sl0 = slot0 + (size_t)rl * nsplit;
