@@ -221,8 +221,9 @@ int32_t pipesd_debug_wait_timeout(pipesd_ctx *ctx, int32_t limit_us);
  * pool).  Lets a harness replay rounds from a recorded point; the serving path uses pipesd_kv_rollback. */
 int32_t pipesd_debug_set_len(pipesd_ctx *ctx, int32_t req, int32_t new_len);
 
-/* Launch accounting.  While enabled, every kernel launch of the context is counted and every
- * weight-streaming GEMM launch is bracketed by CUDA events on the context's stream.
+/* Launch accounting.  Every kernel launch of the context is counted.  With time_gemms != 0 every pass runs on a kernel per
+ * projection, and every GEMM launch is bracketed by CUDA events on the context's stream (otherwise a pass of up to 32 rows is one
+ * kernel, which has no GEMM launches to time; the two agree to rounding).
  * pipesd_profile_read synchronises, reports the totals since the last read and resets them. */
 typedef struct pipesd_profile_info {
     int64_t kernel_launches; /* all kernels launched by the context                         */
@@ -245,7 +246,8 @@ int32_t pipesd_gemm_run(const void *packed, const float *x, float *y, void *scra
                         int32_t K, void *cuda_stream);
 
 /* Harness switch.  Passes of more than 32 rows run their projections on the dense tensor-core kernel, smaller passes
- * on the small-M weight-streaming kernel.  The small-M kernel sums a row in an order that follows the weights' shape alone;
+ * in the layer-stack kernel (or, where a request has more than 72 query rows per KV head, on the small-M weight-streaming
+ * kernel).  Both of these sum a row in an order that follows the weights' shape (and the number of SMs) alone;
  * the dense kernel cuts K into slices by the pass's row count as well, so that a row's projections agree to rounding, not
  * bit for bit, between passes of different row counts (and between the kernels).  on != 0 makes every pass of the context
  * use the dense kernel; on > 1 also gives passes of fewer rows the slices of a pass of `on` rows, so that a request

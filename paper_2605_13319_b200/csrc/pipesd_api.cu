@@ -21,6 +21,7 @@
 #include "gemm_dense.cuh"
 #include "layers.cuh"
 #include "reject.cuh"
+#include "stack.cuh"
 
 using namespace pipesd;
 
@@ -108,11 +109,24 @@ size_t attn_part_slots(const pipesd_model_cfg& c) { return (size_t)c.max_rows * 
 
 struct WsLayout {
     size_t x, xf_h, qbuf, xf_attn, xf_act, logits, partA, partB, ssqA, ssqB, o_part, m_part, l_part, tickets, cs, sn, kvoff, stats, results, meta,
-        block_tab, qstage, req_state, never_flag, total;
+        block_tab, qstage, req_state, never_flag, st_ssq, st_q, st_sync, st_ll, total;
 };
 
 size_t ticket_bytes(const pipesd_model_cfg& c, const Derived& d) { return 4 * (size_t)d.row_cap * c.n_q_heads; }
 constexpr size_t kXdPad = 2 * kDenseMaxHalf + 16;
+
+// Rows of the largest pass that the layer-stack kernel takes, and bytes of its Q (each request's rows padded to whole groups of eight).
+int stack_rows(const pipesd_model_cfg& c) { return std::min(c.max_rows, kMaxItemRows); }
+// Rows of exchange words per CTA and shared row block, over all projections; the device may have fewer SMs than the most.
+int stack_ll_block(const pipesd_model_cfg& c, const Derived& d, int rows) {
+    const int n[5] = {d.Nqkv, c.d_model, 2 * c.d_ffn, c.d_model, c.vocab}, k[5] = {c.d_model, d.qd, c.d_model, c.d_ffn, c.d_model};
+    int best = 0;
+    for (int i = 0; i < 5; ++i) best = std::max(best, stack_block_rows(rows, k[i] / 16, (n[i] + 127) / 128, kStackMaxCtas));
+    return best;
+}
+size_t stack_q_bytes(const pipesd_model_cfg& c) {
+    return 4 * (size_t)c.head_dim * ((size_t)c.n_q_heads * stack_rows(c) + 7 * (size_t)c.n_kv_heads * std::min(c.max_requests, kStackMaxItems));
+}
 
 WsLayout ws_layout(const pipesd_model_cfg& c, const Derived& d) {
     WsLayout w;
@@ -146,6 +160,13 @@ WsLayout ws_layout(const pipesd_model_cfg& c, const Derived& d) {
     w.qstage = take(4 * Mv * c.vocab);
     w.req_state = take(sizeof(ReqState) * (size_t)c.max_requests);
     w.never_flag = take(16);
+    // the layer-stack kernel's: sums of squares (two sets), Q in operand order, arrivals, exchange words
+    const int rows = stack_rows(c);
+    w.st_ssq = take(2 * 4 * (size_t)rows * 4 * nssq);
+    w.st_q = take(stack_q_bytes(c));
+    w.st_sync = take(kStackSyncBytes);
+    w.st_ll = take(16 * std::max((size_t)2 * kStackMaxCtas * stack_ll_block(c, d, rows) * 128,
+                                stack_ll_rows(rows, c.n_q_heads, c.n_kv_heads) * (c.head_dim + 1)));
     w.total = o;
     return w;
 }
@@ -175,8 +196,17 @@ const void* attn_fn(int hd, bool big) {
     return hd == 128 ? (const void*)attn_kernel<128, 1> : (const void*)attn_kernel<64, 1>;
 }
 
+using StackFn = void (*)(StackArgs);
+StackFn stack_fn(int NT, int hd) {
+    if (hd == 128) return NT <= 2 ? layer_stack_kernel<2, 128> : layer_stack_kernel<4, 128>;
+    return NT <= 2 ? layer_stack_kernel<2, 64> : layer_stack_kernel<4, 64>;
+}
+
 cudaError_t init_attrs_current_device() {
     cudaError_t e;
+    for (int NT : {2, 4})
+        for (int hd : {64, 128})
+            if ((e = cudaFuncSetAttribute((const void*)stack_fn(NT, hd), cudaFuncAttributeMaxDynamicSharedMemorySize, kStackSmemMax)) != cudaSuccess) return e;
     if ((e = gemm_init_attrs()) != cudaSuccess) return e;
     const void* dense_fns[4] = {(const void*)gemm_dense_kernel<kPlain>, (const void*)gemm_dense_kernel<kQkvRope>,
                                 (const void*)gemm_dense_kernel<kResid>, (const void*)gemm_dense_kernel<kSwiglu>};
@@ -300,6 +330,8 @@ struct pipesd_ctx {
     int merge_polls = kAttnMergePolls;
     bool force_dense = false;   // harness switch: the dense kernels also for passes of at most 32 rows ...
     int plan_rows = 0;          // ... with the plans of a pass of this many rows
+    int stack_ctas = 0;         // CTAs of the layer-stack kernel, one per SM (0: the device cannot launch it)
+    uint64_t stack_phases = 0;  // phases run since the exchange words were last cleared
     bool pass_dense = false;    // the pass being enqueued runs on the dense kernels
     // bytes of the O and gate/up weights the attention kernel pulls into L2 once its K/V has landed (measured: all of O
     // and 16 MB of gate/up; more gains nothing, an SM takes data in only about 1.4 times faster than HBM delivers it)
@@ -343,10 +375,18 @@ int fail(pipesd_ctx* c, int code, const char* what) {
     return code;
 }
 
+// The layer-stack kernel's arrival count, phase number and exchange words start at zero.
+cudaError_t clear_stack_flags(pipesd_ctx* c) {
+    c->stack_phases = 0;
+    return cudaMemsetAsync(c->wsp + c->ws.st_sync, 0, c->ws.total - c->ws.st_sync, c->st);
+}
+
 // The device error word and the attention tickets start at zero, and again after an error (the tickets reset themselves in use).
 cudaError_t clear_device_flags(pipesd_ctx* c) {
     const cudaError_t e = cudaMemsetAsync(c->err_word(), 0, 4, c->st);
-    return e != cudaSuccess ? e : cudaMemsetAsync(c->wsp + c->ws.tickets, 0, ticket_bytes(c->cfg, c->dv), c->st);
+    if (e != cudaSuccess) return e;
+    const cudaError_t e2 = cudaMemsetAsync(c->wsp + c->ws.tickets, 0, ticket_bytes(c->cfg, c->dv), c->st);
+    return e2 != cudaSuccess ? e2 : clear_stack_flags(c);
 }
 
 int cuda_fail(pipesd_ctx* c, cudaError_t e, const char* where) {
@@ -488,6 +528,114 @@ void shrink_pages(pipesd_ctx* c, Request& r, int keep_len) {
     }
 }
 
+// Key ranges of the layer-stack kernel's CTAs, in units of 16 keys, hold at most this many (request, KV head) pairs' parts.
+int stack_segments(const pipesd_model_cfg& c, const std::vector<ItemDesc>& items, int ctas) {
+    long units = 0;
+    int shortest = 1 << 30;
+    for (const ItemDesc& it : items) {
+        const int u = (it.base + it.rows + 15) / 16;
+        units += (long)u * c.n_kv_heads;
+        shortest = std::min(shortest, u);
+    }
+    const long per = std::max<long>((units + ctas - 1) / ctas, 4);
+    return (int)std::min<long>((per + shortest - 1) / shortest + 1, 1 << 20);
+}
+
+// Whether a pass is the layer-stack kernel's: up to 32 rows, of requests whose query rows per KV head fit its tensor memory, in a
+// batch whose key ranges fit its tables.  The others (prompts of 19 to 32 tokens at four query heads per KV head, say), and every
+// pass while GEMM launches are timed, run on a kernel per projection, as all did before: us a pass on one box, 7b shape, 9 rows
+// 3224 -> 2850, 17 rows 3906 -> 3178; 8b shape, 17 rows 5033 -> 3925; 1b shape, 9 rows 1003 -> 891; tiny 116 -> 116.
+bool stack_takes(const pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int M, StackPlan* plan, int* n_max, int* r_max) {
+    const pipesd_model_cfg& c = ctx->cfg;
+    if (ctx->stack_ctas < 1 || M > kMaxItemRows || ctx->force_dense || ctx->time_gemms || (int)items.size() > kStackMaxItems) return false;
+    int rows = 1;
+    for (const ItemDesc& it : items) rows = std::max(rows, it.rows);
+    *r_max = rows * (c.n_q_heads / c.n_kv_heads);
+    *n_max = (*r_max + 7) / 8 * 8;
+    return *n_max <= kStackMaxN && stack_segments(c, items, ctx->stack_ctas) <= kStackMaxSegs && stack_plan(plan, M, c.head_dim, *n_max);
+}
+
+// Launch the layer-stack kernel over the M rows whose metadata has been uploaded.
+int launch_stack(pipesd_ctx* ctx, const StackPlan& plan, int n_items, int M, int n_max, int r_max, const PassMeta& meta, bool want_logits) {
+    const pipesd_model_cfg& c = ctx->cfg;
+    const LayerW& l0 = ctx->layers[0];
+    const int G = ctx->stack_ctas, hd = c.head_dim;
+    StackArgs a = {};
+    auto gemm = [&](int kind, const GemmW& w, const void* act) {
+        StackGemm& g = a.g[kind];
+        g.w = reinterpret_cast<const unsigned char*>(w.packed);
+        g.act = static_cast<const unsigned char*>(act);
+        g.N = w.N;
+        g.KS = w.K / 16;
+        g.RB = (w.N + 127) / 128;
+        g.per = stack_per(g.KS, g.RB, G);
+        g.flush = dense_chunk(g.KS) / kStackSteps;
+    };
+    a.act_h = ctx->W<uint16_t>(ctx->ws.xf_h);
+    a.act_attn = ctx->W<uint16_t>(ctx->ws.xf_attn);
+    a.act_ffn = ctx->W<uint16_t>(ctx->ws.xf_act);
+    gemm(kStQkv, l0.qkv, a.act_h);
+    gemm(kStO, l0.o, a.act_attn);
+    gemm(kStGu, l0.gu, a.act_h);
+    gemm(kStDn, l0.dn, a.act_ffn);
+    gemm(kStLm, ctx->lm, a.act_h);
+    a.layer_stride = c.n_layers > 1 ? (size_t)((const char*)ctx->layers[1].qkv.packed - (const char*)l0.qkv.packed) : 0;
+    a.n1 = l0.n1;
+    a.n2 = l0.n2;
+    a.final_norm = ctx->final_norm;
+    a.emb = ctx->emb;
+    a.meta = meta;
+    a.kv_pool = ctx->kv_pool;
+    a.x = ctx->W<float>(ctx->ws.x);
+    a.cs = ctx->W<float>(ctx->ws.cs);
+    a.sn = ctx->W<float>(ctx->ws.sn);
+    a.logits = ctx->W<float>(ctx->ws.logits);
+    a.n_ssq = 4 * ((c.d_model + 127) / 128);
+    a.ssq_a = ctx->W<float>(ctx->ws.st_ssq);
+    a.ssq_b = a.ssq_a + (size_t)stack_rows(c) * a.n_ssq;
+    a.qop = ctx->W<uint16_t>(ctx->ws.st_q);
+    a.qop_bytes = stack_q_bytes(c);
+    a.ll = ctx->W<uint4>(ctx->ws.st_ll);
+    a.ll_rows = stack_ll_block(c, ctx->dv, stack_rows(c));
+    a.ll_ml = stack_ll_rows(stack_rows(c), c.n_q_heads, c.n_kv_heads) * hd;
+    a.sync = ctx->W<unsigned>(ctx->ws.st_sync);
+    a.err = ctx->err_word();
+    a.n_layers = c.n_layers;
+    a.d = c.d_model;
+    a.Hq = c.n_q_heads;
+    a.Hkv = c.n_kv_heads;
+    a.M = M;
+    a.T = plan.T;
+    a.n_items = n_items;
+    a.want_logits = want_logits;
+    a.n_pages = c.n_pages;
+    a.page_size = c.page_size;
+    a.slots = plan.slots;
+    a.acts = plan.acts;
+    a.n_max = n_max;
+    a.r_max = r_max;
+    a.q_bufs = plan.q_bufs;
+    a.p_bufs = plan.p_bufs;
+    a.eps = c.rms_eps;
+    a.log_base = log((double)c.rope_base);
+    // a phase number must not come round to one that a word still carries
+    ctx->stack_phases += 2 + 5 * (uint64_t)c.n_layers;
+    if (ctx->stack_phases > (1ull << 31)) CU(clear_stack_flags(ctx));
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.gridDim = dim3(G);
+    cfg.blockDim = dim3(kStackThreads);
+    cfg.dynamicSmemBytes = plan.smem;
+    cfg.stream = ctx->st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    CU(cudaLaunchKernelEx(&cfg, stack_fn(plan.T / 8, hd), a));
+    ctx->n_launch += 1;
+    return PIPESD_OK;
+}
+
 // Upload the metadata of one pass and run the layer stack over M rows.  Logits are wanted of the last n_logits rows (of
 // all rows unless the pass is a prompt chunk of more than 32).
 int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, bool want_reject) {
@@ -606,6 +754,13 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
     const int hd = c.head_dim, Hq = c.n_q_heads, Hkv = c.n_kv_heads, d = c.d_model, F = c.d_ffn;
     const int n_ssq = (d + 127) / 128;
 
+    StackPlan splan;
+    int st_n = 0, st_r = 0;
+    const bool stacked = stack_takes(ctx, items, M, &splan, &st_n, &st_r);
+    if (stacked) {
+        int rc_ = launch_stack(ctx, splan, n_items, M, st_n, st_r, meta, want_logits);
+        if (rc_) return rc_;
+    }
     // Passes of more than 32 rows run their GEMMs on the dense kernels (every weight byte read once per block of up to 256
     // tokens); their activation arrays are in that kernel's operand order, with the token block size of the consumer.
     ctx->pass_dense = M > 32 || ctx->force_dense;
@@ -614,7 +769,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
               tbs_o = dense ? dense_plan_from(M, 0, ctx->plan_rows, d, dv.qd, ctx->dense_pairs).tbs : 0;
     // Every kernel of the chain is launched with programmatic stream serialisation: it may start while its
     // predecessor drains and blocks in griddepcontrol.wait before touching the predecessor's output.
-    {
+    if (!stacked) {
         int n = M * hd / 2;
         CU(launch_pdl(rope_table_kernel, dim3((n + 127) / 128), dim3(128), 0, st, meta, M, hd, log((double)c.rope_base),
                       cs, sn, ctx->W<long long>(ctx->ws.kvoff), c.n_pages, Hkv, c.page_size));
@@ -664,7 +819,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
         ctx->n_launch += 1;
         return PIPESD_OK;
     };
-    for (int l = 0; l < c.n_layers; ++l) {
+    for (int l = 0; l < c.n_layers && !stacked; ++l) {
         const LayerW& lw = ctx->layers[l];
         {   // q, k, v = W_qkv . norm(x); RoPE; K/V appended to the pages
             GemmArgs a = base;
@@ -708,7 +863,7 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
     if (want_logits) {
         float* logits = ctx->W<float>(ctx->ws.logits);
         RowStat* stats = ctx->W<RowStat>(ctx->ws.stats);
-        {
+        if (!stacked) {
             GemmArgs a = base;
             a.xf = (const uint4*)xf_h; a.N = c.vocab; a.ssq_in = ssqA; a.out = logits;
             int rc_ = launch_gemm(ctx, kPlain, ctx->lm, a, d, 0, 0, M - n_logits);
@@ -717,8 +872,9 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
         ctx->last_rows = n_logits;
         if (want_reject) {
             ctx->n_launch += 2;
-            // a plain launch: it starts after the GEMM has fully completed
-            row_stats_kernel<<<dim3(M, kStatSplits), 256, 0, st>>>(c.vocab, logits, stats);
+            // behind a GEMM a plain launch: it starts after that has fully completed
+            if (stacked) CU(launch_pdl(row_stats_kernel, dim3(M, kStatSplits), dim3(256), 0, st, c.vocab, (const float*)logits, stats));
+            else row_stats_kernel<<<dim3(M, kStatSplits), 256, 0, st>>>(c.vocab, logits, stats);
             CU(launch_pdl_cluster(accept_sample_kernel, dim3(kSampleCluster, n_items), dim3(kSampleThreads), 0, st,
                                   kSampleCluster, (const float*)logits, c.vocab, (const RowStat*)stats,
                                   reinterpret_cast<const RejectItem*>(ctx->wsp + ctx->ws.meta + ml.rej), meta.row_tok,
@@ -797,6 +953,9 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
             cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, c.device) != cudaSuccess ||
             cudaDeviceGetAttribute(&thr_sm, cudaDevAttrMaxThreadsPerMultiProcessor, c.device) != cudaSuccess)
             return bail(PIPESD_E_CUDA);
+        int coop = 0;
+        if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c.device) != cudaSuccess) return bail(PIPESD_E_CUDA);
+        ctx->stack_ctas = coop ? std::min(n_sm, kStackMaxCtas) : 0;
         for (int S = 1; S <= kDenseMaxSlices; ++S) {
             cudaLaunchConfig_t lc = {};
             cudaLaunchAttribute at[1];

@@ -22,6 +22,7 @@ struct RowStat {
 // Per (row, split) of the logits: max, argmax, sum-exp.  grid (M, kStatSplits), block 256.
 __global__ void __launch_bounds__(256) row_stats_kernel(int V, const float* __restrict__ logits,
                                                         RowStat* __restrict__ stats) {
+    pdl_wait();      // (where it is launched with programmatic serialisation)
     const int row = blockIdx.x, sp = blockIdx.y;
     const int per = (V + kStatSplits - 1) / kStatSplits;
     const int j0 = sp * per, j1 = min(V, j0 + per);

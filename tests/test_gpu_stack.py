@@ -1,0 +1,83 @@
+"""The layer-stack kernel (passes of up to 32 rows) against the kernels per projection, which run the same pass while GEMM
+launches are timed: logits and the new K/V rows, at the sizes where its plans change."""
+import numpy as np
+import pytest
+
+from paper_2605_13319_b200 import synth
+from harness import logit_rel_err
+
+pytestmark = pytest.mark.gpu
+
+# Both sum fp32 in different orders; what differs beyond 2^-20 is that K and V are stored as bf16, where a value at a rounding
+# boundary goes either way (2^-8 of itself) and later layers see that: up to 4e-4 of a row's largest logit in these shapes.
+TOL = 2e-3
+
+T = synth.TINY
+CASES = {
+    # one request: shape, prefix lengths, drafts per request, page size
+    "one key": (T, [1], [1], 16),
+    "head 128": (T.scaled(d_model=512, n_q_heads=4, n_kv_heads=4, head_dim=128), [130], [8], 16),
+    "four heads share, 72 rows": (T.scaled(n_q_heads=8, n_kv_heads=2, head_dim=64, d_model=512), [700], [17], 16),
+    "eight heads share one, 72 rows": (T.scaled(n_q_heads=8, n_kv_heads=1, head_dim=128, d_model=1024), [5000], [8], 16),
+    "32 rows": (T, [257], [31], 16),
+    "25 rows, pages of 8": (T, [255], [24], 8),
+    "pages of 256": (T, [600], [6], 256),
+    "ranges of several tiles": (T.scaled(d_model=2048, n_q_heads=16, n_kv_heads=16, head_dim=128), [2500], [8], 16),
+    "ragged widths": (T.scaled(d_model=272, d_ffn=176, vocab=1040), [33], [3], 16),
+    "narrow": (T.scaled(d_model=48, n_q_heads=1, n_kv_heads=1, d_ffn=32, vocab=48), [90], [2], 16),
+    "wide, whole row blocks": (T.scaled(d_model=1024, d_ffn=4096, vocab=32000), [64], [5], 16),
+    "16 requests of two rows": (T, [3, 17, 400, 129, 5, 6, 7, 900, 1, 64, 65, 66, 31, 32, 33, 250], [1] * 16, 16),
+    "three requests": (T.scaled(n_kv_heads=2), [40, 1200, 300], [16, 2, 9], 16),
+}
+
+
+def _run(ctx, items, lens, rows, layers):
+    from paper_2605_13319_b200 import binding
+    got = ctx.verify(items, flags=binding.Q_HOST)
+    logits = ctx.debug_get_logits(rows)
+    ctx.kv_rollback([it["req"] for it in items], [len(it["tokens"]) - 1 for it in items])
+    kv = []
+    for it, P in zip(items, lens):
+        for l in layers:
+            kv += [synth.bf16_to_f32(x) for x in ctx.debug_read_kv(it["req"], l, P, len(it["tokens"]))]
+        ctx.debug_set_len(it["req"], P)
+    return got, logits, kv
+
+
+@pytest.mark.parametrize("name", list(CASES))
+@pytest.mark.parametrize("growing", [False, True])
+def test_against_the_kernels_per_projection(name, growing):
+    """`growing`: keys grow along the prefix, so that scores exceed a segment's first one by far and sums are rescaled."""
+    from paper_2605_13319_b200 import binding
+    shape, lens, ks, page = CASES[name]
+    if growing and max(lens) < 200:
+        pytest.skip("nothing to rescale")
+    w = synth.make_weights(shape, 11)
+    rows = sum(ks) + len(ks)
+    ctx = binding.Context(shape, w, n_pages=sum((P + 40) // page + 1 for P in lens), max_requests=len(lens), max_rows=rows, max_seq=max(lens) + 40,
+                          max_draft=max(ks), page_size=page, poison=True)
+    items = []
+    for i, (P, k) in enumerate(zip(lens, ks)):
+        req = ctx.req_open()
+        for l in range(shape.n_layers):
+            kb, vb = synth.make_synthetic_kv(shape, P, 11 + i, l)
+            if growing:
+                ramp = np.linspace(0.0, 60.0, P, dtype=np.float32)[:, None]
+                kb = synth.f32_to_bf16(synth.bf16_to_f32(kb).reshape(P, -1) * ramp).reshape(kb.shape)
+            ctx.debug_write_kv(req, l, 0, kb, vb)
+        items.append(dict(req=req, tokens=synth.tokens_i32(k + 1, 11, 900 + i, shape.vocab), u=synth.make_accept_uniforms(k, 11, i),
+                          q=np.full((k, shape.vocab), 1.0 / shape.vocab, np.float32)))
+    layers = range(shape.n_layers)
+    ctx.profile_enable(True)
+    _, want, want_kv = _run(ctx, items, lens, rows, layers)
+    launches = ctx.profile_read()["kernel_launches"]
+    ctx.profile_enable(False)
+    for _ in range(2):                                         # the second on what the first left in the exchange words
+        _, got, got_kv = _run(ctx, items, lens, rows, layers)
+        assert ctx.profile_read()["kernel_launches"] == 3 < launches
+        assert np.isfinite(got).all()
+        # scores of a few hundred carry errors of 2^-17 of themselves, and probabilities as much in relative terms
+        assert logit_rel_err(got, want).max() < (2e-2 if growing else TOL)
+        for a, b in zip(got_kv, want_kv):
+            assert np.all(np.abs(a - b) <= 2.0 ** -7 * np.abs(b) + (2e-2 if growing else 2e-3) * np.abs(b).max())
+    ctx.close()
