@@ -198,13 +198,14 @@ const void* attn_fn(int hd, bool big) {
 
 using StackFn = void (*)(StackArgs);
 StackFn stack_fn(int NT, int hd) {
-    if (hd == 128) return NT <= 2 ? layer_stack_kernel<2, 128> : layer_stack_kernel<4, 128>;
-    return NT <= 2 ? layer_stack_kernel<2, 64> : layer_stack_kernel<4, 64>;
+    static const StackFn fns[2][4] = {{layer_stack_kernel<1, 64>, layer_stack_kernel<2, 64>, layer_stack_kernel<3, 64>, layer_stack_kernel<4, 64>},
+                                      {layer_stack_kernel<1, 128>, layer_stack_kernel<2, 128>, layer_stack_kernel<3, 128>, layer_stack_kernel<4, 128>}};
+    return fns[hd == 128][NT - 1];
 }
 
 cudaError_t init_attrs_current_device() {
     cudaError_t e;
-    for (int NT : {2, 4})
+    for (int NT : {1, 2, 3, 4})
         for (int hd : {64, 128})
             if ((e = cudaFuncSetAttribute((const void*)stack_fn(NT, hd), cudaFuncAttributeMaxDynamicSharedMemorySize, kStackSmemMax)) != cudaSuccess) return e;
     if ((e = gemm_init_attrs()) != cudaSuccess) return e;
@@ -605,7 +606,6 @@ int launch_stack(pipesd_ctx* ctx, const StackPlan& plan, int n_items, int M, int
     a.Hq = c.n_q_heads;
     a.Hkv = c.n_kv_heads;
     a.M = M;
-    a.T = plan.T;
     a.n_items = n_items;
     a.want_logits = want_logits;
     a.n_pages = c.n_pages;

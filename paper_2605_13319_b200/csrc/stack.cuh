@@ -82,7 +82,7 @@ struct StackArgs {
     int ll_rows;                 // rows of 128 words per CTA and shared row block
     unsigned* sync;
     int* err;
-    int n_layers, d, Hq, Hkv, M, T, n_items, want_logits, n_pages, page_size, n_ssq;
+    int n_layers, d, Hq, Hkv, M, n_items, want_logits, n_pages, page_size, n_ssq;
     int slots, acts;             // ring slots, activation slots
     int n_max, r_max, q_bufs, p_bufs;   // attention: N and rows per KV head of the largest request; buffers of Q and P
     float eps;
@@ -185,6 +185,7 @@ __device__ __forceinline__ bool stack_try(uint32_t bar, uint32_t parity) {
 }
 __device__ __forceinline__ bool stack_wait(uint32_t bar, uint32_t parity) {
     bool done = false;
+#pragma unroll 1
     for (uint32_t it = 0; it < kStackTries; ++it) {
         if (stack_try(bar, parity)) { done = true; break; }
     }
@@ -296,12 +297,15 @@ struct StackRing {
     }
     __device__ __forceinline__ void skip(int k, int n) {
         slot += k;
+#pragma unroll 1
         while (slot >= n) { slot -= n; par ^= 1u; }
     }
 };
 
-// NTM: token tiles of eight that a worker's registers hold (2 or 4).
-template <int NTM, int HD>
+// NT: groups of eight rows of the pass (1 to 4).  A constant, so that the MMA's descriptors differ by constants: the issuing warp's
+// instructions are what a stage costs it.  (us a pass, with the waits' loops not unrolled, 125 KB of code instead of 170: 7b shape, 9
+// rows 2844 -> 2794, 17 rows 3181 -> 3123; 8b shape, 17 rows 3910 -> 3862; 1b shape, 9 rows 888 -> 864.)
+template <int NT, int HD>
 __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __grid_constant__ StackArgs a) {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int HG = HD / 8;
@@ -309,7 +313,8 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
     constexpr int kPerTile = HD == 128 ? 2 : 1;               // ring slots a K/V tile pair takes
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int cta = blockIdx.x, n_cta = gridDim.x;
-    const int NT = a.T / 8;
+    constexpr int T = 8 * NT;
+    constexpr int act_stage = NT * kStackSteps * 512, act_step = NT * 512;
     unsigned char* ones = smem;
     unsigned char* ring = smem + 256;
     unsigned char* scratch = ring + a.slots * kStackSlot;
@@ -319,7 +324,6 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
     float* m_ref = wm + 4 * a.n_max;                          // [N] reference score
     float* alpha = m_ref + a.n_max;                           // [N] rescale factor
     const uint32_t ring_a = smem_u32(ring), scratch_a = smem_u32(scratch);
-    const int act_stage = NT * kStackSteps * 512, act_step = NT * 512;
     const int q_bytes = a.n_max * HD * 4;
     unsigned char* p_op = scratch + a.q_bufs * q_bytes;       // P, hi and lo terms
     volatile int* abort_s = &sm.abort;
@@ -525,7 +529,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
             StackRing rw = {0, 0u}, ra = {0, 0u}, rd = {0, 1u};     // rd: accumulators, `empty` parity
             unsigned tile = 0, q_n = 0, staged = 0;                 // staged: weights' stages in tensor memory
             bool ok = true;
-            const uint32_t idesc = umma_idesc_bf16(128, 16 * NT, 0, 0);
+            constexpr uint32_t idesc = umma_idesc_bf16(128, 16 * NT, 0, 0);
             int put = 0, get = 0;                                   // their places, of kStackStaged
             auto staged_at = [&](int i) { return tmem + 512u - 64u * (uint32_t)(i + 1); };
             auto gemm = [&](const StackGemm& g, int room) -> bool {
@@ -569,7 +573,8 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
 #pragma unroll 1
                         for (int f = 0; f < g.flush && ks < end; ++f) {
                             const int n = min((ks | (kStackSteps - 1)) + 1, end) - ks;
-                            const uint64_t bd = umma_desc(scratch_a + ra.slot * act_stage, 128, 256), bs = (uint64_t)(act_step >> 4);
+                            const uint64_t bd = umma_desc(scratch_a + ra.slot * act_stage, 128, 256);
+                            constexpr uint64_t bs = act_step >> 4;
                             if (!fresh) if (!stack_wait(smem_u32(&sm.full_a[ra.slot]), ra.par)) return false;
                             fresh = false;
                             if (staged > 0) {
@@ -698,6 +703,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 // weights to come before the next K/V tile; tensor memory beside the attention's columns while those are in use
                 if (p == 0) ok = stack_wait(smem_u32(&sm.tables), 0u);
                 int room = 0;
+#pragma unroll 1
                 for (int q = kind, i = p; q != kStAttn && i < n_phase; ++i) {
                     room += sm.geo[q].stages;
                     q = q == kStLm ? kStAttn : q == kStDn ? (i + 1 < 5 * a.n_layers ? kStQkv : kStLm) : q + 1;
@@ -792,6 +798,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
         uint32_t tries = kStackTries;         // one, once a wait has run out
         auto wait = [&](unsigned long long& bar, uint32_t parity) {
             bool done = false;
+#pragma unroll 1
             for (uint32_t it = 0; it < tries; ++it) {
                 if (stack_try(smem_u32(&bar), parity)) { done = true; break; }
             }
@@ -817,9 +824,9 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
         auto act_put = [&](bool live, uint16_t* dst, int t, int k, float v) {
             uint16_t h, l;
             split_bf16(v, h, l);
-            uint16_t* p = dst + (k >> 4) * (a.T * 32) + ((t >> 3) * 2 + ((k >> 3) & 1)) * 64 + (t & 7) * 8 + (k & 7);
+            uint16_t* p = dst + (k >> 4) * (T * 32) + ((t >> 3) * 2 + ((k >> 3) & 1)) * 64 + (t & 7) * 8 + (k & 7);
             st_if(live, p, h);
-            st_if(live, p + a.T * 16, l);
+            st_if(live, p + T * 16, l);
         };
 
         // ---- this CTA's part of the projections, one per warp
@@ -873,12 +880,12 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 *reinterpret_cast<float4*>(a.x + (size_t)row * a.d + e) = v;
                 ss += v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w;
                 const float4 g = *reinterpret_cast<const float4*>(a.n1 + e);
-                uint16_t* xd = a.act_h + act_index_row(row, e >> 4, a.d / 16, 0, a.T) + act_index_col(e & 15, 0, a.T);
+                uint16_t* xd = a.act_h + act_index_row(row, e >> 4, a.d / 16, 0, T) + act_index_col(e & 15, 0, T);
                 uint2 h, lo;
                 split_bf16x2(v.x * g.x, v.y * g.y, h.x, lo.x);
                 split_bf16x2(v.z * g.z, v.w * g.w, h.y, lo.y);
                 *reinterpret_cast<uint2*>(xd) = h;
-                *reinterpret_cast<uint2*>(xd + act_index_lo(a.T)) = lo;
+                *reinterpret_cast<uint2*>(xd + act_index_lo(T)) = lo;
             }
             ss = warp_sum(ss);
             if (lane == 0) sm.red[warp - 4] = ss;
@@ -1007,7 +1014,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 const int q = k / 3;
                 fetch(q < n_ent && k - 3 * q < ent[q].n, row_sel(ent[q].w), ent[q].t + k - 3 * q, xa[k], xb[k]);
             }
-            constexpr int kVals = 4 * NTM > 6 ? 4 * NTM : 6;
+            constexpr int kVals = 4 * NT > 6 ? 4 * NT : 6;
 #pragma unroll 1
             for (;;) {
                 // either a row block of which all K is here, or two groups of shared ones: rows t .. t + n - 1 of `row`, then of `rowb`
@@ -1025,19 +1032,17 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                         wait(sm.d_full[rd.slot], rd.par);
                         tc_fence_after();
                         const uint32_t d = tmem + 64u * rd.slot + lane_sel + (uint32_t)t_half;
-                        float hi[4 * NTM], lo[4 * NTM];
+                        float hi[4 * NT], lo[4 * NT];
 #pragma unroll
-                        for (int k = 0; k < NTM; ++k) {
-                            if (k < NT) {
-                                tmem_ld4(d + 4 * k, hi + 4 * k);
-                                tmem_ld4(d + 8 * NT + 4 * k, lo + 4 * k);
-                            }
+                        for (int k = 0; k < NT; ++k) {
+                            tmem_ld4(d + 4 * k, hi + 4 * k);
+                            tmem_ld4(d + 8 * NT + 4 * k, lo + 4 * k);
                         }
                         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-                        for (int k = 0; k < 4 * NTM; ++k) {
+                        for (int k = 0; k < 4 * NT; ++k) {
                             asm volatile("" : "+f"(hi[k]), "+f"(lo[k]));            // not read ahead of the wait
-                            if (k < 4 * NT) val[k] += hi[k] + lo[k];
+                            val[k] += hi[k] + lo[k];
                         }
                         tc_fence_before();
                         __syncwarp();
@@ -1056,15 +1061,15 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                         uint4* p = a.ll + quarter * 32 + lane;
                         if (gs == 1) {
 #pragma unroll
-                            for (int k = 0; k < 4 * NTM; ++k) ll_store_if(k < n_half, p + (size_t)to[k] * 128, val[k], 0.f, 0.f, epoch);
+                            for (int k = 0; k < 4 * NT; ++k) ll_store_if(k < n_half, p + (size_t)to[k] * 128, val[k], 0.f, 0.f, epoch);
                         } else if (gs == 2) {
 #pragma unroll
-                            for (int k = 0; k < 4 * NTM; k += 2) ll_store_if(k < n_half, p + (size_t)to[k / 2] * 128, val[k], val[k + 1], 0.f, epoch);
+                            for (int k = 0; k < 4 * NT; k += 2) ll_store_if(k < n_half, p + (size_t)to[k / 2] * 128, val[k], val[k + 1], 0.f, epoch);
                         } else {
 #pragma unroll
-                            for (int k = 0; k < 4 * NTM; k += 3)
-                                ll_store_if(k < n_half, p + (size_t)to[k / 3] * 128, val[k], k + 1 < 4 * NTM ? val[k + 1 < 4 * NTM ? k + 1 : 0] : 0.f,
-                                            k + 2 < 4 * NTM ? val[k + 2 < 4 * NTM ? k + 2 : 0] : 0.f, epoch);
+                            for (int k = 0; k < 4 * NT; k += 3)
+                                ll_store_if(k < n_half, p + (size_t)to[k / 3] * 128, val[k], k + 1 < 4 * NT ? val[k + 1 < 4 * NT ? k + 1 : 0] : 0.f,
+                                            k + 2 < 4 * NT ? val[k + 2 < 4 * NT ? k + 2 : 0] : 0.f, epoch);
                         }
                         continue;
                     }
