@@ -721,7 +721,19 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
         const int G = a.Hq / a.Hkv;
         int rows = 0, kb = 0;
         if (lane < a.n_items) { rows = a.meta.it_rows[lane]; kb = a.meta.it_base[lane]; }
-        const int units = (kb + rows + 15) / 16;                     // of 16 keys, per KV head
+        // Units of 16 keys per KV head, `per` of them a CTA's; at least 64 keys: shorter parts would only add partial results to
+        // exchange.  If ranges up to a quarter longer let every range end with its head (so that a CTA has one part), heads are padded
+        // to whole ranges: a second part costs a CTA two to three us, a tile 1.5.  (us a pass, 9 rows: 1b shape, 512 keys 866 -> 798, 7b
+        // shape, 2048 keys 2836 -> 2798; 8b shape, 17 rows and 8192 keys 3892 -> 3713.)
+        int units = (kb + rows + 15) / 16;
+        int per = max((a.Hkv * (int)__reduce_add_sync(0xffffffffu, (unsigned)units) + n_cta - 1) / n_cta, 4);
+#pragma unroll 1
+        for (int longer = per; longer <= per + per / 4; ++longer) {
+            if (a.Hkv * (int)__reduce_add_sync(0xffffffffu, (unsigned)((units + longer - 1) / longer)) > n_cta) continue;
+            per = longer;
+            units = (units + per - 1) / per * per;
+            break;
+        }
         const int N = (G * rows + 7) & ~7;
         int u0 = a.Hkv * units, q0 = a.Hkv * N * HD * 2, rs = a.Hkv * G * rows;      // inclusive sums over the items
 #pragma unroll
@@ -749,8 +761,6 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
             sm.q_r[lane] = lane - sm.it[item].row0;
         }
         if (lane == 0) {
-            // at least 64 keys per CTA: shorter parts would only add partial results to exchange
-            const int per = max((U + n_cta - 1) / n_cta, 4);
             int u = min(cta * per, U), n = 0, tiles = 0, i = 0;
             const int e = min(u + per, U);
             while (u < e && n < kStackMaxSegs) {

@@ -27,6 +27,7 @@ CASES = {
     "narrow": (T.scaled(d_model=48, n_q_heads=1, n_kv_heads=1, d_ffn=32, vocab=48), [90], [2], 16),
     "wide, whole row blocks": (T.scaled(d_model=1024, d_ffn=4096, vocab=32000), [64], [5], 16),
     "16 requests of two rows": (T, [3, 17, 400, 129, 5, 6, 7, 900, 1, 64, 65, 66, 31, 32, 33, 250], [1] * 16, 16),
+    "more heads than SMs": (T.scaled(d_model=1024, n_q_heads=16, n_kv_heads=16), [130, 170, 400, 110, 190, 260, 164, 500, 133, 148, 300, 129], [1, 2] * 6, 16),
     "three requests": (T.scaled(n_kv_heads=2), [40, 1200, 300], [16, 2, 9], 16),
 }
 
