@@ -183,6 +183,13 @@ __device__ __forceinline__ bool stack_try(uint32_t bar, uint32_t parity) {
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+// A look that never suspends, the same for all lanes.
+__device__ __forceinline__ bool stack_look(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    return __all_sync(0xffffffffu, ok != 0u);
+}
 __device__ __forceinline__ bool stack_wait(uint32_t bar, uint32_t parity) {
     bool done = false;
 #pragma unroll 1
@@ -544,10 +551,12 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                     const uint32_t first = smem_u32(&sm.full_a[ra.slot]);
                     if (!stack_wait(smem_u32(&sm.d_empty[rd.slot]), rd.par)) return false;
                     bool open = false;
+                    // (looks, not tries: a try on either barrier would sleep through the other's news)
 #pragma unroll 1
-                    for (uint32_t it = 0; it < kStackTries && !open; ++it) {
-                        open = stack_try(first, ra.par);
-                        if (!open && (int)staged < room && stack_try(smem_u32(&sm.full_w[rw.slot]), rw.par)) {
+                    for (uint32_t it = 0; it < (1u << 24) && !open; ++it) {
+                        open = stack_look(first, ra.par);
+                        if ((it & 1023u) == 1023u && __any_sync(0xffffffffu, *abort_s)) return false;
+                        if (!open && (int)staged < room && stack_look(smem_u32(&sm.full_w[rw.slot]), rw.par)) {
                             tc_fence_after();
                             const uint32_t to = staged_at(put);
                             const uint64_t wd = umma_desc(ring_a + rw.slot * kStackSlot, 128, 256);
@@ -689,6 +698,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 rw.skip(kPerTile * n_tiles, a.slots);
             };
             int n_done = 0;
+            bool in_use = false;                                    // the attention's columns
 #pragma unroll 1
             for (int p = 0; p < n_phase && ok; ++p, ++n_done) {
                 const int kind = p < 5 * a.n_layers ? p % 5 : (int)kStLm;
@@ -697,7 +707,10 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 if (!ok) continue;
                 if (kind == kStAttn) {
                     attn();
-                    if (sm.n_tiles > 0) put = get = 0;                   // (none is staged across an attention with tiles)
+                    if (sm.n_tiles > 0) {
+                        put = get = 0;                                   // (none is staged across an attention with tiles)
+                        in_use = true;
+                    }
                     continue;
                 }
                 // weights to come before the next K/V tile; tensor memory beside the attention's columns while those are in use
@@ -709,8 +722,11 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                     q = q == kStLm ? kStAttn : q == kStDn ? (i + 1 < 5 * a.n_layers ? kStQkv : kStLm) : q + 1;
                     if (q == kStAttn || (kind == kStQkv)) break;
                 }
-                const int beside = kind == kStO && sm.n_tiles > 0 ? (512 - 8 * a.n_max) / 64 : kStackStaged;
+                // (until a phase of which this CTA has a part has opened: where it has none of the output projection, this role is
+                // in the next phase while the workers are still in the attention)
+                const int beside = in_use ? min((512 - 8 * a.n_max) / 64, kStackStaged) : kStackStaged;
                 ok = gemm(a.g[kind], min(room, max(beside, 0)));
+                if (sm.geo[kind].stages > 0) in_use = false;
             }
             if (!ok && go) give_up(13);
             umma_commit_if(go, smem_u32(&sm.last));         // nothing of this CTA runs on the tensor cores when it leaves
