@@ -545,7 +545,7 @@ int stack_segments(const pipesd_model_cfg& c, const std::vector<ItemDesc>& items
 // Whether a pass is the layer-stack kernel's: up to 32 rows, of requests whose query rows per KV head fit its tensor memory, in a
 // batch whose key ranges fit its tables.  The others (prompts of 19 to 32 tokens at four query heads per KV head, say), and every
 // pass while GEMM launches are timed, run on a kernel per projection, as all did before: us a pass on one box, 7b shape, 9 rows
-// 3224 -> 2798, 17 rows 3906 -> 3142; 8b shape, 17 rows 5033 -> 3713; 1b shape, 9 rows 1003 -> 798; tiny 116 -> 112.
+// 3224 -> 2718, 17 rows 3906 -> 3096; 8b shape, 17 rows 5033 -> 3637; 1b shape, 9 rows 1003 -> 801; tiny 116 -> 111.
 bool stack_takes(const pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int M, StackPlan* plan, int* n_max, int* r_max) {
     const pipesd_model_cfg& c = ctx->cfg;
     if (ctx->stack_ctas < 1 || M > kMaxItemRows || ctx->force_dense || ctx->time_gemms || (int)items.size() > kStackMaxItems) return false;
