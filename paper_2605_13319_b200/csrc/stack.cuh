@@ -1156,8 +1156,11 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 }
 #pragma unroll 1
                 for (int k = 0; n > 0; ++k) {
-                    if (!ready) fetch(true, row, t, xa[0], xb[0]);
-                    finish(row, t, val[0], xa[0], xb[0]);
+                    // (rows that nothing was fetched for: a row block that is this CTA's alone comes before the groups, whose inputs stay
+                    // in xa, xb meanwhile)
+                    float fa = xa[0], fb = xb[0];
+                    if (!ready) fetch(true, row, t, fa, fb);
+                    finish(row, t, val[0], fa, fb);
                     ++t;
                     int by = 1;
                     if (--n == 0 && gap == 3) {             // on to the second group
@@ -1172,7 +1175,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
 #pragma unroll
                         for (int m = 0; m + 1 < kVals; ++m) val[m] = val[m + 1];
 #pragma unroll
-                        for (int m = 0; m < 5; ++m) { xa[m] = xa[m + 1]; xb[m] = xb[m + 1]; }
+                        for (int m = 0; m < 5; ++m) { xa[m] = ready ? xa[m + 1] : xa[m]; xb[m] = ready ? xb[m + 1] : xb[m]; }
                     }
                 }
             }

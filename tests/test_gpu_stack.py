@@ -29,6 +29,12 @@ CASES = {
     "16 requests of two rows": (T, [3, 17, 400, 129, 5, 6, 7, 900, 1, 64, 65, 66, 31, 32, 33, 250], [1] * 16, 16),
     "more heads than SMs": (T.scaled(d_model=1024, n_q_heads=16, n_kv_heads=16), [130, 170, 400, 110, 190, 260, 164, 500, 133, 148, 300, 129], [1, 2] * 6, 16),
     "three requests": (T.scaled(n_kv_heads=2), [40, 1200, 300], [16, 2, 9], 16),
+    # CTAs that hold a whole row block and finish rows of one they share, where the epilogue reads memory: a CTA takes eight
+    # k16 steps at least, more than one row block's 6 (or 5) of these
+    "whole and shared row blocks of QKV": (T.scaled(d_model=96), [40], [8], 16),
+    "whole and shared row blocks of QKV, 32 rows": (T.scaled(d_model=80, n_q_heads=8, n_kv_heads=4), [300], [31], 16),
+    "whole and shared row blocks of down": (T.scaled(d_ffn=96), [40], [1], 16),
+    "whole and shared row blocks of down, 32 rows": (T.scaled(d_model=1024, d_ffn=80), [300], [31], 16),
 }
 
 
