@@ -266,6 +266,9 @@ int32_t pipesd_debug_gemm_dense(const void *packed, const float *x, float *y, vo
  * done before it leaves its share of their merge to the last one.  Results do not depend on it, bit for bit: at 0 the last
  * one merges all rows, as it does where other work keeps the splits from running at the same time. */
 int32_t pipesd_debug_merge_polls(pipesd_ctx *ctx, int32_t polls);
+/* Harness switch: CTAs of the layer-stack kernel, 1 up to one per SM (0: one per SM, as always otherwise).  Its plans follow their
+ * number, as they do on a device of fewer SMs.  PIPESD_E_INVALID beyond that. */
+int32_t pipesd_debug_stack_ctas(pipesd_ctx *ctx, int32_t ctas);
 /* Host only: how pipesd_prefill cuts a prompt of n tokens (1..max_seq): *rows of the chunk behind its first `done`, and the
  * last *logits rows of the last chunk whose logits it keeps. */
 int32_t pipesd_debug_prefill_chunk(const pipesd_model_cfg *cfg, int32_t n, int32_t done, int32_t *rows, int32_t *logits);

@@ -331,7 +331,8 @@ struct pipesd_ctx {
     int merge_polls = kAttnMergePolls;
     bool force_dense = false;   // harness switch: the dense kernels also for passes of at most 32 rows ...
     int plan_rows = 0;          // ... with the plans of a pass of this many rows
-    int stack_ctas = 0;         // CTAs of the layer-stack kernel, one per SM (0: the device cannot launch it)
+    int stack_most = 0;         // CTAs of the layer-stack kernel: one per SM (0: the device cannot launch it) ...
+    int stack_ctas = 0;         // ... or as many as a harness asked for
     uint64_t stack_phases = 0;  // phases run since the exchange words were last cleared
     bool pass_dense = false;    // the pass being enqueued runs on the dense kernels
     // bytes of the O and gate/up weights the attention kernel pulls into L2 once its K/V has landed (measured: all of O
@@ -955,7 +956,7 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
             return bail(PIPESD_E_CUDA);
         int coop = 0;
         if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c.device) != cudaSuccess) return bail(PIPESD_E_CUDA);
-        ctx->stack_ctas = coop ? std::min(n_sm, kStackMaxCtas) : 0;
+        ctx->stack_ctas = ctx->stack_most = coop ? std::min(n_sm, kStackMaxCtas) : 0;
         for (int S = 1; S <= kDenseMaxSlices; ++S) {
             cudaLaunchConfig_t lc = {};
             cudaLaunchAttribute at[1];
@@ -1558,6 +1559,12 @@ int32_t pipesd_debug_force_dense(pipesd_ctx* ctx, int32_t on) {
 int32_t pipesd_debug_merge_polls(pipesd_ctx* ctx, int32_t polls) {
     if (!ctx || polls < 0 || polls > 65536) return fail(ctx, PIPESD_E_INVALID, "pipesd_debug_merge_polls");
     ctx->merge_polls = polls;
+    return PIPESD_OK;
+}
+
+int32_t pipesd_debug_stack_ctas(pipesd_ctx* ctx, int32_t ctas) {
+    if (!ctx || ctas < 0 || ctas > ctx->stack_most) return fail(ctx, PIPESD_E_INVALID, "pipesd_debug_stack_ctas");
+    ctx->stack_ctas = ctas ? ctas : ctx->stack_most;
     return PIPESD_OK;
 }
 

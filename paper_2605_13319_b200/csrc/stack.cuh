@@ -893,9 +893,10 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sm.tables));
-        // ---- embedding rows, rotary table, zeros behind the live rows of Q
-        if (cta < a.M) {
-            const int row = cta;
+        // ---- embedding rows (a CTA's first is its only one where there are as many CTAs), rotary table, zeros behind the live rows
+        // of Q
+#pragma unroll 1
+        for (int row = cta; row < a.M; row += n_cta) {
             const uint16_t* er = a.emb + (size_t)a.meta.row_tok[row] * a.d;
             float ss = 0.f;
 #pragma unroll 1
@@ -914,6 +915,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 *reinterpret_cast<uint2*>(xd + act_index_lo(T)) = lo;
             }
             ss = warp_sum(ss);
+            if (row != cta) sync_workers();      // the row before has been summed
             if (lane == 0) sm.red[warp - 4] = ss;
             sync_workers();
 #pragma unroll 1

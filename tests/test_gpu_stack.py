@@ -88,3 +88,45 @@ def test_against_the_kernels_per_projection(name, growing):
         for a, b in zip(got_kv, want_kv):
             assert np.all(np.abs(a - b) <= 2.0 ** -7 * np.abs(b) + (2e-2 if growing else 2e-3) * np.abs(b).max())
     ctx.close()
+
+
+def _context(shape, lens, ks, page=16, seed=11):
+    """A context with these prefixes cached, the items of a pass over them, and the number of its rows."""
+    from paper_2605_13319_b200 import binding
+    rows = sum(ks) + len(ks)
+    ctx = binding.Context(shape, synth.make_weights(shape, seed), n_pages=sum((P + 40) // page + 1 for P in lens), max_requests=len(lens),
+                          max_rows=rows, max_seq=max(lens) + 40, max_draft=max(ks), page_size=page, poison=True)
+    items = []
+    for i, (P, k) in enumerate(zip(lens, ks)):
+        req = ctx.req_open()
+        for l in range(shape.n_layers):
+            ctx.debug_write_kv(req, l, 0, *synth.make_synthetic_kv(shape, P, seed + i, l))
+        items.append(dict(req=req, tokens=synth.tokens_i32(k + 1, seed, 900 + i, shape.vocab), u=synth.make_accept_uniforms(k, seed, i),
+                          q=np.full((k, shape.vocab), 1.0 / shape.vocab, np.float32)))
+    return ctx, items, rows
+
+
+def _close(got, want, got_kv, want_kv, tol=TOL):
+    assert np.isfinite(got).all()
+    assert logit_rel_err(got, want).max() < tol
+    for a, b in zip(got_kv, want_kv):
+        assert np.all(np.abs(a - b) <= 2.0 ** -7 * np.abs(b) + tol * np.abs(b).max())
+
+
+@pytest.mark.parametrize("name, some", [("32 rows", (2, 3, 13, 40)), ("ragged widths", (1, 2, 3, 7)), ("three requests", (10, 26, 27, 40)),
+                                        ("wide, whole row blocks", (2, 3, 13, 40))])
+def test_fewer_ctas(name, some):
+    """As on a device of fewer SMs: fewer CTAs than rows, several whole row blocks to a CTA, and whole and shared ones."""
+    shape, lens, ks, page = CASES[name]
+    ctx, items, rows = _context(shape, lens, ks, page)
+    layers = range(shape.n_layers)
+    ctx.profile_enable(True)
+    _, want, want_kv = _run(ctx, items, lens, rows, layers)
+    ctx.profile_enable(False)
+    for ctas in (*some, 0):
+        ctx.debug_stack_ctas(ctas)
+        ctx.profile_read()
+        _, got, got_kv = _run(ctx, items, lens, rows, layers)
+        assert ctx.profile_read()["kernel_launches"] == 3, ctas
+        _close(got, want, got_kv, want_kv)
+    ctx.close()
