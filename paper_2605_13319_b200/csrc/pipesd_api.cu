@@ -331,7 +331,7 @@ struct pipesd_ctx {
     int merge_polls = kAttnMergePolls;
     bool force_dense = false;   // harness switch: the dense kernels also for passes of at most 32 rows ...
     int plan_rows = 0;          // ... with the plans of a pass of this many rows
-    int stack_most = 0;         // CTAs of the layer-stack kernel: one per SM (0: the device cannot launch it) ...
+    int stack_most = 0;         // CTAs of the layer-stack kernel: one per SM (0: the device or the stream cannot launch it) ...
     int stack_ctas = 0;         // ... or as many as a harness asked for
     uint64_t stack_phases = 0;  // phases run since the exchange words were last cleared
     bool pass_dense = false;    // the pass being enqueued runs on the dense kernels
@@ -557,8 +557,10 @@ bool stack_takes(const pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int 
     return *n_max <= kStackMaxN && stack_segments(c, items, ctx->stack_ctas) <= kStackMaxSegs && stack_plan(plan, M, c.head_dim, *n_max);
 }
 
-// Launch the layer-stack kernel over the M rows whose metadata has been uploaded.
-int launch_stack(pipesd_ctx* ctx, const StackPlan& plan, int n_items, int M, int n_max, int r_max, const PassMeta& meta, bool want_logits) {
+// Launch the layer-stack kernel over the M rows whose metadata has been uploaded.  *refused: the stream has fewer SMs than the kernel
+// has CTAs (one of a green context: its part of the device is no attribute of the device), nothing was launched, and the context's
+// passes run on a kernel per projection from here on.
+int launch_stack(pipesd_ctx* ctx, const StackPlan& plan, int n_items, int M, int n_max, int r_max, const PassMeta& meta, bool want_logits, bool* refused) {
     const pipesd_model_cfg& c = ctx->cfg;
     const LayerW& l0 = ctx->layers[0];
     const int G = ctx->stack_ctas, hd = c.head_dim;
@@ -632,7 +634,14 @@ int launch_stack(pipesd_ctx* ctx, const StackPlan& plan, int n_items, int M, int
     cfg.stream = ctx->st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    CU(cudaLaunchKernelEx(&cfg, stack_fn(plan.T / 8, hd), a));
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, stack_fn(plan.T / 8, hd), a);
+    *refused = e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported;
+    if (*refused) {
+        cudaGetLastError();
+        ctx->stack_ctas = ctx->stack_most = 0;
+        return PIPESD_OK;
+    }
+    CU(e);
     ctx->n_launch += 1;
     return PIPESD_OK;
 }
@@ -757,10 +766,12 @@ int run_pass(pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int n_logits, 
 
     StackPlan splan;
     int st_n = 0, st_r = 0;
-    const bool stacked = stack_takes(ctx, items, M, &splan, &st_n, &st_r);
+    bool stacked = stack_takes(ctx, items, M, &splan, &st_n, &st_r);
     if (stacked) {
-        int rc_ = launch_stack(ctx, splan, n_items, M, st_n, st_r, meta, want_logits);
+        bool refused = false;
+        int rc_ = launch_stack(ctx, splan, n_items, M, st_n, st_r, meta, want_logits, &refused);
         if (rc_) return rc_;
+        stacked = !refused;
     }
     // Passes of more than 32 rows run their GEMMs on the dense kernels (every weight byte read once per block of up to 256
     // tokens); their activation arrays are in that kernel's operand order, with the token block size of the consumer.
@@ -954,9 +965,11 @@ int32_t pipesd_ctx_create(const pipesd_model_cfg* cfg, const pipesd_weights* w, 
             cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, c.device) != cudaSuccess ||
             cudaDeviceGetAttribute(&thr_sm, cudaDevAttrMaxThreadsPerMultiProcessor, c.device) != cudaSuccess)
             return bail(PIPESD_E_CUDA);
-        int coop = 0;
-        if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c.device) != cudaSuccess) return bail(PIPESD_E_CUDA);
-        ctx->stack_ctas = ctx->stack_most = coop ? std::min(n_sm, kStackMaxCtas) : 0;
+        int coop = 0, stack_sm = 0;
+        if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c.device) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&stack_sm, (const void*)stack_fn(4, c.head_dim), kStackThreads, kStackSmemMax) != cudaSuccess)
+            return bail(PIPESD_E_CUDA);
+        ctx->stack_ctas = ctx->stack_most = coop && stack_sm > 0 ? std::min(n_sm, kStackMaxCtas) : 0;
         for (int S = 1; S <= kDenseMaxSlices; ++S) {
             cudaLaunchConfig_t lc = {};
             cudaLaunchAttribute at[1];

@@ -90,12 +90,12 @@ def test_against_the_kernels_per_projection(name, growing):
     ctx.close()
 
 
-def _context(shape, lens, ks, page=16, seed=11):
+def _context(shape, lens, ks, page=16, seed=11, stream=None):
     """A context with these prefixes cached, the items of a pass over them, and the number of its rows."""
     from paper_2605_13319_b200 import binding
     rows = sum(ks) + len(ks)
     ctx = binding.Context(shape, synth.make_weights(shape, seed), n_pages=sum((P + 40) // page + 1 for P in lens), max_requests=len(lens),
-                          max_rows=rows, max_seq=max(lens) + 40, max_draft=max(ks), page_size=page, poison=True)
+                          max_rows=rows, max_seq=max(lens) + 40, max_draft=max(ks), page_size=page, poison=True, stream=stream)
     items = []
     for i, (P, k) in enumerate(zip(lens, ks)):
         req = ctx.req_open()
@@ -130,3 +130,39 @@ def test_fewer_ctas(name, some):
         assert ctx.profile_read()["kernel_launches"] == 3, ctas
         _close(got, want, got_kv, want_kv)
     ctx.close()
+
+
+def _part_of_the_device(sms):
+    """A stream that has `sms` SMs of device 0 to itself (a green context's); skips where that cannot be had."""
+    import torch
+    driver = pytest.importorskip("cuda.bindings.driver")
+
+    def ok(r):
+        if r[0] != driver.CUresult.CUDA_SUCCESS:
+            pytest.skip(f"no green context: {r[0]}")
+        return r[1]
+    torch.zeros(1, device="cuda")
+    dev = ok(driver.cuDeviceGet(0))
+    whole = ok(driver.cuDeviceGetDevResource(dev, driver.CUdevResourceType.CU_DEV_RESOURCE_TYPE_SM))
+    part = ok(driver.cuDevSmResourceSplitByCount(1, whole, 0, sms))[0]
+    green = ok(driver.cuGreenCtxCreate(ok(driver.cuDevResourceGenerateDesc([part], 1)), dev,
+                                       driver.CUgreenCtxCreate_flags.CU_GREEN_CTX_DEFAULT_STREAM))
+    stream = ok(driver.cuGreenCtxStreamCreate(green, driver.CUstream_flags.CU_STREAM_NON_BLOCKING, 0))
+    return torch.cuda.ExternalStream(int(stream))
+
+
+def test_stream_of_fewer_sms():
+    """The kernel wants as many SMs as the device has; on a stream that has fewer its launch is refused, and the pass, and every
+    later one, runs on the kernels per projection."""
+    shape, lens, ks = T, [100], [8]
+    results = []
+    for stream in (None, _part_of_the_device(64)):
+        ctx, items, rows = _context(shape, lens, ks, stream=stream)
+        ctx.profile_read()
+        results += [(_run(ctx, items, lens, rows, range(shape.n_layers)), ctx.profile_read()["kernel_launches"]) for _ in range(2)]
+        ctx.close()
+    (want, n), _, (first, n1), (second, n2) = results
+    assert n == 3 < n1 == n2
+    for got in (first, second):
+        _close(got[1], want[1], got[2], want[2])
+    assert first[0] == second[0] and np.array_equal(first[1], second[1])
