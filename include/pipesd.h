@@ -156,6 +156,14 @@ int32_t pipesd_ctx_destroy(pipesd_ctx *ctx);
  * flight are then void (status PIPESD_E_CUDA each), nothing of them is committed, and the context stays usable. */
 int32_t pipesd_ctx_sync(pipesd_ctx *ctx);
 
+/* Whether other work shares the device with the context's passes (share = 0, as after pipesd_ctx_create: none does).  Unless told so,
+ * a pass of up to 32 rows is one kernel that takes every SM at once: it begins when kernels of other streams have left all of them,
+ * and they begin when it has ended.  With share != 0 such a pass is a kernel per projection from the next call on, none of
+ * which waits for a CTA that is not running: slower by itself (1.1 to 1.4 times), but it runs beside a kernel that holds some
+ * SMs for long -- one that waits for the pass itself included -- and the passes of several contexts on one device overlap.  The two
+ * agree to rounding, not bit for bit.  (Set-up around the method: the paper says nothing about what else the GPU runs.) */
+int32_t pipesd_share_device(pipesd_ctx *ctx, int32_t share);
+
 /* Request slots, one per edge device served by this cloud model (App. I: every edge is independent, one target model
  * handles the requests of all): an empty block table / return of all its pages to the pool. */
 int32_t pipesd_req_open(pipesd_ctx *ctx, int32_t *req);

@@ -97,6 +97,7 @@ _SIGNATURES = {
     "pipesd_sched_trigger_step": (i32, [ctypes.POINTER(ctypes.c_double), ctypes.c_double, ctypes.c_double,
                                         ctypes.c_double, ctypes.POINTER(i32)]),
     "pipesd_debug_force_dense": (i32, [vp, i32]),
+    "pipesd_share_device": (i32, [vp, i32]),
     "pipesd_debug_merge_polls": (i32, [vp, i32]),
     "pipesd_debug_stack_ctas": (i32, [vp, i32]),
     "pipesd_debug_prefill_chunk": (i32, [ctypes.POINTER(ModelCfg), i32, i32, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]),
@@ -220,6 +221,10 @@ class Context:
     def ctx_sync(self):
         self._check(lib().pipesd_ctx_sync(self._h), "pipesd_ctx_sync")
         self._alive = []
+
+    def share_device(self, share: bool = True):
+        """Other work shares the device: no pass takes all of its SMs at once."""
+        self._check(lib().pipesd_share_device(self._h, int(share)), "pipesd_share_device")
 
     def req_open(self) -> int:
         r = i32()

@@ -333,6 +333,7 @@ struct pipesd_ctx {
     int plan_rows = 0;          // ... with the plans of a pass of this many rows
     int stack_most = 0;         // CTAs of the layer-stack kernel: one per SM (0: the device or the stream cannot launch it) ...
     int stack_ctas = 0;         // ... or as many as a harness asked for
+    bool shared = false;        // other work shares the device: no kernel that takes all of it
     uint64_t stack_phases = 0;  // phases run since the exchange words were last cleared
     bool pass_dense = false;    // the pass being enqueued runs on the dense kernels
     // bytes of the O and gate/up weights the attention kernel pulls into L2 once its K/V has landed (measured: all of O
@@ -549,7 +550,7 @@ int stack_segments(const pipesd_model_cfg& c, const std::vector<ItemDesc>& items
 // 3224 -> 2718, 17 rows 3906 -> 3096; 8b shape, 17 rows 5033 -> 3637; 1b shape, 9 rows 1003 -> 801; tiny 116 -> 111.
 bool stack_takes(const pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int M, StackPlan* plan, int* n_max, int* r_max) {
     const pipesd_model_cfg& c = ctx->cfg;
-    if (ctx->stack_ctas < 1 || M > kMaxItemRows || ctx->force_dense || ctx->time_gemms || (int)items.size() > kStackMaxItems) return false;
+    if (ctx->stack_ctas < 1 || ctx->shared || M > kMaxItemRows || ctx->force_dense || ctx->time_gemms || (int)items.size() > kStackMaxItems) return false;
     int rows = 1;
     for (const ItemDesc& it : items) rows = std::max(rows, it.rows);
     *r_max = rows * (c.n_q_heads / c.n_kv_heads);
@@ -1126,6 +1127,16 @@ int32_t pipesd_ctx_sync(pipesd_ctx* ctx) {
         }
     }
     ctx->inflight.clear();
+    return PIPESD_OK;
+}
+
+// What a pass that takes all SMs costs where it is not alone, and what one that does not costs where it is: ms a pass beside a one-warp
+// kernel of 50 ms, 1b shape, 9 rows 46 against 1.2, tiny 45 against 0.14; passes a second of two contexts (a stream and a thread
+// each) 1307 against 1524, tiny 11283 against 15065, 1b with 17 rows 1101 against 1115; of one 1250 against 1007, 8881 against 8558,
+// 1064 against 713.
+int32_t pipesd_share_device(pipesd_ctx* ctx, int32_t share) {
+    if (!ctx) return PIPESD_E_INVALID;
+    ctx->shared = share != 0;
     return PIPESD_OK;
 }
 

@@ -166,3 +166,31 @@ def test_stream_of_fewer_sms():
     for got in (first, second):
         _close(got[1], want[1], got[2], want[2])
     assert first[0] == second[0] and np.array_equal(first[1], second[1])
+
+
+def test_shared_device():
+    """A pass of a context that shares its device is done while another stream's kernel still holds an SM; and agrees with the
+    one that takes them all."""
+    import torch
+    from paper_2605_13319_b200 import binding
+    shape, lens, ks = T, [100], [8]
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    (ctx, items, rows), (other, _, _) = (_context(shape, lens, ks, stream=s) for s in streams)
+    layers = range(shape.n_layers)
+    _, want, want_kv = _run(ctx, items, lens, rows, layers)
+    ctx.share_device()
+    _run(ctx, items, lens, rows, layers)
+    held = torch.cuda.Event()
+    other.debug_wait_timeout(100000)                           # one warp for 100 ms
+    held.record(streams[1])
+    got, logits, kv = _run(ctx, items, lens, rows, layers)
+    assert not held.query()                                    # it is still there
+    _close(logits, want, kv, want_kv)
+    with pytest.raises(binding.PipesdError):
+        other.ctx_sync()
+    ctx.share_device(False)
+    ctx.profile_read()
+    _, again, _ = _run(ctx, items, lens, rows, layers)
+    assert ctx.profile_read()["kernel_launches"] == 3 and np.array_equal(again, want)
+    ctx.close()
+    other.close()
