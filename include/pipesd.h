@@ -277,6 +277,10 @@ int32_t pipesd_debug_merge_polls(pipesd_ctx *ctx, int32_t polls);
 /* Harness switch: CTAs of the layer-stack kernel, 1 up to one per SM (0: one per SM, as always otherwise).  Its plans follow their
  * number, as they do on a device of fewer SMs.  PIPESD_E_INVALID beyond that. */
 int32_t pipesd_debug_stack_ctas(pipesd_ctx *ctx, int32_t ctas);
+/* Harness switch: looks, a trip to the L2 each, after which a CTA of the layer-stack kernel no longer waits for what the others write:
+ * 1 to 2^22 (0: 2^22, seconds, as always otherwise).  Whoever gives up sets the device error word, the kernel's other waits run
+ * out within a second or two, and the pass ends like any other whose device-side wait timed out (pipesd_ctx_sync). */
+int32_t pipesd_debug_stack_looks(pipesd_ctx *ctx, int32_t looks);
 /* Host only: how pipesd_prefill cuts a prompt of n tokens (1..max_seq): *rows of the chunk behind its first `done`, and the
  * last *logits rows of the last chunk whose logits it keeps. */
 int32_t pipesd_debug_prefill_chunk(const pipesd_model_cfg *cfg, int32_t n, int32_t done, int32_t *rows, int32_t *logits);

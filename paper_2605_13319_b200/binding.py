@@ -100,6 +100,7 @@ _SIGNATURES = {
     "pipesd_share_device": (i32, [vp, i32]),
     "pipesd_debug_merge_polls": (i32, [vp, i32]),
     "pipesd_debug_stack_ctas": (i32, [vp, i32]),
+    "pipesd_debug_stack_looks": (i32, [vp, i32]),
     "pipesd_debug_prefill_chunk": (i32, [ctypes.POINTER(ModelCfg), i32, i32, ctypes.POINTER(ctypes.c_int32), ctypes.POINTER(ctypes.c_int32)]),
     "pipesd_debug_gemm_dense_scratch_bytes": (u64, [i32, i32, i32]),
     "pipesd_debug_gemm_dense": (i32, [vp, vp, vp, vp, i32, i32, i32, i32, i32, vp]),
@@ -300,6 +301,10 @@ class Context:
     def debug_stack_ctas(self, ctas: int):
         """CTAs of the layer-stack kernel; 0: one per SM."""
         self._check(lib().pipesd_debug_stack_ctas(self._h, ctas), "pipesd_debug_stack_ctas")
+
+    def debug_stack_looks(self, looks: int):
+        """Looks after which a CTA of the layer-stack kernel no longer waits for the others; 0: its own limit."""
+        self._check(lib().pipesd_debug_stack_looks(self._h, looks), "pipesd_debug_stack_looks")
 
     def debug_attn_slots(self, rows_per_kv_head: int):
         out = (ctypes.c_int32 * 2)()

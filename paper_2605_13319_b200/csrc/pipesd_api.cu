@@ -333,6 +333,7 @@ struct pipesd_ctx {
     int plan_rows = 0;          // ... with the plans of a pass of this many rows
     int stack_most = 0;         // CTAs of the layer-stack kernel: one per SM (0: the device or the stream cannot launch it) ...
     int stack_ctas = 0;         // ... or as many as a harness asked for
+    unsigned stack_looks = kStackLooks;      // of the layer-stack kernel, at other CTAs' arrivals and words
     bool shared = false;        // other work shares the device: no kernel that takes all of it
     uint64_t stack_phases = 0;  // phases run since the exchange words were last cleared
     bool pass_dense = false;    // the pass being enqueued runs on the dense kernels
@@ -612,6 +613,7 @@ int launch_stack(pipesd_ctx* ctx, const StackPlan& plan, int n_items, int M, int
     a.M = M;
     a.n_items = n_items;
     a.want_logits = want_logits;
+    a.looks = ctx->stack_looks;
     a.n_pages = c.n_pages;
     a.page_size = c.page_size;
     a.slots = plan.slots;
@@ -1589,6 +1591,12 @@ int32_t pipesd_debug_merge_polls(pipesd_ctx* ctx, int32_t polls) {
 int32_t pipesd_debug_stack_ctas(pipesd_ctx* ctx, int32_t ctas) {
     if (!ctx || ctas < 0 || ctas > ctx->stack_most) return fail(ctx, PIPESD_E_INVALID, "pipesd_debug_stack_ctas");
     ctx->stack_ctas = ctas ? ctas : ctx->stack_most;
+    return PIPESD_OK;
+}
+
+int32_t pipesd_debug_stack_looks(pipesd_ctx* ctx, int32_t looks) {
+    if (!ctx || looks < 0 || looks > (int32_t)kStackLooks) return fail(ctx, PIPESD_E_INVALID, "pipesd_debug_stack_looks");
+    ctx->stack_looks = looks ? (unsigned)looks : kStackLooks;
     return PIPESD_OK;
 }
 

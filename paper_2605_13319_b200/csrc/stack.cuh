@@ -83,6 +83,7 @@ struct StackArgs {
     unsigned* sync;
     int* err;
     int n_layers, d, Hq, Hkv, M, n_items, want_logits, n_pages, page_size, n_ssq;
+    unsigned looks;              // kStackLooks, unless a harness asks for less
     int slots, acts;             // ring slots, activation slots
     int n_max, r_max, q_bufs, p_bufs;   // attention: N and rows per KV head of the largest request; buffers of Q and P
     float eps;
@@ -110,7 +111,7 @@ struct StackSmall {
     unsigned long long full_w[kStackMaxSlots], empty_w[kStackMaxSlots], full_a[kStackMaxActs], empty_a[kStackMaxActs], d_full[2], d_empty[2],
         q_full[2], q_empty[2], s_full[2], p_full, pv_done[2], phase, tables, last;
     uint32_t tmem;
-    int abort;
+    int go, abort;               // the launch has work to do; a role has given up
     unsigned base, epoch, issued_w, issued_a, issued_q;
     int n_seg, n_tiles;
     float rstd[32], red[8];
@@ -174,9 +175,9 @@ static inline size_t stack_ll_rows(int rows, int Hq, int Hkv) {
     return (size_t)kStackMaxCtas * r + (size_t)Hq * rows;
 }
 
-// ---- waits.  Bounded by counts (a try suspends for a hardware-chosen time; 2^20 of them take a second or so); a role gives up at
-// its first wait that runs out, so that all of them are through within a few of these.
-constexpr uint32_t kStackTries = 1u << 20;
+// ---- waits.  Bounded by counts (a try suspends for a hardware-chosen time, some 4 us: 2^18 of them take a second); a role gives up at its
+// first wait that runs out, so that all of them are through within a few of these.
+constexpr uint32_t kStackTries = 1u << 18;
 __device__ __forceinline__ bool stack_try(uint32_t bar, uint32_t parity) {
     uint32_t ok;
     asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
@@ -190,12 +191,17 @@ __device__ __forceinline__ bool stack_look(uint32_t bar, uint32_t parity) {
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return __all_sync(0xffffffffu, ok != 0u);
 }
+// (a converged warp, whose lanes have to leave with one answer: those that disagreed about a wait that runs out would go separate ways.
+// A lane whose tries ran out therefore looks once more, behind the others' last tries: if one of those succeeded, the phase is over and
+// this one does too; if none did, they are all here, and one's sight is the others'.  This costs nothing, and a vote behind every
+// wait 0.5 %.  The limit is a constant: as an argument it cost 0.8 % of a pass (1b shape, 9 rows 796 -> 803 us, 7b shape 2634 -> 2646).)
 __device__ __forceinline__ bool stack_wait(uint32_t bar, uint32_t parity) {
     bool done = false;
 #pragma unroll 1
     for (uint32_t it = 0; it < kStackTries; ++it) {
         if (stack_try(bar, parity)) { done = true; break; }
     }
+    if (!done) done = __any_sync(__activemask(), stack_try(bar, parity));
     return done;
 }
 __device__ __forceinline__ int ld_relaxed(const int* p) {
@@ -206,14 +212,15 @@ __device__ __forceinline__ int ld_relaxed(const int* p) {
 // Looks that find nothing, a trip to the L2 each, before a reader of other CTAs' words gives up: seconds.
 constexpr uint32_t kStackLooks = 1u << 22;
 // (a converged warp: one lane looks, and its sight is the others' too)
-__device__ __forceinline__ bool stack_arrived(const unsigned* ctr, unsigned target, const volatile int* abort_s, const int* err, int lane) {
+__device__ __forceinline__ bool stack_arrived(const unsigned* ctr, unsigned target, const volatile int* abort_s, const int* err, int lane, uint32_t looks) {
+    uint32_t it = 0;
 #pragma unroll 1
-    for (uint32_t it = 0; it < kStackLooks; ++it) {
+    do {
         unsigned v = 0u;
         asm volatile("{\n .reg .pred q;\n setp.eq.s32 q, %2, 0;\n @q ld.acquire.gpu.global.u32 %0, [%1];\n}" : "+r"(v) : "l"(ctr), "r"(lane) : "memory");
         if ((int)(__shfl_sync(0xffffffffu, v, 0) - target) >= 0) return true;
         if ((it & 63u) == 63u && __any_sync(0xffffffffu, *abort_s || ld_relaxed(err) != 0)) return false;
-    }
+    } while (++it < looks);
     return false;
 }
 // Orders what this thread has seen of other CTAs' ordinary stores before its later copies from global memory.
@@ -338,7 +345,8 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
 
     if (tid == 0) {
         // an earlier launch gave up and the host has not seen it yet: its results are void, and so would be these
-        sm.abort = ld_relaxed(a.err);
+        sm.go = ld_relaxed(a.err) == 0;
+        sm.abort = 0;
         sm.base = a.sync[32];
         sm.epoch = a.sync[64];
         sm.issued_w = sm.issued_a = sm.issued_q = 0;
@@ -383,7 +391,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
     const bool wide_l = a.n_max <= 64;       // denominators of hi and lo terms in columns of their own
 
     // registers: 104 x 128 threads + 200 x 256, of the 168 x 384 the kernel is launched with
-    const bool run = sm.abort == 0;
+    const bool run = sm.go != 0;             // (the abort flag may be up by the time that a slow warp looks)
     if (warp < 4) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
     if (warp == 0 && run) {
@@ -432,7 +440,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 for (int j0 = sg.k0; j0 < k1 && ok; j0 += kAttnTile) {
                     const int je = min(j0 + kAttnTile, k1), j1 = (je + 7) & ~7;
                     if (je > sg.base && !fresh) {
-                        ok = stack_arrived(ctr, target, abort_s, a.err, lane);
+                        ok = stack_arrived(ctr, target, abort_s, a.err, lane, a.looks);
                         if (!ok) break;
                         fence_proxy_async_global();
                         fresh = true;
@@ -484,7 +492,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 // everything but the look itself comes before it: what follows it is on every phase's critical path
                 if (p == 0) ok = stack_wait(smem_u32(&sm.tables), 0u);
                 if (kind == kStAttn) {
-                    ok = ok && stack_arrived(ctr, target, abort_s, a.err, lane);
+                    ok = ok && stack_arrived(ctr, target, abort_s, a.err, lane, a.looks);
                     if (!ok) break;
                     fence_proxy_async_global();
 #pragma unroll 1
@@ -503,7 +511,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                     const int KS = a.g[kind].KS, e = sm.geo[kind].e;
                     int s = sm.geo[kind].s, ks = sm.geo[kind].ks;
                     bool told = false;
-                    ok = ok && stack_wait(smem_u32(&sm.empty_a[r.slot]), r.par) && stack_arrived(ctr, target, abort_s, a.err, lane);
+                    ok = ok && stack_wait(smem_u32(&sm.empty_a[r.slot]), r.par) && stack_arrived(ctr, target, abort_s, a.err, lane, a.looks);
                     if (!ok) break;
                     fence_proxy_async_global();
 #pragma unroll 1
@@ -729,7 +737,10 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 if (sm.geo[kind].stages > 0) in_use = false;
             }
             if (!ok && go) give_up(13);
-            umma_commit_if(go, smem_u32(&sm.last));         // nothing of this CTA runs on the tensor cores when it leaves
+            // nothing of this CTA runs on the tensor cores when it leaves (one commit after the other: a wait for the newer one alone
+            // would be satisfied by the phase before an older one that ran out)
+            if (n_done > 0) stack_wait(smem_u32(&sm.last), (uint32_t)(n_done - 1) & 1u);
+            umma_commit_if(go, smem_u32(&sm.last));
             stack_wait(smem_u32(&sm.last), (uint32_t)n_done & 1u);
         }
     } else if (warp == 3 && run) {
@@ -811,6 +822,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
         }
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sm.tables));
+        asm volatile("bar.arrive 2, %0;" ::"n"(32 + kStackWorkers) : "memory");
     }
     } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
@@ -829,14 +841,14 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                 if (stack_try(smem_u32(&bar), parity)) { done = true; break; }
             }
             if (!__all_sync(0xffffffffu, done)) {
-                if (tries > 1u && lane == 0) give_up(14);
+                if (ok && lane == 0) give_up(14);
                 tries = 1u;
                 ok = false;
             }
         };
         // between two looks at other CTAs' words: false once it is time to give up (the whole warp)
         auto look_on = [&](uint32_t look) {
-            if (ok && (look & 63u) == 63u && __any_sync(0xffffffffu, *abort_s || ld_relaxed(a.err) != 0 || look == kStackLooks - 1)) {
+            if (ok && (look & 63u) == 63u && __any_sync(0xffffffffu, *abort_s || ld_relaxed(a.err) != 0 || look >= a.looks)) {
                 ok = false;
                 if (lane == 0) give_up(15);
             }
@@ -940,6 +952,8 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
         for (size_t i = (size_t)cta * kStackWorkers + wt; i < a.qop_bytes / 16; i += (size_t)n_cta * kStackWorkers)
             reinterpret_cast<uint4*>(a.qop)[i] = make_uint4(0u, 0u, 0u, 0u);
         arrive_grid();
+        // (a barrier and not a wait that may run out: workers go on after one that did, and where they store follows from the tables)
+        asm volatile("bar.sync 2, %0;" ::"n"(32 + kStackWorkers) : "memory");
 
         StackRing rw = {0, 0u}, rd = {0, 0u};
         unsigned tile = 0;
@@ -950,7 +964,6 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
             const StackGemm& g = a.g[kind];
             const int KS = g.KS;
             const bool normed = kind == kStQkv || kind == kStGu || kind == kStLm;
-            if (kind == kStQkv && l == 0) wait(sm.tables, 0u);
             if (normed) {
                 const float* ssq = kind == kStGu ? a.ssq_b : a.ssq_a;
 #pragma unroll 1
@@ -1120,7 +1133,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                             vb[u] = make_uint4(0u, 0u, 0u, j0 + u < eb.C ? ~epoch : epoch);
                         }
 #pragma unroll 1
-                        for (uint32_t look = 0; look < kStackLooks; ++look) {
+                        for (uint32_t look = 0;; ++look) {
 #pragma unroll
                             for (int u = 0; u < 8; ++u) {
                                 ll_load_if(va[u].w != epoch, va[u], pa + u * 128);
@@ -1188,7 +1201,6 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
         // ---- attention: this CTA's segments, then its share of their merges
         auto attn = [&](unsigned epoch) {
             constexpr int kGroups = kStackWorkers / HD;
-            wait(sm.tables, 0u);
             const int kt = quarter * 32 + lane;                         // key within the tile; head dimension of O^T
             const int n_seg = sm.n_seg;
             auto product_done = [&](unsigned t) { wait(sm.pv_done[t & 1u], (t >> 1) & 1u); };       // second product of tile t
@@ -1395,7 +1407,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
 #pragma unroll
                             for (int u = 0; u < 8; ++u) v[u] = make_uint4(0u, 0u, 0u, k0 + u < nj ? ~epoch : epoch);
 #pragma unroll 1
-                            for (uint32_t look = 0; look < kStackLooks; ++look) {
+                            for (uint32_t look = 0;; ++look) {
                                 ll_load_if(ml[0].w != epoch, ml[0], pm);
                                 ll_load_if(ml[1].w != epoch, ml[1], pm + 1);
 #pragma unroll

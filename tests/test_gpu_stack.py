@@ -194,3 +194,68 @@ def test_shared_device():
     assert ctx.profile_read()["kernel_launches"] == 3 and np.array_equal(again, want)
     ctx.close()
     other.close()
+
+
+@pytest.mark.parametrize("name", ["one key", "ranges of several tiles", "three requests", "whole and shared row blocks of down"])
+def test_waits_that_run_out(name):
+    """So few looks at what other CTAs write that roles give up: the pass ends, the error is reported, and the next pass of the
+    context is what it was before, bit for bit.  At one look nobody gets past the first phase; at more of them each gives up
+    somewhere else, or nowhere."""
+    from paper_2605_13319_b200 import binding
+    shape, lens, ks, page = CASES[name]
+    ctx, items, rows = _context(shape, lens, ks, page)
+    reqs, layers = [it["req"] for it in items], range(shape.n_layers)
+    want, logits, kv = _run(ctx, items, lens, rows, layers)
+    for looks in (1, 4, 16, 1):
+        ctx.debug_stack_looks(looks)
+        failed = None
+        try:
+            got = ctx.verify(items, flags=binding.Q_HOST)
+        except binding.PipesdError as e:
+            failed = e
+        if failed is None:
+            assert looks > 1 and got == want and np.array_equal(ctx.debug_get_logits(rows), logits), looks
+        else:
+            assert failed.code == binding.E_CUDA and "timed out" in str(failed)
+        ctx.kv_rollback(reqs, [0] * len(reqs))
+        for req, P in zip(reqs, lens):
+            ctx.debug_set_len(req, P)
+        ctx.debug_stack_looks(0)
+        again = _run(ctx, items, lens, rows, layers)
+        assert again[0] == want and np.array_equal(again[1], logits), looks
+        assert all(np.array_equal(a, b) for a, b in zip(again[2], kv)), looks
+    with pytest.raises(binding.PipesdError):
+        ctx.debug_stack_looks(-1)
+    ctx.close()
+
+
+def test_pass_behind_a_wait_that_ran_out():
+    """A pass enqueued behind a wait that ran out, before the host has seen that, leaves at once: what it would have written stays
+    as it was."""
+    from paper_2605_13319_b200 import binding
+    shape, n = T, 20
+    ctx, items, rows = _context(shape, [100], [8])
+    want, logits, kv = _run(ctx, items, [100], rows, range(shape.n_layers))
+    ctx.close()
+    ctx = binding.Context(shape, synth.make_weights(shape, 11), n_pages=20, max_requests=2, max_rows=32, max_seq=140, max_draft=8, poison=True)
+    (req, other), tokens = (ctx.req_open(), ctx.req_open()), synth.tokens_i32(n, 11, 77, shape.vocab)
+    there = [synth.make_synthetic_kv(shape, n, 5, l) for l in range(shape.n_layers)]
+    for l in range(shape.n_layers):
+        ctx.debug_write_kv(req, l, 0, *synth.make_synthetic_kv(shape, 100, 11, l))
+        ctx.debug_write_kv(other, l, 0, *there[l])
+    ctx.debug_set_len(other, 0)
+    ctx.debug_wait_timeout(1000)
+    ctx.prefill(other, tokens)                                 # into the same page
+    with pytest.raises(binding.PipesdError):
+        ctx.ctx_sync()
+    for l in range(shape.n_layers):
+        for a, b in zip(ctx.debug_read_kv(other, l, 0, n), there[l]):
+            assert np.array_equal(np.asarray(a).ravel(), np.asarray(b).ravel())
+    items[0]["req"] = req
+    again = _run(ctx, items, [100], rows, range(shape.n_layers))
+    assert again[0] == want and np.array_equal(again[1], logits) and all(np.array_equal(a, b) for a, b in zip(again[2], kv))
+    ctx.debug_set_len(other, 0)
+    ctx.prefill(other, tokens)
+    ctx.ctx_sync()
+    assert not np.array_equal(np.asarray(ctx.debug_read_kv(other, 0, 0, n)[0]).ravel(), np.asarray(there[0][0]).ravel())
+    ctx.close()
