@@ -196,6 +196,26 @@ def test_shared_device():
     other.close()
 
 
+@pytest.mark.parametrize("long, fits", [(2174, True), (2175, False)])
+def test_long_request_beside_a_short_one(long, fits):
+    """A CTA's table holds 16 parts of key ranges.  At 32 KV heads, beside a request of two 16-key units per head, ranges of 30 units
+    have at most 16 of them, ranges of 31 may have 17: such a pass runs on the kernels per projection."""
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("ranges are other ones")
+    shape, lens, ks = T.scaled(n_q_heads=32, n_kv_heads=32), [30, long], [1, 1]
+    ctx, items, rows = _context(shape, lens, ks)
+    layers = range(shape.n_layers)
+    ctx.profile_enable(True)
+    _, want, want_kv = _run(ctx, items, lens, rows, layers)
+    ctx.profile_enable(False)
+    _, got, got_kv = _run(ctx, items, lens, rows, layers)
+    assert (ctx.profile_read()["kernel_launches"] == 3) == fits
+    assert np.array_equal(got, want) != fits
+    _close(got, want, got_kv, want_kv)
+    ctx.close()
+
+
 @pytest.mark.parametrize("name", ["one key", "ranges of several tiles", "three requests", "whole and shared row blocks of down"])
 def test_waits_that_run_out(name):
     """So few looks at what other CTAs write that roles give up: the pass ends, the error is reported, and the next pass of the
