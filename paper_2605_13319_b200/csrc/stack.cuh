@@ -1340,26 +1340,18 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                     if (wt == 0) mbar_arrive(smem_u32(&sm.p_full));
                     rv.skip(kPerTile, a.slots);
                 }
-                // ---- partial result: thread = head dimension of O^T; the denominators are the same in lanes 0-7 of L
+                // ---- the result of this range: thread = head dimension of O^T; the denominators are the same in lanes 0-7 of L.  A head
+                // whose keys are all here is finished, by division; of others, the contributors exchange partial results.  (Through the
+                // exchange, a head of one's own took its CTA a trip to the L2 per eight rows, four at 128 dimensions: prompts of 24 to
+                // 32 tokens at d_model 512 to 1024 were up to 13 % slower than with a kernel per projection.)
                 product_done(tile - 1u);
                 tc_fence_after();
                 const int ll_row = sg.ll0 + sg.idx * a.r_max;
-                const bool pairs = n_rows > kGroups * sg.C;
+                const bool alone = sg.C == 1, pairs = n_rows > kGroups * sg.C;
+                if (quarter == 0) {
 #pragma unroll 1
-                for (int cb = half; cb < NG; cb += 2) {
-                    float o[8];
-                    read_8(t_O + lane_sel + cb * 8, o);
-                    // rows in pairs where the merge takes them so
-                    uint4* p = a.ll + (size_t)(ll_row + cb * 8) * HD + kt;
-                    const int n = kt < HD ? n_rows - cb * 8 : 0;
-                    if (pairs) {
-#pragma unroll
-                        for (int i = 0; i < 8; i += 2) ll_store_if(i < n, p + i / 2 * HD, o[i], o[i + 1], 0.f, epoch);
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) ll_store_if(i < n, p + i * HD, o[i], 0.f, 0.f, epoch);
-                    }
-                    if (quarter == 0) {
+                    for (int cb = half; cb < NG; cb += 2) {
+                        float o[8];
                         if (wide_l) {
                             read_8(t_L + cb * 8, o);
                         } else {
@@ -1370,7 +1362,33 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
 #pragma unroll
                         for (int i = 1; i < 8; ++i) l = lane == i ? o[i] : l;                 // lane = row
                         const float m = lane < 8 ? m_ref[cb * 8 + lane] : 0.f;
-                        ll_store_if(lane < 8 && cb * 8 + lane < n_rows, a.ll + a.ll_ml + ll_row + cb * 8 + lane, m == INFINITY ? -INFINITY : m, l, 0.f, epoch);
+                        if (alone && lane < 8) wm[cb * 8 + lane] = l;
+                        ll_store_if(!alone && lane < 8 && cb * 8 + lane < n_rows, a.ll + a.ll_ml + ll_row + cb * 8 + lane, m == INFINITY ? -INFINITY : m, l, 0.f, epoch);
+                    }
+                }
+                if (alone) sync_workers();
+#pragma unroll 1
+                for (int cb = half; cb < NG; cb += 2) {
+                    float o[8];
+                    read_8(t_O + lane_sel + cb * 8, o);
+                    // rows in pairs where the merge takes them so
+                    uint4* p = a.ll + (size_t)(ll_row + cb * 8) * HD + kt;
+                    const int n = kt < HD ? n_rows - cb * 8 : 0;
+                    if (alone) {
+#pragma unroll 1
+                        for (int i = 0; i < min(n, 8); ++i) {
+                            const int r = cb * 8 + i;
+                            act_put(true, a.act_attn, sg.row0 + r / G, (sg.kvh * G + r % G) * HD + kt, o[0] / wm[r]);
+#pragma unroll
+                            for (int k = 0; k < 7; ++k) o[k] = o[k + 1];
+                        }
+                        __syncwarp();
+                    } else if (pairs) {
+#pragma unroll
+                        for (int i = 0; i < 8; i += 2) ll_store_if(i < n, p + i / 2 * HD, o[i], o[i + 1], 0.f, epoch);
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) ll_store_if(i < n, p + i * HD, o[i], 0.f, 0.f, epoch);
                     }
                 }
                 tc_fence_before();
@@ -1387,6 +1405,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
             for (int s = 0; s < n_seg; ++s) {
                 const StackSeg& sg = sm.seg[s];
                 const int C = sg.C, gs = sg.n_rows > kGroups * C ? 2 : 1;
+                if (C == 1) continue;
 #pragma unroll 1
                 for (int q = sg.idx + grp * C; q * gs < sg.n_rows; q += kGroups * C) {
                     // a row's words: of pair q, word q of its eight rows' block
