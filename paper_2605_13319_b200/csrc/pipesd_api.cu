@@ -494,7 +494,7 @@ int push_inflight(pipesd_ctx* ctx, pipesd_verify_result* dst, std::vector<pipesd
     return PIPESD_OK;
 }
 
-// Rows of the chunk of a prompt of n tokens that follows the first `done`.  Up to 32 tokens are passes of the small-M kernels;
+// Rows of the chunk of a prompt of n tokens that follows the first `done`.  Up to 32 tokens are small passes;
 // more of them go through the dense kernels in chunks of up to row_cap rows, no two of which differ by more than one, so that
 // none is as short as a small-M pass: the last one leaves logits of its last rows only, which the dense kernels alone can do.
 int prompt_chunk(const pipesd_model_cfg& c, const Derived& d, int n, int done) {
@@ -546,14 +546,26 @@ int stack_segments(const pipesd_model_cfg& c, const std::vector<ItemDesc>& items
 }
 
 // Whether a pass is the layer-stack kernel's: up to 32 rows, of requests whose query rows per KV head fit its tensor memory, in a
-// batch whose key ranges fit its tables.  The others (prompts of 19 to 32 tokens at four query heads per KV head, say), and every
-// pass while GEMM launches are timed, run on a kernel per projection, as all did before: us a pass on one box, 7b shape, 9 rows
+// batch whose key ranges fit its tables and are not many and short.  The others (prompts of 19 to 32 tokens at four query heads per KV head,
+// or a request of 4000 keys beside one of 30 at 32 KV heads, say), every pass of a context that shares its device or a part of one, and
+// every pass while GEMM launches are timed, run on a kernel per projection, as all did before: us a pass on one box, 7b shape, 9 rows
 // 3224 -> 2718, 17 rows 3906 -> 3096; 8b shape, 17 rows 5033 -> 3637; 1b shape, 9 rows 1003 -> 801; tiny 116 -> 111.
 bool stack_takes(const pipesd_ctx* ctx, const std::vector<ItemDesc>& items, int M, StackPlan* plan, int* n_max, int* r_max) {
     const pipesd_model_cfg& c = ctx->cfg;
     if (ctx->stack_ctas < 1 || ctx->shared || M > kMaxItemRows || ctx->force_dense || ctx->time_gemms || (int)items.size() > kStackMaxItems) return false;
     int rows = 1;
-    for (const ItemDesc& it : items) rows = std::max(rows, it.rows);
+    long keys = 0;
+    for (const ItemDesc& it : items) {
+        rows = std::max(rows, it.rows);
+        keys += it.base + it.rows;
+    }
+    // Many short (request, KV head) pairs of a small model: a CTA's parts run one after the other, two to three us each, where the attention
+    // kernel has two CTAs per SM, and there is little weight to stream meanwhile.  Time with a kernel per projection over time with
+    // one: 256 pairs of 50 to 400 keys, a layer of 3 to 34 MB 0.88 to 0.93, of 40 to 57 MB 1.05 to 1.12; 192 pairs 0.95 to 1.02; 256
+    // pairs of 500 to 1000 keys 1.01 to 1.10.
+    const long pairs = (long)items.size() * c.n_kv_heads;
+    const double layer_bytes = 2.0 * c.d_model * ((double)ctx->dv.Nqkv + ctx->dv.qd + 3.0 * c.d_ffn);
+    if (10 * pairs > 13 * ctx->stack_most && keys < 400 * (long)items.size() && layer_bytes < 36e6) return false;
     *r_max = rows * (c.n_q_heads / c.n_kv_heads);
     *n_max = (*r_max + 7) / 8 * 8;
     return *n_max <= kStackMaxN && stack_segments(c, items, ctx->stack_ctas) <= kStackMaxSegs && stack_plan(plan, M, c.head_dim, *n_max);

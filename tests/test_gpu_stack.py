@@ -216,6 +216,24 @@ def test_long_request_beside_a_short_one(long, fits):
     ctx.close()
 
 
+@pytest.mark.parametrize("keys, one", [(60, False), (398, True), (700, True)])
+def test_many_short_requests(keys, one):
+    """256 (request, KV head) pairs of a small model: below 400 keys each (the pass's own two among them) a kernel per projection."""
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count > 196:
+        pytest.skip("no more pairs than the device has SMs for")
+    shape, lens, ks = T.scaled(d_model=512, n_q_heads=16, n_kv_heads=16), [keys] * 16, [1] * 16
+    ctx, items, rows = _context(shape, lens, ks)
+    layers = range(shape.n_layers)
+    ctx.profile_enable(True)
+    _, want, want_kv = _run(ctx, items, lens, rows, layers)
+    ctx.profile_enable(False)
+    _, got, got_kv = _run(ctx, items, lens, rows, layers)
+    assert (ctx.profile_read()["kernel_launches"] == 3) == one
+    _close(got, want, got_kv, want_kv)
+    ctx.close()
+
+
 @pytest.mark.parametrize("name", ["one key", "ranges of several tiles", "three requests", "whole and shared row blocks of down"])
 def test_waits_that_run_out(name):
     """So few looks at what other CTAs write that roles give up: the pass ends, the error is reported, and the next pass of the
