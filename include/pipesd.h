@@ -254,8 +254,9 @@ int32_t pipesd_gemm_run(const void *packed, const float *x, float *y, void *scra
                         int32_t K, void *cuda_stream);
 
 /* Harness switch.  Passes of more than 32 rows run their projections on the dense tensor-core kernel, smaller passes
- * in the layer-stack kernel (or, where a request has more than 72 query rows per KV head, on the small-M weight-streaming
- * kernel).  Both of these sum a row in an order that follows the weights' shape (and the number of SMs) alone;
+ * in the layer-stack kernel or, where they are not that kernel's, on the small-M weight-streaming kernel (a request with more
+ * than 72 query rows per KV head; a short request beside a long one at many KV heads; many short requests of a small model; a
+ * device that is shared, or a part of one; GEMM launches that are timed).  Both of these sum a row in an order that follows the weights' shape (and the number of SMs) alone;
  * the dense kernel cuts K into slices by the pass's row count as well, so that a row's projections agree to rounding, not
  * bit for bit, between passes of different row counts (and between the kernels).  on != 0 makes every pass of the context
  * use the dense kernel; on > 1 also gives passes of fewer rows the slices of a pass of `on` rows, so that a request
@@ -272,7 +273,8 @@ int32_t pipesd_debug_gemm_dense(const void *packed, const float *x, float *y, vo
                                 int32_t tokens_per_cta, int32_t slices, void *cuda_stream);
 /* Harness switch: how often (0..65536) a CTA of the attention kernel looks whether the other key splits of its rows are
  * done before it leaves its share of their merge to the last one.  Results do not depend on it, bit for bit: at 0 the last
- * one merges all rows, as it does where other work keeps the splits from running at the same time. */
+ * one merges all rows, as it does where other work keeps the splits from running at the same time.  Passes that the
+ * layer-stack kernel takes do not run that kernel. */
 int32_t pipesd_debug_merge_polls(pipesd_ctx *ctx, int32_t polls);
 /* Harness switch: CTAs of the layer-stack kernel, 1 up to one per SM (0: one per SM, as always otherwise).  Its plans follow their
  * number, as they do on a device of fewer SMs.  PIPESD_E_INVALID beyond that. */

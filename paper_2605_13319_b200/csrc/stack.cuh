@@ -21,8 +21,8 @@
 //
 // Attention.  The keys of all (request, KV head) pairs form one line, cut into equal ranges, one per CTA; a range's parts
 // (segments) run through the algorithm of attention.cuh (keys on the M side; S^T, O^T and denominators in tensor memory;
-// exponentials relative to the segment's first key), K/V from the same copy stream, Q already in operand order.  Partial
-// results are exchanged like partial sums, each contributor merges every C-th row.
+// exponentials relative to the segment's first key), K/V from the same copy stream, Q already in operand order.  A head whose keys are
+// one CTA's is finished there; of others, partial results are exchanged like partial sums, each contributor merges every C-th row.
 //
 // What a phase costs beyond its stream (7b shape, 9 rows, us): look 0.5, activations 0.8, exchange and epilogue 2, release 1; the
 // attention 12.  Every phase runs code that the one before it did not, so the hot paths are kept short and rolled: code that
@@ -225,14 +225,8 @@ __device__ __forceinline__ bool stack_arrived(const unsigned* ctr, unsigned targ
 }
 // Orders what this thread has seen of other CTAs' ordinary stores before its later copies from global memory.
 __device__ __forceinline__ void fence_proxy_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
-// Exchange words: three values and the phase number that vouches for them, 16 bytes written and read as one.
-__device__ __forceinline__ void ll_store(uint4* p, float x, float y, float z, unsigned epoch) {
-    asm volatile("{\n .reg .b64 l, h;\n .reg .b128 w;\n mov.b64 l, {%1, %2};\n mov.b64 h, {%3, %4};\n mov.b128 w, {l, h};\n st.relaxed.gpu.global.b128 [%0], w;\n}" ::"l"(p),
-                 "r"(__float_as_uint(x)), "r"(__float_as_uint(y)), "r"(__float_as_uint(z)), "r"(epoch)
-                 : "memory");
-}
-// The same, and ordinary accesses, where a condition holds, without a branch: a point that lanes meet again at costs more than
-// the access.
+// Exchange words: three values and the phase number that vouches for them, 16 bytes written and read as one.  These, and ordinary
+// accesses, where a condition holds, without a branch: a point that lanes meet again at costs more than the access.
 __device__ __forceinline__ void ll_store_if(bool c, uint4* p, float x, float y, float z, unsigned epoch) {
     asm volatile("{\n .reg .pred q;\n .reg .b64 l, h;\n .reg .b128 w;\n setp.ne.u32 q, %5, 0;\n mov.b64 l, {%1, %2};\n mov.b64 h, {%3, %4};\n mov.b128 w, {l, h};\n"
                  " @q st.relaxed.gpu.global.b128 [%0], w;\n}" ::"l"(p), "r"(__float_as_uint(x)), "r"(__float_as_uint(y)), "r"(__float_as_uint(z)), "r"(epoch), "r"((uint32_t)c)
@@ -461,7 +455,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                                      (uint32_t)(jp - js) * (HD * 2), smem_u32(&sm.full_w[r.slot]));
                         if (kv == 1 || kPerTile == 2) {
                             ++issued;
-                                        r.step(a.slots);
+                            r.step(a.slots);
                         }
                     }
                 }
