@@ -1453,7 +1453,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                     }
 #pragma unroll 1
                     for (int z = 0; z < gs && r + z < sg.n_rows; ++z) {
-                        act_put(true, a.act_attn, sg.row0 + (r + z) / G, (sg.kvh * G + (r + z) % G) * HD + dim, num[0] / den[0]);
+                    act_put(true, a.act_attn, sg.row0 + (r + z) / G, (sg.kvh * G + (r + z) % G) * HD + dim, num[0] * (1.f / den[0]));
                         num[0] = num[1];
                         den[0] = den[1];
                     }
