@@ -1335,8 +1335,8 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                     rv.skip(kPerTile, a.slots);
                 }
                 // ---- the result of this range: thread = head dimension of O^T; the denominators are the same in lanes 0-7 of L.  A head
-                // whose keys are all here is finished, by division; of others, the contributors exchange partial results.  (Through the
-                // exchange, a head of one's own took its CTA a trip to the L2 per eight rows, four at 128 dimensions: prompts of 24 to
+                // whose keys are all here is finished; of others, the contributors exchange partial results.  (The reciprocal, as in the
+                // merges, rounds 2^-24 of the value; the terms that are stored keep 2^-17.  Through the exchange, a head of one's own took its CTA a trip to the L2 per eight rows, four at 128 dimensions: prompts of 24 to
                 // 32 tokens at d_model 512 to 1024 were up to 13 % slower than with a kernel per projection.)
                 product_done(tile - 1u);
                 tc_fence_after();
@@ -1372,7 +1372,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
 #pragma unroll 1
                         for (int i = 0; i < min(n, 8); ++i) {
                             const int r = cb * 8 + i;
-                            act_put(true, a.act_attn, sg.row0 + r / G, (sg.kvh * G + r % G) * HD + kt, o[0] / wm[r]);
+                            act_put(true, a.act_attn, sg.row0 + r / G, (sg.kvh * G + r % G) * HD + kt, o[0] * (1.f / wm[r]));
 #pragma unroll
                             for (int k = 0; k < 7; ++k) o[k] = o[k + 1];
                         }
@@ -1453,7 +1453,7 @@ __global__ void __launch_bounds__(kStackThreads, 1) layer_stack_kernel(const __g
                     }
 #pragma unroll 1
                     for (int z = 0; z < gs && r + z < sg.n_rows; ++z) {
-                    act_put(true, a.act_attn, sg.row0 + (r + z) / G, (sg.kvh * G + (r + z) % G) * HD + dim, num[0] * (1.f / den[0]));
+                        act_put(true, a.act_attn, sg.row0 + (r + z) / G, (sg.kvh * G + (r + z) % G) * HD + dim, num[0] * (1.f / den[0]));
                         num[0] = num[1];
                         den[0] = den[1];
                     }
