@@ -35,6 +35,10 @@ CASES = {
     "whole and shared row blocks of QKV, 32 rows": (T.scaled(d_model=80, n_q_heads=8, n_kv_heads=4), [300], [31], 16),
     "whole and shared row blocks of down": (T.scaled(d_ffn=96), [40], [1], 16),
     "whole and shared row blocks of down, 32 rows": (T.scaled(d_model=1024, d_ffn=80), [300], [31], 16),
+    # heads whose keys are one CTA's: finished from tensor memory
+    "a head of one's own, 72 rows": (T.scaled(n_q_heads=8, n_kv_heads=1, head_dim=128, d_model=1024), [40], [8], 16),
+    "heads of one's own, 25 rows": (T.scaled(d_model=512, n_q_heads=4, n_kv_heads=4, head_dim=128), [20], [24], 16),
+    "heads of one's own, 7 and 21 rows": (T.scaled(n_q_heads=6, n_kv_heads=2), [30, 5], [6, 20], 8),
 }
 
 
